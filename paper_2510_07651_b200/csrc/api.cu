@@ -74,6 +74,7 @@ obc_status resolve_score(const obc_score_params* p, ScoreShape* s) {
 // launch agree.  The dtype is not known to the size query, so the workspace covers both.
 bool want_tc(const obc_score_params* p, const ScoreShape& s, int dtype, const TensorView& q) {
     if (p->path == OBC_PATH_SIMT) return false;
+    if (p->path == OBC_PATH_TC && s.R < 64) return false;          // the explicit choice keeps its stated minimum
     return tc_supported(s, dtype, q);
 }
 
@@ -90,7 +91,7 @@ obc_status obc_score_workspace(const obc_score_params* p, size_t* bytes) {
     obc_status st = resolve_score(p, &s);
     if (st != OBC_OK) return st;
     size_t need = make_simt_plan(s, s.R, false).bytes;
-    if (p->path != OBC_PATH_SIMT && tc_shape_supported(s)) {
+    if (p->path != OBC_PATH_SIMT) {
         size_t t = tc_workspace_bytes(s);
         if (t > need) need = t;
     }

@@ -53,11 +53,11 @@ struct SimtPlan {
     int tiles_per_split;
     int tile_tokens;                     // tokens per tile of the pass-1 kernel the plan is for
     int rows_out;                        // rows per unit in the combined arrays (R, or R padded)
-    int want_obf;                        // also write the bf16 copy of -2*O (tensor-core pass 2)
+    int want_obf;                        // also write the bf16 copy of -2*O (tensor-core pass 2); 2: as a high and a low part
     size_t off_flag;                             // 256-byte header: device status word, kernel spans at kSpanOffset
     size_t off_part_m, off_part_l, off_part_o;   // partial softmax stats / outputs per split
     size_t off_lse2, off_onorm, off_o;           // combined: log2-sum-exp, ||o||^2, O (fp32)
-    size_t off_obf;                              // bf16 [units][rows_out][d] = -2 * O
+    size_t off_obf;                              // bf16 [units][want_obf][rows_out][d] = -2 * O (high part, low part)
     size_t off_cpair;                            // float4 per row pair: (-lse2_0, -lse2_1, |o_0|^2, |o_1|^2)
     size_t off_nv;                               // fp32 [units][Nmax]: ||v_p||^2 (written by tensor-core pass 1)
     size_t bytes;
@@ -126,8 +126,7 @@ obc_status launch_decode(const DecodeShape& s, TensorView q, TensorView kt, Tens
                          int step_pos, void* ws, cudaStream_t stream);
 
 // ---- tensor-core (tcgen05) score path -----------------------------------------------------------
-bool tc_shape_supported(const ScoreShape& s);                       // R large enough for the MMA tiles
-bool tc_supported(const ScoreShape& s, int dtype, const TensorView& q);   // + bf16, uniformly strided Q rows
+bool tc_supported(const ScoreShape& s, int dtype, const TensorView& q);   // bf16, uniformly strided Q rows
 size_t tc_workspace_bytes(const ScoreShape& s);
 obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, TensorView v,
                            float* scores, void* ws, cudaStream_t stream, const GivenAttention* given = nullptr,

@@ -187,6 +187,14 @@ __device__ __forceinline__ int active_splits(const SimtPlan& plan, int N) {
     const int tiles = (N + plan.tile_tokens - 1) / plan.tile_tokens;
     return min(plan.n_splits, (tiles + plan.tiles_per_split - 1) / plan.tiles_per_split);
 }
+// -2 O in bf16, row `r` of a unit; with plan.want_obf == 2 as a high part and, rows_out rows further, what it leaves out
+__device__ __forceinline__ void store_obf(const SimtPlan& plan, float* ws, int unit, int r, int c, float o) {
+    __nv_bfloat16* at = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + plan.off_obf) +
+                        ((size_t)unit * plan.rows_out * plan.want_obf + r) * kD + c;
+    const __nv_bfloat16 hi = __float2bfloat16(-2.f * o);
+    *at = hi;
+    if (plan.want_obf == 2) at[(size_t)plan.rows_out * kD] = __float2bfloat16(fmaf(-2.f, o, -__bfloat162float(hi)));
+}
 constexpr int CMB_INFLIGHT = 10;                       // float4 loads in flight per thread
 
 __device__ __forceinline__ float block128_reduce(float x, bool take_max, float* red) {
@@ -203,11 +211,10 @@ simt_combine_kernel(ScoreShape s, SimtPlan plan, float* ws) {
     const int r = blockIdx.x % plan.rows_out, unit = blockIdx.x / plan.rows_out;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t orow = (size_t)unit * plan.rows_out + r;
-    __nv_bfloat16* obf = plan.want_obf ? reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + plan.off_obf) : nullptr;
     float* cpair = plan.want_obf ? ws + plan.off_cpair / 4 + (orow >> 1) * 4 + (orow & 1) : nullptr;
     if (r >= s.R) {
         (ws + plan.off_o / 4)[orow * kD + tid] = 0.f;
-        if (obf) obf[orow * kD + tid] = __float2bfloat16(0.f);
+        if (plan.want_obf) store_obf(plan, ws, unit, r, tid, 0.f);
         if (tid == 0) {
             (ws + plan.off_lse2 / 4)[orow] = INFINITY; (ws + plan.off_onorm / 4)[orow] = 0.f;
             if (cpair) { cpair[0] = -INFINITY; cpair[2] = 0.f; }
@@ -265,7 +272,7 @@ simt_combine_kernel(ScoreShape s, SimtPlan plan, float* ws) {
     const float oc = L > 0.f ? ((sAcc[0][tid] + sAcc[1][tid]) + (sAcc[2][tid] + sAcc[3][tid])) / L : 0.f;
     const float onorm = block128_reduce(oc * oc, false, red);
     (ws + plan.off_o / 4)[orow * kD + tid] = oc;
-    if (obf) obf[orow * kD + tid] = __float2bfloat16(-2.f * oc);
+    if (plan.want_obf) store_obf(plan, ws, unit, r, tid, oc);
     if (tid == 0) {
         const float lse2 = Mrun + log2f(L);
         (ws + plan.off_lse2 / 4)[orow] = lse2;
@@ -287,7 +294,6 @@ simt_combine_rows_kernel(ScoreShape s, SimtPlan plan, float* ws) {
     const long long orow = (long long)blockIdx.x * (CMB_NT / 32) + (threadIdx.x >> 5);
     if (orow >= rows_total) return;
     const int r = (int)(orow % plan.rows_out), unit = (int)(orow / plan.rows_out);
-    __nv_bfloat16* obf = plan.want_obf ? reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + plan.off_obf) : nullptr;
     float* cpair = plan.want_obf ? ws + plan.off_cpair / 4 + (orow >> 1) * 4 + (orow & 1) : nullptr;
     float4 oc = make_float4(0.f, 0.f, 0.f, 0.f);
     float lse2 = INFINITY, onorm = 0.f;                    // padding rows weigh 0
@@ -335,10 +341,18 @@ simt_combine_rows_kernel(ScoreShape s, SimtPlan plan, float* ws) {
         lse2 = M + log2f(L);
     }
     *reinterpret_cast<float4*>(ws + plan.off_o / 4 + orow * kD + lane * 4) = oc;
-    if (obf) {
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(-2.f * oc.x, -2.f * oc.y), hi = __floats2bfloat162_rn(-2.f * oc.z, -2.f * oc.w);
-        *reinterpret_cast<uint2*>(obf + orow * kD + lane * 4) =
-            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    if (plan.want_obf) {
+        __nv_bfloat16* at = reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + plan.off_obf) +
+                            ((size_t)unit * plan.rows_out * plan.want_obf + r) * kD + lane * 4;
+        const __nv_bfloat162 a = __floats2bfloat162_rn(-2.f * oc.x, -2.f * oc.y), b = __floats2bfloat162_rn(-2.f * oc.z, -2.f * oc.w);
+        *reinterpret_cast<uint2*>(at) = make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+        if (plan.want_obf == 2) {                          // what the high part leaves out
+            const float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
+            const __nv_bfloat162 la = __floats2bfloat162_rn(fmaf(-2.f, oc.x, -fa.x), fmaf(-2.f, oc.y, -fa.y));
+            const __nv_bfloat162 lb = __floats2bfloat162_rn(fmaf(-2.f, oc.z, -fb.x), fmaf(-2.f, oc.w, -fb.y));
+            *reinterpret_cast<uint2*>(at + (size_t)plan.rows_out * kD) =
+                make_uint2(*reinterpret_cast<const uint32_t*>(&la), *reinterpret_cast<const uint32_t*>(&lb));
+        }
     }
     if (lane == 0) {
         (ws + plan.off_lse2 / 4)[orow] = lse2;
@@ -359,7 +373,6 @@ given_prep_kernel(ScoreShape s, SimtPlan plan, TensorView o, const float* lse, f
     const int r = blockIdx.x % plan.rows_out, unit = blockIdx.x / plan.rows_out;
     const int tid = threadIdx.x;
     const size_t orow = (size_t)unit * plan.rows_out + r;
-    __nv_bfloat16* obf = plan.want_obf ? reinterpret_cast<__nv_bfloat16*>(reinterpret_cast<char*>(ws) + plan.off_obf) : nullptr;
     float* cpair = plan.want_obf ? ws + plan.off_cpair / 4 + (orow >> 1) * 4 + (orow & 1) : nullptr;
     __shared__ float red[4];
     float oc = 0.f, lse2 = INFINITY;             // padding rows weigh 0
@@ -370,7 +383,7 @@ given_prep_kernel(ScoreShape s, SimtPlan plan, TensorView o, const float* lse, f
     }
     const float onorm = block128_reduce(oc * oc, false, red);
     (ws + plan.off_o / 4)[orow * kD + tid] = oc;
-    if (obf) obf[orow * kD + tid] = __float2bfloat16(-2.f * oc);
+    if (plan.want_obf) store_obf(plan, ws, unit, r, tid, oc);
     if (tid == 0) {
         (ws + plan.off_lse2 / 4)[orow] = lse2;
         (ws + plan.off_onorm / 4)[orow] = onorm;

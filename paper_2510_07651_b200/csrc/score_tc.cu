@@ -351,14 +351,21 @@ __device__ __forceinline__ void score_rows16(const uint32_t (&zr)[16], const uin
 // One (tile, chunk) item of one token: all rows of the chunk, one batch of 16 rows in registers at a time.  (Loading
 // the next batch ahead of the math, which doubles the registers, was slower in both kernels: the other epilogue
 // warps of the SM sub-partition cover the wait for a batch.)
-template <unsigned VARS, bool MASKED>
+// HILO: the columns of T' come twice, `lo` columns apart (from the high and from the low part of -2 O): their sum is T'.
+template <unsigned VARS, bool MASKED, bool HILO = false>
 __device__ __forceinline__ void score_chunk(uint32_t zt, uint32_t tt, int chunk_rows, const float4* cst,
-                                                 float2 sl2, float2 sc, RowSums& S, int ptok, int mask_base, int W, int wi) {
+                                                 float2 sl2, float2 sc, RowSums& S, int ptok, int mask_base, int W, int wi, int lo = 0) {
     uint32_t z0[16], t0[16];
 #pragma unroll 1
     for (int c0 = 0; c0 < chunk_rows; c0 += 16) {
-        tc_ld16(zt + c0, z0);
         tc_ld16(tt + c0, t0);
+        if (HILO) {
+            tc_ld16(tt + lo + c0, z0);
+            tc_wait_ld16x2(z0, t0);
+#pragma unroll
+            for (int i = 0; i < 16; ++i) t0[i] = __float_as_uint(__uint_as_float(t0[i]) + __uint_as_float(z0[i]));
+        }
+        tc_ld16(zt + c0, z0);
         tc_wait_ld16x2(z0, t0);
         score_rows16<VARS, MASKED>(z0, t0, cst + (c0 >> 1), sl2, sc, S, ptok, mask_base, W, wi);
     }
@@ -366,7 +373,10 @@ __device__ __forceinline__ void score_chunk(uint32_t zt, uint32_t tt, int chunk_
 
 // VARS: variants this instantiation computes (a superset of p.variants).  OWN_NV: no pass 1 ran (the
 // caller supplied the attention outputs), so warps 2-3 compute the value norms from the V tiles here.
-template <unsigned VARS, bool OWN_NV>
+// HILO: fewer than 64 window rows.  Such a call is summed in 32 bits throughout: -2 O enters as the sum of two bf16
+// parts, which stand side by side on the MMA's N dimension (at most 2 x 64 rows) and meet in the epilogue.  The
+// kernel stays bound by the K/V tiles it streams, with half of the epilogue's rows idle.
+template <unsigned VARS, bool OWN_NV, bool HILO>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
                 const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -407,7 +417,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
     bool failed = false;
     int fail_site = 0;                             // source line of the wait that gave up (status word)
-    const uint32_t qo_bytes = (uint32_t)p.chunk_rows * 128u * 2u * 2u;   // Q and O chunks, two halves each
+    const uint32_t qo_bytes = (uint32_t)p.chunk_rows * 256u * (HILO ? 3u : 2u);   // Q and O chunks, two halves each (O: high and low part)
 
     // Every role walks the same tiles (TileWalk); all window rows of a unit (at most 128) are one chunk.
     // Tiles go to the two epilogue groups alternately.  What an epilogue group waits for (accumulators
@@ -449,7 +459,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     if (!mbar_wait(bar(BAR_QO_EMPTY), (qo_loads & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
                     mbar_expect_tx(bar(BAR_QO_FULL), qo_bytes);
                     const int qrow = (b * p.Hkv * p.G + g * p.G) * p.W;
-                    const int orow = unit * p.rows_out;
+                    const int orow = unit * p.rows_out * (HILO ? 2 : 1);
                     tma_load_2d(sbase + OFF_Q, &map_q, bar(BAR_QO_FULL), 0, qrow);
                     tma_load_2d(sbase + OFF_Q + kHalfBytes, &map_q, bar(BAR_QO_FULL), 64, qrow);
                     tma_load_2d(sbase + OFF_O, &map_o, bar(BAR_QO_FULL), 0, orow);
@@ -468,7 +478,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     } else if (warp == 1) {
         // ===================================== MMA issuer =======================================
         if (lane == 0) {
-            const uint32_t idesc = idesc_bf16(p.chunk_rows);
+            const uint32_t idesc = idesc_bf16(p.chunk_rows), idesc_t = idesc_bf16(HILO ? 2 * p.chunk_rows : p.chunk_rows);
             uint32_t item = 0, qo_loads = 0, tile_seq = 0;
             int qo_unit = -1;
             for (; !tw.done() && !failed; tw.next(), ++tile_seq) {
@@ -491,7 +501,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     tc_mma(zt, desc_make(ak + desc_kstep(ks, kHalfBytes)), desc_make(bq + desc_kstep(ks, kHalfBytes)), idesc, ks > 0);
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
-                    tc_mma(tt, desc_make(av + desc_kstep(ks, kHalfBytes)), desc_make(bo + desc_kstep(ks, kHalfBytes)), idesc, ks > 0);
+                    tc_mma(tt, desc_make(av + desc_kstep(ks, kHalfBytes)), desc_make(bo + desc_kstep(ks, kHalfBytes)), idesc_t, ks > 0);
                 tc_commit(bar(BAR_TM_FULL + owner * 2 + buf)); // accumulators ready for the tile's epilogue group
                 tc_commit(bar(BAR_EMPTY + st));                // K/V stage no longer read by the MMA
                 // Q / O may be overwritten once these MMAs are done, if the next item needs others
@@ -578,9 +588,9 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const uint32_t zt = tmem_base + ((uint32_t)(lane_grp * 32) << 16) + buf * 256u + (uint32_t)r_begin, tt = zt + 128u;
             if (r_count > 0) {
                 if (masked_tile)
-                    score_chunk<VARS, true>(zt, tt, r_count, cst, sl2, sc, S, ptok, Nm - p.W, p.W, r_begin % p.W);
+                    score_chunk<VARS, true, HILO>(zt, tt, r_count, cst, sl2, sc, S, ptok, Nm - p.W, p.W, r_begin % p.W, p.chunk_rows);
                 else
-                    score_chunk<VARS, false>(zt, tt, r_count, cst, sl2, sc, S, ptok, 0, 0, 0);
+                    score_chunk<VARS, false, HILO>(zt, tt, r_count, cst, sl2, sc, S, ptok, 0, 0, 0, p.chunk_rows);
             }
             tc_fence_before();
             __syncwarp();
@@ -1090,6 +1100,8 @@ __device__ __forceinline__ void p1_chunk_of_block(const P1Params& p, int vu, int
     c = p.n_chunks - 1 - vu % p.n_chunks;
 }
 
+// HILO: fewer than 64 window rows; MMA rows 64.. repeat rows 0.. and carry the low part of P
+template <bool HILO>
 __global__ void __launch_bounds__(kThreadsP1, 1)
 tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ P1Params p) {
@@ -1144,10 +1156,14 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     } else if (warp == 0) {
         // ===================================== TMA producer =====================================
         if (lane == 0 && n_tiles > 0) {
-            mbar_expect_tx(bar(P1_QFULL), (uint32_t)p.chunk_rows * 256u);
+            mbar_expect_tx(bar(P1_QFULL), (uint32_t)p.chunk_rows * (HILO ? 512u : 256u));
             const int qrow = (b * p.Hq + g * p.G) * p.W + c * p.chunk_rows;
             tma_load_2d(sbase + P1_OFF_Q, &map_q, bar(P1_QFULL), 0, qrow);
             tma_load_2d(sbase + P1_OFF_Q + kHalfBytes, &map_q, bar(P1_QFULL), 64, qrow);
+            if (HILO) {
+                tma_load_2d(sbase + P1_OFF_Q + kHalfBytes / 2, &map_q, bar(P1_QFULL), 0, qrow);
+                tma_load_2d(sbase + P1_OFF_Q + kHalfBytes + kHalfBytes / 2, &map_q, bar(P1_QFULL), 64, qrow);
+            }
             int issued = 0;
             const uint64_t pol_stream = l2_policy_evict_first();
             for (int i = 0; i < n_tiles; ++i) {
@@ -1250,8 +1266,10 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const int lane_grp = warp & 3;
         const int row = lane_grp * 32 + lane;                                // row within the chunk
         const int rows_valid = min(p.chunk_rows, p.R - c * p.chunk_rows);
-        const int r = c * p.chunk_rows + row;
-        const bool valid = row < rows_valid;
+        const bool low_part = HILO && lane_grp >= 2;                       // this warp's rows are the second copies of rows 0..63
+        const int row_q = HILO ? row & 63 : row;
+        const int r = c * p.chunk_rows + row_q;
+        const bool valid = row_q < rows_valid;
         const int last = valid ? (p.causal ? min(Nm - p.W + (r % p.W), N - 1) : N - 1) : -1;   // last visible token
         const int first_masked = min(p.causal ? Nm - p.W + 1 : N, N);        // tiles reaching it need the mask
         const float sl2 = p.scale * kLog2e;
@@ -1330,6 +1348,10 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                         const float2 e = make_float2(fast_exp2(x.x), fast_exp2(x.y));
                         lsum = __fadd2_rn(lsum, e);
                         pk[j >> 1] = pack_bf16x2(e.x, e.y);
+                        if (low_part) {                                      // P = bf16(P) + bf16(P - bf16(P)): the second term
+                            const float2 h = bf16x2_to_f32x2(pk[j >> 1]);
+                            pk[j >> 1] = pack_bf16x2(e.x - h.x, e.y - h.y);
+                        }
                     }
                     tc_st16(tS + pc * 16, pk);
                 };
@@ -1389,7 +1411,7 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const float o_scale = fin ? (Lrow > 0.f ? 1.f / Lrow : 0.f) : 1.f;
             const float g0 = f0 * o_scale, g1 = f1 * o_scale;
             float sq = 0.f;                                                  // squared norm of this thread's 64 output columns
-            if (w == 0 && valid && !fin) { p.part_m[prow0 + row] = M; p.part_l[prow0 + row] = Lrow; }
+            if (w == 0 && valid && !fin && !low_part) { p.part_m[prow0 + row] = M; p.part_l[prow0 + row] = Lrow; }
 #pragma unroll 1
             for (int q = 0; q < 2; ++q) {
                 // CTA-uniform: warpgroup 0 owns tiles iff the split has any, warpgroup 1 iff it has two or more
@@ -1425,6 +1447,15 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             for (int rr = 0; rr < 16; ++rr) {
                 const int orow = row_lo + rr;
                 rowv[rr] = *reinterpret_cast<const uint4*>(xo + orow * 512 + ((lane ^ (orow & 31)) << 4));
+            }
+            if (HILO) {                                                    // rows 64.. hold what the low part of P added to rows 0..
+#pragma unroll
+                for (int rr = 0; rr < 16; ++rr) {
+                    const int orow = (row_lo + rr) | 64;
+                    const float4 lo = *reinterpret_cast<const float4*>(xo + orow * 512 + ((lane ^ (orow & 31)) << 4));
+                    rowv[rr] = make_uint4(__float_as_uint(__uint_as_float(rowv[rr].x) + lo.x), __float_as_uint(__uint_as_float(rowv[rr].y) + lo.y),
+                                          __float_as_uint(__uint_as_float(rowv[rr].z) + lo.z), __float_as_uint(__uint_as_float(rowv[rr].w) + lo.w));
+                }
             }
             if (fin) {
                 // rows of the unit are rows of the outputs (one split, no padding rows): O, -2 O in bf16, and per row
@@ -1502,10 +1533,14 @@ int sm_count() {
 
 }  // namespace
 
-bool tc_shape_supported(const ScoreShape& s) { return s.R >= 64; }
+// Fewer than 64 window rows fill half of the MMA's M dimension at most.  Pass 1 then runs every row twice, the second
+// copy with the low part of P, and pass 2 takes -2 O as two parts on its N dimension, so that such a call keeps the 32-bit
+// sums of the CUDA-core kernels at the tensor cores' rate (32 heads x 8191 tokens x 32 rows: one score call 489 us on CUDA cores, 63 us here, of which K and V twice
+// through HBM are 41; 8 heads x 2547 tokens x 32 rows: 87 against 26 us).
+static bool tc_hilo(const ScoreShape& s) { return s.R < 64; }
 
 bool tc_supported(const ScoreShape& s, int dtype, const TensorView& q) {
-    if (dtype != OBC_BF16 || !tc_shape_supported(s)) return false;
+    if (dtype != OBC_BF16) return false;
     // the window rows of a KV head's group must be one uniformly strided run of rows
     return q.sh == (long long)s.W * q.st && q.sb == (long long)s.Hq * q.sh;
 }
@@ -1540,7 +1575,7 @@ static SimtPlan make_tc_plan(const ScoreShape& s) {
     p.n_splits = (tiles + p.tiles_per_split - 1) / p.tiles_per_split;          // CTAs, and partial results, per unit
     p.tile_tokens = TILE;
     p.rows_out = ch.rows_out;
-    p.want_obf = 1;
+    p.want_obf = tc_hilo(s) ? 2 : 1;
     const size_t rows = (size_t)units * s.R, prow = rows * p.n_splits, orow = (size_t)units * ch.rows_out;
     size_t off = 0;
     p.off_flag = off;   off = 256;
@@ -1550,7 +1585,7 @@ static SimtPlan make_tc_plan(const ScoreShape& s) {
     p.off_lse2 = off;   off = align_up(off + orow * 4, 256);
     p.off_onorm = off;  off = align_up(off + orow * 4, 256);
     p.off_o = off;      off = align_up(off + orow * kD * 4, 256);
-    p.off_obf = off;    off = align_up(off + orow * kD * 2, 1024);
+    p.off_obf = off;    off = align_up(off + orow * kD * 2 * p.want_obf, 1024);
     p.off_cpair = off;  off = align_up(off + orow * 8, 256);
     p.off_nv = off;     off = align_up(off + (size_t)units * s.Nmax * 4, 256);
     p.bytes = off;
@@ -1577,11 +1612,12 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     const SimtPlan plan = make_tc_plan(s);
     char* wsb = (char*)ws;
     const int units = s.B * s.Hkv;
+    const bool hilo = tc_hilo(s);
     CUtensorMap mq, mo, mk, mv;
     {
         const uint64_t qd[2] = {(uint64_t)kD, (uint64_t)s.B * s.Hq * s.W};
         const uint64_t qs[1] = {(uint64_t)q.st * 2};
-        const uint64_t od[2] = {(uint64_t)kD, (uint64_t)units * ch.rows_out};
+        const uint64_t od[2] = {(uint64_t)kD, (uint64_t)units * ch.rows_out * plan.want_obf};
         const uint64_t os[1] = {(uint64_t)kD * 2};
         const uint64_t kd[4] = {(uint64_t)kD, (uint64_t)s.Nmax, (uint64_t)s.Hkv, (uint64_t)s.B};
         const uint64_t ks[3] = {(uint64_t)k.st * 2, (uint64_t)(s.Hkv > 1 ? k.sh : k.st * s.Nmax) * 2,
@@ -1589,7 +1625,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         const uint64_t vs[3] = {(uint64_t)v.st * 2, (uint64_t)(s.Hkv > 1 ? v.sh : v.st * s.Nmax) * 2,
                                 (uint64_t)(s.B > 1 ? v.sb : (s.Hkv > 1 ? v.sh * s.Hkv : v.st * s.Nmax)) * 2};
         if (!make_map(&mq, q.ptr, 2, qd, qs, (uint32_t)ch.chunk_rows) ||
-            !make_map(&mo, wsb + plan.off_obf, 2, od, os, (uint32_t)ch.chunk_rows) ||
+            !make_map(&mo, wsb + plan.off_obf, 2, od, os, (uint32_t)(ch.chunk_rows * plan.want_obf)) ||
             !make_map(&mk, k.ptr, 4, kd, ks, TILE) || !make_map(&mv, v.ptr, 4, kd, vs, TILE)) {
             set_last_cuda_error((int)cudaErrorInvalidValue);
             return OBC_ERR_CUDA;
@@ -1618,15 +1654,17 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         p1.status = (unsigned int*)(wsb + plan.off_flag);
         p1.span = (unsigned long long*)(wsb + plan.off_flag + kSpanOffset);
         // with one CTA per (unit, row chunk) and no padding rows there is nothing to merge: pass 1 writes the results itself
-        const bool direct = plan.n_splits == 1 && ch.rows_out == s.R;
+        // (two MMA rows per window row still have to be added up)
+        const bool direct = plan.n_splits == 1 && ch.rows_out == s.R && !hilo;
         if (direct) {
             p1.out_o = (float*)(wsb + plan.off_o); p1.out_obf = (__nv_bfloat16*)(wsb + plan.off_obf);
             p1.out_lse2 = (float*)(wsb + plan.off_lse2); p1.out_onorm = (float*)(wsb + plan.off_onorm);
             p1.out_cpair = (float*)(wsb + plan.off_cpair);
         }
-        OBC_CUDA_TRY(cudaFuncSetAttribute(tc_pass1_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemP1));
+        const auto pass1 = hilo ? tc_pass1_kernel<true> : tc_pass1_kernel<false>;
+        OBC_CUDA_TRY(cudaFuncSetAttribute(pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemP1));
         { ProfScope ps("tc_pass1", stream);
-          OBC_CUDA_TRY(launch_pdl(tc_pass1_kernel, dim3(plan.n_splits, units * ch.n_chunks), dim3(kThreadsP1), kSmemP1, stream, 1, mq, mk, mv, p1)); }
+          OBC_CUDA_TRY(launch_pdl(pass1, dim3(plan.n_splits, units * ch.n_chunks), dim3(kThreadsP1), kSmemP1, stream, 1, mq, mk, mv, p1)); }
         if (!direct) {
             obc_status st = launch_combine(s, plan, ws, stream);
             if (st != OBC_OK) return st;
@@ -1688,16 +1726,16 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         { ProfScope ps("tc_pass2", stream); OBC_CUDA_TRY(launch_pdl(kernel, dim3(grid), dim3(kThreads), kSmemBytes, stream, 1, mq, mo, mk, mv, p)); }
         return OBC_OK;
     };
-    if (given) {
-        if (s.variants == OBC_VAR_VK) return launch(tc_pass2_kernel<OBC_VAR_VK, true>);
-        if (s.variants == (OBC_VAR_K | OBC_VAR_VK)) return launch(tc_pass2_kernel<OBC_VAR_K | OBC_VAR_VK, true>);
-        return launch(tc_pass2_kernel<kAllVariants, true>);
+    // pass 1 leaves only ||v||^2; without it, and for the l1 variant, the norms come from the V tiles in pass 2
+    const bool own_nv = given || (s.variants & OBC_VAR_VATP);
+    if (hilo) {
+        if (s.variants == OBC_VAR_VK) return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, true>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, true>);
+        return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, true>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, true>);
     }
-    if (s.variants == OBC_VAR_VK) return launch(tc_pass2_kernel<OBC_VAR_VK, false>);
-    if (s.variants == (OBC_VAR_K | OBC_VAR_VK)) return launch(tc_pass2_kernel<OBC_VAR_K | OBC_VAR_VK, false>);
-    // pass 1 leaves only ||v||^2; the l1 variant takes both norms from the V tiles in pass 2
-    if (s.variants & OBC_VAR_VATP) return launch(tc_pass2_kernel<kAllVariants, true>);
-    return launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false>);
+    if (s.variants == OBC_VAR_VK) return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, false>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, false>);
+    if (s.variants == (OBC_VAR_K | OBC_VAR_VK))
+        return own_nv ? launch(tc_pass2_kernel<OBC_VAR_K | OBC_VAR_VK, true, false>) : launch(tc_pass2_kernel<OBC_VAR_K | OBC_VAR_VK, false, false>);
+    return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, false>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, false>);
 }
 
 }  // namespace obc

@@ -79,6 +79,27 @@ def test_tensor_core_row_counts(N, W, Hq, Hkv):
     _check(case, ["V", "K", "VK", "ATTN", "VATP"], path="tc", tight=2e-2)
 
 
+@pytest.mark.parametrize("N,W,Hq,Hkv", [
+    (1, 1, 2, 2),            # one token, one row: 15 padding rows in the chunk of 16
+    (127, 1, 7, 1),          # just under one tile
+    (128, 16, 1, 1),         # one whole tile, a chunk without padding
+    (129, 17, 1, 1),         # one token in the last tile, chunk of 32
+    (3001, 32, 4, 4),        # several tiles per split, no groups
+    (1500, 12, 12, 3),       # R = 48: the row halves of pass 2 are 32 and 16
+    (700, 63, 1, 1),         # R = 63: the largest row count of this path, one padding row
+])
+def test_fewer_than_64_window_rows(N, W, Hq, Hkv):
+    """bf16 caches with fewer than 64 window rows: attention weights and outputs travel as two bf16 parts, so the scores
+    agree with the double-precision ones as 32-bit sums do.  Bound: the parts leave out 2^-17 of a weight or of an output,
+    and 128-term and N-term fp32 sums add a few 2^-24 each; 1e-5 of the largest score covers both with a margin of four."""
+    case = synth.make_prefill("fewrows", B=2, Hq=Hq, Hkv=Hkv, d=128, W=W, N=[N, max(W, N - 40)], dtype="bf16", seed=31 + N, hh_frac=0.02)
+    for variants in (["VK"], ["V", "K", "VK", "ATTN"], ["V", "K", "VK", "ATTN", "VATP"]):
+        want, got = H.oracle_scores(case, variants), H.gpu_scores(case, variants)
+        mx = max(np.abs(want[n]).max() for n in variants if n in ("V", "K", "VK"))
+        for n in variants:
+            H.assert_scores_close(got[n], want[n], "f32", what=f"{case.name}/{n}", mx=None if n in ("ATTN", "VATP") else mx)
+
+
 @pytest.mark.parametrize("N,Hq,Hkv,dtype,path", [
     (96, 2, 1, "f32", "auto"),            # R = 192 on CUDA cores
     (384, 2, 2, "bf16", "simt"),
