@@ -4,6 +4,7 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <stdint.h>
+#include <type_traits>
 #include <utility>
 #include "obcache.h"
 
@@ -52,6 +53,7 @@ struct SimtPlan {
     int n_splits;                        // KV splits of pass 1
     int tiles_per_split;
     int tile_tokens;                     // tokens per tile of the pass-1 kernel the plan is for
+    int row_chunk;                       // window rows per chunk of the CUDA-core kernels
     int rows_out;                        // rows per unit in the combined arrays (R, or R padded)
     int want_obf;                        // also write the bf16 copy of -2*O (tensor-core pass 2); 2: as a high and a low part
     size_t off_flag;                             // 256-byte header: device status word, kernel spans at kSpanOffset

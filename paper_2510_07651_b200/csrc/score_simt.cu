@@ -1,5 +1,5 @@
-// CUDA-core (fp32 FMA) score kernels: the path for fp32 caches and for row counts too small or
-// too irregular for the tensor-core kernels.  Two passes over K/V per (batch item, KV head):
+// CUDA-core (fp32 FMA) score kernels: the path for fp32 caches (and for bf16 caches on request, or when the
+// queries' strides rule the tensor-core kernels out).  Two passes over K/V per (batch item, KV head):
 //
 //   pass 1  split-KV streaming softmax over the window rows: per split, running max / sum of
 //           exp2 and the un-normalised partial output  (Sec. 3: A = softmax(QK^T/sqrt(d)), O = AV)
@@ -14,8 +14,12 @@
 namespace obc {
 
 namespace {
-constexpr int TN = 64;        // tokens per tile
-constexpr int RC = 32;        // window rows per chunk (8 warps x 4 rows)
+// Kernel shapes: TN tokens per tile, RPW window rows per warp and hence 8 RPW rows per chunk.  Large problems take
+// <64, 4>.  A problem that leaves SMs idle with it (fewer tile-chunk items than two per SM) takes tiles of 32 tokens, and
+// one with at most 16 rows chunks of 16, so that no warp of a small window is without rows: one fp32 head of 1024 tokens
+// and 16 rows, pass 1 on 32 CTAs of one tile each instead of 2 CTAs of eight (52.7 -> 5.4 us), pass 2 on 32 instead of 16
+// CTAs (13.6 -> 6.3 us); 8 heads of 2681 tokens and 128 rows on <64, 4>, with the split rule of make_simt_plan and a round
+// trip per tile instead of several, 78.7 -> 56.4 and 94.5 -> 81.1 us.
 constexpr int KS = kD + 4;    // padded row stride (floats) of the token-major smem tiles
 constexpr int NT = 256;
 
@@ -38,14 +42,21 @@ __device__ __forceinline__ float elem_to_float(__nv_bfloat16 x) { return __bfloa
 
 // cooperative load of `rows` x 128 elements into fp32 smem (row stride `stride` floats);
 // rows >= valid are zero-filled.  get(row) returns the global row pointer.
-template <typename T, typename F>
-__device__ __forceinline__ void load_rows(float* dst, int stride, int rows, int valid, F get) {
-    for (int idx = threadIdx.x; idx < rows * (kD / 4); idx += NT) {
-        int row = idx >> 5, c4 = idx & 31;
-        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (row < valid) f = load4<T>(get(row) + c4 * 4);
-        *reinterpret_cast<float4*>(dst + row * stride + c4 * 4) = f;
+// All of a thread's loads are issued before its first store: one round trip to memory per call.
+template <typename T, int ROWS, typename F>
+__device__ __forceinline__ void load_rows(float* dst, int stride, int valid, F get) {
+    constexpr int PER = ROWS * (kD / 4) / NT;
+    static_assert(PER * NT == ROWS * (kD / 4), "rows split evenly over the threads");
+    const int row0 = threadIdx.x >> 5, c4 = threadIdx.x & 31;
+    float4 f[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int row = row0 + u * (NT / 32);
+        f[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < valid) f[u] = load4<T>(get(row) + c4 * 4);
     }
+#pragma unroll
+    for (int u = 0; u < PER; ++u) *reinterpret_cast<float4*>(dst + (row0 + u * (NT / 32)) * stride + c4 * 4) = f[u];
 }
 
 __device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
@@ -54,26 +65,29 @@ __device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
     return acc;
 }
 
-// acc[i][j] += sum_c A[(warp*4+i)][c] * Bt[(lane+32j)][c]   (A row stride kD, Bt row stride KS)
+// acc[i][j] += sum_c A[(warp*RPW+i)][c] * Bt[(lane+32j)][c]   (A row stride kD, Bt row stride KS)
+template <int RPW, int TPL>
 __device__ __forceinline__ void tile_gemm(const float* __restrict__ sA, const float* __restrict__ sB,
-                                          int warp, int lane, float (&acc)[4][2]) {
+                                          int warp, int lane, float (&acc)[RPW][TPL]) {
 #pragma unroll 4
     for (int c4 = 0; c4 < kD / 4; ++c4) {
-        float4 b0 = *reinterpret_cast<const float4*>(sB + lane * KS + c4 * 4);
-        float4 b1 = *reinterpret_cast<const float4*>(sB + (lane + 32) * KS + c4 * 4);
+        float4 b[TPL];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float4 a = *reinterpret_cast<const float4*>(sA + (warp * 4 + i) * kD + c4 * 4);
-            acc[i][0] = dot4(a, b0, acc[i][0]);
-            acc[i][1] = dot4(a, b1, acc[i][1]);
+        for (int j = 0; j < TPL; ++j) b[j] = *reinterpret_cast<const float4*>(sB + (lane + 32 * j) * KS + c4 * 4);
+#pragma unroll
+        for (int i = 0; i < RPW; ++i) {
+            float4 a = *reinterpret_cast<const float4*>(sA + (warp * RPW + i) * kD + c4 * 4);
+#pragma unroll
+            for (int j = 0; j < TPL; ++j) acc[i][j] = dot4(a, b[j], acc[i][j]);
         }
     }
 }
 
 // ------------------------------------------------------------------------------------------ pass 1
-template <typename T>
+template <typename T, int TN, int RPW>
 __global__ void __launch_bounds__(NT, 2)
 simt_pass1_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, TensorView v, float* ws) {
+    constexpr int RC = 8 * RPW, TPL = TN / 32;
     pdl_wait();
     extern __shared__ __align__(16) float smem[];
     float* sK = smem;                       // [TN][KS]
@@ -90,22 +104,22 @@ simt_pass1_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
     if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0)
         *reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(ws) + plan.off_flag) = 0u;
 
-    load_rows<T>(sQ, kD, RC, min(RC, s.R - r0), [&](int row) {
+    load_rows<T, RC>(sQ, kD, min(RC, s.R - r0), [&](int row) {
         int r = r0 + row;
         return row_ptr<T>(q, b, g * s.G + r / s.W, r % s.W);
     });
 
-    float m2[4], l[4], o[4][4];
+    float m2[RPW], l[RPW], o[RPW][4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < RPW; ++i) {
         m2[i] = -INFINITY; l[i] = 0.f;
 #pragma unroll
         for (int c = 0; c < 4; ++c) o[i][c] = 0.f;
     }
-    long long last[4];
+    long long last[RPW];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int r = r0 + warp * 4 + i;
+    for (int i = 0; i < RPW; ++i) {
+        int r = r0 + warp * RPW + i;
         last[i] = (r < s.R) ? (s.causal ? min((long long)mask_len(s, b) - s.W + (r % s.W), (long long)N - 1) : (long long)N - 1) : -1;
     }
 
@@ -115,44 +129,48 @@ simt_pass1_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
     for (int tile = tile_lo; tile < tile_hi; ++tile) {
         const int t0 = tile * TN;
         __syncthreads();
-        load_rows<T>(sK, KS, TN, min(TN, N - t0), [&](int row) { return row_ptr<T>(k, b, g, t0 + row); });
-        load_rows<T>(sV, kD, TN, min(TN, N - t0), [&](int row) { return row_ptr<T>(v, b, g, t0 + row); });
+        load_rows<T, TN>(sK, KS, min(TN, N - t0), [&](int row) { return row_ptr<T>(k, b, g, t0 + row); });
+        load_rows<T, TN>(sV, kD, min(TN, N - t0), [&](int row) { return row_ptr<T>(v, b, g, t0 + row); });
         __syncthreads();
 
-        float acc[4][2] = {};
-        tile_gemm(sQ, sK, warp, lane, acc);
+        float acc[RPW][TPL] = {};
+        tile_gemm<RPW, TPL>(sQ, sK, warp, lane, acc);
 
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float s0 = (t0 + lane <= last[i]) ? acc[i][0] * sl2 : -INFINITY;
-            float s1 = (t0 + lane + 32 <= last[i]) ? acc[i][1] * sl2 : -INFINITY;
-            float mt = warp_max(fmaxf(s0, s1));
-            float mn = fmaxf(m2[i], mt);
-            float p0 = 0.f, p1 = 0.f, corr = 1.f;
-            if (mn != -INFINITY) {
-                corr = exp2f(m2[i] - mn);              // m2 = -inf -> 0
-                p0 = exp2f(s0 - mn); p1 = exp2f(s1 - mn);
+        for (int i = 0; i < RPW; ++i) {
+            float sc[TPL], mt = -INFINITY;
+#pragma unroll
+            for (int j = 0; j < TPL; ++j) {
+                sc[j] = (t0 + lane + 32 * j <= last[i]) ? acc[i][j] * sl2 : -INFINITY;
+                mt = fmaxf(mt, sc[j]);
             }
-            float ps = warp_sum(p0 + p1);
-            l[i] = l[i] * corr + ps;
+            mt = warp_max(mt);
+            const float mn = fmaxf(m2[i], mt);
+            float corr = 1.f, ps = 0.f;
+            if (mn != -INFINITY) corr = exp2f(m2[i] - mn);         // m2 = -inf -> 0
+#pragma unroll
+            for (int j = 0; j < TPL; ++j) {
+                const float pj = mn != -INFINITY ? exp2f(sc[j] - mn) : 0.f;
+                ps += pj;
+                sP[(warp * RPW + i) * TN + lane + 32 * j] = pj;
+            }
+            l[i] = l[i] * corr + warp_sum(ps);
             m2[i] = mn;
 #pragma unroll
             for (int c = 0; c < 4; ++c) o[i][c] *= corr;
-            sP[(warp * 4 + i) * TN + lane] = p0;
-            sP[(warp * 4 + i) * TN + lane + 32] = p1;
         }
         __syncwarp();
         // O[rows of this warp][lane*4 .. +3] += P[row][p] * V[p][lane*4 .. +3]
 #pragma unroll 2
         for (int p4 = 0; p4 < TN / 4; ++p4) {
-            float4 pr[4];
+            float4 pr[RPW];
 #pragma unroll
-            for (int i = 0; i < 4; ++i) pr[i] = *reinterpret_cast<const float4*>(sP + (warp * 4 + i) * TN + p4 * 4);
+            for (int i = 0; i < RPW; ++i) pr[i] = *reinterpret_cast<const float4*>(sP + (warp * RPW + i) * TN + p4 * 4);
 #pragma unroll
             for (int pp = 0; pp < 4; ++pp) {
                 float4 vv = *reinterpret_cast<const float4*>(sV + (p4 * 4 + pp) * kD + lane * 4);
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+                for (int i = 0; i < RPW; ++i) {
                     float pw = pp == 0 ? pr[i].x : pp == 1 ? pr[i].y : pp == 2 ? pr[i].z : pr[i].w;
                     o[i][0] = fmaf(pw, vv.x, o[i][0]); o[i][1] = fmaf(pw, vv.y, o[i][1]);
                     o[i][2] = fmaf(pw, vv.z, o[i][2]); o[i][3] = fmaf(pw, vv.w, o[i][3]);
@@ -166,8 +184,8 @@ simt_pass1_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
     float* part_l = ws + plan.off_part_l / 4;
     float* part_o = ws + plan.off_part_o / 4;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        int r = r0 + warp * 4 + i;
+    for (int i = 0; i < RPW; ++i) {
+        int r = r0 + warp * RPW + i;
         if (r >= s.R) continue;
         size_t row = ((size_t)unit * plan.n_splits + split) * s.R + r;
         if (lane == 0) { part_m[row] = m2[i]; part_l[row] = l[i]; }
@@ -392,10 +410,11 @@ given_prep_kernel(ScoreShape s, SimtPlan plan, TensorView o, const float* lse, f
 }
 
 // ------------------------------------------------------------------------------------------ pass 2
-template <typename T>
+template <typename T, int TN, int RPW>
 __global__ void __launch_bounds__(NT, 2)
 simt_pass2_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, TensorView v,
                   const float* ws, float* scores) {
+    constexpr int RC = 8 * RPW, TPL = TN / 32;
     pdl_wait();
     extern __shared__ __align__(16) float smem[];
     float* sK = smem;                       // [TN][KS]
@@ -422,11 +441,12 @@ simt_pass2_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
         return;
     }
 
-    load_rows<T>(sK, KS, TN, min(TN, N - t0), [&](int row) { return row_ptr<T>(k, b, g, t0 + row); });
-    load_rows<T>(sV, KS, TN, min(TN, N - t0), [&](int row) { return row_ptr<T>(v, b, g, t0 + row); });
+    load_rows<T, TN>(sK, KS, min(TN, N - t0), [&](int row) { return row_ptr<T>(k, b, g, t0 + row); });
+    load_rows<T, TN>(sV, KS, min(TN, N - t0), [&](int row) { return row_ptr<T>(v, b, g, t0 + row); });
     __syncthreads();
-    // ||v_p||^2: each warp covers 8 tokens
-    for (int tkn = warp * 8; tkn < warp * 8 + 8; ++tkn) {
+    // ||v_p||^2: each warp covers an eighth of the tokens
+#pragma unroll
+    for (int tkn = warp * (TN / 8); tkn < (warp + 1) * (TN / 8); ++tkn) {
         float4 f = *reinterpret_cast<const float4*>(sV + tkn * KS + lane * 4);
         float sq = warp_sum(f.x * f.x + f.y * f.y + f.z * f.z + f.w * f.w);
         float ab = warp_sum((fabsf(f.x) + fabsf(f.y)) + (fabsf(f.z) + fabsf(f.w)));
@@ -438,16 +458,16 @@ simt_pass2_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
     const float* lse_all = ws + plan.off_lse2 / 4 + (size_t)unit * plan.rows_out;
     const float* no_all = ws + plan.off_onorm / 4 + (size_t)unit * plan.rows_out;
 
-    float sv[2] = {0.f, 0.f}, sk[2] = {0.f, 0.f}, sx[2] = {0.f, 0.f}, sa[2] = {0.f, 0.f};
+    float sv[TPL] = {}, sk[TPL] = {}, sx[TPL] = {}, sa[TPL] = {};
 
     for (int r0 = 0; r0 < s.R; r0 += RC) {
         __syncthreads();
         const int valid = min(RC, s.R - r0);
-        load_rows<T>(sQ, kD, RC, valid, [&](int row) {
+        load_rows<T, RC>(sQ, kD, valid, [&](int row) {
             int r = r0 + row;
             return row_ptr<T>(q, b, g * s.G + r / s.W, r % s.W);
         });
-        load_rows<float>(sO, kD, RC, valid, [&](int row) { return o_all + (size_t)(r0 + row) * kD; });
+        load_rows<float, RC>(sO, kD, valid, [&](int row) { return o_all + (size_t)(r0 + row) * kD; });
         if (threadIdx.x < RC) {
             bool ok = threadIdx.x < valid;
             sLse[threadIdx.x] = ok ? lse_all[r0 + threadIdx.x] : 0.f;
@@ -455,18 +475,18 @@ simt_pass2_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
         }
         __syncthreads();
 
-        float az[4][2] = {}, at[4][2] = {};
-        tile_gemm(sQ, sK, warp, lane, az);
-        tile_gemm(sO, sV, warp, lane, at);
+        float az[RPW][TPL] = {}, at[RPW][TPL] = {};
+        tile_gemm<RPW, TPL>(sQ, sK, warp, lane, az);
+        tile_gemm<RPW, TPL>(sO, sV, warp, lane, at);
 
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + warp * 4 + i;
+        for (int i = 0; i < RPW; ++i) {
+            const int r = r0 + warp * RPW + i;
             if (r >= s.R) continue;
             const long long last = s.causal ? min((long long)mask_len(s, b) - s.W + (r % s.W), (long long)N - 1) : (long long)N - 1;
-            const float lse = sLse[warp * 4 + i], no = sNo[warp * 4 + i];
+            const float lse = sLse[warp * RPW + i], no = sNo[warp * RPW + i];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+            for (int j = 0; j < TPL; ++j) {
                 const int tl = lane + 32 * j;
                 if (t0 + tl > last) continue;              // masked pair: contributes 0
                 const float nv = sNv[tl];
@@ -482,11 +502,12 @@ simt_pass2_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
         }
     }
 
-    // sum over the 8 warps (each warp held 4 of every 32 rows)
+    // sum over the 8 warps (each warp held RPW rows of every chunk)
     __syncthreads();
-    float* red = sQ;                        // [8][4][TN]
+    float* red = sQ;                        // [8][4][TN] over Q and O
+    static_assert(32 * TN <= 2 * RC * kD, "the sums fit the Q and O tiles");
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
+    for (int j = 0; j < TPL; ++j) {
         const int tl = lane + 32 * j;
         red[(warp * 4 + 0) * TN + tl] = sv[j];
         red[(warp * 4 + 1) * TN + tl] = sk[j];
@@ -514,41 +535,66 @@ simt_pass2_kernel(ScoreShape s, SimtPlan plan, TensorView q, TensorView k, Tenso
     }
 }
 
-constexpr size_t kSmemPass1 = (size_t)(TN * KS + TN * kD + RC * kD + RC * TN) * 4;
-constexpr size_t kSmemPass2 = (size_t)(2 * TN * KS + 2 * RC * kD + 2 * TN + 2 * RC) * 4;
+constexpr size_t smem_pass1(int tn, int rc) { return (size_t)(tn * KS + tn * kD + rc * kD + rc * tn) * 4; }
+constexpr size_t smem_pass2(int tn, int rc) { return (size_t)(2 * tn * KS + 2 * rc * kD + 2 * tn + 2 * rc) * 4; }
+
+// the kernel shape a plan asks for (see the head of the file)
+template <typename F> obc_status with_shape(const SimtPlan& plan, F f) {
+    if (plan.tile_tokens == 64) return f(std::integral_constant<int, 64>{}, std::integral_constant<int, 4>{});
+    if (plan.row_chunk == 32) return f(std::integral_constant<int, 32>{}, std::integral_constant<int, 4>{});
+    return f(std::integral_constant<int, 32>{}, std::integral_constant<int, 2>{});
+}
 
 template <typename T>
 obc_status launch_pass1_typed(const ScoreShape& s, const SimtPlan& plan, TensorView q, TensorView k, TensorView v,
                               float* ws, cudaStream_t stream) {
-    const int units = s.B * s.Hkv, chunks = (s.R + RC - 1) / RC;
-    OBC_CUDA_TRY(cudaFuncSetAttribute(simt_pass1_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPass1));
-    { ProfScope ps("simt_pass1", stream); OBC_CUDA_TRY(launch_pdl(simt_pass1_kernel<T>, dim3(plan.n_splits, units, chunks), dim3(NT), kSmemPass1, stream, 1, s, plan, q, k, v, ws)); }
-    return launch_combine(s, plan, ws, stream);
+    const int units = s.B * s.Hkv, chunks = (s.R + plan.row_chunk - 1) / plan.row_chunk;
+    obc_status st = with_shape(plan, [&](auto tn, auto rpw) -> obc_status {
+        const auto kernel = simt_pass1_kernel<T, tn.value, rpw.value>;
+        constexpr size_t bytes = smem_pass1(tn.value, 8 * rpw.value);
+        OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        ProfScope ps("simt_pass1", stream);
+        OBC_CUDA_TRY(launch_pdl(kernel, dim3(plan.n_splits, units, chunks), dim3(NT), bytes, stream, 1, s, plan, q, k, v, ws));
+        return OBC_OK;
+    });
+    return st != OBC_OK ? st : launch_combine(s, plan, ws, stream);
 }
 
 template <typename T>
 obc_status launch_pass2_typed(const ScoreShape& s, const SimtPlan& plan, TensorView q, TensorView k, TensorView v,
                               float* scores, float* ws, cudaStream_t stream) {
     const int units = s.B * s.Hkv;
-    OBC_CUDA_TRY(cudaFuncSetAttribute(simt_pass2_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemPass2));
-    { ProfScope ps("simt_pass2", stream); OBC_CUDA_TRY(launch_pdl(simt_pass2_kernel<T>, dim3((s.Nmax + TN - 1) / TN, units), dim3(NT), kSmemPass2, stream, 1, s, plan, q, k, v, ws, scores)); }
-    return OBC_OK;
+    return with_shape(plan, [&](auto tn, auto rpw) -> obc_status {
+        const auto kernel = simt_pass2_kernel<T, tn.value, rpw.value>;
+        constexpr size_t bytes = smem_pass2(tn.value, 8 * rpw.value);
+        OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        ProfScope ps("simt_pass2", stream);
+        OBC_CUDA_TRY(launch_pdl(kernel, dim3((s.Nmax + tn.value - 1) / tn.value, units), dim3(NT), bytes, stream, 1, s, plan, q, k, v, (const float*)ws, scores));
+        return OBC_OK;
+    });
 }
 }  // namespace
 
 SimtPlan make_simt_plan(const ScoreShape& s, int rows_out, bool want_obf) {
     SimtPlan p{};
-    const int units = s.B * s.Hkv, chunks = (s.R + RC - 1) / RC;
-    const int tiles = (s.Nmax + TN - 1) / TN;
-    // enough CTAs for ~2 waves of 148 SMs x 2 resident CTAs, at least 8 tiles per split
-    int want = (148 * 2 * 2 + units * chunks - 1) / (units * chunks);
-    int max_splits = (tiles + 7) / 8;
-    int n = want < 1 ? 1 : want;
-    if (n > max_splits) n = max_splits;
+    const long long units = (long long)s.B * s.Hkv;
+    const long long slots = 148 * 2;                       // two resident CTAs per SM
+    const bool small = units * ((s.Nmax + 63) / 64) * ((s.R + 31) / 32) < slots;
+    const int tn = small ? 32 : 64, rc = small && s.R <= 16 ? 16 : 32;
+    const long long chunks = (s.R + rc - 1) / rc;
+    const int tiles = (s.Nmax + tn - 1) / tn;
+    // pass-1 CTAs for about two waves when every one still has eight tiles, else for one wave of at least one tile each
+    long long n = (2 * slots + units * chunks - 1) / (units * chunks);
+    if (n * 8 > tiles) {
+        n = slots / (units * chunks);
+        if (n < (tiles + 7) / 8) n = (tiles + 7) / 8;
+    }
+    if (n > tiles) n = tiles;
     if (n < 1) n = 1;
-    p.tiles_per_split = (tiles + n - 1) / n;
+    p.tiles_per_split = (int)((tiles + n - 1) / n);
     p.n_splits = (tiles + p.tiles_per_split - 1) / p.tiles_per_split;
-    p.tile_tokens = TN;
+    p.tile_tokens = tn;
+    p.row_chunk = rc;
     p.rows_out = rows_out;
     p.want_obf = want_obf ? 1 : 0;
     size_t rows = (size_t)units * s.R, prow = rows * p.n_splits, orow = (size_t)units * rows_out, off = 0;
