@@ -273,6 +273,16 @@ obc_status obc_compact(int32_t batch, int32_t n_kv_heads, int32_t head_dim, int3
                        obc_tensor k_out, obc_tensor v_out,
                        const float* scores_in, float* scores_out, void* stream);
 
+/*
+ * obc_compact into buffers that the caller has not cleared: where idx[b,g,j] < 0, row j of each output named in
+ * `zero_rows` (OBC_ZERO_* bits) is written as zeros instead of being left untouched.  zero_rows = 0: obc_compact.
+ */
+enum { OBC_ZERO_K = 1, OBC_ZERO_V = 2, OBC_ZERO_SCORES = 4 };
+obc_status obc_compact_padded(int32_t batch, int32_t n_kv_heads, int32_t head_dim, int32_t idx_stride,
+                              int32_t max_len, obc_tensor k, obc_tensor v, const int32_t* idx,
+                              obc_tensor k_out, obc_tensor v_out,
+                              const float* scores_in, float* scores_out, uint32_t zero_rows, void* stream);
+
 /* ------------------------------------------------------------------------------------------
  * obc_decode_step: one decode-time rescoring + eviction step (Sec. 3 "Decoding" and "Cache
  * Eviction"; Sec. 4.2: scores accumulated over decode steps; App. C.2.2: sinks and a recent

@@ -1,9 +1,10 @@
-"""Thin ctypes binding over libobcache.so.  Same names as include/obcache.h; argument
-marshalling only: every step of the path runs in the library's CUDA kernels.
+"""Thin binding over libobcache.so.  Same names as include/obcache.h; argument marshalling only:
+every step of the path runs in the library's CUDA kernels.
 
-torch is used for device memory (`data_ptr()`), strides and the current stream, nothing else.
-There is no fallback: if the shared library is missing or cannot be loaded, importing the
-functions raises.
+torch is used for device memory (`data_ptr()`), strides and the current stream, nothing else.  The
+calls of the hot path (score, select, compact, the whole eviction, the decode step) are marshalled
+in native code (csrc/binding.cpp); the others go through ctypes.  There is no fallback: if a shared
+library is missing or cannot be loaded, the functions raise.
 """
 from __future__ import annotations
 
@@ -24,7 +25,7 @@ POOLS = {"none": OBC_POOL_NONE, "avg": OBC_POOL_AVG, "max": OBC_POOL_MAX}
 PATHS = {"auto": OBC_PATH_AUTO, "simt": OBC_PATH_SIMT, "tc": OBC_PATH_TC}
 
 EXPORTS = ["obc_score_workspace", "obc_score", "obc_score_given", "obc_window_attention", "obc_merge_attention", "obc_shard_indices", "obc_score_status", "obc_score_kernel_spans", "obc_select_workspace", "obc_select",
-           "obc_select_noalloc", "obc_select_adaptive_workspace", "obc_select_adaptive", "obc_compact",
+           "obc_select_noalloc", "obc_select_adaptive_workspace", "obc_select_adaptive", "obc_compact", "obc_compact_padded",
            "obc_decode_workspace", "obc_decode_step", "obc_profile_begin", "obc_profile_end",
            "obc_status_string", "obc_last_cuda_error", "obc_version"]
 
@@ -94,6 +95,7 @@ def lib():
         L.obc_select_adaptive_workspace.argtypes = [C.POINTER(obc_select_params), C.c_float, sz]
         L.obc_select_adaptive.argtypes = [C.POINTER(obc_select_params), C.c_float, vp, vp, vp, vp, C.c_size_t, vp]
         L.obc_compact.argtypes = [C.c_int32] * 5 + [obc_tensor, obc_tensor, vp, obc_tensor, obc_tensor, vp, vp, vp]
+        L.obc_compact_padded.argtypes = [C.c_int32] * 5 + [obc_tensor, obc_tensor, vp, obc_tensor, obc_tensor, vp, vp, C.c_uint32, vp]
         L.obc_decode_workspace.argtypes = [C.POINTER(obc_decode_params), sz]
         L.obc_decode_step.argtypes = [C.POINTER(obc_decode_params)] + [obc_tensor] * 5 + [vp, vp, vp, C.c_int32, vp, C.c_size_t, vp]
         L.obc_profile_begin.argtypes = []
@@ -110,6 +112,26 @@ def lib():
 def _check(st: int, where: str):
     if st != 0:
         raise ObcError(st, where)
+
+
+_native_mod = None
+
+
+def _native():
+    """The native marshalling module (raises ImportError if it has not been built)."""
+    global _native_mod
+    if _native_mod is None:
+        lib()
+        from . import _native as mod
+        _native_mod = mod
+    return _native_mod
+
+
+def _result(r, where: str):
+    """What a native call returned: its result, or the status of a library call that failed."""
+    if r.__class__ is int:
+        raise ObcError(r, where)
+    return r
 
 
 def _dtype_code(t: torch.Tensor) -> int:
@@ -167,15 +189,8 @@ def obc_score(q, k, v, *, seq_lens=None, scale=0.0, causal=True, variants=("VK",
               scores=None, workspace=None):
     """q [B,Hq,W,d], k/v [B,Hkv,Nmax,d] CUDA tensors -> fp32 scores [n_variants,B,Hkv,Nmax]
     (planes in V, K, VK, ATTN, VATP order).  Enqueued on the current stream."""
-    p = score_params(q, k, seq_lens=seq_lens, scale=scale, causal=causal, variants=variants, path=path)
-    B, Hkv, Nmax = k.shape[0], k.shape[1], k.shape[2]
-    n_planes = bin(p.variants).count("1")
-    if scores is None:
-        scores = torch.empty((n_planes, B, Hkv, Nmax), dtype=torch.float32, device=k.device)
-    ws = _workspace(obc_score_workspace(p), k, workspace)
-    _check(lib().obc_score(C.byref(p), as_tensor4(q), as_tensor4(k), as_tensor4(v), scores.data_ptr(),
-                           ws.data_ptr(), ws.numel(), _stream()), "obc_score")
-    return scores
+    return _result(_native().score(q, k, v, None, None, seq_lens, None, scale, 1 if causal else 0, variants_mask(variants),
+                                   PATHS[path] if isinstance(path, str) else path, scores, workspace), "obc_score")
 
 
 def obc_window_attention(q, k, v, *, seq_lens=None, mask_lens=None, scale=0.0, causal=True, path="auto",
@@ -229,20 +244,8 @@ def obc_score_given(q, k, v, o, lse, *, seq_lens=None, scale=0.0, causal=True, v
                     scores=None, workspace=None, mask_lens=None):
     """obc_score from attention outputs the caller already has: o [B,Hq,W,d] (f32 or bf16) and lse
     fp32 [B,Hq,W] (natural log, contiguous) of the window rows; no window attention is recomputed."""
-    p = score_params(q, k, seq_lens=seq_lens, scale=scale, causal=causal, variants=variants, path=path, mask_lens=mask_lens)
-    B, Hkv, Nmax = k.shape[0], k.shape[1], k.shape[2]
-    if tuple(o.shape) != tuple(q.shape) or tuple(lse.shape) != tuple(q.shape[:3]):
-        raise ValueError("o must be shaped like q and lse like q without its last axis")
-    if lse.dtype != torch.float32 or not lse.is_contiguous():
-        raise ValueError("lse must be a contiguous float32 tensor")
-    n_planes = bin(p.variants).count("1")
-    if scores is None:
-        scores = torch.empty((n_planes, B, Hkv, Nmax), dtype=torch.float32, device=k.device)
-    ws = _workspace(obc_score_workspace(p), k, workspace)
-    _check(lib().obc_score_given(C.byref(p), as_tensor4(q), as_tensor4(k), as_tensor4(v), as_tensor4(o),
-                                 lse.data_ptr(), scores.data_ptr(), ws.data_ptr(), ws.numel(), _stream()),
-           "obc_score_given")
-    return scores
+    return _result(_native().score(q, k, v, o, lse, seq_lens, mask_lens, scale, 1 if causal else 0, variants_mask(variants),
+                                   PATHS[path] if isinstance(path, str) else path, scores, workspace), "obc_score_given")
 
 
 def obc_score_status(workspace) -> None:
@@ -278,14 +281,9 @@ def obc_select_workspace(p: obc_select_params) -> int:
 def obc_select(scores, *, budget=0, budgets=None, idx_stride=None, seq_lens=None, n_sink=0, n_recent=0,
                pool="none", pool_kernel=1, idx=None, workspace=None):
     """scores fp32 [B,Hkv,Nmax] -> int32 idx [B,Hkv,idx_stride] (ascending, padded with -1)."""
-    p = select_params(scores, budget=budget, budgets=budgets, idx_stride=idx_stride, seq_lens=seq_lens,
-                      n_sink=n_sink, n_recent=n_recent, pool=pool, pool_kernel=pool_kernel)
-    if idx is None:
-        idx = torch.empty((p.batch, p.n_kv_heads, p.idx_stride), dtype=torch.int32, device=scores.device)
-    ws = _workspace(obc_select_workspace(p), scores, workspace)
-    _check(lib().obc_select(C.byref(p), scores.data_ptr(), idx.data_ptr(), ws.data_ptr(), ws.numel(), _stream()),
-           "obc_select")
-    return idx
+    return _result(_native().select(scores, int(budget), budgets, int(budget if idx_stride is None else idx_stride), seq_lens, n_sink,
+                                    n_recent, POOLS[pool] if isinstance(pool, str) else pool, pool_kernel, idx, workspace, None, None),
+                   "obc_select")
 
 
 def obc_select_adaptive(scores, *, budget, safeguard=0.2, idx_stride=None, seq_lens=None, n_sink=0, n_recent=0,
@@ -293,18 +291,9 @@ def obc_select_adaptive(scores, *, budget, safeguard=0.2, idx_stride=None, seq_l
     """Head-adaptive budgets: scores fp32 [B,Hkv,Nmax] -> (idx int32 [B,Hkv,idx_stride] padded with -1,
     counts int32 [B,Hkv]).  Every head keeps floor(safeguard * n_hh) tokens by its own ranking; the rest of the
     layer's Hkv * n_hh slots go to the best remaining tokens of all heads together."""
-    p = select_params(scores, budget=budget, idx_stride=idx_stride, seq_lens=seq_lens, n_sink=n_sink,
-                      n_recent=n_recent, pool=pool, pool_kernel=pool_kernel)
-    if idx is None:
-        idx = torch.empty((p.batch, p.n_kv_heads, p.idx_stride), dtype=torch.int32, device=scores.device)
-    if counts is None:
-        counts = torch.empty((p.batch, p.n_kv_heads), dtype=torch.int32, device=scores.device)
-    n = C.c_size_t(0)
-    _check(lib().obc_select_adaptive_workspace(C.byref(p), float(safeguard), C.byref(n)), "obc_select_adaptive_workspace")
-    ws = _workspace(n.value, scores, workspace)
-    _check(lib().obc_select_adaptive(C.byref(p), float(safeguard), scores.data_ptr(), idx.data_ptr(), counts.data_ptr(),
-                                     ws.data_ptr(), ws.numel(), _stream()), "obc_select_adaptive")
-    return idx, counts
+    return _result(_native().select(scores, int(budget), None, int(budget if idx_stride is None else idx_stride), seq_lens, n_sink,
+                                    n_recent, POOLS[pool] if isinstance(pool, str) else pool, pool_kernel, idx, workspace,
+                                    float(safeguard), counts), "obc_select_adaptive")
 
 
 SELECT_NOALLOC_MAX_KEYS = 1 << 20
@@ -326,17 +315,7 @@ def obc_select_noalloc(scores, idx, *, budget=0, budgets=None, seq_lens=None, n_
 
 def obc_compact(k, v, idx, *, k_out=None, v_out=None, scores_in=None, scores_out=None):
     """Gather kept rows: k/v [B,Hkv,Nmax,d], idx [B,Hkv,S] -> k_out/v_out [B,Hkv,S,d]."""
-    B, Hkv, Nmax, d = k.shape
-    S = idx.shape[2]
-    if k_out is None:
-        k_out = torch.zeros((B, Hkv, S, d), dtype=k.dtype, device=k.device)
-    if v_out is None:
-        v_out = torch.zeros((B, Hkv, S, d), dtype=v.dtype, device=v.device)
-    if scores_in is not None and scores_out is None:
-        scores_out = torch.zeros((B, Hkv, S), dtype=torch.float32, device=k.device)
-    _check(lib().obc_compact(B, Hkv, d, S, Nmax, as_tensor4(k), as_tensor4(v), idx.data_ptr(), as_tensor4(k_out),
-                             as_tensor4(v_out), _ptr(scores_in), _ptr(scores_out), _stream()), "obc_compact")
-    return (k_out, v_out) if scores_in is None else (k_out, v_out, scores_out)
+    return _result(_native().compact(k, v, idx, k_out, v_out, scores_in, scores_out), "obc_compact")
 
 
 def decode_params(q_t, k_cache, *, budget, n_sink, n_recent, variant="VK", scale=0.0, acc_window=0,
@@ -361,13 +340,9 @@ def obc_decode_step(q_t, k_t, v_t, k_cache, v_cache, s_acc, pos, state, step_pos
     """One in-place decode rescoring + eviction step (see include/obcache.h).  With acc_window = w > 0 the
     accumulator is the sum of the last w steps' scores and s_hist is the zero-initialised fp32 ring
     [B,Hkv,w,capacity] that holds them."""
-    p = decode_params(q_t, k_cache, budget=budget, n_sink=n_sink, n_recent=n_recent, variant=variant, scale=scale,
-                      acc_window=acc_window, s_hist=s_hist)
-    ws = _workspace(obc_decode_workspace(p), k_cache, workspace)
-    _check(lib().obc_decode_step(C.byref(p), as_tensor4(q_t), as_tensor4(k_t), as_tensor4(v_t), as_tensor4(k_cache),
-                                 as_tensor4(v_cache), s_acc.data_ptr(), pos.data_ptr(), state.data_ptr(),
-                                 int(step_pos), ws.data_ptr(), ws.numel(), _stream()), "obc_decode_step")
-    return ws
+    return _result(_native().decode_step(q_t, k_t, v_t, k_cache, v_cache, s_acc, pos, state, int(step_pos), budget, n_sink, n_recent,
+                                         VARIANTS[variant] if isinstance(variant, str) else variant, scale, workspace,
+                                         int(acc_window), s_hist), "obc_decode_step")
 
 
 def obc_profile_begin():
@@ -387,9 +362,15 @@ def evict_prefill(q, k, v, *, budget=0, budgets=None, seq_lens=None, variant="VK
                   pool="none", pool_kernel=1, causal=True, path="auto"):
     """The whole prefill hot path: score -> pool/select -> compact.  Returns (k_out, v_out, idx, scores)."""
     n_recent = q.shape[2] if n_recent is None else n_recent
+    if budgets is None:
+        r = _native().evict(q, k, v, int(budget), seq_lens, variants_mask((variant,)), n_sink, n_recent,
+                            POOLS[pool] if isinstance(pool, str) else pool, pool_kernel, 1 if causal else 0,
+                            PATHS[path] if isinstance(path, str) else path)
+        if r[0].__class__ is int:
+            raise ObcError(r[0], ("obc_score", "obc_select_workspace", "obc_select", "obc_compact")[r[1]])
+        return r
     scores = obc_score(q, k, v, seq_lens=seq_lens, causal=causal, variants=(variant,), path=path)
-    stride = int(budget) if budgets is None else int(budgets.max().item())
-    idx = obc_select(scores[0], budget=budget, budgets=budgets, idx_stride=stride, seq_lens=seq_lens,
+    idx = obc_select(scores[0], budget=budget, budgets=budgets, idx_stride=int(budgets.max().item()), seq_lens=seq_lens,
                      n_sink=n_sink, n_recent=n_recent, pool=pool, pool_kernel=pool_kernel)
     k_out, v_out = obc_compact(k, v, idx)
     return k_out, v_out, idx, scores

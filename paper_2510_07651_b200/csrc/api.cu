@@ -300,6 +300,13 @@ obc_status obc_compact(int32_t batch, int32_t n_kv_heads, int32_t head_dim, int3
                        int32_t max_len, obc_tensor k, obc_tensor v, const int32_t* idx,
                        obc_tensor k_out, obc_tensor v_out,
                        const float* scores_in, float* scores_out, void* stream) {
+    return obc_compact_padded(batch, n_kv_heads, head_dim, idx_stride, max_len, k, v, idx, k_out, v_out, scores_in, scores_out, 0, stream);
+}
+
+obc_status obc_compact_padded(int32_t batch, int32_t n_kv_heads, int32_t head_dim, int32_t idx_stride,
+                              int32_t max_len, obc_tensor k, obc_tensor v, const int32_t* idx,
+                              obc_tensor k_out, obc_tensor v_out,
+                              const float* scores_in, float* scores_out, uint32_t zero_rows, void* stream) {
     if (head_dim != kD) return OBC_ERR_UNSUPPORTED;
     if (batch < 1 || n_kv_heads < 1 || idx_stride < 1 || max_len < 1) return OBC_ERR_SHAPE;
     if ((long long)batch * n_kv_heads > 65535) return OBC_ERR_SHAPE;            // units index gridDim.y
@@ -311,8 +318,9 @@ obc_status obc_compact(int32_t batch, int32_t n_kv_heads, int32_t head_dim, int3
     if ((st = check_tensor(k_out, true)) != OBC_OK) return st;
     if ((st = check_tensor(v_out, true)) != OBC_OK) return st;
     if (k.dtype != v.dtype || k.dtype != k_out.dtype || k.dtype != v_out.dtype) return OBC_ERR_UNSUPPORTED;
+    if (zero_rows & ~(uint32_t)(OBC_ZERO_K | OBC_ZERO_V | OBC_ZERO_SCORES)) return OBC_ERR_UNSUPPORTED;
     return launch_gather(batch, n_kv_heads, idx_stride, max_len, elem_size(k.dtype), view(k), view(v),
-                         view(k_out), view(v_out), idx, scores_in, scores_out, (cudaStream_t)stream);
+                         view(k_out), view(v_out), idx, scores_in, scores_out, zero_rows, (cudaStream_t)stream);
 }
 
 static obc_status resolve_decode(const obc_decode_params* p, DecodeShape* s) {

@@ -595,10 +595,10 @@ obc_status launch_g(const DecodeShape& s, const DecodePlan& plan, const CUtensor
                     int step_pos, char* ws, cudaStream_t stream) {
     const int units = s.B * s.Hkv;
     const size_t stage = kStageBytes + 1024;                            // + room to align the swizzled tile
-    { ProfScope ps("decode_pass1", stream); OBC_CUDA_TRY(cudaFuncSetAttribute(decode_pass1_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage));
+    { ProfScope ps("decode_pass1", stream); OBC_CUDA_TRY(allow_smem(decode_pass1_kernel<G>, stage));
       OBC_CUDA_TRY(launch_pdl(decode_pass1_kernel<G>, dim3(plan.chunks, units), dim3(CH), stage, stream, 1, mk, mv, s, plan, q, kt, vt, kc, vc, s_acc, pos, state, step_pos, ws)); }
     { ProfScope ps("decode_combine", stream); OBC_CUDA_TRY(launch_pdl(decode_combine_kernel, dim3(units * s.G), dim3(kD), 0, stream, 1, s, plan, ws)); }
-    { ProfScope ps("decode_score", stream); OBC_CUDA_TRY(cudaFuncSetAttribute(decode_score_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)stage));
+    { ProfScope ps("decode_score", stream); OBC_CUDA_TRY(allow_smem(decode_score_kernel<G>, stage));
       OBC_CUDA_TRY(launch_pdl(decode_score_kernel<G>, dim3(plan.chunks, units), dim3(CH), stage, stream, 1, mv, s, plan, vc, s_acc, pos, state, step_pos, ws)); }
     { ProfScope ps("decode_final", stream); OBC_CUDA_TRY(launch_pdl(decode_final_kernel, dim3((units + 3) / 4), dim3(128), 0, stream, 1, s, plan, pos, state, ws)); }
     return OBC_OK;

@@ -112,7 +112,7 @@ obc_status launch_shard_indices(int units, int idx_stride, int t0, int n, const 
                                 cudaStream_t stream);
 obc_status launch_gather(int B, int Hkv, int idx_stride, int Nmax, int elem_bytes,
                          TensorView k, TensorView v, TensorView ko, TensorView vo, const int32_t* idx,
-                         const float* s_in, float* s_out, cudaStream_t stream);
+                         const float* s_in, float* s_out, uint32_t zero_rows, cudaStream_t stream);
 
 // ---- decode step --------------------------------------------------------------------------------
 struct DecodeShape {
@@ -165,6 +165,23 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     }
     cfg.attrs = attr;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
+}
+
+// Lets `kernel` use `bytes` of dynamic shared memory on the current device.  The attribute stays with the kernel, so what a
+// host thread has asked for is remembered (per kernel and device) and the call, about a microsecond of host time per
+// launch, is made once.
+template <typename... KArgs>
+inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
+    struct Seen { const void* kernel; int dev; size_t bytes; };
+    thread_local Seen seen[32] = {};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    Seen& at = seen[((uintptr_t)kernel >> 4) % 32];
+    if (at.kernel == (const void*)kernel && at.dev == dev && at.bytes >= bytes) return cudaSuccess;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) at = Seen{(const void*)kernel, dev, bytes};
+    return e;
 }
 
 // ---- device helpers --------------------------------------------------------------------------

@@ -552,7 +552,7 @@ obc_status launch_pass1_typed(const ScoreShape& s, const SimtPlan& plan, TensorV
     obc_status st = with_shape(plan, [&](auto tn, auto rpw) -> obc_status {
         const auto kernel = simt_pass1_kernel<T, tn.value, rpw.value>;
         constexpr size_t bytes = smem_pass1(tn.value, 8 * rpw.value);
-        OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        OBC_CUDA_TRY(allow_smem(kernel, bytes));
         ProfScope ps("simt_pass1", stream);
         OBC_CUDA_TRY(launch_pdl(kernel, dim3(plan.n_splits, units, chunks), dim3(NT), bytes, stream, 1, s, plan, q, k, v, ws));
         return OBC_OK;
@@ -567,7 +567,7 @@ obc_status launch_pass2_typed(const ScoreShape& s, const SimtPlan& plan, TensorV
     return with_shape(plan, [&](auto tn, auto rpw) -> obc_status {
         const auto kernel = simt_pass2_kernel<T, tn.value, rpw.value>;
         constexpr size_t bytes = smem_pass2(tn.value, 8 * rpw.value);
-        OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+        OBC_CUDA_TRY(allow_smem(kernel, bytes));
         ProfScope ps("simt_pass2", stream);
         OBC_CUDA_TRY(launch_pdl(kernel, dim3((s.Nmax + tn.value - 1) / tn.value, units), dim3(NT), bytes, stream, 1, s, plan, q, k, v, (const float*)ws, scores));
         return OBC_OK;

@@ -1662,7 +1662,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
             p1.out_cpair = (float*)(wsb + plan.off_cpair);
         }
         const auto pass1 = hilo ? tc_pass1_kernel<true> : tc_pass1_kernel<false>;
-        OBC_CUDA_TRY(cudaFuncSetAttribute(pass1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemP1));
+        OBC_CUDA_TRY(allow_smem(pass1, kSmemP1));
         { ProfScope ps("tc_pass1", stream);
           OBC_CUDA_TRY(launch_pdl(pass1, dim3(plan.n_splits, units * ch.n_chunks), dim3(kThreadsP1), kSmemP1, stream, 1, mq, mk, mv, p1)); }
         if (!direct) {
@@ -1703,7 +1703,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         const long long positions = (long long)units * (((s.Nmax + TILE - 1) / TILE + 1) / 2) * p.csplit;
         const int mgrid = (int)(positions < sm_count() ? positions : sm_count());
         auto launch_multi = [&](auto kernel) -> obc_status {
-            OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMulti));
+            OBC_CUDA_TRY(allow_smem(kernel, kSmemMulti));
             { ProfScope ps("tc_pass2", stream); OBC_CUDA_TRY(launch_pdl(kernel, dim3(mgrid), dim3(kThreadsMulti), kSmemMulti, stream, 1, mq64, mo64, mk, mv, p)); }
             if (p.csplit > 1) {
                 ProfScope ps("partial_sum", stream);
@@ -1722,7 +1722,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     }
 
     auto launch = [&](auto kernel) -> obc_status {
-        OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes));
+        OBC_CUDA_TRY(allow_smem(kernel, kSmemBytes));
         { ProfScope ps("tc_pass2", stream); OBC_CUDA_TRY(launch_pdl(kernel, dim3(grid), dim3(kThreads), kSmemBytes, stream, 1, mq, mo, mk, mv, p)); }
         return OBC_OK;
     };

@@ -520,7 +520,7 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
 __global__ void __launch_bounds__(256)
 gather_kernel(int units, int Hkv, int idx_stride, int vecs, int elem_bytes,
               TensorView k, TensorView v, TensorView ko, TensorView vo,
-              const int32_t* __restrict__ idx, const float* __restrict__ s_in, float* __restrict__ s_out, int Nmax) {
+              const int32_t* __restrict__ idx, const float* __restrict__ s_in, float* __restrict__ s_out, int Nmax, uint32_t zero_rows) {
     pdl_wait();
     const int unit = blockIdx.y, b = unit / Hkv, g = unit % Hkv;
     const int total = idx_stride * vecs, quarter = (total + 3) / 4;
@@ -537,7 +537,7 @@ gather_kernel(int units, int Hkv, int idx_stride, int vecs, int elem_bytes,
     for (int u = 0; u < 4; ++u) {
         const int e = e0 + u * quarter;
         j[u] = e / vecs; c[u] = e % vecs;
-        src[u] = e < total ? idx[(size_t)unit * idx_stride + j[u]] : -1;
+        src[u] = e < total ? idx[(size_t)unit * idx_stride + j[u]] : -2;         // -2: no row at all
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -551,6 +551,11 @@ gather_kernel(int units, int Hkv, int idx_stride, int vecs, int elem_bytes,
             reinterpret_cast<uint4*>(kob + (size_t)j[u] * ko.st * eb)[c[u]] = kv[u];
             reinterpret_cast<uint4*>(vob + (size_t)j[u] * vo.st * eb)[c[u]] = vv[u];
             if (s_in && c[u] == 0) s_out[(size_t)unit * idx_stride + j[u]] = s_in[(size_t)unit * Nmax + src[u]];
+        } else if (zero_rows && src[u] == -1) {            // padding rows of outputs that nobody has cleared
+            const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+            if (zero_rows & OBC_ZERO_K) reinterpret_cast<uint4*>(kob + (size_t)j[u] * ko.st * eb)[c[u]] = zero;
+            if (zero_rows & OBC_ZERO_V) reinterpret_cast<uint4*>(vob + (size_t)j[u] * vo.st * eb)[c[u]] = zero;
+            if ((zero_rows & OBC_ZERO_SCORES) && c[u] == 0) s_out[(size_t)unit * idx_stride + j[u]] = 0.f;
         }
 }
 
@@ -667,8 +672,7 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
     const int C = select_cluster_size(s.Nmax, &seg_cap);
     if (C > 0) {
         const size_t smem = sizeof(ClusterShared) + (size_t)seg_cap * 8 + (size_t)s.pool_kernel * 4 + 16;
-        OBC_CUDA_TRY(cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        if (C > 8) OBC_CUDA_TRY(cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        OBC_CUDA_TRY(allow_smem(select_cluster_kernel, smem));
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(units * C)); cfg.blockDim = dim3(CL_NT); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
         cudaLaunchAttribute attr[1];
@@ -683,6 +687,7 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
         (void)cudaGetDevice(&dev);
         for (const auto& e : seen) if (e.C == C && e.smem == smem && e.dev == dev) max_clusters = e.max_clusters;
         if (max_clusters < 0) {
+            if (C > 8) OBC_CUDA_TRY(cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
             if (cudaOccupancyMaxActiveClusters(&max_clusters, select_cluster_kernel, &cfg) != cudaSuccess) { max_clusters = 0; (void)cudaGetLastError(); }
             seen[seen_next] = {dev, C, smem, max_clusters};
             seen_next = (seen_next + 1) % 4;
@@ -742,13 +747,13 @@ obc_status launch_select_static(const SelectShape& s, const float* scores, int32
 
 obc_status launch_gather(int B, int Hkv, int idx_stride, int Nmax, int elem_bytes,
                          TensorView k, TensorView v, TensorView ko, TensorView vo, const int32_t* idx,
-                         const float* s_in, float* s_out, cudaStream_t stream) {
+                         const float* s_in, float* s_out, uint32_t zero_rows, cudaStream_t stream) {
     const int vecs = kD * elem_bytes / 16;
     const long long total = ((long long)idx_stride * vecs + 3) / 4;    // four vectors per thread
     {
         ProfScope ps("gather", stream);
         OBC_CUDA_TRY(launch_pdl(gather_kernel, dim3((unsigned)((total + 255) / 256), B * Hkv), dim3(256), 0, stream, 1,
-                                B * Hkv, Hkv, idx_stride, vecs, elem_bytes, k, v, ko, vo, idx, s_in, s_out, Nmax));
+                                B * Hkv, Hkv, idx_stride, vecs, elem_bytes, k, v, ko, vo, idx, s_in, s_out, Nmax, zero_rows));
     }
     return OBC_OK;
 }

@@ -114,6 +114,26 @@ def test_compact_bit_exact(dtype):
             assert np.array_equal(so[b, h, :n].cpu().numpy(), scores[b, h][want_idx[b, h, :n]])
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("kept,stride", [(0, 1), (1, 5), (37, 64)])
+def test_compact_padding_rows(dtype, kept, stride):
+    """Rows whose index is -1: zeros in outputs that the call allocates, untouched in outputs that the caller brings."""
+    g = torch.Generator(device="cuda").manual_seed(kept + stride)
+    k = torch.randn((1, 2, 90, 128), generator=g, device="cuda").to(dtype)
+    v = torch.randn((1, 2, 90, 128), generator=g, device="cuda").to(dtype)
+    s = torch.rand((1, 2, 90), generator=g, device="cuda")
+    idx = torch.full((1, 2, stride), -1, dtype=torch.int32, device="cuda")
+    idx[..., :kept] = torch.arange(kept, dtype=torch.int32, device="cuda") * 2
+    filler = [torch.full((1, 2, stride, 128), 7.0, dtype=dtype, device="cuda") for _ in range(3)]   # so that fresh memory is not zero
+    del filler
+    ko, vo, so = api.obc_compact(k, v, idx, scores_in=s)
+    for out, src in ((ko, k), (vo, v), (so, s)):
+        assert torch.equal(out[:, :, :kept], src[:, :, :2 * kept:2]) and (out[:, :, kept:] == 0).all()
+    mine = torch.full_like(ko, 3.0)
+    ko2, vo2 = api.obc_compact(k, v, idx, k_out=mine)
+    assert ko2 is mine and torch.equal(ko2[:, :, :kept], ko[:, :, :kept]) and (ko2[:, :, kept:] == 3.0).all() and torch.equal(vo2, vo)
+
+
 def test_whole_prefill_path_config1():
     # score -> select -> compact end to end; selection compared on the GPU's own fp32 scores
     case, run = synth.config(1)
