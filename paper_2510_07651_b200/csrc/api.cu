@@ -273,7 +273,7 @@ obc_status obc_select_adaptive_workspace(const obc_select_params* p, float safeg
     SelectShape s; int n_safe = 0;
     obc_status st = resolve_adaptive(p, safeguard, &s, &n_safe);
     if (st != OBC_OK) return st;
-    *bytes = select_adaptive_workspace_bytes(s, n_safe);
+    *bytes = select_adaptive_workspace_bytes(s);
     return OBC_OK;
 }
 
@@ -283,7 +283,7 @@ obc_status obc_select_adaptive(const obc_select_params* p, float safeguard, cons
     obc_status st = resolve_adaptive(p, safeguard, &s, &n_safe);
     if (st != OBC_OK) return st;
     if (!scores || !idx || !counts) return OBC_ERR_NULL;
-    if (!workspace || workspace_bytes < select_adaptive_workspace_bytes(s, n_safe)) return OBC_ERR_WORKSPACE;
+    if (!workspace || workspace_bytes < select_adaptive_workspace_bytes(s)) return OBC_ERR_WORKSPACE;
     if (((uintptr_t)workspace & 255) != 0) return OBC_ERR_ALIGN;
     return launch_select_adaptive(s, n_safe, scores, idx, counts, workspace, (cudaStream_t)stream);
 }

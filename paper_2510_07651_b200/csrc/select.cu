@@ -29,6 +29,26 @@ __device__ __forceinline__ uint32_t float_key(float x) {
 __device__ __forceinline__ int seq_len(const SelectShape& s, int b) { return s.seq_lens ? s.seq_lens[b] : s.Nmax; }
 __device__ __forceinline__ int budget_of(const SelectShape& s, int b) { return s.budgets ? s.budgets[b] : s.budget; }
 
+// key of token p of a head with scores sc: the pooled score of a candidate (lo <= p < hi), 0 (below every candidate) elsewhere
+__device__ __forceinline__ uint32_t pooled_key(const SelectShape& s, const float* __restrict__ sc, int p, int lo, int hi) {
+    if (p < lo || p >= hi) return 0u;
+    const int half = s.pool_kernel / 2;
+    float val;
+    if (s.pool_mode == OBC_POOL_NONE || s.pool_kernel == 1) {
+        val = sc[p];
+    } else if (s.pool_mode == OBC_POOL_MAX) {
+        val = -INFINITY;
+        for (int t = p - half; t <= p + half; ++t)
+            if (t >= lo && t < hi) val = fmaxf(val, sc[t]);
+    } else {
+        val = 0.f;
+        for (int t = p - half; t <= p + half; ++t)
+            if (t >= lo && t < hi) val = __fadd_rn(val, sc[t]);
+        val = __fdiv_rn(val, (float)s.pool_kernel);
+    }
+    return float_key(val);
+}
+
 __global__ void __launch_bounds__(256)
 pool_key_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* __restrict__ keys) {
     pdl_wait();
@@ -36,49 +56,219 @@ pool_key_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* __res
     const int N = seq_len(s, b), lo = s.n_sink, hi = N - s.n_recent;
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= s.Nmax) return;
-    const float* sc = scores + (size_t)unit * s.Nmax;
-    uint32_t key = 0;
-    if (p >= lo && p < hi) {
-        float val;
-        const int half = s.pool_kernel / 2;
-        if (s.pool_mode == OBC_POOL_NONE || s.pool_kernel == 1) {
-            val = sc[p];
-        } else if (s.pool_mode == OBC_POOL_MAX) {
-            val = -INFINITY;
-            for (int t = p - half; t <= p + half; ++t)
-                if (t >= lo && t < hi) val = fmaxf(val, sc[t]);
-        } else {
-            val = 0.f;
-            for (int t = p - half; t <= p + half; ++t)
-                if (t >= lo && t < hi) val = __fadd_rn(val, sc[t]);
-            val = __fdiv_rn(val, (float)s.pool_kernel);
-        }
-        key = float_key(val);
+    keys[(size_t)unit * s.Nmax + p] = pooled_key(s, scores + (size_t)unit * s.Nmax, p, lo, hi);
+}
+
+// ---- head-adaptive budgets --------------------------------------------------------------------------------
+// Every head keeps its n_safe best candidates; the other rem = H (n_hh - n_safe) slots of a batch item go to the best
+// remaining candidates of all its heads.  With cnt_h(x) = candidates of head h whose key is at least x, the heads keep
+// F(x) = sum_h max(0, cnt_h(x) - n_safe) tokens beyond their guaranteed ones if x is the threshold, so the threshold T is
+// the largest key with F(T) >= rem, and what a head keeps is its own best max(n_safe, cnt_h(T + 1)) + (its share of the
+// candidates equal to T) tokens: only the COUNTS have to be found across heads, and the per-head selection does the rest.
+// T comes out of three histogram levels per head (11 + 11 + 10 bits) over the whole chip:
+//   adaptive_pool_kernel   pooled keys, level-1 histograms
+//   adaptive_hist_kernel   (levels 2 and 3) every CTA finds the digit of the level before, then counts its keys below it
+//   the selection kernels  last digit, tie shares, scored tokens of the head
+// Every histogram row comes with 32 sums over equal runs of its bins, so that a digit is found in two round trips to L2
+// (32 runs of every head, then the bins of one run) by any CTA that needs it.
+// Latency bound: 8 heads x 32k keys 5.4 + 4.6 + 5.2 us and 2 us in the selection; 8 x 98k keys 8.1 + 6.1 + 6.0 us.  (Ranking
+// all heads' keys as one sequence in one 16-CTA cluster took 20 us for the former and, where the keys did not fit one, by
+// one CTA, 1.07 ms for the latter.)
+constexpr int AD_NT = 512;
+constexpr int AD_BINS = 2048;                 // bins of levels 1 and 2; level 3 has half of them
+constexpr int AD_ROW = AD_BINS + 32;          // a head's row: bins, then the sums over 32 runs of them
+
+struct AdaptiveLevels {                       // in the workspace; scores across heads are ranked when hist != null
+    uint32_t* hist;                           // [3 levels][units][AD_ROW]
+    uint32_t* above;                          // [2][units]: candidates above the digits of level 1, of levels 1 and 2
+    uint32_t* digit;                          // [B][2]: level-1 and level-2 digit of T
+    int32_t* counts;                          // [units]: tokens kept per head, or -1 (the caller's)
+    uint32_t n_safe;
+    int chunk;                                // keys per CTA of the passes
+    int units;
+    __device__ __forceinline__ uint32_t* row(int level, int unit) const { return hist + ((size_t)level * units + unit) * AD_ROW; }
+};
+
+struct AdaptiveFind { uint32_t run_sum[32], bin_sum[64], run, digit; };     // shared memory of the search
+
+__device__ __forceinline__ uint32_t warp_suffix(uint32_t x) {               // sum over the lanes >= lane
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_down_sync(0xffffffffu, x, o);
+        if (lane + o < 32) x += t;
     }
-    keys[(size_t)unit * s.Nmax + p] = key;
+    return x;
+}
+
+// Largest bin d of level LEVEL (0..2) with sum_h max(0, above[h] + (candidates of head h in bins >= d) - n_safe) >= rem,
+// over the H heads from unit u0 on.  All threads of the block call it.
+template <int LEVEL>
+__device__ uint32_t adaptive_find(const AdaptiveLevels& lv, int u0, int H, uint32_t rem, AdaptiveFind& sh) {
+    constexpr int PER = LEVEL == 2 ? 32 : 64;                  // bins per run
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, warps = (int)blockDim.x >> 5;
+    const uint32_t* above = LEVEL == 0 ? nullptr : lv.above + (size_t)(LEVEL - 1) * lv.units + u0;
+    auto beyond = [&](uint32_t c) { return c > lv.n_safe ? c - lv.n_safe : 0u; };
+    if (tid < 32) sh.run_sum[tid] = 0;
+    if (tid < 64) sh.bin_sum[tid] = 0;
+    if (tid == 0) { sh.run = 0; sh.digit = 0; }
+    __syncthreads();
+    for (int h = warp; h < H; h += warps) {
+        const uint32_t c = warp_suffix(lv.row(LEVEL, u0 + h)[AD_BINS + lane]) + (above ? above[h] : 0u);
+        if (beyond(c)) atomicAdd(&sh.run_sum[lane], beyond(c));
+    }
+    __syncthreads();
+    if (tid < 32 && sh.run_sum[tid] >= rem && (tid == 31 || sh.run_sum[tid + 1] < rem)) sh.run = (uint32_t)tid;
+    __syncthreads();
+    const int run = (int)sh.run;
+    for (int h = warp; h < H; h += warps) {
+        const uint32_t* row = lv.row(LEVEL, u0 + h);
+        const uint32_t runs = row[AD_BINS + lane];
+        const uint32_t x0 = row[run * PER + lane], x1 = PER == 64 ? row[run * PER + 32 + lane] : 0u;
+        uint32_t up = warp_suffix(lane > run ? runs : 0u);     // candidates in the runs above, in lane 0
+        up = __shfl_sync(0xffffffffu, up, 0) + (above ? above[h] : 0u);
+        const uint32_t s1 = warp_suffix(x1), s0 = warp_suffix(x0) + __shfl_sync(0xffffffffu, s1, 0);
+        if (beyond(up + s0)) atomicAdd(&sh.bin_sum[lane], beyond(up + s0));
+        if (PER == 64 && beyond(up + s1)) atomicAdd(&sh.bin_sum[32 + lane], beyond(up + s1));
+    }
+    __syncthreads();
+    if (tid < PER && sh.bin_sum[tid] >= rem && (tid == PER - 1 || sh.bin_sum[tid + 1] < rem)) sh.digit = (uint32_t)(run * PER + tid);
+    __syncthreads();
+    return sh.digit;
+}
+
+// candidates of the unit above the digits found so far, level LEVEL's being d (called by a whole warp, same result in every lane)
+template <int LEVEL>
+__device__ __forceinline__ uint32_t adaptive_above(const AdaptiveLevels& lv, int unit, uint32_t d) {
+    constexpr int PER = LEVEL == 2 ? 32 : 64;
+    const int lane = threadIdx.x & 31, run = (int)d / PER, at = (int)d % PER;
+    const uint32_t* row = lv.row(LEVEL, unit);
+    uint32_t x = lane > run ? row[AD_BINS + lane] : 0u;
+    if (lane > at) x += row[run * PER + lane];
+    if (PER == 64 && lane + 32 > at) x += row[run * PER + 32 + lane];
+    x = __shfl_sync(0xffffffffu, warp_suffix(x), 0);
+    return x + (LEVEL == 0 ? 0u : lv.above[(size_t)(LEVEL - 1) * lv.units + unit]);
+}
+
+// slots of a batch item's heads beyond the guaranteed ones; -1 when the budget does not fit the sequence
+__device__ __forceinline__ int adaptive_rem(const SelectShape& s, int b, uint32_t n_safe) {
+    const int N = seq_len(s, b), lo = s.n_sink, hi = N - s.n_recent, n_hh = s.budget - s.n_sink - s.n_recent;
+    if (N > s.Nmax || hi < lo || n_hh < 0 || n_hh > hi - lo) return -1;
+    return s.Hkv * (n_hh - (int)n_safe);
+}
+
+// Scored tokens that head `unit` keeps (-1: the budget does not fit): the last digit of T and the tie shares.  All threads
+// of the block call it.
+__device__ int adaptive_hh(const SelectShape& s, const AdaptiveLevels& lv, int unit, AdaptiveFind& sh) {
+    const int b = unit / s.Hkv, u0 = b * s.Hkv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
+    const int rem = adaptive_rem(s, b, lv.n_safe);
+    if (rem <= 0) return rem < 0 ? -1 : (int)lv.n_safe;
+    const uint32_t d = adaptive_find<2>(lv, u0, s.Hkv, (uint32_t)rem, sh);
+    auto beyond = [&](uint32_t c) { return c > lv.n_safe ? c - lv.n_safe : 0u; };
+    // sums over the heads: slots that the candidates above T take, and candidates equal to T of the heads before this one
+    if (threadIdx.x < 2) sh.run_sum[threadIdx.x] = 0;
+    __syncthreads();
+    for (int h = warp; h < s.Hkv; h += warps) {
+        const uint32_t up = adaptive_above<2>(lv, u0 + h, d), ties = beyond(up + lv.row(2, u0 + h)[d]) - beyond(up);
+        if (lane == 0) {
+            atomicAdd(&sh.run_sum[0], beyond(up));
+            if (u0 + h < unit) atomicAdd(&sh.run_sum[1], ties);
+            if (u0 + h == unit) { sh.bin_sum[0] = up; sh.bin_sum[1] = ties; }
+        }
+    }
+    __syncthreads();
+    const uint32_t left = (uint32_t)rem - sh.run_sum[0], before = sh.run_sum[1], up = sh.bin_sum[0], ties = sh.bin_sum[1];
+    return (int)(max(lv.n_safe, up) + (before < left ? min(ties, left - before) : 0u));     // ties: lowest head first
+}
+
+// adds a CTA's histogram of `bins` bins to the unit's row, with the sums over its 32 runs
+__device__ __forceinline__ void adaptive_flush(const uint32_t* hist, int bins, uint32_t* row) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, per = bins / 32;
+    for (int i = tid; i < bins; i += AD_NT)
+        if (hist[i]) atomicAdd(&row[i], hist[i]);
+    for (int r = warp; r < 32; r += AD_NT / 32) {
+        uint32_t x = hist[r * per + lane];
+        if (per == 64) x += hist[r * per + 32 + lane];
+        x = warp_suffix(x);
+        if (lane == 0 && x) atomicAdd(&row[AD_BINS + r], x);
+    }
+}
+
+__global__ void __launch_bounds__(AD_NT)
+adaptive_pool_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* __restrict__ keys, AdaptiveLevels lv) {
+    __shared__ uint32_t hist[AD_BINS];
+    const int unit = blockIdx.y, b = unit / s.Hkv, c0 = blockIdx.x * lv.chunk, c1 = min(c0 + lv.chunk, s.Nmax);
+    for (int d = threadIdx.x; d < AD_BINS; d += AD_NT) hist[d] = 0;
+    __syncthreads();
+    pdl_wait();
+    const int lo = s.n_sink, hi = min(seq_len(s, b), s.Nmax) - s.n_recent;
+    const float* sc = scores + (size_t)unit * s.Nmax;
+#pragma unroll 4
+    for (int p = c0 + threadIdx.x; p < c1; p += AD_NT) {
+        const uint32_t key = pooled_key(s, sc, p, lo, hi);
+        keys[(size_t)unit * s.Nmax + p] = key;
+        if (key) atomicAdd(&hist[key >> 21], 1u);
+    }
+    __syncthreads();
+    adaptive_flush(hist, AD_BINS, lv.row(0, unit));
+}
+
+// level 2 or 3: the digit that the level before settles, then the histogram of the keys that share the digits so far
+template <int LEVEL>
+__global__ void __launch_bounds__(AD_NT)
+adaptive_hist_kernel(SelectShape s, const uint32_t* __restrict__ keys, AdaptiveLevels lv) {
+    __shared__ uint32_t hist[AD_BINS];
+    __shared__ AdaptiveFind sh;
+    constexpr int BINS = LEVEL == 2 ? 2048 : 1024;
+    for (int d = threadIdx.x; d < BINS; d += AD_NT) hist[d] = 0;
+    pdl_wait();
+    const int unit = blockIdx.y, b = unit / s.Hkv, u0 = b * s.Hkv, c0 = blockIdx.x * lv.chunk, c1 = min(c0 + lv.chunk, s.Nmax);
+    const int rem = adaptive_rem(s, b, lv.n_safe);
+    if (rem <= 0) return;                                      // nothing to share out (adaptive_hh sees to it)
+    const uint32_t d = adaptive_find<LEVEL - 2>(lv, u0, s.Hkv, (uint32_t)rem, sh);
+    if (unit == u0 && blockIdx.x == 0) {                       // one CTA per batch item leaves the result for the next level
+        for (int h = threadIdx.x >> 5; h < s.Hkv; h += AD_NT / 32) {
+            const uint32_t up = adaptive_above<LEVEL - 2>(lv, u0 + h, d);
+            if ((threadIdx.x & 31) == 0) lv.above[(size_t)(LEVEL - 2) * lv.units + u0 + h] = up;
+        }
+        if (threadIdx.x == 0) lv.digit[b * 2 + (LEVEL - 2)] = d;
+    }
+    const uint32_t prefix = LEVEL == 2 ? d : lv.digit[b * 2] << 11 | d;
+    constexpr int SHIFT = LEVEL == 2 ? 21 : 10, NEXT = LEVEL == 2 ? 10 : 0;
+#pragma unroll 8
+    for (int p = c0 + threadIdx.x; p < c1; p += AD_NT) {
+        const uint32_t key = keys[(size_t)unit * s.Nmax + p];
+        if (key >> SHIFT == prefix) atomicAdd(&hist[(key >> NEXT) & (BINS - 1)], 1u);
+    }
+    __syncthreads();
+    adaptive_flush(hist, BINS, lv.row(LEVEL - 1, unit));
 }
 
 constexpr int SEL_NT = 1024;
 
 __global__ void __launch_bounds__(SEL_NT)
-select_kernel(SelectShape s, const uint32_t* __restrict__ keys_all, int32_t* __restrict__ idx_all) {
+select_kernel(SelectShape s, const uint32_t* __restrict__ keys_all, int32_t* __restrict__ idx_all, AdaptiveLevels ad) {
     pdl_wait();
     __shared__ uint32_t hist[256];
     __shared__ uint32_t sh_prefix, sh_remaining;
     __shared__ uint32_t warp_gt[32], warp_eq[32];
 
     const int unit = blockIdx.x, b = unit / s.Hkv;
-    const int N = seq_len(s, b), budget = budget_of(s, b);
+    const int N = seq_len(s, b);
     const int lo = s.n_sink, hi = N - s.n_recent, n = hi - lo;
-    const int n_hh = budget - s.n_sink - s.n_recent;
+    __shared__ AdaptiveFind ad_sh;
+    const int n_hh = ad.hist ? adaptive_hh(s, ad, unit, ad_sh) : budget_of(s, b) - s.n_sink - s.n_recent;
+    const int budget = n_hh + s.n_sink + s.n_recent;
     const uint32_t* keys = keys_all + (size_t)unit * s.Nmax;
     int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
     if (n_hh < 0 || n_hh > n || budget > s.idx_stride || N > s.Nmax || hi < lo) {   // bad per-sequence budget
         for (int j = tid; j < s.idx_stride; j += SEL_NT) idx[j] = -1;
+        if (ad.hist && tid == 0) ad.counts[unit] = -1;
         return;
     }
+    if (ad.hist && tid == 0) ad.counts[unit] = budget;
     // protected ranges and padding
     for (int j = tid; j < s.n_sink; j += SEL_NT) idx[j] = j;
     for (int j = tid; j < s.n_recent; j += SEL_NT) idx[s.n_sink + n_hh + j] = hi + j;
@@ -235,7 +425,7 @@ __device__ __forceinline__ void find_bin(const uint32_t* hist, uint32_t remainin
 
 __global__ void __launch_bounds__(CL_NT)
 select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* __restrict__ idx_all, int seg_cap,
-                      const uint32_t* __restrict__ keys_in) {
+                      const uint32_t* __restrict__ keys_in, AdaptiveLevels ad) {
     extern __shared__ __align__(16) uint8_t sel_smem[];
     ClusterShared& sh = *reinterpret_cast<ClusterShared*>(sel_smem);
     uint32_t* keys = reinterpret_cast<uint32_t*>(sel_smem + ((sizeof(ClusterShared) + 15) & ~(size_t)15));   // 16-byte aligned
@@ -245,9 +435,11 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
     const int unit = blockIdx.x / C, b = unit / s.Hkv;
-    const int N = seq_len(s, b), budget = budget_of(s, b);
+    const int N = seq_len(s, b);
     const int lo = s.n_sink, hi = N - s.n_recent, n = hi - lo;
-    const int n_hh = budget - s.n_sink - s.n_recent;
+    // (the search across heads borrows the space of a histogram that is cleared below)
+    const int n_hh = ad.hist ? adaptive_hh(s, ad, unit, *reinterpret_cast<AdaptiveFind*>(&sh.local[0])) : budget_of(s, b) - s.n_sink - s.n_recent;
+    const int budget = n_hh + s.n_sink + s.n_recent;
     int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gtid = rank * CL_NT + tid, gthreads = C * CL_NT;
@@ -255,8 +447,10 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     // these tests depend on the unit only, so all CTAs of the cluster leave together
     if (n_hh < 0 || n_hh > n || budget > s.idx_stride || N > s.Nmax || hi < lo) {   // bad per-sequence budget
         for (int j = gtid; j < s.idx_stride; j += gthreads) idx[j] = -1;
+        if (ad.hist && gtid == 0) ad.counts[unit] = -1;
         return;
     }
+    if (ad.hist && gtid == 0) ad.counts[unit] = budget;
     for (int j = gtid; j < s.n_sink; j += gthreads) idx[j] = j;
     for (int j = gtid; j < s.n_recent; j += gthreads) idx[s.n_sink + n_hh + j] = hi + j;
     for (int j = budget + gtid; j < s.idx_stride; j += gthreads) idx[j] = -1;
@@ -560,23 +754,6 @@ gather_kernel(int units, int Hkv, int idx_stride, int vecs, int elem_bytes,
 }
 
 
-// ---- head-adaptive budgets: pieces around the two selection kernels ------------------------------------
-// keys of the tokens every head keeps by its own ranking are raised to the largest key, so that the
-// ranking across heads takes them first
-__global__ void __launch_bounds__(256)
-adaptive_boost_kernel(int units, int Nmax, int n_sink, int n_safe, int safe_stride,
-                      const int32_t* __restrict__ idx_safe, uint32_t* __restrict__ keys) {
-    pdl_wait();
-    const int unit = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (unit >= units || j >= n_safe) return;
-    const int p = idx_safe[(size_t)unit * safe_stride + n_sink + j];
-    if (p >= 0 && p < Nmax) keys[(size_t)unit * Nmax + p] = 0xffffffffu;
-}
-
-// vidx [B][total]: the tokens chosen across the heads of a batch item, ascending in h * Nmax + p.  One block
-// per (b, h) finds its head's stretch by binary search and writes the head's row of idx: sinks, chosen
-// tokens, recent tail, -1 padding; counts[b, h] = tokens kept (or -1, with a row of -1, when the row does
-// not fit idx_stride or the budget does not fit the sequence).
 // First position of the ascending array a[0, n) whose value is >= v (n if none), found by the whole block: every
 // round the threads probe evenly spaced positions of the remaining range at once, so 16384 entries take three
 // round trips to memory where a binary search by one thread takes fourteen.  Called by all threads of the block.
@@ -591,33 +768,6 @@ __device__ __forceinline__ int block_lower_bound(int n, Less value_below) {
         else { const int last = lo + (cnt - 1) * step; lo = last + 1; hi = min(last + step, hi); }
     }
     return lo;
-}
-
-__global__ void __launch_bounds__(256)
-adaptive_split_kernel(SelectShape s, int total, const int32_t* __restrict__ vidx_all,
-                      int32_t* __restrict__ idx_all, int32_t* __restrict__ counts) {
-    pdl_wait();
-    const int unit = blockIdx.x, b = unit / s.Hkv, h = unit % s.Hkv;
-    const int N = seq_len(s, b), lo = s.n_sink, hi = N - s.n_recent;
-    const int n_hh = s.budget - s.n_sink - s.n_recent;
-    const int32_t* vidx = vidx_all + (size_t)b * total;
-    int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
-    auto lower_bound = [&](int v) {                       // first position whose virtual index is >= v
-        return block_lower_bound(total, [&](int i) { return vidx[i] < v; });
-    };
-    const int seg0 = lower_bound(h * s.Nmax), seg1 = lower_bound((h + 1) * s.Nmax), c = seg1 - seg0;
-    const int kept = s.n_sink + c + s.n_recent;
-    const bool bad = N > s.Nmax || hi < lo || n_hh < 0 || n_hh > hi - lo || kept > s.idx_stride;
-    if (bad) {
-        for (int j = threadIdx.x; j < s.idx_stride; j += blockDim.x) idx[j] = -1;
-        if (threadIdx.x == 0) counts[unit] = -1;
-        return;
-    }
-    for (int j = threadIdx.x; j < s.n_sink; j += blockDim.x) idx[j] = j;
-    for (int j = threadIdx.x; j < c; j += blockDim.x) idx[s.n_sink + j] = vidx[seg0 + j] - h * s.Nmax;
-    for (int j = threadIdx.x; j < s.n_recent; j += blockDim.x) idx[s.n_sink + c + j] = hi + j;
-    for (int j = kept + threadIdx.x; j < s.idx_stride; j += blockDim.x) idx[j] = -1;
-    if (threadIdx.x == 0) counts[unit] = kept;
 }
 
 // A token shard's share of the kept indices: row (b, h) of idx is ascending (padding -1 at the end), so the entries
@@ -660,12 +810,12 @@ static int select_cluster_size(int Nmax, int* seg_cap) {
 
 // keys_in: when given, [units][Nmax] keys that take the place of pooling `scores` (which may then be null);
 // `ws` is then not written
-static obc_status launch_select_impl(const SelectShape& s, const float* scores, const uint32_t* keys_in, int32_t* idx,
+static obc_status launch_select_impl(const SelectShape& s, const float* scores, const uint32_t* keys_in, AdaptiveLevels ad, int32_t* idx,
                                      void* ws, cudaStream_t stream);
 obc_status launch_select(const SelectShape& s, const float* scores, int32_t* idx, void* ws, cudaStream_t stream) {
-    return launch_select_impl(s, scores, nullptr, idx, ws, stream);
+    return launch_select_impl(s, scores, nullptr, AdaptiveLevels{}, idx, ws, stream);
 }
-static obc_status launch_select_impl(const SelectShape& s, const float* scores, const uint32_t* keys_in, int32_t* idx,
+static obc_status launch_select_impl(const SelectShape& s, const float* scores, const uint32_t* keys_in, AdaptiveLevels ad, int32_t* idx,
                                      void* ws, cudaStream_t stream) {
     const int units = s.B * s.Hkv;
     int seg_cap = 0;
@@ -694,18 +844,18 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
         }
         if (max_clusters > 0) {
             { ProfScope ps("select_cluster", stream);
-              OBC_CUDA_TRY(launch_pdl(select_cluster_kernel, dim3((unsigned)(units * C)), dim3(CL_NT), smem, stream, C, s, scores, idx, seg_cap, keys_in)); }
+              OBC_CUDA_TRY(launch_pdl(select_cluster_kernel, dim3((unsigned)(units * C)), dim3(CL_NT), smem, stream, C, s, scores, idx, seg_cap, keys_in, ad)); }
             return OBC_OK;
         }
         (void)cudaGetLastError();                  // the device cannot host such a cluster: one CTA per head
     }
     if (keys_in) {
-        { ProfScope ps("select", stream); OBC_CUDA_TRY(launch_pdl(select_kernel, dim3(units), dim3(SEL_NT), 0, stream, 1, s, keys_in, idx)); }
+        { ProfScope ps("select", stream); OBC_CUDA_TRY(launch_pdl(select_kernel, dim3(units), dim3(SEL_NT), 0, stream, 1, s, keys_in, idx, ad)); }
         return OBC_OK;
     }
     uint32_t* keys = (uint32_t*)ws;
     { ProfScope ps("pool_key", stream); OBC_CUDA_TRY(launch_pdl(pool_key_kernel, dim3((s.Nmax + 255) / 256, units), dim3(256), 0, stream, 1, s, scores, keys)); }
-    { ProfScope ps("select", stream); OBC_CUDA_TRY(launch_pdl(select_kernel, dim3(units), dim3(SEL_NT), 0, stream, 1, s, (const uint32_t*)keys, idx)); }
+    { ProfScope ps("select", stream); OBC_CUDA_TRY(launch_pdl(select_kernel, dim3(units), dim3(SEL_NT), 0, stream, 1, s, (const uint32_t*)keys, idx, AdaptiveLevels{})); }
     return OBC_OK;
 }
 
@@ -741,7 +891,7 @@ obc_status launch_select_static(const SelectShape& s, const float* scores, int32
     if (st != OBC_OK) return st;
     // every key a head reads is written by pool_key_kernel of this call: nothing has to be cleared
     { ProfScope ps("pool_key", stream); OBC_CUDA_TRY(launch_pdl(pool_key_kernel, dim3((s.Nmax + 255) / 256, units), dim3(256), 0, stream, 1, s, scores, keys)); }
-    { ProfScope ps("select", stream); OBC_CUDA_TRY(launch_pdl(select_kernel, dim3(units), dim3(SEL_NT), 0, stream, 1, s, (const uint32_t*)keys, idx)); }
+    { ProfScope ps("select", stream); OBC_CUDA_TRY(launch_pdl(select_kernel, dim3(units), dim3(SEL_NT), 0, stream, 1, s, (const uint32_t*)keys, idx, AdaptiveLevels{})); }
     return OBC_OK;
 }
 
@@ -759,50 +909,38 @@ obc_status launch_gather(int B, int Hkv, int idx_stride, int Nmax, int elem_byte
 }
 
 // ---- head-adaptive budgets -------------------------------------------------------------------------------
-// workspace: pooled keys [units][Nmax] | every head's own selection [units][n_sink + n_safe + n_recent] |
-// the selection across heads [B][Hkv * n_hh]
-struct AdaptivePlan { size_t off_keys, off_safe, off_vidx, bytes; int safe_stride, total; };
-static AdaptivePlan make_adaptive_plan(const SelectShape& s, int n_safe) {
+// workspace: the three histogram levels of every head (cleared by the call) | pooled keys | small results of the search
+struct AdaptivePlan { size_t off_hist, off_keys, off_above, off_digit, bytes; };
+static AdaptivePlan make_adaptive_plan(const SelectShape& s) {
     AdaptivePlan p{};
     const size_t units = (size_t)s.B * s.Hkv;
-    const int n_hh = s.budget - s.n_sink - s.n_recent;
-    p.safe_stride = s.n_sink + n_safe + s.n_recent;
-    p.total = s.Hkv * (n_hh > 0 ? n_hh : 0);
     size_t off = 0;
-    p.off_keys = off; off = align_up(off + units * s.Nmax * 4, 256);
-    p.off_safe = off; off = align_up(off + units * (size_t)(p.safe_stride > 0 ? p.safe_stride : 1) * 4, 256);
-    p.off_vidx = off; off = align_up(off + (size_t)s.B * (size_t)(p.total > 0 ? p.total : 1) * 4, 256);
+    p.off_hist = off;  off = align_up(off + 3 * units * AD_ROW * 4, 256);
+    p.off_keys = off;  off = align_up(off + units * s.Nmax * 4, 256);
+    p.off_above = off; off = align_up(off + 2 * units * 4, 256);
+    p.off_digit = off; off = align_up(off + (size_t)s.B * 8, 256);
     p.bytes = off;
     return p;
 }
-size_t select_adaptive_workspace_bytes(const SelectShape& s, int n_safe) { return make_adaptive_plan(s, n_safe).bytes; }
+size_t select_adaptive_workspace_bytes(const SelectShape& s) { return make_adaptive_plan(s).bytes; }
 
 obc_status launch_select_adaptive(const SelectShape& s, int n_safe, const float* scores, int32_t* idx, int32_t* counts,
                                   void* ws, cudaStream_t stream) {
-    const AdaptivePlan plan = make_adaptive_plan(s, n_safe);
+    const AdaptivePlan plan = make_adaptive_plan(s);
     const int units = s.B * s.Hkv;
-    uint32_t* keys = (uint32_t*)((char*)ws + plan.off_keys);
-    int32_t* idx_safe = (int32_t*)((char*)ws + plan.off_safe);
-    int32_t* vidx = (int32_t*)((char*)ws + plan.off_vidx);
-    { ProfScope ps("pool_key", stream); OBC_CUDA_TRY(launch_pdl(pool_key_kernel, dim3((s.Nmax + 255) / 256, units), dim3(256), 0, stream, 1, s, scores, keys)); }
-    if (n_safe > 0) {
-        SelectShape own = s;                              // every head's own ranking, n_safe scored tokens each
-        own.budget = s.n_sink + n_safe + s.n_recent; own.budgets = nullptr; own.idx_stride = plan.safe_stride;
-        obc_status st = launch_select_impl(own, nullptr, keys, idx_safe, nullptr, stream);
-        if (st != OBC_OK) return st;
-        { ProfScope ps("adaptive_boost", stream);
-          OBC_CUDA_TRY(launch_pdl(adaptive_boost_kernel, dim3((n_safe + 255) / 256, units), dim3(256), 0, stream, 1, units, s.Nmax, s.n_sink, n_safe, plan.safe_stride, (const int32_t*)idx_safe, keys)); }
-    }
-    if (plan.total > 0) {
-        // all heads of a batch item as one sequence of Hkv * Nmax keys (the keys of protected and padding
-        // positions are 0 and rank below every candidate); equal keys keep the lowest head, then the lowest index
-        SelectShape all{s.B, 1, s.Hkv * s.Nmax, nullptr, plan.total, nullptr, plan.total, 0, 0, OBC_POOL_NONE, 1};
-        obc_status st = launch_select_impl(all, nullptr, keys, vidx, nullptr, stream);
-        if (st != OBC_OK) return st;
-    }
-    { ProfScope ps("adaptive_split", stream);
-      OBC_CUDA_TRY(launch_pdl(adaptive_split_kernel, dim3(units), dim3(256), 0, stream, 1, s, plan.total, (const int32_t*)vidx, idx, counts)); }
-    return OBC_OK;
+    char* w = (char*)ws;
+    uint32_t* keys = (uint32_t*)(w + plan.off_keys);
+    // about two CTAs per SM: each of them repeats the search through the heads' histograms
+    const long long per = ((long long)units * s.Nmax + 2 * 148 - 1) / (2 * 148);
+    const int chunk = (int)(per < 2048 ? 2048 : (per + AD_NT - 1) / AD_NT * AD_NT);
+    const AdaptiveLevels lv{(uint32_t*)(w + plan.off_hist), (uint32_t*)(w + plan.off_above), (uint32_t*)(w + plan.off_digit), counts,
+                            (uint32_t)n_safe, chunk, units};
+    const dim3 grid((unsigned)((s.Nmax + chunk - 1) / chunk), (unsigned)units);
+    OBC_CUDA_TRY(cudaMemsetAsync(w + plan.off_hist, 0, 3 * (size_t)units * AD_ROW * 4, stream));
+    { ProfScope ps("adaptive_pool", stream); OBC_CUDA_TRY(launch_pdl(adaptive_pool_kernel, grid, dim3(AD_NT), 0, stream, 1, s, scores, keys, lv)); }
+    { ProfScope ps("adaptive_hist", stream); OBC_CUDA_TRY(launch_pdl(adaptive_hist_kernel<2>, grid, dim3(AD_NT), 0, stream, 1, s, (const uint32_t*)keys, lv)); }
+    { ProfScope ps("adaptive_hist", stream); OBC_CUDA_TRY(launch_pdl(adaptive_hist_kernel<3>, grid, dim3(AD_NT), 0, stream, 1, s, (const uint32_t*)keys, lv)); }
+    return launch_select_impl(s, nullptr, keys, lv, idx, nullptr, stream);
 }
 
 }  // namespace obc

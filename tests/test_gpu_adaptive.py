@@ -45,6 +45,22 @@ def test_adaptive_ragged_lengths_and_random_scores():
     assert np.array_equal(cnt, want_cnt) and np.array_equal(idx, want_idx)
 
 
+@pytest.mark.parametrize("B,Hkv,N,budget,levels", [
+    (1, 1, 50, 20, 3),             # one head: the ranking across heads is its own
+    (2, 33, 700, 90, 5),           # more heads than a warp has lanes, ties in every head
+    (1, 17, 2049, 300, 1),         # all scores equal: the lowest heads take the shared slots; one key in the second chunk
+    (3, 2, 9000, 2000, 1 << 20),   # several chunks per head, all three digits matter
+    (1, 2, 330000, 5000, 1 << 22), # heads too long for a cluster
+])
+def test_adaptive_counts_across_heads(B, Hkv, N, budget, levels):
+    rng = np.random.default_rng(N + levels)
+    scores = (1.0 + rng.integers(0, levels, (B, Hkv, N)) / np.float32(levels)).astype(np.float32)
+    for safeguard in (0.0, 0.3):
+        stride = N          # equal scores send all shared slots to the first heads
+        idx, cnt, want_idx, want_cnt = _both(scores, [N] * B, budget, 1, 7, "none", 1, safeguard, stride)
+        assert np.array_equal(cnt, want_cnt) and np.array_equal(idx, want_idx)
+
+
 def test_adaptive_degenerate_budgets():
     rng = np.random.default_rng(6)
     scores = rng.random((1, 2, 400), dtype=np.float32)
