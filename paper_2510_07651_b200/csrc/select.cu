@@ -798,13 +798,23 @@ obc_status launch_shard_indices(int units, int idx_stride, int t0, int n, const 
 
 size_t select_workspace_bytes(int B, int Hkv, int Nmax) { return align_up((size_t)B * Hkv * Nmax * 4, 256); }
 
-// Cluster size for the one-cluster-per-head path, or 0 when a head does not fit a cluster's shared memory.
-static int select_cluster_size(int Nmax, int* seg_cap) {
-    int C = 8;
-    if ((Nmax + C - 1) / C > 8192) C = 16;
-    const int seg = ((Nmax + C - 1) / C + 31) / 32 * 32;
-    if (seg > CL_MAX_SEG) return 0;
-    *seg_cap = seg;
+// Cluster size for the one-cluster-per-head path, or 0 when a head does not fit a cluster's shared memory.  A CTA's phases
+// cost the same for 32 as for 2048 keys, so short heads take one CTA; few longer heads take eight CTAs (8 heads of 8192
+// tokens: 13.8 / 11.6 / 10.5 / 10.2 us for 1 / 2 / 4 / 8; of 2048: 9.8 / 10.2 / 9.9 / 9.9); many heads take what still runs
+// side by side, two CTAs per SM (64 heads of 2048: 9.8 / 10.2 / 11.7 / 21.5 us, of 8192: 14.0 / 12.0 / 13.3 / 23.1, of 32768:
+// - / 22.1 / 20.8 / 30.5; 256 heads of 4096: 14.1 / 24.7 / 42.9 / 83.1), but no share above 8192 candidates, of which an SM
+// holds only one CTA (64 ragged heads of up to 65536: 37 us with four CTAs, 33 with eight; 256 of 32768: 84 with two, 76 with four).
+static int select_cluster_size(int units, int Nmax, int* seg_cap) {
+    auto seg_of = [&](int C) { return ((Nmax + C - 1) / C + 31) / 32 * 32; };
+    int C = 1;
+    if (units * 8LL <= 148) {
+        if (Nmax > 2048) C = seg_of(8) > 8192 ? 16 : 8;
+    } else {
+        while (C < 8 && Nmax > 4096 * C && (units * 2LL * C <= 2 * 148 || seg_of(C) > 8192)) C *= 2;
+    }
+    while (C < 16 && seg_of(C) > CL_MAX_SEG) C *= 2;
+    if (seg_of(C) > CL_MAX_SEG) return 0;
+    *seg_cap = seg_of(C);
     return C;
 }
 
@@ -819,7 +829,7 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
                                      void* ws, cudaStream_t stream) {
     const int units = s.B * s.Hkv;
     int seg_cap = 0;
-    const int C = select_cluster_size(s.Nmax, &seg_cap);
+    const int C = select_cluster_size(units, s.Nmax, &seg_cap);
     if (C > 0) {
         const size_t smem = sizeof(ClusterShared) + (size_t)seg_cap * 8 + (size_t)s.pool_kernel * 4 + 16;
         OBC_CUDA_TRY(allow_smem(select_cluster_kernel, smem));

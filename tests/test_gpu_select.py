@@ -36,6 +36,15 @@ def test_select_bit_exact_on_random_scores(pool, kern, N, budget, n_sink, n_rece
     assert np.array_equal(got.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("Hkv,N", [(3, 2048), (3, 2049), (40, 4096), (40, 4097), (70, 16500), (160, 8192), (160, 8193)])
+def test_select_every_cluster_size(Hkv, N):
+    # one CTA per head, eight for a few heads, two and four for many, one for very many, two where its share would pass 8192
+    rng = np.random.default_rng(N)
+    scores = (rng.integers(0, 300, (1, Hkv, N)) / 64).astype(np.float32)
+    got, want = _select_both(scores, [N], [N // 7 + 40], 4, 32, "max", 7)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
 def test_select_ties_keep_lowest_index_and_all_equal_scores():
     N = 3000
     rng = np.random.default_rng(0)
