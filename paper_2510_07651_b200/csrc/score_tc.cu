@@ -32,6 +32,7 @@ namespace obc {
 namespace {
 
 constexpr int TILE = 128;                       // tokens per tile = MMA M
+constexpr unsigned kObcVariants = OBC_VAR_V | OBC_VAR_K | OBC_VAR_VK;      // Eq. 4-6
 constexpr unsigned kAllVariants = OBC_VAR_V | OBC_VAR_K | OBC_VAR_VK | OBC_VAR_ATTN | OBC_VAR_VATP;
 constexpr int NSTAGE = 2;
 constexpr uint32_t kHalfBytes = 128 * 128;      // [128 rows][64 bf16] = 16 KB, one swizzle-128B block
@@ -48,7 +49,7 @@ constexpr uint32_t OFF_V = OFF_K + NSTAGE * kOperandBytes;        // NSTAGE x 32
 constexpr uint32_t OFF_CONST = OFF_V + NSTAGE * kOperandBytes;    // 16 epilogue warps x 32 float4 (row-pair constants of the warp's half)
 constexpr int NSLOT = 4;                                          // ring depth of the per-tile value norms
 constexpr uint32_t OFF_NV = OFF_CONST + 16 * 32 * 16;             // NSLOT x 128 x (||v||^2, ||v||_1), own-norm kernels only
-constexpr int kNumSums = 7;                                       // running sums a token carries (RowSums)
+constexpr int kNumSums = 6;                                       // running sums a token carries (RowSums)
 constexpr uint32_t OFF_XCH = OFF_NV + NSLOT * TILE * 8;           // [tile parity][2][kNumSums][128] floats: the second half's sums
 constexpr uint32_t OFF_BAR = OFF_XCH + 2 * 2 * kNumSums * TILE * 4;
 constexpr uint32_t kNumBars = 2 * NSTAGE + 2 + 4 + 2 + 2 * NSLOT + 4;
@@ -299,17 +300,26 @@ __device__ __forceinline__ void value_norms(const uint8_t* vt, int tok, float& l
     l1 = sab.x + sab.y;
 }
 
-// Running sums of one token over the window rows, two rows per packed fp32x2 lane.  With
-// a = A_rp, u = a z (z the unscaled logit), b = a + scale u = a (1 + Z):
-//   Eq. 6   sum_r a^2 ||(1+Z) v - Z o_r||^2 = |v|^2 S1 + scale S2 + scale^2 S3
-//   Eq. 5   sum_r a^2 Z^2 ||v - o_r||^2     = scale^2 (|v|^2 S5 + S3 + S4)
-//   Eq. 4   |v|^2 S6;   attention-only: S7
-// with S1 = sum b^2, S2 = sum u b t', S3 = sum u^2 |o_r|^2, S4 = sum u^2 t', S5 = sum u^2,
-// S6 = sum a^2, S7 = sum a and t' = -2 v.o_r (the expanded norms of Algorithm 1).
-struct RowSums { float2 s1, s2, s3, s4, s5, s6, s7; };
+// Running sums of one token over the window rows, two rows per packed fp32x2 lane.  With a = A_rp, z the unscaled logit,
+// Z = scale z and t' = -2 v.o_r (the expanded norms of Algorithm 1):
+//   Eq. 4   sum_r a^2 |v|^2                 = |v|^2 S1
+//   Eq. 5   sum_r a^2 Z^2 ||v - o_r||^2     = scale^2 (|v|^2 S3 + S5)
+//   Eq. 6   sum_r a^2 ||(1+Z) v - Z o_r||^2 = |v|^2 (S1 + 2 scale S2 + scale^2 S3) + scale S4 + scale^2 S5
+// and S6 = sum a (attention-only), with S1 = sum a^2, S2 = sum a^2 z, S3 = sum a^2 z^2, S4 = sum a^2 z t',
+// S5 = sum a^2 z^2 (t' + |o_r|^2).  a^2 comes straight out of the exponential, of twice the argument: nine packed
+// instructions per row pair and one exponential per row serve Eq. 4-6 together (the sums over u = a z and
+// b = a (1 + Z) that they replace took ten for Eq. 5 and 6 and thirteen with the rest: 512 rows per head, four sequences of
+// up to 26550 tokens, Eq. 4-6: 265 -> 228 us for pass 2; Eq. 5 and 6 of the 128k layer with 448 rows: 163 -> 157 us).
+// The joint score alone is cheaper in u and b: s1 = sum b^2, s2 = sum u (b t' + u scale |o_r|^2), and the score is
+// |v|^2 s1 + scale s2 with seven instructions per row pair.
+struct RowSums { float2 s1, s2, s3, s4, s5, s6; };
 
-// 16 rows of one token: zr = logits, tr = -2 v.o_r, cst = per row pair (-lse2_0, -lse2_1, |o_0|^2, |o_1|^2);
-// when only the joint score is computed (VARS == OBC_VAR_VK) the |o|^2 entries arrive multiplied by scale
+template <unsigned VARS> constexpr bool kWantsA = VARS == OBC_VAR_VK || (VARS & (OBC_VAR_ATTN | OBC_VAR_VATP)) != 0;
+// what the exponent is multiplied with: a^2 alone is wanted, or a
+template <unsigned VARS> constexpr float kExpFactor = kWantsA<VARS> ? 1.f : 2.f;
+
+// 16 rows of one token: zr = logits, tr = -2 v.o_r, cst = per row pair (-lse2_0, -lse2_1, |o_0|^2, |o_1|^2), the
+// first two times kExpFactor (as sl2); when only the joint score is computed the |o|^2 entries arrive multiplied by scale
 template <unsigned VARS, bool MASKED>
 __device__ __forceinline__ void score_rows16(const uint32_t (&zr)[16], const uint32_t (&tr)[16], const float4* cst,
                                              float2 sl2, float2 sc, RowSums& S, int ptok, int mask_base, int W, int& wi) {
@@ -326,26 +336,37 @@ __device__ __forceinline__ void score_rows16(const uint32_t (&zr)[16], const uin
             wi = wi + 1 == W ? 0 : wi + 1;
         }
         const float2 a = make_float2(fast_exp2(e.x), fast_exp2(e.y));
-        const float2 u = __fmul2_rn(a, z);
         if (VARS == OBC_VAR_VK) {
-            // joint score alone: the constants hold scale |o_r|^2, and s2 collects u (b t' + u scale |o_r|^2),
-            // i.e. S2 + scale S3 of the general form below, with one packed instruction less
+            const float2 u = __fmul2_rn(a, z);
             const float2 b = __ffma2_rn(u, sc, a);
             S.s1 = __ffma2_rn(b, b, S.s1);
             S.s2 = __ffma2_rn(u, __ffma2_rn(u, make_float2(cp.z, cp.w), __fmul2_rn(b, t2)), S.s2);
-        } else if (VARS & OBC_VAR_VK) {
-            const float2 b = __ffma2_rn(u, sc, a);
-            S.s1 = __ffma2_rn(b, b, S.s1);
-            S.s2 = __ffma2_rn(__fmul2_rn(u, b), t2, S.s2);
+        } else {
+            float2 c0 = a;                              // a^2 already
+            if (kWantsA<VARS>) { c0 = __fmul2_rn(a, a); S.s6 = __fadd2_rn(a, S.s6); }
+            const float2 c1 = __fmul2_rn(c0, z), c2 = __fmul2_rn(c1, z);
+            S.s1 = __fadd2_rn(c0, S.s1);
+            S.s2 = __fadd2_rn(c1, S.s2);
+            S.s3 = __fadd2_rn(c2, S.s3);
+            S.s4 = __ffma2_rn(c1, t2, S.s4);
+            S.s5 = __ffma2_rn(c2, __fadd2_rn(t2, make_float2(cp.z, cp.w)), S.s5);
         }
-        if ((VARS & (OBC_VAR_VK | OBC_VAR_K)) && VARS != OBC_VAR_VK) {
-            const float2 uu = __fmul2_rn(u, u);
-            S.s3 = __ffma2_rn(uu, make_float2(cp.z, cp.w), S.s3);
-            if (VARS & OBC_VAR_K) { S.s4 = __ffma2_rn(uu, t2, S.s4); S.s5 = __fadd2_rn(uu, S.s5); }
-        }
-        if (VARS & OBC_VAR_V) S.s6 = __ffma2_rn(a, a, S.s6);
-        if (VARS & (OBC_VAR_ATTN | OBC_VAR_VATP)) S.s7 = __fadd2_rn(a, S.s7);
     }
+}
+
+// stores the planes of one token from its sums (packed lanes folded)
+template <unsigned VARS>
+__device__ __forceinline__ void store_scores(const float (&sum)[kNumSums], float nv, float nv1, float scale, unsigned variants, float* out,
+                                             size_t plane, bool live) {
+    int pl = 0;
+    if (VARS == OBC_VAR_VK) { out[0] = live ? fmaf(nv, sum[0], scale * sum[1]) : 0.f; return; }
+    const float s2 = scale * scale;
+    if (variants & OBC_VAR_V)    out[(size_t)(pl++) * plane] = live ? nv * sum[0] : 0.f;
+    if (variants & OBC_VAR_K)    out[(size_t)(pl++) * plane] = live ? s2 * fmaf(nv, sum[2], sum[4]) : 0.f;
+    if (variants & OBC_VAR_VK)   out[(size_t)(pl++) * plane] =
+        live ? fmaf(nv, fmaf(s2, sum[2], fmaf(2.f * scale, sum[1], sum[0])), fmaf(scale, sum[3], s2 * sum[4])) : 0.f;
+    if (variants & OBC_VAR_ATTN) out[(size_t)(pl++) * plane] = live ? sum[5] : 0.f;
+    if (variants & OBC_VAR_VATP) out[(size_t)(pl++) * plane] = live ? nv1 * sum[5] : 0.f;
 }
 
 // One (tile, chunk) item of one token: all rows of the chunk, one batch of 16 rows in registers at a time.  (Loading
@@ -541,7 +562,8 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // the chunk's rows in two runs of whole 16-row batches
         const int rows0 = min(p.chunk_rows, (p.chunk_rows / 2 + 15) / 16 * 16);
         const int r_begin = half ? rows0 : 0, r_count = half ? p.chunk_rows - rows0 : rows0;
-        const float2 sl2 = make_float2(p.scale * kLog2e, p.scale * kLog2e), sc = make_float2(p.scale, p.scale);
+        const float ksl = p.scale * kLog2e * kExpFactor<VARS>;
+        const float2 sl2 = make_float2(ksl, ksl), sc = make_float2(p.scale, p.scale);
         const size_t plane = (size_t)units * p.Nmax;
         uint32_t item = 0, tile_seq = 0, mine_seq = 0;
         uint32_t full_par = 0, nv_par = 0;                         // phase parity of this group's barriers, one bit each
@@ -559,7 +581,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const int Nm = tc_mask_len(p, b);
             const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
             RowSums S;
-            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
+            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = make_float2(0.f, 0.f);
             const uint32_t buf = item & 1;
             float nv = 0.f, nv1 = 0.f;                             // used after the row loop
             if (!OWN_NV && half == 0 && ptok < N) nv = p.nv[(size_t)unit * p.Nmax + ptok];
@@ -569,6 +591,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     const int rp = (r_begin >> 1) + lane;          // row pair of the chunk
                     float4 c4 = lane * 2 < r_count ? p.cpair[(((size_t)unit * p.rows_out) >> 1) + rp] : make_float4(-INFINITY, -INFINITY, 0.f, 0.f);
                     if (VARS == OBC_VAR_VK) { c4.z *= p.scale; c4.w *= p.scale; }
+                    c4.x *= kExpFactor<VARS>; c4.y *= kExpFactor<VARS>;
                     my_const[lane] = c4;
                 }
                 __syncwarp();
@@ -596,9 +619,8 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(BAR_TM_EMPTY + buf));
             ++item;
-            // the two row halves of the token meet: sums 1..7 of RowSums, packed lanes folded
-            float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y,
-                                   S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
+            // the two row halves of the token meet: the sums of RowSums, packed lanes folded
+            float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y};
             // slot xs was last used two of this group's tiles ago; the first half read it before it released the
             // accumulators of the tile after that one, without which the tile at hand could not have been computed
             const uint32_t xs = mine_seq & 1;
@@ -606,7 +628,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (half == 1) {
 #pragma unroll
                 for (int j = 0; j < kNumSums; ++j) {
-                    const bool used = VARS == OBC_VAR_VK ? j < 2 : true;
+                    const bool used = VARS == OBC_VAR_VK ? j < 2 : j < 5 || kWantsA<VARS>;
                     if (used) xch[j * TILE] = sum[j];
                 }
                 __syncwarp();
@@ -618,21 +640,10 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             ++mine_seq;
 #pragma unroll
             for (int j = 0; j < kNumSums; ++j) {
-                const bool used = VARS == OBC_VAR_VK ? j < 2 : true;
+                const bool used = VARS == OBC_VAR_VK ? j < 2 : j < 5 || kWantsA<VARS>;
                 if (used) sum[j] += xch[j * TILE];
             }
-            if (ptok < p.Nmax) {
-                const bool live = ptok < N;
-                const float s2 = p.scale * p.scale;
-                int pl = 0;
-                if (p.variants & OBC_VAR_V)    out[(size_t)(pl++) * plane + ptok] = live ? nv * sum[5] : 0.f;
-                if (p.variants & OBC_VAR_K)    out[(size_t)(pl++) * plane + ptok] =
-                    live ? s2 * (fmaf(nv, sum[4], sum[2]) + sum[3]) : 0.f;
-                if (p.variants & OBC_VAR_VK)   out[(size_t)(pl++) * plane + ptok] =
-                    live ? fmaf(nv, sum[0], fmaf(p.scale, sum[1], s2 * sum[2])) : 0.f;
-                if (p.variants & OBC_VAR_ATTN) out[(size_t)(pl++) * plane + ptok] = live ? sum[6] : 0.f;
-                if (p.variants & OBC_VAR_VATP) out[(size_t)(pl++) * plane + ptok] = live ? nv1 * sum[6] : 0.f;
-            }
+            if (ptok < p.Nmax) store_scores<VARS>(sum, nv, nv1, p.scale, p.variants, out + ptok, plane, ptok < N);
         }
         // padding beyond the last tile of a shorter sequence: zeros
         if (p.seq_lens) {
@@ -858,7 +869,7 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 if (may_skip && rows_last_token(c * MC_ROWS, min(c * MC_ROWS + MC_ROWS, p.R) - 1, p.W, Nu, 1) < pair_first) continue;
                 const uint32_t cs = citem & 3;
                 const size_t crow = (size_t)unit * p.rows_out + (size_t)c * MC_ROWS + t64;
-                const float2 cst = make_float2(-p.lse2[crow], p.onorm[crow] * (VARS == OBC_VAR_VK ? p.scale : 1.f));
+                const float2 cst = make_float2(-kExpFactor<VARS> * p.lse2[crow], p.onorm[crow] * (VARS == OBC_VAR_VK ? p.scale : 1.f));
                 // slot cs was last read by the chunk four back; the chunk two back has been summed once
                 // the TMEM buffers this chunk is going to use are free again
                 const uint32_t i0 = 2 * citem, i1 = i0 + 1;
@@ -878,7 +889,8 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         const int wg = (warp - 4) >> 2;                            // owns tile wg of every pair
         const int lane_grp = warp & 3;                             // TMEM lanes 32*lane_grp .. +31
         const int tok = lane_grp * 32 + lane;                      // token within the tile
-        const float2 sl2 = make_float2(p.scale * kLog2e, p.scale * kLog2e), sc = make_float2(p.scale, p.scale);
+        const float ksl = p.scale * kLog2e * kExpFactor<VARS>;
+        const float2 sl2 = make_float2(ksl, ksl), sc = make_float2(p.scale, p.scale);
         const size_t plane = (size_t)units * p.Nmax;
         uint32_t pitem = 0, citem = 0;
         for (; !tw.done() && !failed; tw.next(), ++pitem) {
@@ -889,7 +901,7 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             const int ptok = t0 + tok;
             const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
             RowSums S;
-            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
+            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = make_float2(0.f, 0.f);
             const int pair_first = pair * 2 * TILE;
             for (int c = cs; c < nc; c += cstep) {
                 if (may_skip && rows_last_token(c * MC_ROWS, min(c * MC_ROWS + MC_ROWS, p.R) - 1, p.W, Nm, 1) < pair_first) continue;
@@ -923,16 +935,8 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 // with the chunks of the pair shared by several CTAs each writes its part of the sums (the scores are
                 // linear in them) into its own copy of the planes; tc_partial_sum_kernel adds the copies in order
                 float* out = (cstep > 1 ? p.partial + (size_t)cs * __popc(p.variants) * plane : p.scores) + (size_t)unit * p.Nmax;
-                const bool live = ptok < N;
-                const float s2 = p.scale * p.scale;
-                int pl = 0;
-                if (p.variants & OBC_VAR_V)    out[(size_t)(pl++) * plane + ptok] = live ? nv * (S.s6.x + S.s6.y) : 0.f;
-                if (p.variants & OBC_VAR_K)    out[(size_t)(pl++) * plane + ptok] =
-                    live ? s2 * (fmaf(nv, S.s5.x + S.s5.y, S.s3.x + S.s3.y) + (S.s4.x + S.s4.y)) : 0.f;
-                if (p.variants & OBC_VAR_VK)   out[(size_t)(pl++) * plane + ptok] =
-                    live ? fmaf(nv, S.s1.x + S.s1.y, fmaf(p.scale, S.s2.x + S.s2.y, s2 * (S.s3.x + S.s3.y))) : 0.f;
-                if (p.variants & OBC_VAR_ATTN) out[(size_t)(pl++) * plane + ptok] = live ? S.s7.x + S.s7.y : 0.f;
-                if (p.variants & OBC_VAR_VATP) out[(size_t)(pl++) * plane + ptok] = live ? nv1 * (S.s7.x + S.s7.y) : 0.f;
+                const float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y};
+                store_scores<VARS>(sum, nv, nv1, p.scale, p.variants, out + ptok, plane, ptok < N);
             }
         }
         // padding beyond the last tile of a shorter sequence: zeros
@@ -1711,14 +1715,12 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
             }
             return OBC_OK;
         };
-        if (p.csplit > 1 || (s.causal && s.W > MC_ROWS)) {
-            if (s.variants == OBC_VAR_VK) return launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, true>);
-            if (s.variants == (OBC_VAR_K | OBC_VAR_VK)) return launch_multi(tc_pass2_multi_kernel<OBC_VAR_K | OBC_VAR_VK, true>);
-            return launch_multi(tc_pass2_multi_kernel<kAllVariants, true>);
-        }
-        if (s.variants == OBC_VAR_VK) return launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, false>);
-        if (s.variants == (OBC_VAR_K | OBC_VAR_VK)) return launch_multi(tc_pass2_multi_kernel<OBC_VAR_K | OBC_VAR_VK, false>);
-        return launch_multi(tc_pass2_multi_kernel<kAllVariants, false>);
+        const bool split = p.csplit > 1 || (s.causal && s.W > MC_ROWS);
+        if (s.variants == OBC_VAR_VK)
+            return split ? launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, true>) : launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, false>);
+        if (!(s.variants & ~kObcVariants))
+            return split ? launch_multi(tc_pass2_multi_kernel<kObcVariants, true>) : launch_multi(tc_pass2_multi_kernel<kObcVariants, false>);
+        return split ? launch_multi(tc_pass2_multi_kernel<kAllVariants, true>) : launch_multi(tc_pass2_multi_kernel<kAllVariants, false>);
     }
 
     auto launch = [&](auto kernel) -> obc_status {
@@ -1728,13 +1730,15 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     };
     // pass 1 leaves only ||v||^2; without it, and for the l1 variant, the norms come from the V tiles in pass 2
     const bool own_nv = given || (s.variants & OBC_VAR_VATP);
-    if (hilo) {
-        if (s.variants == OBC_VAR_VK) return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, true>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, true>);
-        return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, true>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, true>);
+    if (s.variants == OBC_VAR_VK) {
+        if (hilo) return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, true>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, true>);
+        return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, false>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, false>);
     }
-    if (s.variants == OBC_VAR_VK) return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, false>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, false>);
-    if (s.variants == (OBC_VAR_K | OBC_VAR_VK))
-        return own_nv ? launch(tc_pass2_kernel<OBC_VAR_K | OBC_VAR_VK, true, false>) : launch(tc_pass2_kernel<OBC_VAR_K | OBC_VAR_VK, false, false>);
+    if (!(s.variants & ~kObcVariants)) {
+        if (hilo) return own_nv ? launch(tc_pass2_kernel<kObcVariants, true, true>) : launch(tc_pass2_kernel<kObcVariants, false, true>);
+        return own_nv ? launch(tc_pass2_kernel<kObcVariants, true, false>) : launch(tc_pass2_kernel<kObcVariants, false, false>);
+    }
+    if (hilo) return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, true>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, true>);
     return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, false>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, false>);
 }
 
