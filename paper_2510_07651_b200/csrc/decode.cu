@@ -14,7 +14,11 @@
 //   decode_score   v_p . o_r and ||v_p||^2 per slot, score, s_acc += score, per-chunk argmin of
 //                  the evictable slots
 //   decode_final   per (b, g): pick the slot to free, update pos / state
+// Few units take one kernel for all of it instead (decode_fused.cuh).
 #include "obc_common.cuh"
+
+#include <cooperative_groups.h>
+namespace cg = cooperative_groups;
 
 namespace obc {
 namespace {
@@ -64,9 +68,11 @@ __device__ __forceinline__ void chunk_bar_init(uint64_t* bar) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 // hint: 0 = default L2 policy, 1 = evict first (rows that are not read again this step), 2 = evict last
+template <int N = CH>
 __device__ __forceinline__ void copy_chunk_tma(uint4* dst, const CUtensorMap* map, uint64_t* bar, int b, int g, int c0, int hint = 0) {
     const uint32_t d = smem_addr(dst), mb = smem_addr(bar);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"((uint32_t)kStageBytes) : "memory");
+    constexpr uint32_t kBytes = (uint32_t)N * 256u;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(kBytes) : "memory");
     if (hint) {
         uint64_t pol;
         if (hint == 1) asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
@@ -74,13 +80,13 @@ __device__ __forceinline__ void copy_chunk_tma(uint4* dst, const CUtensorMap* ma
         asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
                      ::"r"(d), "l"(map), "r"(mb), "r"(0), "r"(c0), "r"(g), "r"(b), "l"(pol) : "memory");
         asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%3, %4, %5, %6}], [%2], %7;"
-                     ::"r"(d + (uint32_t)(kStageBytes / 2)), "l"(map), "r"(mb), "r"(64), "r"(c0), "r"(g), "r"(b), "l"(pol) : "memory");
+                     ::"r"(d + kBytes / 2), "l"(map), "r"(mb), "r"(64), "r"(c0), "r"(g), "r"(b), "l"(pol) : "memory");
         return;
     }
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
                  ::"r"(d), "l"(map), "r"(mb), "r"(0), "r"(c0), "r"(g), "r"(b) : "memory");
     asm volatile("cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5, %6}], [%2];"
-                 ::"r"(d + (uint32_t)(kStageBytes / 2)), "l"(map), "r"(mb), "r"(64), "r"(c0), "r"(g), "r"(b) : "memory");
+                 ::"r"(d + kBytes / 2), "l"(map), "r"(mb), "r"(64), "r"(c0), "r"(g), "r"(b) : "memory");
 }
 // bounded wait for the copy of the given phase: false after two seconds
 __device__ __forceinline__ bool chunk_wait(uint64_t* bar, uint32_t parity) {
@@ -98,8 +104,9 @@ __device__ __forceinline__ bool chunk_wait(uint64_t* bar, uint32_t parity) {
     }
 }
 // piece `piece` (0..15) of staged row `row`
+template <int N = CH>
 __device__ __forceinline__ int staged_piece(int row, int piece) {
-    return (piece >> 3) * (CH * 8) + row * 8 + ((piece & 7) ^ (row & 7));
+    return (piece >> 3) * (N * 8) + row * 8 + ((piece & 7) ^ (row & 7));
 }
 
 // ---- warp-level tensor-core pieces ------------------------------------------------------------------
@@ -124,11 +131,12 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 // address of the 8x8 tile that lane `lane` names for an x4 load covering 16 staged rows from `row0` and the two
 // 16-byte pieces `piece0`, `piece0 + 1`.  rows_major: tiles ordered (rows 0-7, p0), (rows 8-15, p0), (rows 0-7, p1),
 // (rows 8-15, p1), the A operand of slots x channels; otherwise (rows 0-7, p0), (rows 0-7, p1), (rows 8-15, p0), ...
+template <int N = CH>
 __device__ __forceinline__ const uint4* tile_addr(const uint4* sRows, int row0, int piece0, int lane, bool rows_major) {
     const int mi = lane >> 3, rr = lane & 7;
     const int row = row0 + (rows_major ? (mi & 1) : (mi >> 1)) * 8 + rr;
     const int piece = piece0 + (rows_major ? (mi >> 1) : (mi & 1));
-    return sRows + staged_piece(row, piece);
+    return sRows + staged_piece<N>(row, piece);
 }
 // x = hi + lo with both halves bf16: two MMAs then carry an fp32 operand to about 16 bits
 __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, uint32_t& lo) {
@@ -136,6 +144,39 @@ __device__ __forceinline__ void split_bf16x2(float x0, float x1, uint32_t& hi, u
     const __nv_bfloat162 l = __floats2bfloat162_rn(x0 - __low2float(h), x1 - __high2float(h));
     hi = *reinterpret_cast<const uint32_t*>(&h);
     lo = *reinterpret_cast<const uint32_t*>(&l);
+}
+
+// Eq. 4-6 (or the attention-only score) of one slot for the newest query of G heads: log2-scaled logits z2, log2-sum-exp, |o|^2
+// and v . o per head, |v|^2
+template <int G>
+__device__ __forceinline__ float slot_score(unsigned variant, const float (&z2)[G], const float* lse, const float* no, const float (&t)[G], float nv) {
+    float sc = 0.f;
+#pragma unroll
+    for (int r = 0; r < G; ++r) {
+        const float a = exp2f(z2[r] - lse[r]);
+        const float Z = z2[r] * 0.6931471805599453f;           // back from log2 units: scale * q.k
+        const float a2 = a * a;
+        if (variant == OBC_VAR_V) sc = fmaf(a2, nv, sc);
+        else if (variant == OBC_VAR_K) sc = fmaf(a2 * Z * Z, no[r] + nv - 2.f * t[r], sc);
+        else if (variant == OBC_VAR_VK)
+            sc += a2 * nv + a2 * Z * Z * (no[r] + nv - 2.f * t[r]) + 2.f * a2 * Z * (nv - t[r]);
+        else sc += a;
+    }
+    return sc;
+}
+// eviction order: smallest accumulator, equal values -> highest position
+__device__ __forceinline__ bool goes_first(const MinCand& a, const MinCand& b) {
+    return a.slot >= 0 && (b.slot < 0 || a.val < b.val || (a.val == b.val && a.pos > b.pos));
+}
+__device__ __forceinline__ void min_over_warp(MinCand& c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        MinCand other;
+        other.val = __shfl_xor_sync(0xffffffffu, c.val, o);
+        other.pos = __shfl_xor_sync(0xffffffffu, c.pos, o);
+        other.slot = __shfl_xor_sync(0xffffffffu, c.slot, o);
+        if (goes_first(other, c)) { c.val = other.val; c.pos = other.pos; c.slot = other.slot; }
+    }
 }
 
 // The chunks arrive as tiled bulk copies through the two tensor maps.  A bulk copy that does not complete within its
@@ -485,19 +526,7 @@ decode_score_kernel(const __grid_constant__ CUtensorMap map_v, DecodeShape s, De
         float nv = sT[G][tid], t[G];
 #pragma unroll
         for (int r = 0; r < G; ++r) t[r] = sT[r][tid];
-        float sc = 0.f;
-#pragma unroll
-        for (int r = 0; r < G; ++r) {
-            const float z2 = zin[r];
-            const float a = exp2f(z2 - sLse[r]);
-            const float Z = z2 * 0.6931471805599453f;          // back from log2 units: scale * q.k
-            const float a2 = a * a;
-            if (s.variant == OBC_VAR_V) sc = fmaf(a2, nv, sc);
-            else if (s.variant == OBC_VAR_K) sc = fmaf(a2 * Z * Z, sNo[r] + nv - 2.f * t[r], sc);
-            else if (s.variant == OBC_VAR_VK)
-                sc += a2 * nv + a2 * Z * Z * (sNo[r] + nv - 2.f * t[r]) + 2.f * a2 * Z * (nv - t[r]);
-            else sc += a;
-        }
+        const float sc = slot_score<G>(s.variant, zin, sLse, sNo, t, nv);
         float acc = acc_in + sc;
         if (s.acc_window > 0) {                                // the last acc_window steps only, summed afresh in ring order
             float* hcol = s.s_hist + (size_t)unit * s.acc_window * s.cap + slot;
@@ -515,23 +544,13 @@ decode_score_kernel(const __grid_constant__ CUtensorMap map_v, DecodeShape s, De
         s_acc[(size_t)unit * s.cap + slot] = acc;
         if (my_pos >= s.n_sink && my_pos <= step_pos - s.n_recent) cand = MinCand{acc, my_pos, slot, 0};
     }
-    // argmin of (value, -pos): smallest accumulator, equal values -> highest position
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        MinCand other;
-        other.val = __shfl_xor_sync(0xffffffffu, cand.val, o);
-        other.pos = __shfl_xor_sync(0xffffffffu, cand.pos, o);
-        other.slot = __shfl_xor_sync(0xffffffffu, cand.slot, o);
-        if (other.slot >= 0 && (cand.slot < 0 || other.val < cand.val || (other.val == cand.val && other.pos > cand.pos)))
-            { cand.val = other.val; cand.pos = other.pos; cand.slot = other.slot; }
-    }
+    min_over_warp(cand);
     if (lane == 0) sMin[warp] = cand;
     __syncthreads();
     if (tid == 0) {
         MinCand best = sMin[0];
         for (int w = 1; w < NWARP; ++w) {
-            const MinCand o2 = sMin[w];
-            if (o2.slot >= 0 && (best.slot < 0 || o2.val < best.val || (o2.val == best.val && o2.pos > best.pos))) best = o2;
+            if (goes_first(sMin[w], best)) best = sMin[w];
         }
         *part_min = best;
     }
@@ -555,17 +574,9 @@ decode_final_kernel(DecodeShape s, DecodePlan plan, int32_t* pos, int32_t* state
         MinCand best{INFINITY, -1, -1, 0};
         for (int ch = lane; ch < plan.chunks; ch += 32) {
             const MinCand o2 = pm[ch];
-            if (o2.slot >= 0 && (best.slot < 0 || o2.val < best.val || (o2.val == best.val && o2.pos > best.pos))) best = o2;
+            if (goes_first(o2, best)) best = o2;
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            MinCand other;
-            other.val = __shfl_xor_sync(0xffffffffu, best.val, o);
-            other.pos = __shfl_xor_sync(0xffffffffu, best.pos, o);
-            other.slot = __shfl_xor_sync(0xffffffffu, best.slot, o);
-            if (other.slot >= 0 && (best.slot < 0 || other.val < best.val || (other.val == best.val && other.pos > best.pos)))
-                { best.val = other.val; best.pos = other.pos; best.slot = other.slot; }
-        }
+        min_over_warp(best);
         if (best.slot >= 0) {
             if (lane == 0) pos[(size_t)unit * s.cap + best.slot] = -1;
             live -= 1;
@@ -579,20 +590,27 @@ decode_final_kernel(DecodeShape s, DecodePlan plan, int32_t* pos, int32_t* state
     }
 }
 
+#include "decode_fused.cuh"
+
 // a tensor map over a cache [B, Hkv, cap, d]: its base 16-byte aligned and its strides whole 16-byte units
-bool cache_map(CUtensorMap* map, const TensorView& t, const DecodeShape& s) {
+bool cache_map(CUtensorMap* map, const TensorView& t, const DecodeShape& s, int box_rows) {
     if (((uintptr_t)t.ptr & 15) || (t.st & 7) || (t.sh & 7) || (t.sb & 7) || t.st < kD) return false;
     const uint64_t dims[4] = {(uint64_t)kD, (uint64_t)s.cap, (uint64_t)s.Hkv, (uint64_t)s.B};
     const uint64_t strides[3] = {(uint64_t)t.st * 2, (uint64_t)(s.Hkv > 1 ? t.sh : t.st * s.cap) * 2,
                                  (uint64_t)(s.B > 1 ? t.sb : (s.Hkv > 1 ? t.sh * s.Hkv : t.st * s.cap)) * 2};
-    return make_map(map, t.ptr, 4, dims, strides, CH);
+    return make_map(map, t.ptr, 4, dims, strides, (uint32_t)box_rows);
 }
 
 template <int G>
-obc_status launch_g(const DecodeShape& s, const DecodePlan& plan, const CUtensorMap& mk, const CUtensorMap& mv,
-                    TensorView q, TensorView kt, TensorView vt,
-                    TensorView kc, TensorView vc, float* s_acc, int32_t* pos, int32_t* state,
-                    int step_pos, char* ws, cudaStream_t stream) {
+obc_status launch_g(const DecodeShape& s, TensorView q, TensorView kt, TensorView vt, TensorView kc, TensorView vc, float* s_acc, int32_t* pos,
+                    int32_t* state, int step_pos, char* ws, cudaStream_t stream) {
+    // (the entry point has checked what a tensor map asks of the caches: 16-byte aligned base, strides whole 16-byte units)
+    CUtensorMap mk, mv;
+    const int fused = fused_chunk<G>(s), rows = fused ? fused : CH;
+    if (!cache_map(&mk, kc, s, rows) || !cache_map(&mv, vc, s, rows)) { set_last_cuda_error((int)cudaErrorInvalidValue); return OBC_ERR_CUDA; }
+    if (fused == 128) return launch_fused<G, 128>(mk, mv, s, q, kt, vt, kc, vc, s_acc, pos, state, step_pos, stream);
+    if (fused == 256) return launch_fused<G, 256>(mk, mv, s, q, kt, vt, kc, vc, s_acc, pos, state, step_pos, stream);
+    const DecodePlan plan = make_plan(s);
     const int units = s.B * s.Hkv;
     const size_t stage = kStageBytes + 1024;                            // + room to align the swizzled tile
     { ProfScope ps("decode_pass1", stream); OBC_CUDA_TRY(allow_smem(decode_pass1_kernel<G>, stage));
@@ -611,12 +629,8 @@ size_t decode_workspace_bytes(const DecodeShape& s) { return make_plan(s).bytes;
 obc_status launch_decode(const DecodeShape& s, TensorView q, TensorView kt, TensorView vt,
                          TensorView kc, TensorView vc, float* s_acc, int32_t* pos, int32_t* state,
                          int step_pos, void* ws, cudaStream_t stream) {
-    const DecodePlan plan = make_plan(s);
     char* w = (char*)ws;
-    // (the entry point has checked what a tensor map asks of the caches: 16-byte aligned base, strides whole 16-byte units)
-    CUtensorMap mk, mv;
-    if (!cache_map(&mk, kc, s) || !cache_map(&mv, vc, s)) { set_last_cuda_error((int)cudaErrorInvalidValue); return OBC_ERR_CUDA; }
-#define OBC_DECODE_CASE(Gv) case Gv: return launch_g<Gv>(s, plan, mk, mv, q, kt, vt, kc, vc, s_acc, pos, state, step_pos, w, stream)
+#define OBC_DECODE_CASE(Gv) case Gv: return launch_g<Gv>(s, q, kt, vt, kc, vc, s_acc, pos, state, step_pos, w, stream)
     switch (s.G) {
         OBC_DECODE_CASE(1); OBC_DECODE_CASE(2); OBC_DECODE_CASE(3); OBC_DECODE_CASE(4);
         OBC_DECODE_CASE(5); OBC_DECODE_CASE(6); OBC_DECODE_CASE(7); OBC_DECODE_CASE(8);

@@ -100,6 +100,21 @@ def test_decode_every_group_size(G):
     _run(B=1, Hq=2 * G, Hkv=2, n0=290, budget=300, cap=301, n_sink=3, n_recent=20, steps=24)
 
 
+@pytest.mark.parametrize("G", [1, 2, 3, 5, 6, 8])
+def test_decode_many_units(G):
+    # more units than clusters fit on the chip at once: the step in four kernels (three chunks, an odd extent)
+    _run(B=80, Hq=2 * G, Hkv=2, n0=299, budget=300, cap=301, n_sink=3, n_recent=20, steps=3)
+
+
+@pytest.mark.parametrize("cap,G,window", [
+    (127, 1, 0), (128, 4, 0), (129, 7, 17),        # one chunk not quite, exactly, and a second one of a single slot
+    (2048, 4, 0), (2049, 7, 16), (4096, 8, 0),     # sixteen chunks of 128 slots, nine and sixteen of 256
+    (4097, 2, 3),                                  # one slot too many for a cluster: the step in four kernels
+])
+def test_decode_cluster_sizes(cap, G, window):
+    _run(B=1, Hq=G, Hkv=1, n0=cap - 2, budget=cap - 1, cap=cap, n_sink=3, n_recent=20, steps=5, window=window)
+
+
 @pytest.mark.parametrize("window", [1, 5, 16])
 def test_decode_accumulation_window(window):
     """Scores accumulated over the last `window` steps only: steady-state eviction with slot reuse, several
