@@ -35,6 +35,7 @@ constexpr int TILE = 128;                       // tokens per tile = MMA M
 constexpr unsigned kObcVariants = OBC_VAR_V | OBC_VAR_K | OBC_VAR_VK;      // Eq. 4-6
 constexpr unsigned kAllVariants = OBC_VAR_V | OBC_VAR_K | OBC_VAR_VK | OBC_VAR_ATTN | OBC_VAR_VATP;
 constexpr int NSTAGE = 2;
+constexpr int MC_ROWS = 64;                     // window rows per chunk of the multi-chunk pass 2
 constexpr uint32_t kHalfBytes = 128 * 128;      // [128 rows][64 bf16] = 16 KB, one swizzle-128B block
 constexpr uint32_t kOperandBytes = 2 * kHalfBytes;
 constexpr int kThreads = 640;                   // single-chunk pass 2: 4 service warps + 4 epilogue warpgroups
@@ -191,8 +192,10 @@ struct TcParams {
     unsigned int* status;                     // device status word (workspace header)
     unsigned long long* span;                 // [2]: ~(earliest CTA start), latest CTA end, in globaltimer ns
     int l2_stream;                            // K/V copies carry the "evict first" L2 hint (their last use)
-    int csplit;                               // multi-chunk kernel: CTAs that share the row chunks of one tile pair
-    float* partial;                           // csplit > 1: [csplit][planes][units][Nmax] partial scores
+    int csplit;                               // multi-chunk kernel: the most CTAs that share the row chunks of one tile pair; 1: whole pairs
+    float* partial;                           // csplit > 1: [csplit - 1][planes][units][Nmax] scores of every pair's second, third, ... CTA
+    int* copies;                              // csplit > 1: [units][pairs of Nmax tokens] how many of them a pair has
+    int max_pairs;
 };
 
 // (a device-side length is clamped to [0, max_len]: the host cannot check it)
@@ -208,17 +211,6 @@ __device__ __forceinline__ int rows_last_token(int r0, int r1, int W, int N, int
     return (causal && r0 / W == r1 / W) ? N - W + (r1 % W) : N - 1;
 }
 
-// Multi-chunk pass 2 with the row chunks of a tile pair shared by `csplit` CTAs: position t of a unit with
-// P pairs stands for pair zigzag(t mod P) and the chunks c = t / P, t / P + csplit, ...  The zigzag (first,
-// last, second, second to last, ...) puts a pair that many rows see next to one that few rows see, so that
-// the contiguous runs of positions that the CTAs take weigh about the same under a causal window.
-__device__ __forceinline__ void split_position(int t, int positions_in_unit, int csplit, int& pair, int& cs) {
-    if (csplit == 1) { pair = t; cs = 0; return; }
-    const int P = positions_in_unit / csplit, q = t % P;
-    cs = t / P;
-    pair = (q & 1) ? P - 1 - (q >> 1) : (q >> 1);
-}
-
 // Walks the CTA's share of the token tiles.  All non-empty 128-token tiles of all (batch item,
 // KV head) units, in (unit, tile) order, are cut into gridDim.x contiguous, equally long runs, so
 // that a CTA stays inside one unit for as long as possible (its Q / O operands stay in shared
@@ -227,13 +219,9 @@ struct TileWalk {
     int unit, tile, tiles_in_unit;            // current position
     long long left;                           // positions still to visit, including the current one
     const TcParams* p;
-    int span;                                 // consecutive tiles of a unit that one position stands for
-    int reps;                                 // positions per such group of tiles (CTAs that share its row chunks)
-    __device__ __forceinline__ int tiles_of(int b) const {
-        return ((tc_seq_len(*p, b) + TILE - 1) / TILE + span - 1) / span * reps;
-    }
-    __device__ void init(const TcParams& prm, int tiles_per_position = 1, int positions_per_group = 1) {
-        p = &prm; span = tiles_per_position; reps = positions_per_group;
+    __device__ __forceinline__ int tiles_of(int b) const { return (tc_seq_len(*p, b) + TILE - 1) / TILE; }
+    __device__ void init(const TcParams& prm) {
+        p = &prm;
         long long total = 0;
         if (p->seq_lens) { for (int b = 0; b < p->B; ++b) total += (long long)p->Hkv * tiles_of(b); }
         else total = (long long)p->B * p->Hkv * tiles_of(0);
@@ -258,6 +246,121 @@ struct TileWalk {
         if (++tile < tiles_in_unit || left <= 0) return;
         tile = 0;
         do { ++unit; tiles_in_unit = tiles_of(unit / p->Hkv); } while (tiles_in_unit == 0);
+    }
+};
+
+// Walks the CTA's share of the multi-chunk pass 2.  A tile pair's items are the row chunks that see it; the items of all
+// pairs of all units, in order, are cut into gridDim.x equal runs, so that a CTA stays with a pair (128 KB of K and V) for
+// as long as possible and all do the same work, however many rows see a pair.  Only a CTA's first pair can have been begun
+// by another: the CTA's number within that pair is its `slot`, and every slot has its own copy of the score planes.
+// With csplit == 1 the runs consist of whole pairs.
+// (Dealing the chunks of every pair round to up to eight CTAs loaded each pair eight times and balanced the runs by the order
+// of the pairs only.  Pass 2 of the 4k whole-sequence window 268 -> 221 us, of 256 rows x 7043 tokens x 8 heads 32 -> 26, of 448
+// rows x 9000 tokens x 4 heads 33.5 -> 21.3.)
+template <bool SKIP>
+struct ItemWalk {
+    const TcParams* p;
+    int unit, pair, pairs;                    // current segment: chunks v0 .. v1 - 1 of those that see the pair
+    int v0, v1, slot;
+    int left;                                 // items still to visit, including the segment's
+    int past;                                 // tokens between the first one that not every row sees and the pair's first: > 0 where chunks can be hidden
+    __device__ __forceinline__ static int pairs_of(const TcParams& p, int b) { return ((tc_seq_len(p, b) + TILE - 1) / TILE + 1) / 2; }
+    __device__ __forceinline__ static int past_of(const TcParams& p, int b, int j) {
+        // (chunks of up to 64 rows of a head hold its last query, which sees everything)
+        return SKIP && p.causal && p.W > MC_ROWS ? j * 2 * TILE - (tc_mask_len(p, b) - p.W) : 0;
+    }
+    // a chunk inside head h whose last row lies `past` rows behind the head's first sees nothing of the pair: chunks lo .. hi - 1
+    __device__ __forceinline__ static void hidden_run(const TcParams& p, int h, int past, int& lo, int& hi) {
+        lo = (h * p.W + MC_ROWS - 1) / MC_ROWS;
+        hi = (h * p.W + min(past, p.W - 1)) / MC_ROWS;         // (a head's last query is never hidden)
+    }
+    __device__ __forceinline__ static int visible(const TcParams& p, int past) {
+        int n = p.n_chunks;
+        if (past > 0)
+            for (int h = 0, lo, hi; h < p.G; ++h) { hidden_run(p, h, past, lo, hi); n -= max(hi - lo, 0); }
+        return n;
+    }
+    // (the lanes of a warp take the pairs side by side: called by whole warps, as run_length and init)
+    __device__ __forceinline__ static int items_of(const TcParams& p, int b) {
+        const int n = pairs_of(p, b);
+        if (p.csplit == 1) return n;
+        int t = 0;
+        for (int j = threadIdx.x & 31; j < n; j += 32) t += visible(p, past_of(p, b, j));
+        return __reduce_add_sync(0xffffffffu, t);
+    }
+    // items per CTA; a pair is then shared by at most csplit of them
+    __device__ __forceinline__ static int run_length(const TcParams& p, int grid) {
+        long long total = 0;
+        if (p.seq_lens || p.mask_lens) { for (int b = 0; b < p.B; ++b) total += (long long)p.Hkv * items_of(p, b); }
+        else total = (long long)p.B * p.Hkv * items_of(p, 0);
+        const int run = (int)((total + grid - 1) / grid);
+        return max(run, p.csplit == 1 || p.csplit >= p.n_chunks ? 1 : (p.n_chunks + p.csplit - 2) / (p.csplit - 1));
+    }
+    // the segment that begins at item r of the current pair
+    __device__ __forceinline__ void segment(int b, int r) {
+        past = past_of(*p, b, pair);
+        const int n = visible(*p, past);
+        v0 = r;
+        v1 = p->csplit == 1 ? n : min(n, r + left);
+    }
+    __device__ void init(const TcParams& prm) {
+        p = &prm; slot = 0; left = 0; unit = pair = pairs = v0 = v1 = past = 0;
+        const int run = run_length(prm, (int)gridDim.x);
+        long long x = (long long)run * blockIdx.x;
+        int b = 0, t = 0;
+        for (; b < p->B; ++b) {
+            t = items_of(*p, b);
+            const long long blk = (long long)p->Hkv * t;
+            if (x < blk) break;
+            x -= blk;
+        }
+        if (b == p->B) return;
+        long long rest = (long long)p->Hkv * t - x;            // items from here to the end of everything, as far as the run goes
+        for (int bb = b + 1; bb < p->B && rest < run; ++bb) rest += (long long)p->Hkv * items_of(*p, bb);
+        left = (int)min((long long)run, rest);
+        unit = b * p->Hkv + (int)(x / t); pairs = pairs_of(*p, b);
+        int r = (int)(x % t);
+        if (p->csplit == 1) { pair = r; r = 0; }
+        else {
+            const int lane = threadIdx.x & 31;
+            for (;; pair += 32) {
+                const int n = pair + lane < pairs ? visible(*p, past_of(*p, b, pair + lane)) : 0;
+                int incl = n;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int up = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (lane >= o) incl += up;
+                }
+                const unsigned past_r = __ballot_sync(0xffffffffu, incl > r);
+                if (past_r) {
+                    const int f = __ffs(past_r) - 1;
+                    r -= __shfl_sync(0xffffffffu, incl - n, f);
+                    pair += f;
+                    break;
+                }
+                r -= __shfl_sync(0xffffffffu, incl, 31);
+            }
+        }
+        segment(b, r);
+        if (r > 0) slot = (int)blockIdx.x - (int)(((long long)run * blockIdx.x - r) / run);   // the pair was begun by the CTA of its first item
+    }
+    __device__ __forceinline__ bool done() const { return left <= 0; }
+    __device__ __forceinline__ bool ends_pair() const { return v1 == visible(*p, past); }
+    __device__ __forceinline__ void next() {
+        left -= p->csplit == 1 ? 1 : v1 - v0;
+        slot = 0;
+        if (left <= 0) return;
+        if (++pair == pairs) {
+            pair = 0;
+            do { ++unit; pairs = pairs_of(*p, unit / p->Hkv); } while (pairs == 0);
+        }
+        segment(unit / p->Hkv, 0);
+    }
+    // the v-th chunk that sees the pair
+    __device__ __forceinline__ int chunk(int v) const {
+        if (SKIP && past > 0)
+            for (int h = 0, lo, hi; h < p->G; ++h) { hidden_run(*p, h, past, lo, hi); if (hi > lo && v >= lo) v += hi - lo; }
+        return v;
     }
 };
 
@@ -675,7 +778,6 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // of the next chunk hides behind twice the tensor work.  Epilogue warpgroup j owns tile j of the
 // pair: it sums all chunks of its 128 tokens in registers and stores their scores itself.
 // =================================================================================================
-constexpr int MC_ROWS = 64;                                       // window rows per chunk
 constexpr uint32_t kHalfB64 = 64 * 128;                           // B operand block: [64 rows][64 bf16]
 constexpr uint32_t kQoBuf = 4 * kHalfB64;                         // Q chunk (2 x 8 KB) + -2 O chunk (2 x 8 KB)
 constexpr uint32_t MC_OFF_QO = 0;                                 // 2 buffers x 32 KB
@@ -709,7 +811,6 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     span_begin(p.span);
     const int units = p.B * p.Hkv;
-    const int nc = p.n_chunks;                                   // chunks of MC_ROWS rows
 
     if (threadIdx.x == 0) {
         prefetch_tmap(&map_k); prefetch_tmap(&map_v); prefetch_tmap(&map_q); prefetch_tmap(&map_o);
@@ -734,17 +835,13 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     int fail_site = 0;                             // source line of the wait that gave up (status word)
     const uint32_t qo_bytes = MC_ROWS * 128u * 2u * 2u;
 
-    // A position of the walk is a pair of tiles (2 * tw.tile + j, j = 0, 1; the second one may lie past
-    // the end of a unit with an odd tile count: it is computed all the same and stores only zeros).
+    // A position of the walk is a pair of tiles (2 * tw.pair + j, j = 0, 1; the second one may lie past
+    // the end of a unit with an odd tile count: it is computed all the same and stores only zeros) and a run of row chunks.
     // `pitem` counts positions, `citem` row chunks over all positions; the chunk's two MMA pairs are
     // items 2 * citem + j.  Rings: K/V stage j; Q/O buffer citem & 1; constant slot citem & 3; TMEM
     // buffer item & 3, so that epilogue group j always sees buffers j and j + 2.
-    TileWalk tw;
-    tw.init(p, 2, SPLIT ? p.csplit : 1);
-    const int cstep = SPLIT ? p.csplit : 1;
-    // a chunk of 64 rows can lose sight of a tile pair only if the window is longer than the chunk (with up to
-    // 64 window rows per head every chunk holds some head's last query, which sees the whole cache)
-    const bool may_skip = SPLIT && p.causal && p.W > MC_ROWS;
+    ItemWalk<SPLIT> tw;
+    tw.init(p);
     if (!(warp == 0 && lane == 0)) pdl_wait();       // the producer thread waits after its first K/V copies
     if (warp == 0) {
         // ===================================== TMA producer =====================================
@@ -752,11 +849,9 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             uint32_t pitem = 0, citem = 0;
             for (; !tw.done() && !failed; tw.next(), ++pitem) {
                 const int unit = tw.unit, b = unit / p.Hkv, g = unit % p.Hkv;
-                int pair, cs;
-                if (SPLIT) split_position(tw.tile, tw.tiles_in_unit, cstep, pair, cs); else { pair = tw.tile; cs = 0; }
                 for (int j = 0; j < 2 && !failed; ++j) {
                     if (!mbar_wait(bar(MC_EMPTY + j), (pitem & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
-                    const int t0 = (pair * 2 + j) * TILE;
+                    const int t0 = (tw.pair * 2 + j) * TILE;
                     mbar_expect_tx(bar(MC_FULL + j), 2 * kOperandBytes);
                     const uint32_t dk = sbase + MC_OFF_K + j * kOperandBytes, dv = sbase + MC_OFF_V + j * kOperandBytes;
                     tma_load_4d(dk, &map_k, bar(MC_FULL + j), 0, t0, g, b);
@@ -765,9 +860,8 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     tma_load_4d(dv + kHalfBytes, &map_v, bar(MC_FULL + j), 64, t0, g, b);
                 }
                 if (pitem == 0) pdl_wait();                        // K and V were read by pass 1; -2 O is the preceding kernel's output
-                const int pair_first = pair * 2 * TILE, Nu = tc_mask_len(p, b);
-                for (int c = cs; c < nc && !failed; c += cstep) {
-                    if (may_skip && rows_last_token(c * MC_ROWS, min(c * MC_ROWS + MC_ROWS, p.R) - 1, p.W, Nu, 1) < pair_first) continue;
+                for (int v = tw.v0; v < tw.v1 && !failed; ++v) {
+                    const int c = tw.chunk(v);
                     const uint32_t qb = citem & 1;
                     if (!mbar_wait(bar(MC_QO_EMPTY + qb), ((citem >> 1) & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
                     mbar_expect_tx(bar(MC_QO_FULL + qb), qo_bytes);
@@ -803,11 +897,7 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             uint32_t pitem = 0, citem = 0;
             for (; !tw.done() && !failed; tw.next(), ++pitem) {
                 if (!mbar_wait(bar(MC_FULL + 0), pitem & 1) || !mbar_wait(bar(MC_FULL + 1), pitem & 1)) { failed = true; fail_site = __LINE__; break; }
-                int pair, cs;
-                if (SPLIT) split_position(tw.tile, tw.tiles_in_unit, cstep, pair, cs); else { pair = tw.tile; cs = 0; }
-                const int pair_first = pair * 2 * TILE, Nu = tc_mask_len(p, tw.unit / p.Hkv);
-                for (int c = cs; c < nc && !failed; c += cstep) {
-                    if (may_skip && rows_last_token(c * MC_ROWS, min(c * MC_ROWS + MC_ROWS, p.R) - 1, p.W, Nu, 1) < pair_first) continue;
+                for (int v = tw.v0; v < tw.v1 && !failed; ++v) {
                     const uint32_t qb = citem & 1;
                     if (!mbar_wait(bar(MC_QO_FULL + qb), (citem >> 1) & 1)) { failed = true; fail_site = __LINE__; break; }
                     const uint32_t bq = desc_lo_k(sbase + MC_OFF_QO + qb * kQoBuf), bo = bq + ((2 * kHalfB64) >> 4);
@@ -862,11 +952,8 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 return true;
             };
             bool norms_done = false;
-            int pair, cs;
-            if (SPLIT) split_position(tw.tile, tw.tiles_in_unit, cstep, pair, cs); else { pair = tw.tile; cs = 0; }
-            const int pair_first = pair * 2 * TILE, Nu = tc_mask_len(p, unit / p.Hkv);
-            for (int c = cs; c < nc && !failed; c += cstep) {
-                if (may_skip && rows_last_token(c * MC_ROWS, min(c * MC_ROWS + MC_ROWS, p.R) - 1, p.W, Nu, 1) < pair_first) continue;
+            for (int v = tw.v0; v < tw.v1 && !failed; ++v) {
+                const int c = tw.chunk(v);
                 const uint32_t cs = citem & 3;
                 const size_t crow = (size_t)unit * p.rows_out + (size_t)c * MC_ROWS + t64;
                 const float2 cst = make_float2(-kExpFactor<VARS> * p.lse2[crow], p.onorm[crow] * (VARS == OBC_VAR_VK ? p.scale : 1.f));
@@ -895,16 +982,13 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
         uint32_t pitem = 0, citem = 0;
         for (; !tw.done() && !failed; tw.next(), ++pitem) {
             const int unit = tw.unit, b = unit / p.Hkv;
-            int pair, cs;
-            if (SPLIT) split_position(tw.tile, tw.tiles_in_unit, cstep, pair, cs); else { pair = tw.tile; cs = 0; }
-            const int N = tc_seq_len(p, b), Nm = tc_mask_len(p, b), t0 = (pair * 2 + wg) * TILE;
+            const int N = tc_seq_len(p, b), Nm = tc_mask_len(p, b), t0 = (tw.pair * 2 + wg) * TILE;
             const int ptok = t0 + tok;
             const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
             RowSums S;
             S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = make_float2(0.f, 0.f);
-            const int pair_first = pair * 2 * TILE;
-            for (int c = cs; c < nc; c += cstep) {
-                if (may_skip && rows_last_token(c * MC_ROWS, min(c * MC_ROWS + MC_ROWS, p.R) - 1, p.W, Nm, 1) < pair_first) continue;
+            for (int v = tw.v0; v < tw.v1; ++v) {
+                const int c = tw.chunk(v);
                 const uint32_t item = 2 * citem + wg, buf = item & 3, cs = citem & 3;
                 if (!mbar_wait(bar(MC_CONST + cs), (citem >> 2) & 1)) { failed = true; fail_site = __LINE__; break; }
                 if (!mbar_wait(bar(MC_TM_FULL + buf), (item >> 2) & 1)) { failed = true; fail_site = __LINE__; break; }
@@ -933,8 +1017,9 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             const float nv = nv21.x, nv1 = nv21.y;
             if (ptok < p.Nmax) {
                 // with the chunks of the pair shared by several CTAs each writes its part of the sums (the scores are
-                // linear in them) into its own copy of the planes; tc_partial_sum_kernel adds the copies in order
-                float* out = (cstep > 1 ? p.partial + (size_t)cs * __popc(p.variants) * plane : p.scores) + (size_t)unit * p.Nmax;
+                // linear in them), the first into the scores, the others into copies that tc_partial_sum_kernel adds in order
+                if (SPLIT && p.csplit > 1 && threadIdx.x == 128 && tw.ends_pair()) p.copies[(size_t)unit * p.max_pairs + tw.pair] = tw.slot;
+                float* out = (tw.slot > 0 ? p.partial + (size_t)(tw.slot - 1) * __popc(p.variants) * plane : p.scores) + (size_t)unit * p.Nmax;
                 const float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y};
                 store_scores<VARS>(sum, nv, nv1, p.scale, p.variants, out + ptok, plane, ptok < N);
             }
@@ -961,22 +1046,24 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
     }
 }
 
-// scores = sum over the csplit partial copies, in order, for the tokens that pass 2 visited (whole tile
-// pairs up to the unit's length; the zero padding beyond is written by pass 2 itself)
-__global__ void __launch_bounds__(256)
+// Adds to the scores of every tile pair that several CTAs shared what its second, third, ... CTA left in its copy, in that
+// order.  One block per pair.
+__global__ void __launch_bounds__(2 * TILE)
 tc_partial_sum_kernel(TcParams p, int n_planes) {
     pdl_wait();
-    const int unit = blockIdx.y, b = unit / p.Hkv;
-    const int N = tc_seq_len(p, b);
-    const int end = min((N + 2 * TILE - 1) / (2 * TILE) * (2 * TILE), p.Nmax);
+    const int unit = blockIdx.y, j = blockIdx.x, tok = j * 2 * TILE + threadIdx.x;
+    if (j * 2 * TILE >= tc_seq_len(p, unit / p.Hkv) || tok >= p.Nmax) return;
+    // (bounded: after a wait that gave up nobody may have written the count)
+    const int copies = min(p.copies[(size_t)unit * p.max_pairs + j], p.csplit - 1);
+    if (copies <= 0) return;
     const size_t plane = (size_t)p.B * p.Hkv * p.Nmax;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < end; i += gridDim.x * blockDim.x)
-        for (int pl = 0; pl < n_planes; ++pl) {
-            const size_t at = (size_t)pl * plane + (size_t)unit * p.Nmax + i;
-            float sum = 0.f;
-            for (int cs = 0; cs < p.csplit; ++cs) sum += p.partial[(size_t)cs * n_planes * plane + at];
-            p.scores[at] = sum;
-        }
+    for (int pl = 0; pl < n_planes; ++pl) {
+        const size_t at = (size_t)pl * plane + (size_t)unit * p.Nmax + tok;
+        float sum = p.scores[at];
+#pragma unroll 4
+        for (int cp = 0; cp < copies; ++cp) sum += p.partial[(size_t)cp * n_planes * plane + at];
+        p.scores[at] = sum;
+    }
 }
 
 // =================================================================================================
@@ -1549,19 +1636,17 @@ bool tc_supported(const ScoreShape& s, int dtype, const TensorView& q) {
     return q.sh == (long long)s.W * q.st && q.sb == (long long)s.Hq * q.sh;
 }
 
-// Multi-chunk pass 2: with fewer tile pairs than about two per SM (a short cache scored over a long window)
-// the row chunks of every pair are shared by several CTAs.
+// Multi-chunk pass 2: with fewer tile pairs than about two per SM (a short cache scored over a long window) the row chunks
+// of a pair may be shared by several CTAs (see ItemWalk): as many as an equal share of the items allows, where at least half
+// of all (pair, chunk) items are visible.  With more pairs whole ones balance well enough and no partial scores have to be
+// added up.
 static int tc_chunk_split(const ScoreShape& s, const TcChunks& ch) {
     if (ch.n_chunks <= 1) return 1;
     const long long pairs = (long long)s.B * s.Hkv * (((s.Nmax + TILE - 1) / TILE + 1) / 2);
-    const int nc = ch.rows_out / MC_ROWS, sms = sm_count();
-    if (pairs >= 2LL * sms) return 1;
-    // about seven positions per SM: on the 4k whole-sequence window 8 CTAs per pair took 272 us, 4 took 305, 3 took 326,
-    // 12 took 270 and 16 took 282 (every position loads its tile pair again and adds a copy of the score planes)
-    int c = (int)((7LL * sms + pairs - 1) / pairs);
-    if (c > 8) c = 8;
-    if (c > nc) c = nc;
-    return c < 1 ? 1 : c;
+    if (pairs >= 2LL * sm_count()) return 1;
+    const int nc = ch.rows_out / MC_ROWS;
+    const int run = (int)(pairs * nc / (2 * sm_count())), c = (nc + run) / (run > 1 ? run : 1) + 1;
+    return c < 2 ? 2 : c > 32 ? 32 : c > nc ? nc : c;
 }
 
 // Workspace plan of the tensor-core path: the SIMT plan's layout with splits counted in 128-token tiles.
@@ -1599,7 +1684,8 @@ static SimtPlan make_tc_plan(const ScoreShape& s) {
 // the partial score planes of a shared multi-chunk pass 2 follow the plan's arrays
 static size_t tc_partial_bytes(const ScoreShape& s) {
     const int cs = tc_chunk_split(s, tc_chunks(s.R));
-    return cs > 1 ? (size_t)cs * s.n_planes * s.B * s.Hkv * s.Nmax * 4 : 0;
+    const size_t units = (size_t)s.B * s.Hkv;
+    return cs > 1 ? (size_t)(cs - 1) * s.n_planes * units * s.Nmax * 4 + units * ((s.Nmax + 2 * TILE - 1) / (2 * TILE)) * 4 : 0;
 }
 
 size_t tc_workspace_bytes(const ScoreShape& s) { return make_tc_plan(s).bytes + tc_partial_bytes(s); }
@@ -1704,14 +1790,17 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         p.n_chunks = ch.rows_out / MC_ROWS; p.chunk_rows = MC_ROWS;
         p.csplit = tc_chunk_split(s, ch);
         p.partial = (float*)(wsb + plan.bytes);
-        const long long positions = (long long)units * (((s.Nmax + TILE - 1) / TILE + 1) / 2) * p.csplit;
+        const int pairs = (s.Nmax + 2 * TILE - 1) / (2 * TILE);
+        p.max_pairs = pairs;
+        p.copies = (int*)(p.partial + (size_t)(p.csplit - 1) * s.n_planes * units * s.Nmax);
+        const long long positions = (long long)units * pairs * (p.csplit > 1 ? p.n_chunks : 1);
         const int mgrid = (int)(positions < sm_count() ? positions : sm_count());
         auto launch_multi = [&](auto kernel) -> obc_status {
             OBC_CUDA_TRY(allow_smem(kernel, kSmemMulti));
             { ProfScope ps("tc_pass2", stream); OBC_CUDA_TRY(launch_pdl(kernel, dim3(mgrid), dim3(kThreadsMulti), kSmemMulti, stream, 1, mq64, mo64, mk, mv, p)); }
             if (p.csplit > 1) {
                 ProfScope ps("partial_sum", stream);
-                OBC_CUDA_TRY(launch_pdl(tc_partial_sum_kernel, dim3((s.Nmax + 255) / 256, units), dim3(256), 0, stream, 1, p, s.n_planes));
+                OBC_CUDA_TRY(launch_pdl(tc_partial_sum_kernel, dim3(pairs, units), dim3(2 * TILE), 0, stream, 1, p, s.n_planes));
             }
             return OBC_OK;
         };

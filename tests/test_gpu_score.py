@@ -114,6 +114,19 @@ def test_full_history_window(N, Hq, Hkv, dtype, path):
     _check(case, ["V", "K", "VK", "ATTN", "VATP"], path=path, tight=2e-2 if dtype == "bf16" else None)
 
 
+@pytest.mark.parametrize("N,W,Hq,Hkv,lens", [
+    (1641, 1641, 4, 1, None),             # chunks that straddle heads, a pair shared by many CTAs
+    (700, 300, 6, 2, [700, 431]),         # hidden chunks in the last pairs only, two lengths
+    (513, 513, 8, 8, None),               # one token in the last pair
+    (2300, 130, 5, 1, None),              # three chunks per head and a bit
+    (257, 65, 3, 1, [257, 65]),           # the shorter sequence is all window
+])
+def test_row_chunks_shared_by_several_ctas(N, W, Hq, Hkv, lens):
+    case = synth.make_prefill("items", B=len(lens) if lens else 1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=lens or N, dtype="bf16", seed=N + W, hh_frac=0.02)
+    _check(case, ["VK"], tight=2e-2)
+    _check(case, ["V", "K", "VK", "ATTN"], tight=2e-2)
+
+
 def test_peaky_attention_cancellation_case():
     # some attention weights approach 1, so ||v_p - o_i||^2 cancels heavily
     case = synth.make_prefill("peaky", B=1, Hq=8, Hkv=2, d=128, W=16, N=2048, dtype="bf16", seed=5,
