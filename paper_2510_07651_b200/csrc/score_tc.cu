@@ -1113,10 +1113,11 @@ struct P1Params {
     float* nv;                                             // [units][Nmax]: ||v_p||^2, written by the CTAs of the last row chunk; null: not wanted
     unsigned int* status;
     unsigned long long* span;                              // [2]: ~(earliest CTA start), latest CTA end, in globaltimer ns
-    // One CTA per (unit, row chunk) and no padding rows: the CTA writes the merged results itself (what the combine
-    // kernel would make of its single partial) and no combine kernel runs.  Null out_o: partial results as above.
-    float* out_o; __nv_bfloat16* out_obf;                  // [units][R][d]: O and -2 O
-    float* out_lse2; float* out_onorm; float* out_cpair;   // [units][R]; row-pair constants as float4 per pair
+    // One CTA per (unit, row chunk): the CTA writes the merged results itself (what the combine kernel would make of its
+    // single partial), the last chunk's also the padding rows, and no combine kernel runs.  Null out_o: partial results as above.
+    int rows_out;
+    float* out_o; __nv_bfloat16* out_obf;                  // [units][rows_out][d]: O; -2 O (HILO: a high and a low part per unit)
+    float* out_lse2; float* out_onorm; float* out_cpair;   // [units][rows_out]; row-pair constants as float4 per pair
 };
 
 __device__ __forceinline__ void tc_ld32(uint32_t taddr, uint32_t* r) {
@@ -1549,26 +1550,47 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 }
             }
             if (fin) {
-                // rows of the unit are rows of the outputs (one split, no padding rows): O, -2 O in bf16, and per row
-                // the log2-sum-exp, ||o||^2 and the row's half of its pair's constants
+                // O, -2 O in bf16, and per row the log2-sum-exp, ||o||^2 and the row's half of its pair's constants
+                const size_t out0 = (size_t)unit * p.rows_out + (size_t)c * p.chunk_rows;
+                __nv_bfloat16* obf = p.out_obf + ((size_t)unit * p.rows_out * (HILO ? 2 : 1) + (size_t)c * p.chunk_rows) * kD + lane * 4;
+                float on = 0.f;                                              // of row row_lo + lane
+                if (!HILO && lane < 16) on = xs[row_lo + lane] + xs[128 + row_lo + lane];
 #pragma unroll
                 for (int rr = 0; rr < 16; ++rr) {
                     const int orow = row_lo + rr;
                     if (orow < rows_valid) {
-                        *reinterpret_cast<uint4*>(p.out_o + (prow0 + orow) * kD + lane * 4) = rowv[rr];
-                        const uint32_t b0 = pack_bf16x2(-2.f * __uint_as_float(rowv[rr].x), -2.f * __uint_as_float(rowv[rr].y));
-                        const uint32_t b1 = pack_bf16x2(-2.f * __uint_as_float(rowv[rr].z), -2.f * __uint_as_float(rowv[rr].w));
-                        *reinterpret_cast<uint2*>(p.out_obf + (prow0 + orow) * kD + lane * 4) = make_uint2(b0, b1);
+                        const float4 o = make_float4(__uint_as_float(rowv[rr].x), __uint_as_float(rowv[rr].y), __uint_as_float(rowv[rr].z), __uint_as_float(rowv[rr].w));
+                        *reinterpret_cast<float4*>(p.out_o + (out0 + orow) * kD + lane * 4) = o;
+                        const uint32_t b0 = pack_bf16x2(-2.f * o.x, -2.f * o.y), b1 = pack_bf16x2(-2.f * o.z, -2.f * o.w);
+                        *reinterpret_cast<uint2*>(obf + (size_t)orow * kD) = make_uint2(b0, b1);
+                        if (HILO) {                                          // what the high part leaves out; the norm of both parts of O
+                            const float2 h0 = bf16x2_to_f32x2(b0), h1 = bf16x2_to_f32x2(b1);
+                            *reinterpret_cast<uint2*>(obf + (size_t)(p.rows_out + orow) * kD) =
+                                make_uint2(pack_bf16x2(fmaf(-2.f, o.x, -h0.x), fmaf(-2.f, o.y, -h0.y)), pack_bf16x2(fmaf(-2.f, o.z, -h1.x), fmaf(-2.f, o.w, -h1.y)));
+                            const float n = warp_sum((o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w));
+                            if (lane == rr) on = n;
+                        }
                     }
                 }
                 if (lane < 16 && row_lo + lane < rows_valid) {
-                    const int orow = row_lo + lane;
-                    const size_t gr = prow0 + orow;
-                    const float lse2 = xs[256 + orow], on = xs[orow] + xs[128 + orow];
+                    const size_t gr = out0 + row_lo + lane;
+                    const float lse2 = xs[256 + row_lo + lane];
                     p.out_lse2[gr] = lse2; p.out_onorm[gr] = on;
                     float* cp = p.out_cpair + (gr >> 1) * 4 + (gr & 1);
                     cp[0] = -lse2; cp[2] = on;
                 }
+                if (c == p.n_chunks - 1)                                     // padding rows: O = 0, weight 0
+                    for (int r0 = p.R - c * p.chunk_rows + warp - 4; r0 < p.rows_out - c * p.chunk_rows; r0 += 8) {
+                        *reinterpret_cast<float4*>(p.out_o + (out0 + r0) * kD + lane * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+                        *reinterpret_cast<uint2*>(obf + (size_t)r0 * kD) = make_uint2(0u, 0u);
+                        if (HILO) *reinterpret_cast<uint2*>(obf + (size_t)(p.rows_out + r0) * kD) = make_uint2(0u, 0u);
+                        if (lane == 0) {
+                            const size_t gr = out0 + r0;
+                            p.out_lse2[gr] = INFINITY; p.out_onorm[gr] = 0.f;
+                            float* cp = p.out_cpair + (gr >> 1) * 4 + (gr & 1);
+                            cp[0] = -INFINITY; cp[2] = 0.f;
+                        }
+                    }
             } else {
 #pragma unroll
                 for (int rr = 0; rr < 16; ++rr) {                            // one coalesced 512-byte row per instruction
@@ -1743,10 +1765,10 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         p1.nv = want_nv ? (float*)(wsb + plan.off_nv) : nullptr;
         p1.status = (unsigned int*)(wsb + plan.off_flag);
         p1.span = (unsigned long long*)(wsb + plan.off_flag + kSpanOffset);
-        // with one CTA per (unit, row chunk) and no padding rows there is nothing to merge: pass 1 writes the results itself
-        // (two MMA rows per window row still have to be added up)
-        const bool direct = plan.n_splits == 1 && ch.rows_out == s.R && !hilo;
+        // with one CTA per (unit, row chunk) there is nothing to merge: pass 1 writes the results itself
+        const bool direct = plan.n_splits == 1;
         if (direct) {
+            p1.rows_out = plan.rows_out;
             p1.out_o = (float*)(wsb + plan.off_o); p1.out_obf = (__nv_bfloat16*)(wsb + plan.off_obf);
             p1.out_lse2 = (float*)(wsb + plan.off_lse2); p1.out_onorm = (float*)(wsb + plan.off_onorm);
             p1.out_cpair = (float*)(wsb + plan.off_cpair);

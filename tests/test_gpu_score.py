@@ -114,6 +114,13 @@ def test_full_history_window(N, Hq, Hkv, dtype, path):
     _check(case, ["V", "K", "VK", "ATTN", "VATP"], path=path, tight=2e-2 if dtype == "bf16" else None)
 
 
+@pytest.mark.parametrize("N,W,Hq,Hkv", [(100, 40, 2, 2), (90, 20, 160, 80), (300, 5, 320, 160), (150, 16, 640, 160), (131, 50, 480, 160)])
+def test_one_cta_per_head_and_chunk(N, W, Hq, Hkv):
+    # pass 1 writes the merged rows itself, padding rows included: R = 40 (two bf16 parts), 40, 10, 64 and 150 (two chunks)
+    case = synth.make_prefill("direct", B=1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=N + W, hh_frac=0.02)
+    _check(case, ["K", "VK"], tight=2e-2)
+
+
 @pytest.mark.parametrize("N,W,Hq,Hkv,lens", [
     (1641, 1641, 4, 1, None),             # chunks that straddle heads, a pair shared by many CTAs
     (700, 300, 6, 2, [700, 431]),         # hidden chunks in the last pairs only, two lengths
