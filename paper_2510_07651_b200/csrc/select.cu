@@ -157,12 +157,14 @@ __device__ __forceinline__ int adaptive_rem(const SelectShape& s, int b, uint32_
     return s.Hkv * (n_hh - (int)n_safe);
 }
 
-// Scored tokens that head `unit` keeps (-1: the budget does not fit): the last digit of T and the tie shares.  All threads
-// of the block call it.
-__device__ int adaptive_hh(const SelectShape& s, const AdaptiveLevels& lv, int unit, AdaptiveFind& sh) {
+// What head `unit` keeps: n_hh scored tokens (-1: the budget does not fit), found from the last digit of T and the tie
+// shares.  Where the head has n_safe candidates at or above T they are those above T and the first k_eq equal to T, and
+// the head needs no search of its own (`known`).  All threads of the block call it.
+struct HeadShare { int n_hh; bool known; uint32_t T, k_eq; };
+__device__ HeadShare adaptive_share(const SelectShape& s, const AdaptiveLevels& lv, int unit, AdaptiveFind& sh) {
     const int b = unit / s.Hkv, u0 = b * s.Hkv, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, warps = (int)blockDim.x >> 5;
     const int rem = adaptive_rem(s, b, lv.n_safe);
-    if (rem <= 0) return rem < 0 ? -1 : (int)lv.n_safe;
+    if (rem <= 0) return HeadShare{rem < 0 ? -1 : (int)lv.n_safe, false, 0u, 0u};
     const uint32_t d = adaptive_find<2>(lv, u0, s.Hkv, (uint32_t)rem, sh);
     auto beyond = [&](uint32_t c) { return c > lv.n_safe ? c - lv.n_safe : 0u; };
     // sums over the heads: slots that the candidates above T take, and candidates equal to T of the heads before this one
@@ -173,12 +175,15 @@ __device__ int adaptive_hh(const SelectShape& s, const AdaptiveLevels& lv, int u
         if (lane == 0) {
             atomicAdd(&sh.run_sum[0], beyond(up));
             if (u0 + h < unit) atomicAdd(&sh.run_sum[1], ties);
-            if (u0 + h == unit) { sh.bin_sum[0] = up; sh.bin_sum[1] = ties; }
+            if (u0 + h == unit) { sh.bin_sum[0] = up; sh.bin_sum[1] = ties; sh.bin_sum[2] = lv.row(2, unit)[d]; }
         }
     }
     __syncthreads();
     const uint32_t left = (uint32_t)rem - sh.run_sum[0], before = sh.run_sum[1], up = sh.bin_sum[0], ties = sh.bin_sum[1];
-    return (int)(max(lv.n_safe, up) + (before < left ? min(ties, left - before) : 0u));     // ties: lowest head first
+    const uint32_t hh = max(lv.n_safe, up) + (before < left ? min(ties, left - before) : 0u);           // ties: lowest head first
+    const uint32_t T = lv.digit[b * 2] << 21 | lv.digit[b * 2 + 1] << 10 | d;
+    const bool known = up + sh.bin_sum[2] >= lv.n_safe;
+    return HeadShare{(int)hh, known, known ? T : 0u, known ? hh - up : 0u};
 }
 
 // adds a CTA's histogram of `bins` bins to the unit's row, with the sums over its 32 runs
@@ -224,7 +229,7 @@ adaptive_hist_kernel(SelectShape s, const uint32_t* __restrict__ keys, AdaptiveL
     pdl_wait();
     const int unit = blockIdx.y, b = unit / s.Hkv, u0 = b * s.Hkv, c0 = blockIdx.x * lv.chunk, c1 = min(c0 + lv.chunk, s.Nmax);
     const int rem = adaptive_rem(s, b, lv.n_safe);
-    if (rem <= 0) return;                                      // nothing to share out (adaptive_hh sees to it)
+    if (rem <= 0) return;                                      // nothing to share out (adaptive_share sees to it)
     const uint32_t d = adaptive_find<LEVEL - 2>(lv, u0, s.Hkv, (uint32_t)rem, sh);
     if (unit == u0 && blockIdx.x == 0) {                       // one CTA per batch item leaves the result for the next level
         for (int h = threadIdx.x >> 5; h < s.Hkv; h += AD_NT / 32) {
@@ -257,7 +262,9 @@ select_kernel(SelectShape s, const uint32_t* __restrict__ keys_all, int32_t* __r
     const int N = seq_len(s, b);
     const int lo = s.n_sink, hi = N - s.n_recent, n = hi - lo;
     __shared__ AdaptiveFind ad_sh;
-    const int n_hh = ad.hist ? adaptive_hh(s, ad, unit, ad_sh) : budget_of(s, b) - s.n_sink - s.n_recent;
+    HeadShare share{budget_of(s, b) - s.n_sink - s.n_recent, false, 0u, 0u};
+    if (ad.hist) share = adaptive_share(s, ad, unit, ad_sh);
+    const int n_hh = share.n_hh;
     const int budget = n_hh + s.n_sink + s.n_recent;
     const uint32_t* keys = keys_all + (size_t)unit * s.Nmax;
     int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
@@ -276,8 +283,8 @@ select_kernel(SelectShape s, const uint32_t* __restrict__ keys_all, int32_t* __r
     if (n_hh == 0) return;
 
     // ---- radix search for the key T of the n_hh-th largest candidate -----------------------
-    uint32_t prefix = 0, mask = 0, remaining = (uint32_t)n_hh;
-    for (int shift = 24; shift >= 0; shift -= 8) {
+    uint32_t prefix = share.T, mask = 0, remaining = share.known ? share.k_eq : (uint32_t)n_hh;
+    for (int shift = 24; shift >= 0 && !share.known; shift -= 8) {
         if (tid < 256) hist[tid] = 0;
         __syncthreads();
         for (int base = 0; base < n; base += SEL_NT) {
@@ -438,7 +445,9 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     const int N = seq_len(s, b);
     const int lo = s.n_sink, hi = N - s.n_recent, n = hi - lo;
     // (the search across heads borrows the space of a histogram that is cleared below)
-    const int n_hh = ad.hist ? adaptive_hh(s, ad, unit, *reinterpret_cast<AdaptiveFind*>(&sh.local[0])) : budget_of(s, b) - s.n_sink - s.n_recent;
+    HeadShare share{budget_of(s, b) - s.n_sink - s.n_recent, false, 0u, 0u};
+    if (ad.hist) share = adaptive_share(s, ad, unit, *reinterpret_cast<AdaptiveFind*>(&sh.local[0]));
+    const int n_hh = share.n_hh;
     const int budget = n_hh + s.n_sink + s.n_recent;
     int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -460,10 +469,11 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     const int seg = ((n + C - 1) / C + 31) / 32 * 32;
     const int c0 = min(rank * seg, n), c1 = min(c0 + seg, n), m = c1 - c0;
     if (tid == 0) sh.n_list = 0;
-    if (keys_in) for (int i = tid; i < 4 * CL_BINS; i += CL_NT) (&sh.sum[0][0])[i] = 0;   // sum[3][] and local[]
+    if (keys_in && !share.known) for (int i = tid; i < 4 * CL_BINS; i += CL_NT) (&sh.sum[0][0])[i] = 0;   // sum[3][] and local[]
 
     if (keys_in) {                                 // the caller has the (pooled) keys already: [units][Nmax]
         const uint32_t* kin = keys_in + (size_t)unit * s.Nmax + lo + c0;
+#pragma unroll 8
         for (int i = tid; i < m; i += CL_NT) keys[i] = kin[i];
         __syncthreads();
         cluster.barrier_arrive();
@@ -534,10 +544,12 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     // what the CTAs before it keep, without further exchanges.  Only when the lists do not fit their slots (keys
     // that all but coincide) do passes 1 and 2 run across the cluster as pass 0 did.
     uint32_t* list = reinterpret_cast<uint32_t*>(stage);
-    uint32_t prefix = 0, mask = 0, remaining = (uint32_t)n_hh;
+    // (A threshold that the ranking across heads has settled needs no search.)
+    uint32_t prefix = share.T, mask = 0, remaining = share.known ? share.k_eq : (uint32_t)n_hh;
     const int slot_cap = CL_GATHER / C;
     bool gathered_path = false;
-    for (int ps = 0; ps < 3 && !gathered_path; ++ps) {
+    if (share.known) cluster.barrier_wait();
+    for (int ps = 0; ps < 3 && !gathered_path && !share.known; ++ps) {
         const int shift = ps == 0 ? 21 : ps == 1 ? 10 : 0;
         const uint32_t dmask = ps == 2 ? 1023u : 2047u;
         const uint32_t* src = ps == 0 ? keys : list;
