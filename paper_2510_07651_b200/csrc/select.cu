@@ -199,6 +199,14 @@ __device__ __forceinline__ void adaptive_flush(const uint32_t* hist, int bins, u
     }
 }
 
+// (a kernel instead of a memset, which would keep the kernels before and after it from overlapping its ends)
+__global__ void __launch_bounds__(AD_NT)
+adaptive_clear_kernel(uint4* hist, long long n) {
+    pdl_wait();
+    const long long i = (long long)blockIdx.x * AD_NT + threadIdx.x;
+    if (i < n) hist[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
 __global__ void __launch_bounds__(AD_NT)
 adaptive_pool_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* __restrict__ keys, AdaptiveLevels lv) {
     __shared__ uint32_t hist[AD_BINS];
@@ -958,7 +966,9 @@ obc_status launch_select_adaptive(const SelectShape& s, int n_safe, const float*
     const AdaptiveLevels lv{(uint32_t*)(w + plan.off_hist), (uint32_t*)(w + plan.off_above), (uint32_t*)(w + plan.off_digit), counts,
                             (uint32_t)n_safe, chunk, units};
     const dim3 grid((unsigned)((s.Nmax + chunk - 1) / chunk), (unsigned)units);
-    OBC_CUDA_TRY(cudaMemsetAsync(w + plan.off_hist, 0, 3 * (size_t)units * AD_ROW * 4, stream));
+    const long long n_clear = 3LL * units * AD_ROW / 4;
+    { ProfScope ps("adaptive_clear", stream);
+      OBC_CUDA_TRY(launch_pdl(adaptive_clear_kernel, dim3((unsigned)((n_clear + AD_NT - 1) / AD_NT)), dim3(AD_NT), 0, stream, 1, (uint4*)lv.hist, n_clear)); }
     { ProfScope ps("adaptive_pool", stream); OBC_CUDA_TRY(launch_pdl(adaptive_pool_kernel, grid, dim3(AD_NT), 0, stream, 1, s, scores, keys, lv)); }
     { ProfScope ps("adaptive_hist", stream); OBC_CUDA_TRY(launch_pdl(adaptive_hist_kernel<2>, grid, dim3(AD_NT), 0, stream, 1, s, (const uint32_t*)keys, lv)); }
     { ProfScope ps("adaptive_hist", stream); OBC_CUDA_TRY(launch_pdl(adaptive_hist_kernel<3>, grid, dim3(AD_NT), 0, stream, 1, s, (const uint32_t*)keys, lv)); }
