@@ -301,10 +301,11 @@ simt_combine_kernel(ScoreShape s, SimtPlan plan, float* ws) {
 
 // The same merge with one warp per (unit, output row), for many rows (a window of thousands of queries, a large
 // batch): no block-wide barrier, lane t holds head-dim elements 4t..4t+3, the splits are added in order, eight at a time.
-constexpr int CMBW_MAX_SPLITS = 8;
-// FEW: at most CMBW_MAX_SPLITS splits, one batch of loads and the maximum taken from it (one round trip to L2 in all)
-template <bool FEW>
-__global__ void __launch_bounds__(CMB_NT)
+// BATCH: splits whose loads travel together.  FEW: there are no more splits than that, and the maximum comes from the one batch
+// (one round trip to L2 in all).  With two splits a batch of two leaves registers for
+// twice the warps of a batch of eight (8192 rows of two splits: 7.8 -> 5.7 us).
+template <int BATCH, bool FEW>
+__global__ void __launch_bounds__(CMB_NT, BATCH <= 2 ? 12 : 1)
 simt_combine_rows_kernel(ScoreShape s, SimtPlan plan, float* ws) {
     pdl_wait();
     const int lane = threadIdx.x & 31;
@@ -322,11 +323,11 @@ simt_combine_rows_kernel(ScoreShape s, SimtPlan plan, float* ws) {
         const size_t row0 = (size_t)unit * plan.n_splits * s.R + r;          // split sp: row0 + sp * R
         const int n_act = active_splits(plan, seq_len(s, unit / s.Hkv));
         float M = -INFINITY, L = 0.f;
-        float m[CMBW_MAX_SPLITS], l[CMBW_MAX_SPLITS];
-        float4 o4[CMBW_MAX_SPLITS];
+        float m[BATCH], l[BATCH];
+        float4 o4[BATCH];
         auto load_batch = [&](int base) {                                    // every load of the batch before the first use
 #pragma unroll
-            for (int u = 0; u < CMBW_MAX_SPLITS; ++u) {
+            for (int u = 0; u < BATCH; ++u) {
                 const int sp = base + u;
                 const bool on = sp < n_act;
                 m[u] = on ? part_m[row0 + (size_t)sp * s.R] : -INFINITY;
@@ -340,14 +341,14 @@ simt_combine_rows_kernel(ScoreShape s, SimtPlan plan, float* ws) {
         // otherwise the lanes read the splits' maxima side by side
         float mrest = -INFINITY;
         if (!FEW)
-            for (int sp = CMBW_MAX_SPLITS + lane; sp < n_act; sp += 32) mrest = fmaxf(mrest, part_m[row0 + (size_t)sp * s.R]);
+            for (int sp = BATCH + lane; sp < n_act; sp += 32) mrest = fmaxf(mrest, part_m[row0 + (size_t)sp * s.R]);
 #pragma unroll
-        for (int u = 0; u < CMBW_MAX_SPLITS; ++u) M = fmaxf(M, m[u]);
-        if (!FEW && n_act > CMBW_MAX_SPLITS) M = fmaxf(M, warp_max(mrest));
-        for (int base = 0; base < (FEW ? 1 : n_act); base += CMBW_MAX_SPLITS) {
+        for (int u = 0; u < BATCH; ++u) M = fmaxf(M, m[u]);
+        if (!FEW && n_act > BATCH) M = fmaxf(M, warp_max(mrest));
+        for (int base = 0; base < (FEW ? 1 : n_act); base += BATCH) {
             if (base > 0) load_batch(base);
 #pragma unroll
-            for (int u = 0; u < CMBW_MAX_SPLITS; ++u) {
+            for (int u = 0; u < BATCH; ++u) {
                 const float w = m[u] == -INFINITY ? 0.f : exp2f(m[u] - M);
                 L = fmaf(l[u], w, L);
                 oc.x = fmaf(o4[u].x, w, oc.x); oc.y = fmaf(o4[u].y, w, oc.y);
@@ -672,11 +673,12 @@ obc_status launch_combine(const ScoreShape& s, const SimtPlan& plan, void* ws, c
     const long long rows = (long long)s.B * s.Hkv * plan.rows_out;
     // a warp per row when there are many rows: with 8192 rows of 16 splits (ragged batch of 8) 23 us against 31 us for a
     // block per row; with 1024 rows of 18 splits (one 32k layer) the block per row wins, 8.5 us against 14.5 us
-    if ((plan.n_splits <= CMBW_MAX_SPLITS && rows >= 1024) || rows >= 4096) {
+    if ((plan.n_splits <= 8 && rows >= 1024) || rows >= 4096) {
         ProfScope ps("combine", stream);
         const dim3 grid((unsigned)((rows + CMB_NT / 32 - 1) / (CMB_NT / 32)));
-        if (plan.n_splits <= CMBW_MAX_SPLITS) OBC_CUDA_TRY(launch_pdl(simt_combine_rows_kernel<true>, grid, dim3(CMB_NT), 0, stream, 1, s, plan, (float*)ws));
-        else OBC_CUDA_TRY(launch_pdl(simt_combine_rows_kernel<false>, grid, dim3(CMB_NT), 0, stream, 1, s, plan, (float*)ws));
+        const auto kernel = plan.n_splits <= 2 ? simt_combine_rows_kernel<2, true> : plan.n_splits <= 8 ? simt_combine_rows_kernel<8, true>
+                                                                                                        : simt_combine_rows_kernel<8, false>;
+        OBC_CUDA_TRY(launch_pdl(kernel, grid, dim3(CMB_NT), 0, stream, 1, s, plan, (float*)ws));
         return OBC_OK;
     }
     { ProfScope ps("combine", stream); OBC_CUDA_TRY(launch_pdl(simt_combine_kernel, dim3(s.B * s.Hkv * plan.rows_out), dim3(CMB_NT), 0, stream, 1, s, plan, (float*)ws)); }
