@@ -3,10 +3,17 @@
 //
 //   select_cluster_kernel  one thread-block cluster per (batch item, KV head).  Every CTA pools
 //                     its contiguous share of the candidates into order-preserving uint32 keys
-//                     held in shared memory; three radix passes (11 + 11 + 10 bits) whose
-//                     histograms are summed in the leading CTA's shared memory find the key of
-//                     the n_hh-th largest candidate and how many of its ties are kept; the
-//                     CTAs exchange their counts and emit the kept indices in ascending order
+//                     held in shared memory; a histogram of their top 11 bits, summed over the
+//                     cluster, leaves a few hundred keys, on which every CTA finds the key of the
+//                     n_hh-th largest candidate and how many of its ties are kept; the CTAs emit
+//                     the kept indices in ascending order.  Bound by the chain of its phases, not
+//                     by memory (1 MB of scores at 8 heads of 32768): what a phase costs is barrier
+//                     latency and issue slots that all 16 warps spend on the same scalar work, so
+//                     sums go through warp reductions, scans run in the one warp that needs them,
+//                     four candidates travel per shared-memory access and the last 10 bits are
+//                     settled by ranking the few keys left.  8 heads of 32768: 12.0 -> 8.4 us, one
+//                     of 1024: 8.8 -> 5.4 (against scans in all warps, one candidate per access
+//                     and a third histogram)
 //   pool_key_kernel + select_kernel   the same selection with one CTA per head and the keys in
 //                     global memory: the path for sequences too long for a cluster's shared memory
 //   gather_kernel     16-byte vector copy of the kept K/V rows (and optionally their scores)
@@ -386,8 +393,9 @@ constexpr int CL_GATHER = 2 * CL_BINS;        // survivors of the first pass tha
 struct ClusterShared {                        // fixed part of the CTA's shared memory
     uint32_t sum[3][CL_BINS];                 // per radix pass: histogram of the whole head (every CTA adds into every copy)
     uint32_t local[CL_BINS];                  // this CTA's histogram of the current pass
-    uint32_t found[2];                        // result of a pass: prefix, remaining
-    uint32_t n_list;                          // candidates of this CTA that survive the first pass
+    uint32_t found[3];                        // result of a pass: digit, remaining, keys that share the digit
+    uint32_t n_list, n_above;                 // candidates of this CTA that survive the first pass, and that lie in higher bins
+    uint32_t n_few, few[32];                  // keys that share all but the last 10 bits of T, if there are no more than 32
     uint32_t rank_gt[16], rank_eq[16];        // kept-candidate counts of every CTA of the cluster
     uint32_t rank_list[16], rank_above[16];   // per CTA: survivors of the first pass, candidates in higher bins
     uint32_t before[2];                       // kept candidates (greater, equal) in the CTAs before this one
@@ -398,44 +406,52 @@ struct ClusterShared {                        // fixed part of the CTA's shared 
 };
 
 // The highest bin D of hist[0 .. CL_BINS) with count(bins > D) < remaining <= count(bins >= D), found by the
-// whole CTA (thread t owns bins [4t, 4t+4)); found[0] = D, found[1] = remaining - count(bins > D).
+// whole CTA (thread t owns bins [4t, 4t+4)); found = D, remaining - count(bins > D), count(bin D).  Only the warp that
+// owns D looks further than its total: with all of them scanning, issue slots were what this step waited for.
 __device__ __forceinline__ void find_bin(const uint32_t* hist, uint32_t remaining, uint32_t* scan, uint32_t* found) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    uint32_t loc[4], tot = 0;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) { loc[j] = hist[tid * 4 + j]; tot += loc[j]; }
-    uint32_t incl = tot;                           // suffix sum over the lanes >= lane
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t t = __shfl_down_sync(0xffffffffu, incl, o);
-        if (lane + o < 32) incl += t;
-    }
-    if (lane == 0) scan[warp] = incl;
+    const uint4 q = reinterpret_cast<const uint4*>(hist)[tid];
+    const uint32_t tot = q.x + q.y + q.z + q.w, wtot = __reduce_add_sync(0xffffffffu, tot);
+    if (lane == 0) scan[warp] = wtot;
     __syncthreads();
-    uint32_t wsum = lane < CL_NT / 32 ? scan[lane] : 0u;          // suffix sum over the warps > warp
-#pragma unroll
-    for (int o = 1; o < CL_NT / 32; o <<= 1) {
-        const uint32_t t = __shfl_down_sync(0xffffffffu, wsum, o);
-        if (lane + o < CL_NT / 32) wsum += t;
-    }
-    const uint32_t above_warps = __shfl_sync(0xffffffffu, wsum, min(warp + 1, 31));
-    const uint32_t above = incl - tot + (warp + 1 < CL_NT / 32 ? above_warps : 0u);
-    if (above < remaining && remaining <= above + tot) {
-        uint32_t run = above;
-#pragma unroll
-        for (int j = 3; j >= 0; --j) {
-            if (run != 0xffffffffu) {
-                if (remaining <= run + loc[j]) {
-                    found[0] = (uint32_t)(tid * 4 + j);
-                    found[1] = remaining - run;
-                    run = 0xffffffffu;
-                } else {
-                    run += loc[j];
-                }
-            }
+    const uint32_t above_w = __reduce_add_sync(0xffffffffu, lane > warp && lane < CL_NT / 32 ? scan[lane] : 0u);
+    if (above_w < remaining && remaining <= above_w + wtot) {
+        uint32_t run = above_w + warp_suffix(tot) - tot;           // keys in the bins above this thread's
+        if (run < remaining && remaining <= run + tot) {
+            int d = 3;
+            uint32_t c = q.w;
+            if (remaining > run + c) { run += c; d = 2; c = q.z; }
+            if (d == 2 && remaining > run + c) { run += c; d = 1; c = q.y; }
+            if (d == 1 && remaining > run + c) { run += c; d = 0; c = q.x; }
+            found[0] = (uint32_t)(tid * 4 + d);
+            found[1] = remaining - run;
+            found[2] = c;
         }
     }
     __syncthreads();
+}
+
+// Four consecutive pooled values from the twelve staged scores f that begin with the first value's first tap; 2 H + 1 taps
+template <int H>
+__device__ __forceinline__ float4 pool4(const float (&f)[12], int mode, float kernel) {
+    float v[4];
+    if (mode == OBC_POOL_MAX) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[j] = -INFINITY;
+#pragma unroll
+            for (int t = 0; t <= 2 * H; ++t) v[j] = fmaxf(v[j], f[j + t]);     // padding taps are -inf
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {                                          // ascending index order; padding adds +0
+            v[j] = 0.f;
+#pragma unroll
+            for (int t = 0; t <= 2 * H; ++t) v[j] = __fadd_rn(v[j], f[j + t]);
+            v[j] = __fdiv_rn(v[j], kernel);
+        }
+    }
+    return make_float4(v[0], v[1], v[2], v[3]);
 }
 
 __global__ void __launch_bounds__(CL_NT)
@@ -444,21 +460,34 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     extern __shared__ __align__(16) uint8_t sel_smem[];
     ClusterShared& sh = *reinterpret_cast<ClusterShared*>(sel_smem);
     uint32_t* keys = reinterpret_cast<uint32_t*>(sel_smem + ((sizeof(ClusterShared) + 15) & ~(size_t)15));   // 16-byte aligned
-    float* stage = reinterpret_cast<float*>(keys + seg_cap);          // seg_cap + pool_kernel - 1 floats
+    float* stage = reinterpret_cast<float*>(keys + seg_cap);          // seg_cap + pool_kernel - 1 floats, and room to read four more
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    pdl_wait();
     cg::cluster_group cluster = cg::this_cluster();
     const int C = (int)cluster.num_blocks(), rank = (int)cluster.block_rank();
-    const int unit = blockIdx.x / C, b = unit / s.Hkv;
+    const int lC = __ffs(C) - 1;                   // C is a power of two, up to the number of warps
+    auto clear = [&](uint32_t* hist) { reinterpret_cast<uint4*>(hist)[tid] = make_uint4(0u, 0u, 0u, 0u); };
+    static_assert(CL_BINS == 4 * CL_NT, "four bins per thread");
+    auto reset = [&]() {
+        clear(sh.sum[0]);
+        clear(sh.local);
+        if (tid == 0) { sh.n_list = 0; sh.n_above = 0; sh.n_few = 0; sh.before[0] = 0; sh.before[1] = 0; }
+    };
+    if (!ad.hist) reset();
+    pdl_wait();
+    const int unit = blockIdx.x >> lC, b = unit / s.Hkv;
     const int N = seq_len(s, b);
     const int lo = s.n_sink, hi = N - s.n_recent, n = hi - lo;
-    // (the search across heads borrows the space of a histogram that is cleared below)
+    // (the search across heads borrows the space of a histogram that is cleared behind it)
     HeadShare share{budget_of(s, b) - s.n_sink - s.n_recent, false, 0u, 0u};
-    if (ad.hist) share = adaptive_share(s, ad, unit, *reinterpret_cast<AdaptiveFind*>(&sh.local[0]));
+    if (ad.hist) {
+        share = adaptive_share(s, ad, unit, *reinterpret_cast<AdaptiveFind*>(&sh.local[0]));
+        __syncthreads();
+        reset();
+    }
     const int n_hh = share.n_hh;
     const int budget = n_hh + s.n_sink + s.n_recent;
     int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gtid = rank * CL_NT + tid, gthreads = C * CL_NT;
 
     // these tests depend on the unit only, so all CTAs of the cluster leave together
@@ -474,17 +503,16 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     if (n_hh == 0) return;
 
     // ---- this CTA's share of the candidates: [c0, c1) of [0, n) --------------------------------
-    const int seg = ((n + C - 1) / C + 31) / 32 * 32;
+    const int seg = (((n + C - 1) >> lC) + 31) / 32 * 32;
     const int c0 = min(rank * seg, n), c1 = min(c0 + seg, n), m = c1 - c0;
-    if (tid == 0) sh.n_list = 0;
-    if (keys_in && !share.known) for (int i = tid; i < 4 * CL_BINS; i += CL_NT) (&sh.sum[0][0])[i] = 0;   // sum[3][] and local[]
-
     if (keys_in) {                                 // the caller has the (pooled) keys already: [units][Nmax]
         const uint32_t* kin = keys_in + (size_t)unit * s.Nmax + lo + c0;
 #pragma unroll 8
         for (int i = tid; i < m; i += CL_NT) keys[i] = kin[i];
         __syncthreads();
         cluster.barrier_arrive();
+        if (!share.known)
+            for (int i = tid; i < m; i += CL_NT) atomicAdd(&sh.local[keys[i] >> 21], 1u);
     } else {
         // pooled keys: stage the scores with their halo, then pool out of shared memory
         const float* sc = scores + (size_t)unit * s.Nmax;
@@ -499,52 +527,51 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
                 const int i = base + u * CL_NT + tid, p = lo + c0 + i - half;
                 val[u] = (i < m + 2 * half && p >= lo && p < hi) ? sc[p] : pad;
             }
-            if (base == 0)                             // the histograms are cleared while the loads travel
-                for (int i = tid; i < 4 * CL_BINS; i += CL_NT) (&sh.sum[0][0])[i] = 0;   // sum[3][] and local[]
     #pragma unroll
             for (int u = 0; u < LD; ++u) {
                 const int i = base + u * CL_NT + tid;
                 if (i < m + 2 * half) stage[i] = val[u];
             }
         }
-        if (m + 2 * half <= 0)                         // a CTA without candidates issued no loads above
-            for (int i = tid; i < 4 * CL_BINS; i += CL_NT) (&sh.sum[0][0])[i] = 0;
         __syncthreads();
         cluster.barrier_arrive();                      // this CTA's histograms are clear: others may add to them after their wait
-        for (int i = tid; i < m; i += CL_NT) {
-            float val;
-            if (half == 0) {
-                val = stage[i];
-            } else if (half <= 3) {                    // kernels up to 7: all taps read before they are combined
-                float tap[7];
-    #pragma unroll
-                for (int t = 0; t < 7; ++t) tap[t] = t <= 2 * half ? stage[i + t] : pad;
-                if (s.pool_mode == OBC_POOL_MAX) {
-                    val = -INFINITY;
-    #pragma unroll
-                    for (int t = 0; t < 7; ++t) val = fmaxf(val, tap[t]);      // padding taps are -inf
-                } else {                               // taps in ascending index order; padding adds +0
-                    val = 0.f;
-    #pragma unroll
-                    for (int t = 0; t < 7; ++t) if (t <= 2 * half) val = __fadd_rn(val, tap[t]);
-                    val = __fdiv_rn(val, (float)s.pool_kernel);
-                }
-            } else if (s.pool_mode == OBC_POOL_MAX) {
-                val = -INFINITY;
-                for (int t = 0; t <= 2 * half; ++t) val = fmaxf(val, stage[i + t]);
+        // four candidates per thread and step; the top 11 bits of their keys go straight into the first histogram
+        for (int i = tid * 4; i < m; i += CL_NT * 4) {
+            float4 v;
+            if (half <= 3) {                           // kernels up to 7: twelve staged scores in three reads
+                float f[12];
+                *reinterpret_cast<float4*>(&f[0]) = *reinterpret_cast<const float4*>(stage + i);
+                if (half > 0) *reinterpret_cast<float4*>(&f[4]) = *reinterpret_cast<const float4*>(stage + i + 4);
+                if (half > 2) *reinterpret_cast<float4*>(&f[8]) = *reinterpret_cast<const float4*>(stage + i + 8);
+                if (half == 0) v = make_float4(f[0], f[1], f[2], f[3]);
+                else if (half == 1) v = pool4<1>(f, s.pool_mode, (float)s.pool_kernel);
+                else if (half == 2) v = pool4<2>(f, s.pool_mode, (float)s.pool_kernel);
+                else v = pool4<3>(f, s.pool_mode, (float)s.pool_kernel);
             } else {
-                val = 0.f;
-                for (int t = 0; t <= 2 * half; ++t) val = __fadd_rn(val, stage[i + t]);
-                val = __fdiv_rn(val, (float)s.pool_kernel);
+                float* out = reinterpret_cast<float*>(&v);
+                for (int j = 0; j < 4; ++j) {
+                    const float* at = stage + min(i + j, m - 1);
+                    float val = s.pool_mode == OBC_POOL_MAX ? -INFINITY : 0.f;
+                    if (s.pool_mode == OBC_POOL_MAX) for (int t = 0; t <= 2 * half; ++t) val = fmaxf(val, at[t]);
+                    else for (int t = 0; t <= 2 * half; ++t) val = __fadd_rn(val, at[t]);
+                    out[j] = s.pool_mode == OBC_POOL_MAX ? val : __fdiv_rn(val, (float)s.pool_kernel);
+                }
             }
-            keys[i] = float_key(val);
+            const uint4 k4 = make_uint4(float_key(v.x), float_key(v.y), float_key(v.z), float_key(v.w));
+            *reinterpret_cast<uint4*>(keys + i) = k4;      // (a share has room for a multiple of 32 keys)
+            atomicAdd(&sh.local[k4.x >> 21], 1u);
+            if (i + 1 < m) atomicAdd(&sh.local[k4.y >> 21], 1u);
+            if (i + 2 < m) atomicAdd(&sh.local[k4.z >> 21], 1u);
+            if (i + 3 < m) atomicAdd(&sh.local[k4.w >> 21], 1u);
         }
     }
+    __syncthreads();                               // keys and this CTA's histogram of their top bits are complete
     // (the first cluster barrier is split: arrival above, once this CTA's histograms were clear; the wait comes just
     // before the first remote additions, behind the pooling and the first local histogram)
+    cluster.barrier_wait();
 
     // ---- radix search for the key T of the n_hh-th largest candidate ---------------------------
-    // Pass 0 histograms the top 11 bits of all keys of the CTA.  Every CTA adds its non-empty bins into the `sum`
+    // The top 11 bits come from the histogram of all keys.  Every CTA adds its non-empty bins into the `sum`
     // copy of every CTA of the cluster, so that after one cluster barrier each CTA finds by itself the bin D that
     // holds the n_hh-th largest key.  The keys of bin D (a few hundred of a 32k-token head) are copied to a list,
     // and every CTA hands its list, and how many of its candidates lie in the bins above D, to all the others:
@@ -553,143 +580,137 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     // that all but coincide) do passes 1 and 2 run across the cluster as pass 0 did.
     uint32_t* list = reinterpret_cast<uint32_t*>(stage);
     // (A threshold that the ranking across heads has settled needs no search.)
-    uint32_t prefix = share.T, mask = 0, remaining = share.known ? share.k_eq : (uint32_t)n_hh;
-    const int slot_cap = CL_GATHER / C;
-    bool gathered_path = false;
-    if (share.known) cluster.barrier_wait();
-    for (int ps = 0; ps < 3 && !gathered_path && !share.known; ++ps) {
-        const int shift = ps == 0 ? 21 : ps == 1 ? 10 : 0;
-        const uint32_t dmask = ps == 2 ? 1023u : 2047u;
-        const uint32_t* src = ps == 0 ? keys : list;
-        const int cnt = ps == 0 ? m : (int)sh.n_list;
-        for (int base = 0; base < cnt; base += CL_NT) {
-            const int i = base + tid;
-            const bool pred = i < cnt && (ps < 2 || (src[i] & mask) == prefix);   // the list holds pass 0's bin only
-            if (pred) atomicAdd(&sh.local[(src[i] >> shift) & dmask], 1u);
-        }
-        __syncthreads();
-        if (ps == 0) cluster.barrier_wait();       // every CTA of the cluster runs and has cleared its histograms
-        for (int bin = tid; bin < CL_BINS; bin += CL_NT) {
-            const uint32_t c = sh.local[bin];
-            if (c) for (int r = 0; r < C; ++r) atomicAdd(cluster.map_shared_rank(&sh.sum[ps][bin], r), c);
-        }
-        cluster.sync();                            // every copy of sum[ps] holds the whole head
-        find_bin(sh.sum[ps], remaining, sh.scan, sh.found);
+    uint32_t T = share.T, k_eq = share.k_eq;       // keep all keys > T and the first k_eq keys == T
+    bool before_known = C == 1;                    // sh.before[] holds what the CTAs before this one keep
+    if (!share.known) {
+        auto spread = [&](int pass) {              // this CTA's histogram into every copy of the head's
+            for (int bin = tid; bin < CL_BINS; bin += CL_NT) {
+                const uint32_t c = sh.local[bin];
+                if (c) for (int r = 0; r < C; ++r) atomicAdd(cluster.map_shared_rank(&sh.sum[pass][bin], r), c);
+            }
+            cluster.sync();
+        };
+        if (C > 1) spread(0);
+        find_bin(C > 1 ? sh.sum[0] : sh.local, (uint32_t)n_hh, sh.scan, sh.found);
         const uint32_t digit = sh.found[0];
-        remaining = sh.found[1];
-        prefix |= digit << shift; mask |= dmask << shift;
-        if (ps == 0) {
-            // survivors of the first pass -> list (any order); candidates of this CTA in the bins above D
-            uint32_t above = 0;
-            for (int bin = (int)digit + 1 + tid; bin < CL_BINS; bin += CL_NT) above += sh.local[bin];
-            for (int i = tid; i < m; i += CL_NT) {        // survivors are few: one shared-memory atomic each
-                const uint32_t key = keys[i];
-                if ((key & mask) == prefix) list[atomicAdd(&sh.n_list, 1u)] = key;
-            }
-            if (tid < 2) sh.before[tid] = 0;
+        T = digit << 21;
+        k_eq = sh.found[1];
+        // the keys of bin D -> list (any order); candidates of this CTA in the bins above D
+        uint32_t above = 0;
+        for (int i = tid * 4; i < m; i += CL_NT * 4) {
+            const uint4 q = *reinterpret_cast<const uint4*>(keys + i);
+            const uint32_t k4[4] = {q.x, q.y, q.z, q.w};
+            uint32_t c = 0;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) above += __shfl_xor_sync(0xffffffffu, above, o);
-            if (lane == 0) sh.scan[warp] = above;
-            __syncthreads();                       // the list and its length are complete
-            const int nl = (int)sh.n_list;
+            for (int j = 0; j < 4; ++j) { above += i + j < m && k4[j] >> 21 > digit; c += i + j < m && k4[j] >> 21 == digit; }
+            if (c) {                               // few threads: one shared-memory atomic each
+                uint32_t at = atomicAdd(&sh.n_list, c);
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (i + j < m && k4[j] >> 21 == digit) list[at++] = k4[j];
+            }
+        }
+        above = __reduce_add_sync(0xffffffffu, above);
+        if (lane == 0 && above) atomicAdd(&sh.n_above, above);
+        __syncthreads();                           // the list and its length are complete
+        clear(sh.local);
+        const int nl = (int)sh.n_list, slot_cap = C > 1 ? CL_GATHER >> lC : m;
+        const int slot = warp & (C - 1), first = (warp >> lC) * 32 + lane, step = (CL_NT / 32 >> lC) * 32;   // warp w serves CTA w mod C
+        if (C > 1) {
             if (tid < C) {                         // length and higher-bin count into every CTA
-                uint32_t ab = 0;
-                for (int w = 0; w < CL_NT / 32; ++w) ab += sh.scan[w];
                 cluster.map_shared_rank(&sh.rank_list[0], tid)[rank] = (uint32_t)nl;
-                cluster.map_shared_rank(&sh.rank_above[0], tid)[rank] = ab;
+                cluster.map_shared_rank(&sh.rank_above[0], tid)[rank] = sh.n_above;
             }
-            if (nl <= slot_cap)                    // the keys themselves, into slot `rank` of every CTA (warp w serves CTA w mod C)
-                for (int r = warp % C; r < C; r += CL_NT / 32) {
-                    uint32_t* dst = cluster.map_shared_rank(sh.gathered(), r) + rank * slot_cap;
-                    const int step = (CL_NT / 32 >= C ? CL_NT / 32 / C : 1) * 32;
-                    for (int i = (CL_NT / 32 >= C ? warp / C : 0) * 32 + lane; i < nl; i += step) dst[i] = list[i];
-                }
-            for (int bin = tid; bin < CL_BINS; bin += CL_NT) sh.local[bin] = 0;
+            if (nl <= slot_cap) {                  // the keys themselves, into slot `rank` of every CTA
+                uint32_t* dst = cluster.map_shared_rank(sh.gathered(), slot) + rank * slot_cap;
+                for (int i = first; i < nl; i += step) dst[i] = list[i];
+            }
             cluster.sync();                        // lists and counts have arrived everywhere
-            bool fits = true;
-            for (int r = 0; r < C; ++r) fits = fits && (int)sh.rank_list[r] <= slot_cap;   // the same answer in every CTA
-            if (fits) {
-                // ---- the remaining 21 bits, on this CTA's copy of all lists (no cluster traffic) ----
-                for (int half_pass = 0; half_pass < 2; ++half_pass) {
-                    const int sh2 = half_pass == 0 ? 10 : 0;
-                    const uint32_t dm2 = half_pass == 0 ? 2047u : 1023u;
-                    for (int r = warp % C; r < C; r += CL_NT / 32) {          // warp w reads slot w mod C
-                        const int nr = (int)sh.rank_list[r];
-                        const uint32_t* g = sh.gathered() + r * slot_cap;
-                        const int step = (CL_NT / 32 >= C ? CL_NT / 32 / C : 1) * 32;
-                        for (int i = (CL_NT / 32 >= C ? warp / C : 0) * 32 + lane; i < nr; i += step)
-                            if ((g[i] & mask) == prefix) atomicAdd(&sh.local[(g[i] >> sh2) & dm2], 1u);
-                    }
-                    __syncthreads();
-                    find_bin(sh.local, remaining, sh.scan, sh.found);
-                    prefix |= sh.found[0] << sh2; mask |= dm2 << sh2; remaining = sh.found[1];
-                    if (half_pass == 0) {
-                        for (int bin = tid; bin < CL_BINS; bin += CL_NT) sh.local[bin] = 0;
-                        __syncthreads();
-                    }
+        } else {
+            __syncthreads();
+        }
+        const uint32_t my_len = C > 1 ? (lane < C ? sh.rank_list[lane] : 0u) : (uint32_t)nl;
+        if ((int)__reduce_max_sync(0xffffffffu, my_len) <= slot_cap) {         // (the same answer in every CTA)
+            // ---- the remaining 21 bits, on this CTA's copy of all lists (no cluster traffic) ----
+            const uint32_t* g = C > 1 ? sh.gathered() + slot * slot_cap : list;
+            const int ng = C > 1 ? (int)sh.rank_list[slot] : nl;
+            for (int i = first; i < ng; i += step) atomicAdd(&sh.local[(g[i] >> 10) & 2047u], 1u);
+            __syncthreads();
+            find_bin(sh.local, k_eq, sh.scan, sh.found);
+            T |= sh.found[0] << 10;
+            k_eq = sh.found[1];
+            const int same = (int)sh.found[2];
+            if (same <= 32) {                      // all but always: every warp ranks the keys that are left
+                for (int i = first; i < ng; i += step)
+                    if (g[i] >> 10 == T >> 10) sh.few[atomicAdd(&sh.n_few, 1u)] = g[i];
+                __syncthreads();
+                const uint32_t key = lane < same ? sh.few[lane] : 0u;
+                uint32_t gt = 0, ge = 0;
+                for (int j = 0; j < same; ++j) {
+                    const uint32_t other = __shfl_sync(0xffffffffu, key, j);
+                    gt += other > key;
+                    ge += other >= key;
                 }
-                // what the CTAs before this one keep: their candidates above bin D, and of their lists the keys > T, == T
-                uint32_t bg = 0, be = 0;
-                if (tid < rank) bg = sh.rank_above[tid];
-                for (int r = warp % C; r < rank; r += CL_NT / 32) {
-                    const int nr = (int)sh.rank_list[r];
-                    const uint32_t* g = sh.gathered() + r * slot_cap;
-                    const int step = (CL_NT / 32 >= C ? CL_NT / 32 / C : 1) * 32;
-                    for (int i = (CL_NT / 32 >= C ? warp / C : 0) * 32 + lane; i < nr; i += step) { bg += g[i] > prefix; be += g[i] == prefix; }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    bg += __shfl_xor_sync(0xffffffffu, bg, o);
-                    be += __shfl_xor_sync(0xffffffffu, be, o);
-                }
-                if (lane == 0 && (bg | be)) { atomicAdd(&sh.before[0], bg); atomicAdd(&sh.before[1], be); }
-                gathered_path = true;              // leaves the pass loop; the barrier below publishes `before`
+                const int at = __ffs(__ballot_sync(0xffffffffu, lane < same && gt < k_eq && k_eq <= ge)) - 1;
+                T = __shfl_sync(0xffffffffu, key, at);
+                k_eq -= __shfl_sync(0xffffffffu, gt, at);
             } else {
-                // the exchanged passes 1 and 2 add into the histograms that the lists have overwritten: clear them
-                // everywhere before any CTA adds to another's copy
-                for (int i = tid; i < 2 * CL_BINS; i += CL_NT) sh.gathered()[i] = 0;
-                cluster.sync();
+                clear(sh.local);
+                __syncthreads();
+                for (int i = first; i < ng; i += step)
+                    if (g[i] >> 10 == T >> 10) atomicAdd(&sh.local[g[i] & 1023u], 1u);
+                __syncthreads();
+                find_bin(sh.local, k_eq, sh.scan, sh.found);
+                T |= sh.found[0];
+                k_eq = sh.found[1];
+            }
+            if (C > 1) {
+                // what the CTAs before this one keep: their candidates above bin D, and of their lists the keys > T, == T
+                uint32_t bg = tid < rank ? sh.rank_above[tid] : 0u, be = 0;
+                if (slot < rank)
+                    for (int i = first; i < ng; i += step) { bg += g[i] > T; be += g[i] == T; }
+                bg = __reduce_add_sync(0xffffffffu, bg);
+                be = __reduce_add_sync(0xffffffffu, be);
+                if (lane == 0 && (bg | be)) { atomicAdd(&sh.before[0], bg); atomicAdd(&sh.before[1], be); }
+                before_known = true;               // published by the barrier behind the counts below
             }
         } else {
-            for (int bin = tid; bin < CL_BINS; bin += CL_NT) sh.local[bin] = 0;
+            // the exchanged passes 1 and 2 add into the histograms that the lists have overwritten: clear them
+            // everywhere before any CTA adds to another's copy
+            clear(sh.sum[1]);
+            clear(sh.sum[2]);
+            cluster.sync();
+            for (int pass = 1; pass < 3; ++pass) {
+                const int known = pass == 1 ? 21 : 10, shift = pass == 1 ? 10 : 0;
+                for (int i = tid; i < nl; i += CL_NT)
+                    if (list[i] >> known == T >> known) atomicAdd(&sh.local[(list[i] >> shift) & (pass == 1 ? 2047u : 1023u)], 1u);
+                __syncthreads();
+                spread(pass);
+                clear(sh.local);
+                find_bin(sh.sum[pass], k_eq, sh.scan, sh.found);
+                T |= sh.found[0] << shift;
+                k_eq = sh.found[1];
+            }
         }
-        __syncthreads();
     }
-    const uint32_t T = prefix, k_eq = remaining;   // keep all keys > T and the first k_eq keys == T
 
-    // ---- ordered emission: each warp owns a contiguous run of this CTA's candidates, in blocks of 256 keys of
-    // which a lane holds eight consecutive ones (two 16-byte reads) ------------------------------------------------
-    const int wseg = ((m + CL_NT / 32 - 1) / (CL_NT / 32) + 255) / 256 * 256;
+    // ---- ordered emission: each warp owns a contiguous run of this CTA's candidates ------------------------------
+    const int wseg = ((m + CL_NT / 32 - 1) / (CL_NT / 32) + 31) / 32 * 32;
     const int s0 = min(warp * wseg, m), s1 = min(s0 + wseg, m);
-    auto load8 = [&](int i, uint32_t (&k8)[8]) -> unsigned {           // returns the mask of keys that exist
-        if (i + 8 <= s1) {
-            const uint4 a = *reinterpret_cast<const uint4*>(keys + i), b = *reinterpret_cast<const uint4*>(keys + i + 4);
-            k8[0] = a.x; k8[1] = a.y; k8[2] = a.z; k8[3] = a.w; k8[4] = b.x; k8[5] = b.y; k8[6] = b.z; k8[7] = b.w;
-            return 0xffu;
-        }
-        unsigned have = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { const bool in = i + j < s1; k8[j] = in ? keys[i + j] : 0u; have |= (unsigned)in << j; }
-        return have;
-    };
     uint32_t cgt = 0, ceq = 0;
-    for (int base = s0; base < s1; base += 256) {
-        uint32_t k8[8];
-        const unsigned have = load8(base + lane * 8, k8);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { cgt += ((have >> j) & 1u) && k8[j] > T; ceq += ((have >> j) & 1u) && k8[j] == T; }
+#pragma unroll 4
+    for (int i = s0 + lane; i < s1; i += 32) {
+        const uint32_t key = keys[i];
+        cgt += key > T; ceq += key == T;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cgt += __shfl_xor_sync(0xffffffffu, cgt, o);
-        ceq += __shfl_xor_sync(0xffffffffu, ceq, o);
-    }
+    cgt = __reduce_add_sync(0xffffffffu, cgt);
+    ceq = __reduce_add_sync(0xffffffffu, ceq);
     if (lane == 0) { sh.warp_gt[warp] = cgt; sh.warp_eq[warp] = ceq; }
     __syncthreads();
-    if (!gathered_path) {                          // the CTAs' totals were not derived from the lists: exchange them
+    const uint32_t wg = lane < CL_NT / 32 ? sh.warp_gt[lane] : 0u, we = lane < CL_NT / 32 ? sh.warp_eq[lane] : 0u;
+    if (!before_known) {                           // the CTAs' totals were not derived from the lists: exchange them
+        const uint32_t tg = __reduce_add_sync(0xffffffffu, wg), te = __reduce_add_sync(0xffffffffu, we);
         if (tid < C) {                             // this CTA's totals into every CTA of the cluster
-            uint32_t tg = 0, te = 0;
-            for (int w = 0; w < CL_NT / 32; ++w) { tg += sh.warp_gt[w]; te += sh.warp_eq[w]; }
             cluster.map_shared_rank(&sh.rank_gt[0], tid)[rank] = tg;
             cluster.map_shared_rank(&sh.rank_eq[0], tid)[rank] = te;
         }
@@ -701,31 +722,20 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
         }
         __syncthreads();
     }
-    uint32_t gt_run = sh.before[0], eq_run = sh.before[1];             // kept candidates before the block at hand
-    for (int w = 0; w < warp; ++w) { gt_run += sh.warp_gt[w]; eq_run += sh.warp_eq[w]; }
-    for (int base = s0; base < s1; base += 256) {
-        uint32_t k8[8];
-        const int i = base + lane * 8;
-        const unsigned have = load8(i, k8);
-        uint32_t g = 0, e = 0;
-#pragma unroll
-        for (int j = 0; j < 8; ++j) { g += ((have >> j) & 1u) && k8[j] > T; e += ((have >> j) & 1u) && k8[j] == T; }
-        uint32_t gi = g, ei = e;                   // inclusive scans over the lanes
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t tg = __shfl_up_sync(0xffffffffu, gi, o), te = __shfl_up_sync(0xffffffffu, ei, o);
-            if (lane >= o) { gi += tg; ei += te; }
-        }
-        uint32_t eq_at = eq_run + ei - e;          // equal keys before this lane's first key: the first k_eq of them are kept
-        uint32_t out = s.n_sink + gt_run + (gi - g) + min(eq_at, k_eq);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            if (!((have >> j) & 1u)) continue;
-            if (k8[j] > T) idx[out++] = lo + c0 + i + j;
-            else if (k8[j] == T) { if (eq_at < k_eq) idx[out++] = lo + c0 + i + j; ++eq_at; }
-        }
-        gt_run += __shfl_sync(0xffffffffu, gi, 31);
-        eq_run += __shfl_sync(0xffffffffu, ei, 31);
+    uint32_t gt_run = sh.before[0] + __reduce_add_sync(0xffffffffu, lane < warp ? wg : 0u);   // kept candidates before the block at hand
+    uint32_t eq_run = sh.before[1] + __reduce_add_sync(0xffffffffu, lane < warp ? we : 0u);
+    const unsigned lt_mask = (1u << lane) - 1u;
+    int32_t* out = idx + s.n_sink;
+#pragma unroll 4
+    for (int base = s0; base < s1; base += 32) {
+        const int i = base + lane;
+        const uint32_t key = i < s1 ? keys[i] : 0u;
+        const bool is_gt = i < s1 && key > T, is_eq = i < s1 && key == T;
+        const unsigned mg = __ballot_sync(0xffffffffu, is_gt), me = __ballot_sync(0xffffffffu, is_eq);
+        const uint32_t eq_at = eq_run + __popc(me & lt_mask);       // equal keys before this one: the first k_eq of them are kept
+        if (is_gt || (is_eq && eq_at < k_eq)) out[gt_run + __popc(mg & lt_mask) + min(eq_at, k_eq)] = lo + c0 + i;
+        gt_run += __popc(mg);
+        eq_run += __popc(me);
     }
 }
 
@@ -818,20 +828,20 @@ obc_status launch_shard_indices(int units, int idx_stride, int t0, int n, const 
 
 size_t select_workspace_bytes(int B, int Hkv, int Nmax) { return align_up((size_t)B * Hkv * Nmax * 4, 256); }
 
-// Cluster size for the one-cluster-per-head path, or 0 when a head does not fit a cluster's shared memory.  A CTA's phases
-// cost the same for 32 as for 2048 keys, so short heads take one CTA; few longer heads take eight CTAs (8 heads of 8192
-// tokens: 13.8 / 11.6 / 10.5 / 10.2 us for 1 / 2 / 4 / 8; of 2048: 9.8 / 10.2 / 9.9 / 9.9); many heads take what still runs
-// side by side, two CTAs per SM (64 heads of 2048: 9.8 / 10.2 / 11.7 / 21.5 us, of 8192: 14.0 / 12.0 / 13.3 / 23.1, of 32768:
-// - / 22.1 / 20.8 / 30.5; 256 heads of 4096: 14.1 / 24.7 / 42.9 / 83.1), but no share above 8192 candidates, of which an SM
-// holds only one CTA (64 ragged heads of up to 65536: 37 us with four CTAs, 33 with eight; 256 of 32768: 84 with two, 76 with four).
+// Cluster size for the one-cluster-per-head path, or 0 when a head does not fit a cluster's shared memory.  A CTA takes
+// 4.3 us and 0.57 us per 1024 candidates, a cluster 1.2 to 1.8 us more, so heads of up to 4096 tokens take one CTA (8 heads:
+// 6.2 / 6.7 / 6.5 / 6.4 us for 1 / 2 / 4 / 8 CTAs) and longer ones as many as run side by side, one CTA per SM (8 heads of
+// 8192: 8.7 / 7.8 / 6.9 / 6.7; 16 heads: 8.9 / 7.9 / 6.9 / 7.9; 64 heads: 9.0 / 8.1 / 8.8 / 15.6; 128 heads: 9.2 / 10.4 / 16.4 /
+// 29.8; 32 heads of 32768: - / 15.5 / 11.0 / 11.6), sixteen only above 2048 candidates per CTA (4 heads of 16384: 7.1 with
+// eight, 7.2 with sixteen; of 32768: 8.6 / 8.0).  Above 8192 candidates an SM holds one CTA only: such shares are split
+// further whatever runs side by side (256 heads of 32768: 60 us with two CTAs, 56 with four; 16 heads of 65536: 16.1 with
+// four, 14.9 with eight; of 131072: 36 with eight, 32 with sixteen; 128 heads of 131072: 163 / 172).
 static int select_cluster_size(int units, int Nmax, int* seg_cap) {
     auto seg_of = [&](int C) { return ((Nmax + C - 1) / C + 31) / 32 * 32; };
+    auto side_by_side = [](int C) { return C == 2 ? 74 : C == 4 ? 33 : C == 8 ? 15 : 7; };     // clusters, one CTA per SM
     int C = 1;
-    if (units * 8LL <= 148) {
-        if (Nmax > 2048) C = seg_of(8) > 8192 ? 16 : 8;
-    } else {
-        while (C < 8 && Nmax > 4096 * C && (units * 2LL * C <= 2 * 148 || seg_of(C) > 8192)) C *= 2;
-    }
+    if (Nmax > 4096)
+        while (C < 16 && (units <= side_by_side(2 * C) ? C < 8 || seg_of(C) > 2048 : seg_of(C) > 8192 && (C < 8 || units <= 32))) C *= 2;
     while (C < 16 && seg_of(C) > CL_MAX_SEG) C *= 2;
     if (seg_of(C) > CL_MAX_SEG) return 0;
     *seg_cap = seg_of(C);
@@ -851,7 +861,7 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
     int seg_cap = 0;
     const int C = select_cluster_size(units, s.Nmax, &seg_cap);
     if (C > 0) {
-        const size_t smem = sizeof(ClusterShared) + (size_t)seg_cap * 8 + (size_t)s.pool_kernel * 4 + 16;
+        const size_t smem = sizeof(ClusterShared) + (size_t)seg_cap * 8 + (size_t)s.pool_kernel * 4 + 32;
         OBC_CUDA_TRY(allow_smem(select_cluster_kernel, smem));
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(units * C)); cfg.blockDim = dim3(CL_NT); cfg.dynamicSmemBytes = smem; cfg.stream = stream;

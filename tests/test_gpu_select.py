@@ -75,6 +75,31 @@ def test_select_when_the_first_radix_pass_leaves_too_many_survivors(N, budget):
         assert np.array_equal(got.cpu().numpy(), want), (pool, kern)
 
 
+@pytest.mark.parametrize("Hkv,N", [(2, 1003), (2, 4097), (20, 4099), (60, 4101), (2, 16400)])
+@pytest.mark.parametrize("same", [1, 32, 33, 300])
+def test_select_when_few_or_many_keys_share_all_but_the_last_bits(Hkv, N, same):
+    """The threshold lies among `same` keys that differ in their last ten bits alone: up to 32 of them are ranked, more go
+    through a histogram.  Heads on 1, 8, 4, 2 and 16 CTAs; the last candidates do not fill a group of four."""
+    rng = np.random.default_rng(N + same)
+    above = N // 5
+    scores = rng.random((1, Hkv, N), dtype=np.float32) * 0.5
+    for h in range(Hkv):
+        at = rng.permutation(N)
+        scores[0, h, at[:above]] = 2.0 + rng.random(above)
+        scores[0, h, at[above:above + same]] = 1.0 + rng.integers(0, 1 + min(same, 1023) * 3 // 4, same) * 2.0 ** -23    # with ties
+    got, want = _select_both(scores, [N], [above + (same + 1) // 2], 0, 0, "none", 1)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("pool,kern", [("max", 3), ("max", 5), ("avg", 3), ("avg", 7), ("avg", 9), ("max", 9)])
+@pytest.mark.parametrize("N", [37, 1022, 4105])
+def test_select_every_pool_width_at_ragged_ends(pool, kern, N):
+    rng = np.random.default_rng(N + kern)
+    scores = rng.random((1, 2, N), dtype=np.float32)
+    got, want = _select_both(scores, [N], [N // 3 + 3], 1, 2, pool, kern)
+    assert np.array_equal(got.cpu().numpy(), want)
+
+
 def test_select_ragged_lengths_and_per_sequence_budgets():
     rng = np.random.default_rng(1)
     lens = np.array([4096, 517, 2300], np.int32)
