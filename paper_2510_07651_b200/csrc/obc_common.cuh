@@ -145,9 +145,15 @@ bool make_map(CUtensorMap* map, const void* base, int rank, const uint64_t* dims
 // become resident while the preceding kernel of the stream is still draining.  A kernel executes
 // pdl_wait() before its first access to memory that an earlier kernel may have written (or may
 // still read, for its own writes); what precedes the wait is set-up that touches no such memory.
-// (Releasing the next kernel earlier, with griddepcontrol.launch_dependents after the wait, was measured
-// and is not done: CTAs of the next kernel that sit waiting on an SM slowed the kernel at work.)
+// pdl_release() lets the next kernel's CTAs start before this one's are done.  It stands right behind the wait of the small
+// kernels between the two passes on tensor cores (8 heads of 1024 tokens: 15.0 -> 14.0 us per call, because pass 2 sets up
+// and fetches its first tiles meanwhile), and not in kernels that do the bulk of the work, which the waiting CTAs slowed
+// (with a release in every kernel the 131072-token Qwen layer took 358 instead of 346 us; at the tail of pass 1: 349), nor
+// where the successor has little to do before its wait (fp32 head of 1024 tokens: 20.2 -> 20.4 us; decode: no change).
+// A kernel that starts early may touch before its wait whatever the kernels BEFORE its predecessor wrote or read: the
+// predecessor released it behind its own wait, so those are complete.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,

@@ -226,6 +226,7 @@ __device__ __forceinline__ float block128_reduce(float x, bool take_max, float* 
 __global__ void __launch_bounds__(CMB_NT)
 simt_combine_kernel(ScoreShape s, SimtPlan plan, float* ws) {
     pdl_wait();
+    if (plan.want_obf) pdl_release();            // pass 2 on tensor cores follows
     const int r = blockIdx.x % plan.rows_out, unit = blockIdx.x / plan.rows_out;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const size_t orow = (size_t)unit * plan.rows_out + r;
@@ -308,6 +309,7 @@ template <int BATCH, bool FEW>
 __global__ void __launch_bounds__(CMB_NT, BATCH <= 2 ? 12 : 1)
 simt_combine_rows_kernel(ScoreShape s, SimtPlan plan, float* ws) {
     pdl_wait();
+    if (plan.want_obf) pdl_release();            // pass 2 on tensor cores follows
     const int lane = threadIdx.x & 31;
     const long long rows_total = (long long)s.B * s.Hkv * plan.rows_out;
     const long long orow = (long long)blockIdx.x * (CMB_NT / 32) + (threadIdx.x >> 5);
@@ -387,6 +389,7 @@ template <typename T>
 __global__ void __launch_bounds__(CMB_NT)
 given_prep_kernel(ScoreShape s, SimtPlan plan, TensorView o, const float* lse, float* ws) {
     pdl_wait();
+    if (plan.want_obf) pdl_release();            // pass 2 on tensor cores follows
     if (blockIdx.x == 0 && threadIdx.x == 0)     // no wait of this call can have given up yet
         *reinterpret_cast<unsigned int*>(reinterpret_cast<char*>(ws) + plan.off_flag) = 0u;
     const int r = blockIdx.x % plan.rows_out, unit = blockIdx.x / plan.rows_out;
