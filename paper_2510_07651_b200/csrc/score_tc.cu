@@ -1107,7 +1107,7 @@ struct P1Params {
     float scale;
     int causal;
     int n_chunks, chunk_rows;
-    int head_chunks;                                       // whole row chunks that a head's W rows fill, under a causal window; else 0
+    int head_chunks;                                       // whole row chunks (pairs of them) that a head's W rows fill, under a causal window; else 0
     int n_splits, tiles_per_split;                         // CTAs per (unit, chunk); each writes one partial
     int l2_stream;                                         // K/V copies carry the "evict first" L2 hint
     float* part_m; float* part_l; float* part_o;           // [units][n_splits][R] (x d for part_o)
@@ -1176,13 +1176,14 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return r;
 }
 
-// Row chunk of a block.  Under a causal window a chunk of rows visits the tiles up to its last row's position, and all
+// Row chunk of a block (PAIR: pair of consecutive row chunks, in place of a chunk below).  Under a causal window a chunk of rows visits the tiles up to its last row's position, and all
 // of them if it holds the end of a head and the start of the next.  With more CTAs than SMs the chunks that visit most
 // tiles are handed out first: where a head has several chunks, blocks are ordered by the chunk's place counted back from
 // the chunk of its head's last row.  (Heads need not end where chunks do: by chunk number alone pass 1 took 63 instead
 // of 46 us for 2 KV heads x 4 heads x 3500 queries, 136 instead of 126 us for 8 x 4 x 3001.)  Otherwise by chunk, last first.
+template <bool PAIR>
 __device__ __forceinline__ void p1_chunk_of_block(const P1Params& p, int vu, int& unit, int& c) {
-    const int rows = p.chunk_rows, n = p.n_chunks;
+    const int rows = PAIR ? 2 * p.chunk_rows : p.chunk_rows, n = PAIR ? (p.n_chunks + 1) / 2 : p.n_chunks;
     const int base = p.head_chunks;                         // a head has this many chunks or one more; 0: by chunk number
     if (base) {
         auto end = [&](int h) { return ((h + 1) * p.W - 1) / rows; };       // the chunk of head h's last row
@@ -1208,8 +1209,11 @@ __device__ __forceinline__ void p1_chunk_of_block(const P1Params& p, int vu, int
     c = n - 1 - vu % n;
 }
 
-// HILO: fewer than 64 window rows; MMA rows 64.. repeat rows 0.. and carry the low part of P
-template <bool HILO>
+// HILO: fewer than 64 window rows; MMA rows 64.. repeat rows 0.. and carry the low part of P.
+// PAIR: the CTA takes two row chunks, one per softmax warpgroup, and each warpgroup sees every tile: a tile is fetched for
+// both, there are half as many CTAs to set up and to drain, and nothing to merge between the warpgroups.  Warpgroup 0 has the
+// chunk that visits more tiles.  Two K/V stages make room for the second Q chunk; a tile lasts twice as long.
+template <bool HILO, bool PAIR>
 __global__ void __launch_bounds__(kThreadsP1, 1)
 tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
                 const __grid_constant__ CUtensorMap map_v, const __grid_constant__ P1Params p) {
@@ -1223,14 +1227,17 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     span_begin(p.span);
 
     const int split = blockIdx.x;
+    constexpr int NST = PAIR ? 2 : P1_NSTAGE;
+    constexpr uint32_t OFF_K1 = PAIR ? P1_OFF_Q + 2 * kOperandBytes : P1_OFF_K, OFF_V1 = OFF_K1 + NST * kOperandBytes;
+    static_assert(OFF_V1 + NST * kOperandBytes <= P1_OFF_BAR && !(HILO && PAIR), "layout");
     int unit, c;
-    p1_chunk_of_block(p, blockIdx.y, unit, c);
+    p1_chunk_of_block<PAIR>(p, blockIdx.y, unit, c);
     const int b = unit / p.Hkv, g = unit % p.Hkv;
-    const bool nv_job = p.nv != nullptr && c == p.n_chunks - 1;     // this CTA also writes ||v_p||^2 of the tiles it visits
+    const bool nv_job = !PAIR && p.nv != nullptr && c == p.n_chunks - 1;     // this CTA also writes ||v_p||^2 of the tiles it visits
     if (threadIdx.x == 0) {
         prefetch_tmap(&map_q); prefetch_tmap(&map_k); prefetch_tmap(&map_v);
         // a K/V stage is released by the MMA commit and, where they are at work, by the two ||v||^2 warps
-        for (int i = 0; i < P1_NSTAGE; ++i) { mbar_init(bar(P1_FULL + i), 1); mbar_init(bar(P1_EMPTY + i), nv_job ? 3 : 1); }
+        for (int i = 0; i < NST; ++i) { mbar_init(bar(P1_FULL + i), 1); mbar_init(bar(P1_EMPTY + i), nv_job ? 3 : 1); }
         mbar_init(bar(P1_QFULL), 1); mbar_init(bar(P1_ODONE), 1);
         for (int i = 0; i < 2; ++i) { mbar_init(bar(P1_SFULL + i), 1); mbar_init(bar(P1_PFULL + i), 4); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1255,30 +1262,45 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const int tile_lo = split * p.tiles_per_split;
     // tiles past the last token that any row of this chunk sees are not visited
     const int Nm = p.mask_lens ? p.mask_lens[b] : N;       // a shard of a longer sequence: its distance to that sequence's end
-    const int chunk_last = rows_last_token(c * p.chunk_rows, min((c + 1) * p.chunk_rows, p.R) - 1, p.W, Nm, p.causal);
-    const int tile_hi = min(min(tile_lo + p.tiles_per_split, (N + TILE - 1) / TILE), chunk_last / TILE + 1);
-    const int n_tiles = max(tile_hi - tile_lo, 0);
+    auto tiles_of_chunk = [&](int ch) -> int {
+        if (ch >= p.n_chunks) return 0;
+        const int chunk_last = rows_last_token(ch * p.chunk_rows, min((ch + 1) * p.chunk_rows, p.R) - 1, p.W, Nm, p.causal);
+        return max(min(min(tile_lo + p.tiles_per_split, (N + TILE - 1) / TILE), chunk_last / TILE + 1) - tile_lo, 0);
+    };
+    int c0 = c, c1 = c, n_tiles, n1 = 0;                   // chunks of the two warpgroups; tiles of the first (PAIR: and of the second)
+    if (PAIR) {
+        c0 = 2 * c + 1; c1 = 2 * c;
+        n_tiles = tiles_of_chunk(c0); n1 = tiles_of_chunk(c1);
+        if (n1 > n_tiles) { c0 = 2 * c; c1 = 2 * c + 1; const int t = n1; n1 = n_tiles; n_tiles = t; }
+    } else {
+        n_tiles = tiles_of_chunk(c);
+    }
 
     if (idle_split) {
         // nothing to compute and nothing to store
     } else if (warp == 0) {
         // ===================================== TMA producer =====================================
         if (lane == 0 && n_tiles > 0) {
-            mbar_expect_tx(bar(P1_QFULL), (uint32_t)p.chunk_rows * (HILO ? 512u : 256u));
-            const int qrow = (b * p.Hq + g * p.G) * p.W + c * p.chunk_rows;
+            mbar_expect_tx(bar(P1_QFULL), (uint32_t)p.chunk_rows * (HILO || (PAIR && n1 > 0) ? 512u : 256u));
+            const int qrow = (b * p.Hq + g * p.G) * p.W + c0 * p.chunk_rows;
             tma_load_2d(sbase + P1_OFF_Q, &map_q, bar(P1_QFULL), 0, qrow);
             tma_load_2d(sbase + P1_OFF_Q + kHalfBytes, &map_q, bar(P1_QFULL), 64, qrow);
             if (HILO) {
                 tma_load_2d(sbase + P1_OFF_Q + kHalfBytes / 2, &map_q, bar(P1_QFULL), 0, qrow);
                 tma_load_2d(sbase + P1_OFF_Q + kHalfBytes + kHalfBytes / 2, &map_q, bar(P1_QFULL), 64, qrow);
             }
+            if (PAIR && n1 > 0) {
+                const int qrow1 = (b * p.Hq + g * p.G) * p.W + c1 * p.chunk_rows;
+                tma_load_2d(sbase + P1_OFF_Q + kOperandBytes, &map_q, bar(P1_QFULL), 0, qrow1);
+                tma_load_2d(sbase + P1_OFF_Q + kOperandBytes + kHalfBytes, &map_q, bar(P1_QFULL), 64, qrow1);
+            }
             int issued = 0;
             const uint64_t pol_stream = l2_policy_evict_first();
             for (int i = 0; i < n_tiles; ++i) {
-                const uint32_t st = i % P1_NSTAGE;
-                if (!mbar_wait(bar(P1_EMPTY + st), ((i / P1_NSTAGE) & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
+                const uint32_t st = i % NST;
+                if (!mbar_wait(bar(P1_EMPTY + st), ((i / NST) & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
                 mbar_expect_tx(bar(P1_FULL + st), 2 * kOperandBytes);
-                const uint32_t dk = sbase + P1_OFF_K + st * kOperandBytes, dv = sbase + P1_OFF_V + st * kOperandBytes;
+                const uint32_t dk = sbase + OFF_K1 + st * kOperandBytes, dv = sbase + OFF_V1 + st * kOperandBytes;
                 const int t0 = (tile_lo + i) * TILE;
                 if (p.l2_stream) {                             // the cache cannot hold K and V until pass 2 anyway
                     tma_load_4d_hint(dk, &map_k, bar(P1_FULL + st), 0, t0, g, b, pol_stream);
@@ -1293,9 +1315,9 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 }
                 ++issued;
             }
-            for (int back = 0; back < P1_NSTAGE && back < issued; ++back) {   // drain own copies
+            for (int back = 0; back < NST && back < issued; ++back) {         // drain own copies
                 const int it = issued - 1 - back;
-                (void)mbar_wait(bar(P1_FULL + it % P1_NSTAGE), (it / P1_NSTAGE) & 1);
+                (void)mbar_wait(bar(P1_FULL + it % NST), (it / NST) & 1);
             }
             (void)mbar_wait(bar(P1_QFULL), 0);
         }
@@ -1304,11 +1326,15 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         if (lane == 0 && n_tiles > 0) {
             const uint32_t idesc_s = idesc_bf16(TILE);
             const uint32_t idesc_pv = idesc_bf16(kD) | (1u << 16);           // B operand (V) is MN-major
+            // Item i: tile i, warpgroup i mod 2; in pairs tile i / 2 (items of warpgroup 1 past its tiles are left out).
+            auto tile_at = [&](int i) { return PAIR ? i >> 1 : i; };
+            auto is_item = [&](int i) { return PAIR ? (i >> 1) < ((i & 1) ? n1 : n_tiles) : i < n_tiles; };
             auto issue_s = [&](int j) -> bool {                              // S_w = Q . K_j^T
-                const uint32_t st = j % P1_NSTAGE;
-                if (!mbar_wait(bar(P1_FULL + st), (j / P1_NSTAGE) & 1)) return false;
+                const uint32_t tl = tile_at(j), st = tl % NST;
+                if (!mbar_wait(bar(P1_FULL + st), (tl / NST) & 1)) return false;
                 tc_fence_after();
-                const uint32_t ak = desc_lo_k(sbase + P1_OFF_K + st * kOperandBytes), aq = desc_lo_k(sbase + P1_OFF_Q);
+                const uint32_t ak = desc_lo_k(sbase + OFF_K1 + st * kOperandBytes);
+                const uint32_t aq = desc_lo_k(sbase + P1_OFF_Q + (PAIR ? (j & 1) * kOperandBytes : 0u));
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
                     tc_mma(tmem_base + (j & 1) * 128u, desc_make(aq + desc_kstep(ks, kHalfBytes)), desc_make(ak + desc_kstep(ks, kHalfBytes)), idesc_s, ks > 0);
@@ -1317,20 +1343,23 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             };
             failed = !mbar_wait(bar(P1_QFULL), 0);
             if (!failed) failed = !issue_s(0);
-            if (!failed && n_tiles > 1) failed = !issue_s(1);
+            if (!failed && is_item(1)) failed = !issue_s(1);
             if (failed) fail_site = __LINE__;
-            for (int i = 0; i < n_tiles && !failed; ++i) {
-                const uint32_t w = i & 1;
+            const int n_items = PAIR ? 2 * n_tiles : n_tiles;
+            for (int i = 0; i < n_items && !failed; ++i) {
+                const uint32_t w = i & 1, tl = tile_at(i);
+                if (PAIR && !is_item(i)) continue;
                 if (!mbar_wait(bar(P1_PFULL + w), (i >> 1) & 1)) { failed = true; fail_site = __LINE__; break; }
                 tc_fence_after();
-                const uint32_t av = desc_lo_mn(sbase + P1_OFF_V + (i % P1_NSTAGE) * kOperandBytes);
+                const uint32_t av = desc_lo_mn(sbase + OFF_V1 + (tl % NST) * kOperandBytes);
                 const uint32_t first = i > 1;                                // the warpgroup's first tile initialises O_w
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)                               // 128 tokens = 8 steps of K = 16 (2048 bytes of V each)
                     tc_mma_ts(tmem_base + 256u + w * 128u, tmem_base + w * 128u + ks * 8, desc_make(av + ks * (2048 >> 4)),
                               idesc_pv, ks > 0 ? 1u : first);
-                tc_commit(bar(P1_EMPTY + (i % P1_NSTAGE)));                  // S(i) and P.V(i) have read the stage
-                if (i + 2 < n_tiles && !issue_s(i + 2)) { failed = true; fail_site = __LINE__; break; }
+                if (!PAIR || w == 1 || !is_item(i + 1))
+                    tc_commit(bar(P1_EMPTY + (tl % NST)));                   // S(i) and P.V(i) have read the stage (in pairs: both warpgroups')
+                if (is_item(i + 2) && !issue_s(i + 2)) { failed = true; fail_site = __LINE__; break; }
             }
             if (!failed) tc_commit(bar(P1_ODONE));
         }
@@ -1343,9 +1372,9 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         if (nv_job) {
             const int t64 = threadIdx.x - 64;                                // 0..63
             for (int i = 0; i < n_tiles && !failed; ++i) {
-                const uint32_t st = i % P1_NSTAGE;
-                if (!mbar_wait(bar(P1_FULL + st), (i / P1_NSTAGE) & 1)) { failed = true; fail_site = __LINE__; break; }
-                const uint8_t* vt = smem + P1_OFF_V + st * kOperandBytes;
+                const uint32_t st = i % NST;
+                if (!mbar_wait(bar(P1_FULL + st), (i / NST) & 1)) { failed = true; fail_site = __LINE__; break; }
+                const uint8_t* vt = smem + OFF_V1 + st * kOperandBytes;
                 const int t0 = (tile_lo + i) * TILE;
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
@@ -1373,10 +1402,11 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         const int w = (warp - 4) >> 2;                                       // warpgroup: tiles w, w+2, ...
         const int lane_grp = warp & 3;
         const int row = lane_grp * 32 + lane;                                // row within the chunk
-        const int rows_valid = min(p.chunk_rows, p.R - c * p.chunk_rows);
+        const int cw = PAIR && w == 1 ? c1 : c0;                             // this warpgroup's row chunk
+        const int rows_valid = min(p.chunk_rows, p.R - cw * p.chunk_rows);
         const bool low_part = HILO && lane_grp >= 2;                       // this warp's rows are the second copies of rows 0..63
         const int row_q = HILO ? row & 63 : row;
-        const int r = c * p.chunk_rows + row_q;
+        const int r = cw * p.chunk_rows + row_q;
         const bool valid = row_q < rows_valid;
         const int last = valid ? (p.causal ? min(Nm - p.W + (r % p.W), N - 1) : N - 1) : -1;   // last visible token
         const int first_masked = min(p.causal ? Nm - p.W + 1 : N, N);        // tiles reaching it need the mask
@@ -1386,7 +1416,8 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         float m_used = -INFINITY, l = 0.f;
         int my_tiles = 0;
 
-        for (int i = w; i < n_tiles && !failed; i += 2, ++my_tiles) {
+        const int i_end = PAIR && w == 1 ? n1 : n_tiles;
+        for (int i = PAIR ? 0 : w; i < i_end && !failed; i += PAIR ? 1 : 2, ++my_tiles) {
             const int t0 = (tile_lo + i) * TILE;
             if (!mbar_wait(bar(P1_SFULL + w), my_tiles & 1)) { failed = true; fail_site = __LINE__; break; }
             tc_fence_after();
@@ -1477,7 +1508,7 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             l += lsum.x + lsum.y;
             tc_wait_st();
             if (t0 + TILE > N && t0 + row >= N) {                            // tail: V rows past the sequence must not reach the MMA
-                uint8_t* vrow = smem + P1_OFF_V + (i % P1_NSTAGE) * kOperandBytes + row * 128;
+                uint8_t* vrow = smem + OFF_V1 + (i % NST) * kOperandBytes + row * 128;
 #pragma unroll
                 for (int ch = 0; ch < 8; ++ch) {
                     *reinterpret_cast<uint4*>(vrow + (ch << 4)) = make_uint4(0, 0, 0, 0);
@@ -1498,12 +1529,76 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // (16-byte chunks XOR-swizzled by the row), and all eight warps store 512-byte rows.
         float* xm = reinterpret_cast<float*>(smem + P1_OFF_Q);               // [2][128]
         float* xl = xm + 256;                                                // [2][128]
-        uint8_t* xo = smem + P1_OFF_K;
+        uint8_t* xo = smem + OFF_K1;
         bool have = my_tiles > 0 && !failed;
         if (n_tiles > 0) {                                                   // all MMAs done: accumulators final, smem free
             if (!mbar_wait(bar(P1_ODONE), 0)) { failed = true; fail_site = __LINE__; have = false; }
             tc_fence_after();
         }
+        if constexpr (PAIR) {
+            // every row is this thread's alone: normalised, turned through shared memory (the K stages are warpgroup 0's,
+            // the V stages warpgroup 1's) and stored in whole rows
+            xo += w * 2 * kOperandBytes;
+            const bool fin = p.out_o != nullptr;
+            const float M = have ? m_used : -INFINITY;
+            const float o_scale = fin ? (l > 0.f ? 1.f / l : 0.f) : 1.f;
+            float sq = 0.f;
+#pragma unroll 1
+            for (int q = 0; q < 4; ++q) {
+                uint32_t oa[32];
+                if (my_tiles > 0) { tc_ld32(tO + q * 32, oa); tc_wait_ld32(oa); }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (my_tiles > 0)
+                        o = make_float4(__uint_as_float(oa[4 * j]) * o_scale, __uint_as_float(oa[4 * j + 1]) * o_scale,
+                                        __uint_as_float(oa[4 * j + 2]) * o_scale, __uint_as_float(oa[4 * j + 3]) * o_scale);
+                    sq = fmaf(o.x, o.x, fmaf(o.y, o.y, fmaf(o.z, o.z, fmaf(o.w, o.w, sq))));
+                    *reinterpret_cast<float4*>(xo + row * 512 + (((q * 8 + j) ^ (row & 31)) << 4)) = o;
+                }
+            }
+            const size_t out0 = (size_t)unit * p.rows_out + (size_t)cw * p.chunk_rows;                          // row 0 of the chunk
+            const size_t prow0 = ((size_t)unit * p.n_splits + split) * p.R + (size_t)cw * p.chunk_rows;
+            if (valid && fin) {
+                const float lse2 = M + log2f(l);
+                p.out_lse2[out0 + row] = lse2; p.out_onorm[out0 + row] = sq;
+                float* cp = p.out_cpair + ((out0 + row) >> 1) * 4 + ((out0 + row) & 1);
+                cp[0] = -lse2; cp[2] = sq;
+            } else if (valid) {
+                p.part_m[prow0 + row] = M; p.part_l[prow0 + row] = l;
+            }
+            __syncwarp();                                                    // a warp stores the 32 rows it has turned
+            __nv_bfloat16* obf = p.out_obf + out0 * kD + lane * 4;
+#pragma unroll 1
+            for (int h = 0; h < 2; ++h) {
+                float4 rowv[16];
+#pragma unroll
+                for (int rr = 0; rr < 16; ++rr) {
+                    const int orow = lane_grp * 32 + h * 16 + rr;
+                    rowv[rr] = *reinterpret_cast<const float4*>(xo + orow * 512 + ((lane ^ (orow & 31)) << 4));
+                }
+#pragma unroll
+                for (int rr = 0; rr < 16; ++rr) {
+                    const int orow = lane_grp * 32 + h * 16 + rr;
+                    if (orow >= rows_valid) continue;
+                    const float4 o = rowv[rr];
+                    if (!fin) { *reinterpret_cast<float4*>(p.part_o + (prow0 + orow) * kD + lane * 4) = o; continue; }
+                    *reinterpret_cast<float4*>(p.out_o + (out0 + orow) * kD + lane * 4) = o;
+                    *reinterpret_cast<uint2*>(obf + (size_t)orow * kD) =
+                        make_uint2(pack_bf16x2(-2.f * o.x, -2.f * o.y), pack_bf16x2(-2.f * o.z, -2.f * o.w));
+                }
+            }
+            if (fin && cw == p.n_chunks - 1)                                 // padding rows: O = 0, weight 0
+                for (int r0 = p.R - cw * p.chunk_rows + lane_grp; r0 < p.rows_out - cw * p.chunk_rows; r0 += 4) {
+                    *reinterpret_cast<float4*>(p.out_o + (out0 + r0) * kD + lane * 4) = make_float4(0.f, 0.f, 0.f, 0.f);
+                    *reinterpret_cast<uint2*>(obf + (size_t)r0 * kD) = make_uint2(0u, 0u);
+                    if (lane == 0) {
+                        p.out_lse2[out0 + r0] = INFINITY; p.out_onorm[out0 + r0] = 0.f;
+                        float* cp = p.out_cpair + ((out0 + r0) >> 1) * 4 + ((out0 + r0) & 1);
+                        cp[0] = -INFINITY; cp[2] = 0.f;
+                    }
+                }
+        } else {
         xm[w * 128 + row] = have ? m_used : -INFINITY;
         xl[w * 128 + row] = l;
         asm volatile("bar.sync 1, 256;" ::: "memory");                       // both softmax warpgroups
@@ -1615,6 +1710,7 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 }
             }
         }
+        }
         tc_fence_before();
     }
 
@@ -1685,6 +1781,15 @@ static int tc_chunk_split(const ScoreShape& s, const TcChunks& ch) {
     const int nc = ch.rows_out / MC_ROWS;
     const int run = (int)(pairs * nc / (2 * sm_count())), c = (nc + run) / (run > 1 ? run : 1) + 1;
     return c < 2 ? 2 : c > 32 ? 32 : c > nc ? nc : c;
+}
+
+// Pass 1 takes the row chunks of a unit two by two (tc_pass1_kernel, PAIR) where the pairs alone give every SM a CTA and
+// the cache is longer than ten tiles.  Whole-sequence windows of 8 KV heads x 4 heads, chunks / pairs: 1100 queries (144
+// pairs) 31 / 35 us, 1300 (168) 42 / 39, 2048 68 / 57, 3001 126 / 120, 4096 188 / 174; 2 x 4 x 4096 (128 pairs) 49 / 79; 8 x 4 x 1024
+// (eight tiles) 26.5 / 28.2.  With several splits per pair (few rows, a long cache) the gain in pass 1 (56691 to 93869 tokens: from 10 %
+// faster to 16 % slower) went to the merge of twice as many partial results.
+static bool p1_pairs(const ScoreShape& s, const TcChunks& ch) {
+    return ch.n_chunks > 1 && (long long)s.B * s.Hkv * ((ch.n_chunks + 1) / 2) >= sm_count() && s.Nmax > 10 * TILE;
 }
 
 // Workspace plan of the tensor-core path: the SIMT plan's layout with splits counted in 128-token tiles.
@@ -1768,11 +1873,12 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         obc_status st = launch_given_prep(s, plan, *given, ws, stream);
         if (st != OBC_OK) return st;
     } else {       // pass 1 + combine
+        const bool pairs = p1_pairs(s, ch);
         P1Params p1{};
         p1.B = s.B; p1.Hq = s.Hq; p1.Hkv = s.Hkv; p1.G = s.G; p1.W = s.W; p1.R = s.R; p1.Nmax = s.Nmax;
         p1.seq_lens = s.seq_lens; p1.mask_lens = s.mask_lens; p1.scale = s.scale; p1.causal = s.causal;
         p1.n_chunks = ch.n_chunks; p1.chunk_rows = ch.chunk_rows;
-        p1.head_chunks = s.causal && ch.n_chunks > 1 ? s.W / ch.chunk_rows : 0;
+        p1.head_chunks = s.causal && ch.n_chunks > 1 ? s.W / (pairs ? 2 * ch.chunk_rows : ch.chunk_rows) : 0;
         p1.n_splits = plan.n_splits; p1.tiles_per_split = plan.tiles_per_split;
         p1.l2_stream = l2_stream ? 1 : 0;
         p1.part_m = (float*)(wsb + plan.off_part_m); p1.part_l = (float*)(wsb + plan.off_part_l);
@@ -1790,10 +1896,10 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
             p1.out_lse2 = (float*)(wsb + plan.off_lse2); p1.out_onorm = (float*)(wsb + plan.off_onorm);
             p1.out_cpair = (float*)(wsb + plan.off_cpair);
         }
-        const auto pass1 = hilo ? tc_pass1_kernel<true> : tc_pass1_kernel<false>;
+        const auto pass1 = hilo ? tc_pass1_kernel<true, false> : pairs ? tc_pass1_kernel<false, true> : tc_pass1_kernel<false, false>;
         OBC_CUDA_TRY(allow_smem(pass1, kSmemP1));
         { ProfScope ps("tc_pass1", stream);
-          OBC_CUDA_TRY(launch_pdl(pass1, dim3(plan.n_splits, units * ch.n_chunks), dim3(kThreadsP1), kSmemP1, stream, 1, mq, mk, mv, p1)); }
+          OBC_CUDA_TRY(launch_pdl(pass1, dim3(plan.n_splits, units * (pairs ? (ch.n_chunks + 1) / 2 : ch.n_chunks)), dim3(kThreadsP1), kSmemP1, stream, 1, mq, mk, mv, p1)); }
         if (!direct) {
             obc_status st = launch_combine(s, plan, ws, stream);
             if (st != OBC_OK) return st;

@@ -122,6 +122,17 @@ def test_one_cta_per_head_and_chunk(N, W, Hq, Hkv):
 
 
 @pytest.mark.parametrize("N,W,Hq,Hkv,lens", [
+    (1281, 130, 160, 80, None),           # three chunks, the last pair half empty; one token in the last tile
+    (1300, 1300, 26, 26, None),           # whole-sequence window, the chunks of a pair visit different tiles
+    (1400, 150, 148, 74, [1400, 333]),    # chunks that straddle heads, two lengths
+    (6200, 130, 74, 74, [6200, 100 + 130]),   # two splits of a pair: partial results
+])
+def test_row_chunks_in_pairs(N, W, Hq, Hkv, lens):
+    case = synth.make_prefill("pairs", B=len(lens) if lens else 1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=lens or N, dtype="bf16", seed=N + W, hh_frac=0.02)
+    _check(case, ["K", "VK"], tight=2e-2)
+
+
+@pytest.mark.parametrize("N,W,Hq,Hkv,lens", [
     (1641, 1641, 4, 1, None),             # chunks that straddle heads, a pair shared by many CTAs
     (700, 300, 6, 2, [700, 431]),         # hidden chunks in the last pairs only, two lengths
     (513, 513, 8, 8, None),               # one token in the last pair
