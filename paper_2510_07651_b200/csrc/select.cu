@@ -56,6 +56,42 @@ __device__ __forceinline__ uint32_t pooled_key(const SelectShape& s, const float
     return float_key(val);
 }
 
+// Four consecutive pooled values from the twelve staged scores f that begin with the first value's first tap; 2 H + 1 taps
+template <int H>
+__device__ __forceinline__ float4 pool4(const float (&f)[12], int mode, float kernel) {
+    float v[4];
+    if (mode == OBC_POOL_MAX) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            v[j] = -INFINITY;
+#pragma unroll
+            for (int t = 0; t <= 2 * H; ++t) v[j] = fmaxf(v[j], f[j + t]);     // padding taps are -inf
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {                                          // ascending index order; padding adds +0
+            v[j] = 0.f;
+#pragma unroll
+            for (int t = 0; t <= 2 * H; ++t) v[j] = __fadd_rn(v[j], f[j + t]);
+            v[j] = __fdiv_rn(v[j], kernel);
+        }
+    }
+    return make_float4(v[0], v[1], v[2], v[3]);
+}
+
+// The same for stage[i ..], i a multiple of four, with three reads of four scores each; kernels up to 7 (half <= 3).
+// stage[i] holds the first tap of value i, and is readable up to stage[i + 11].
+__device__ __forceinline__ float4 pool4_staged(const float* stage, int half, int mode, int kernel) {
+    float f[12];
+    *reinterpret_cast<float4*>(&f[0]) = *reinterpret_cast<const float4*>(stage);
+    if (half > 0) *reinterpret_cast<float4*>(&f[4]) = *reinterpret_cast<const float4*>(stage + 4);
+    if (half > 2) *reinterpret_cast<float4*>(&f[8]) = *reinterpret_cast<const float4*>(stage + 8);
+    if (half == 0) return make_float4(f[0], f[1], f[2], f[3]);
+    if (half == 1) return pool4<1>(f, mode, (float)kernel);
+    if (half == 2) return pool4<2>(f, mode, (float)kernel);
+    return pool4<3>(f, mode, (float)kernel);
+}
+
 __global__ void __launch_bounds__(256)
 pool_key_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* __restrict__ keys) {
     pdl_wait();
@@ -74,14 +110,18 @@ pool_key_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* __res
 // candidates equal to T) tokens: only the COUNTS have to be found across heads, and the per-head selection does the rest.
 // T comes out of three histogram levels per head (11 + 11 + 10 bits) over the whole chip:
 //   adaptive_pool_kernel   pooled keys, level-1 histograms
-//   adaptive_hist_kernel   (levels 2 and 3) every CTA finds the digit of the level before, then counts its keys below it
+//   adaptive_hist_kernel   (levels 2 and 3) every CTA finds the digit of the level before, then counts its keys below it,
+//                          the first of which it asked for before the search
 //   the selection kernels  last digit, tie shares, scored tokens of the head
 // Every histogram row comes with 32 sums over equal runs of its bins, so that a digit is found in two round trips to L2
 // (32 runs of every head, then the bins of one run) by any CTA that needs it.
-// Latency bound: 8 heads x 32k keys 5.4 + 4.6 + 5.2 us and 2 us in the selection; 8 x 98k keys 8.1 + 6.1 + 6.0 us.  (Ranking
+// Latency bound: 8 heads x 32k keys 3.5 + 4.2 + 4.7 us and 7.7 us in the selection, which asks for its keys before the search
+// as well (with the keys asked for behind the searches, and one candidate pooled at a time from global memory instead of four
+// from shared memory, 5.4 + 4.6 + 5.2 and 8.4 us).  (Ranking
 // all heads' keys as one sequence in one 16-CTA cluster took 20 us for the former and, where the keys did not fit one, by
 // one CTA, 1.07 ms for the latter.)
 constexpr int AD_NT = 512;
+constexpr int AD_EARLY = 4;                                    // keys per thread that a histogram kernel asks for first
 constexpr int AD_BINS = 2048;                 // bins of levels 1 and 2; level 3 has half of them
 constexpr int AD_ROW = AD_BINS + 32;          // a head's row: bins, then the sums over 32 runs of them
 
@@ -223,11 +263,42 @@ adaptive_pool_kernel(SelectShape s, const float* __restrict__ scores, uint32_t* 
     pdl_wait();
     const int lo = s.n_sink, hi = min(seq_len(s, b), s.Nmax) - s.n_recent;
     const float* sc = scores + (size_t)unit * s.Nmax;
-#pragma unroll 4
-    for (int p = c0 + threadIdx.x; p < c1; p += AD_NT) {
-        const uint32_t key = pooled_key(s, sc, p, lo, hi);
-        keys[(size_t)unit * s.Nmax + p] = key;
-        if (key) atomicAdd(&hist[key >> 21], 1u);
+    uint32_t* out = keys + (size_t)unit * s.Nmax;
+    const int half = s.pool_mode == OBC_POOL_NONE ? 0 : s.pool_kernel / 2, tid = threadIdx.x;
+    if (half <= 3) {                                           // four values per thread out of staged scores
+        constexpr int BLOCK = 4 * AD_NT;
+        __shared__ __align__(16) float stage[BLOCK + 8];
+        const float pad = s.pool_mode == OBC_POOL_MAX ? -INFINITY : 0.f;
+        for (int base = c0; base < c1; base += BLOCK) {
+            float val[5];
+#pragma unroll
+            for (int u = 0; u < 5; ++u) {
+                const int i = u * AD_NT + tid, p = base + i - half;
+                val[u] = i < BLOCK + 2 * half && p >= lo && p < hi ? sc[p] : pad;
+            }
+#pragma unroll
+            for (int u = 0; u < 5; ++u)
+                if (u * AD_NT + tid < BLOCK + 2 * half) stage[u * AD_NT + tid] = val[u];
+            __syncthreads();
+            const int p0 = base + tid * 4;
+            const float4 v = pool4_staged(stage + tid * 4, half, s.pool_mode, s.pool_kernel);
+            const float v4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int p = p0 + j;
+                if (p >= c1) continue;
+                const uint32_t key = p >= lo && p < hi ? float_key(v4[j]) : 0u;
+                out[p] = key;
+                if (key) atomicAdd(&hist[key >> 21], 1u);
+            }
+            __syncthreads();
+        }
+    } else {
+        for (int p = c0 + tid; p < c1; p += AD_NT) {
+            const uint32_t key = pooled_key(s, sc, p, lo, hi);
+            out[p] = key;
+            if (key) atomicAdd(&hist[key >> 21], 1u);
+        }
     }
     __syncthreads();
     adaptive_flush(hist, AD_BINS, lv.row(0, unit));
@@ -243,6 +314,13 @@ adaptive_hist_kernel(SelectShape s, const uint32_t* __restrict__ keys, AdaptiveL
     for (int d = threadIdx.x; d < BINS; d += AD_NT) hist[d] = 0;
     pdl_wait();
     const int unit = blockIdx.y, b = unit / s.Hkv, u0 = b * s.Hkv, c0 = blockIdx.x * lv.chunk, c1 = min(c0 + lv.chunk, s.Nmax);
+    const uint32_t* kin = keys + (size_t)unit * s.Nmax;
+    uint32_t early[AD_EARLY];                                  // these keys travel while the digit is looked for
+#pragma unroll
+    for (int u = 0; u < AD_EARLY; ++u) {
+        const int p = c0 + u * AD_NT + threadIdx.x;
+        early[u] = p < c1 ? kin[p] : 0u;
+    }
     const int rem = adaptive_rem(s, b, lv.n_safe);
     if (rem <= 0) return;                                      // nothing to share out (adaptive_share sees to it)
     const uint32_t d = adaptive_find<LEVEL - 2>(lv, u0, s.Hkv, (uint32_t)rem, sh);
@@ -255,9 +333,12 @@ adaptive_hist_kernel(SelectShape s, const uint32_t* __restrict__ keys, AdaptiveL
     }
     const uint32_t prefix = LEVEL == 2 ? d : lv.digit[b * 2] << 11 | d;
     constexpr int SHIFT = LEVEL == 2 ? 21 : 10, NEXT = LEVEL == 2 ? 10 : 0;
+#pragma unroll
+    for (int u = 0; u < AD_EARLY; ++u)
+        if (c0 + u * AD_NT + (int)threadIdx.x < c1 && early[u] >> SHIFT == prefix) atomicAdd(&hist[(early[u] >> NEXT) & (BINS - 1)], 1u);
 #pragma unroll 8
-    for (int p = c0 + threadIdx.x; p < c1; p += AD_NT) {
-        const uint32_t key = keys[(size_t)unit * s.Nmax + p];
+    for (int p = c0 + AD_EARLY * AD_NT + threadIdx.x; p < c1; p += AD_NT) {
+        const uint32_t key = kin[p];
         if (key >> SHIFT == prefix) atomicAdd(&hist[(key >> NEXT) & (BINS - 1)], 1u);
     }
     __syncthreads();
@@ -431,29 +512,8 @@ __device__ __forceinline__ void find_bin(const uint32_t* hist, uint32_t remainin
     __syncthreads();
 }
 
-// Four consecutive pooled values from the twelve staged scores f that begin with the first value's first tap; 2 H + 1 taps
-template <int H>
-__device__ __forceinline__ float4 pool4(const float (&f)[12], int mode, float kernel) {
-    float v[4];
-    if (mode == OBC_POOL_MAX) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            v[j] = -INFINITY;
-#pragma unroll
-            for (int t = 0; t <= 2 * H; ++t) v[j] = fmaxf(v[j], f[j + t]);     // padding taps are -inf
-        }
-    } else {
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {                                          // ascending index order; padding adds +0
-            v[j] = 0.f;
-#pragma unroll
-            for (int t = 0; t <= 2 * H; ++t) v[j] = __fadd_rn(v[j], f[j + t]);
-            v[j] = __fdiv_rn(v[j], kernel);
-        }
-    }
-    return make_float4(v[0], v[1], v[2], v[3]);
-}
-
+// ADAPTIVE: the budgets are shared out across the heads, and the pooled keys are there already (keys_in, [units][Nmax])
+template <bool ADAPTIVE>
 __global__ void __launch_bounds__(CL_NT)
 select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* __restrict__ idx_all, int seg_cap,
                       const uint32_t* __restrict__ keys_in, AdaptiveLevels ad) {
@@ -473,18 +533,27 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
         clear(sh.local);
         if (tid == 0) { sh.n_list = 0; sh.n_above = 0; sh.n_few = 0; sh.before[0] = 0; sh.before[1] = 0; }
     };
-    if (!ad.hist) reset();
+    if (!ADAPTIVE) reset();
     pdl_wait();
     const int unit = blockIdx.x >> lC, b = unit / s.Hkv;
     const int N = seq_len(s, b);
     const int lo = s.n_sink, hi = N - s.n_recent, n = hi - lo;
+    // this CTA's share of the candidates: [c0, c1) of [0, n)
+    const int seg = (((n + C - 1) >> lC) + 31) / 32 * 32;
+    const int c0 = min(rank * seg, n), c1 = min(c0 + seg, n), m = c1 - c0;
+    if (ADAPTIVE && N <= s.Nmax) {                 // the keys travel while the head's share is looked for
+        const uint32_t* kin = keys_in + (size_t)unit * s.Nmax + lo + c0;
+        for (int i = tid; i < m; i += CL_NT)
+            asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(keys + i)), "l"(kin + i) : "memory");
+    }
     // (the search across heads borrows the space of a histogram that is cleared behind it)
     HeadShare share{budget_of(s, b) - s.n_sink - s.n_recent, false, 0u, 0u};
-    if (ad.hist) {
+    if (ADAPTIVE) {
         share = adaptive_share(s, ad, unit, *reinterpret_cast<AdaptiveFind*>(&sh.local[0]));
         __syncthreads();
         reset();
     }
+    if (ADAPTIVE) asm volatile("cp.async.wait_all;" ::: "memory");  // (before any way out of the kernel)
     const int n_hh = share.n_hh;
     const int budget = n_hh + s.n_sink + s.n_recent;
     int32_t* idx = idx_all + (size_t)unit * s.idx_stride;
@@ -493,22 +562,16 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
     // these tests depend on the unit only, so all CTAs of the cluster leave together
     if (n_hh < 0 || n_hh > n || budget > s.idx_stride || N > s.Nmax || hi < lo) {   // bad per-sequence budget
         for (int j = gtid; j < s.idx_stride; j += gthreads) idx[j] = -1;
-        if (ad.hist && gtid == 0) ad.counts[unit] = -1;
+        if (ADAPTIVE && gtid == 0) ad.counts[unit] = -1;
         return;
     }
-    if (ad.hist && gtid == 0) ad.counts[unit] = budget;
+    if (ADAPTIVE && gtid == 0) ad.counts[unit] = budget;
     for (int j = gtid; j < s.n_sink; j += gthreads) idx[j] = j;
     for (int j = gtid; j < s.n_recent; j += gthreads) idx[s.n_sink + n_hh + j] = hi + j;
     for (int j = budget + gtid; j < s.idx_stride; j += gthreads) idx[j] = -1;
     if (n_hh == 0) return;
 
-    // ---- this CTA's share of the candidates: [c0, c1) of [0, n) --------------------------------
-    const int seg = (((n + C - 1) >> lC) + 31) / 32 * 32;
-    const int c0 = min(rank * seg, n), c1 = min(c0 + seg, n), m = c1 - c0;
-    if (keys_in) {                                 // the caller has the (pooled) keys already: [units][Nmax]
-        const uint32_t* kin = keys_in + (size_t)unit * s.Nmax + lo + c0;
-#pragma unroll 8
-        for (int i = tid; i < m; i += CL_NT) keys[i] = kin[i];
+    if (ADAPTIVE) {
         __syncthreads();
         cluster.barrier_arrive();
         if (!share.known)
@@ -538,15 +601,8 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
         // four candidates per thread and step; the top 11 bits of their keys go straight into the first histogram
         for (int i = tid * 4; i < m; i += CL_NT * 4) {
             float4 v;
-            if (half <= 3) {                           // kernels up to 7: twelve staged scores in three reads
-                float f[12];
-                *reinterpret_cast<float4*>(&f[0]) = *reinterpret_cast<const float4*>(stage + i);
-                if (half > 0) *reinterpret_cast<float4*>(&f[4]) = *reinterpret_cast<const float4*>(stage + i + 4);
-                if (half > 2) *reinterpret_cast<float4*>(&f[8]) = *reinterpret_cast<const float4*>(stage + i + 8);
-                if (half == 0) v = make_float4(f[0], f[1], f[2], f[3]);
-                else if (half == 1) v = pool4<1>(f, s.pool_mode, (float)s.pool_kernel);
-                else if (half == 2) v = pool4<2>(f, s.pool_mode, (float)s.pool_kernel);
-                else v = pool4<3>(f, s.pool_mode, (float)s.pool_kernel);
+            if (half <= 3) {
+                v = pool4_staged(stage + i, half, s.pool_mode, s.pool_kernel);
             } else {
                 float* out = reinterpret_cast<float*>(&v);
                 for (int j = 0; j < 4; ++j) {
@@ -862,7 +918,9 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
     const int C = select_cluster_size(units, s.Nmax, &seg_cap);
     if (C > 0) {
         const size_t smem = sizeof(ClusterShared) + (size_t)seg_cap * 8 + (size_t)s.pool_kernel * 4 + 32;
-        OBC_CUDA_TRY(allow_smem(select_cluster_kernel, smem));
+        const bool adaptive = keys_in != nullptr;
+        const auto kernel = adaptive ? select_cluster_kernel<true> : select_cluster_kernel<false>;
+        OBC_CUDA_TRY(allow_smem(kernel, smem));
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3((unsigned)(units * C)); cfg.blockDim = dim3(CL_NT); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
         cudaLaunchAttribute attr[1];
@@ -870,21 +928,21 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
         attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         // whether the device can host such a cluster depends on the cluster size and the shared memory alone: asked once
-        // per (device, size, bytes) and remembered (the query costs as much host time as the launch)
-        thread_local struct { int dev, C; size_t smem; int max_clusters; } seen[4] = {};
+        // per (kernel, device, size, bytes) and remembered (the query costs as much host time as the launch)
+        thread_local struct { bool adaptive; int dev, C; size_t smem; int max_clusters; } seen[8] = {};
         thread_local int seen_next = 0;
         int dev = -1, max_clusters = -1;
         (void)cudaGetDevice(&dev);
-        for (const auto& e : seen) if (e.C == C && e.smem == smem && e.dev == dev) max_clusters = e.max_clusters;
+        for (const auto& e : seen) if (e.C == C && e.smem == smem && e.dev == dev && e.adaptive == adaptive) max_clusters = e.max_clusters;
         if (max_clusters < 0) {
-            if (C > 8) OBC_CUDA_TRY(cudaFuncSetAttribute(select_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-            if (cudaOccupancyMaxActiveClusters(&max_clusters, select_cluster_kernel, &cfg) != cudaSuccess) { max_clusters = 0; (void)cudaGetLastError(); }
-            seen[seen_next] = {dev, C, smem, max_clusters};
-            seen_next = (seen_next + 1) % 4;
+            if (C > 8) OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            if (cudaOccupancyMaxActiveClusters(&max_clusters, kernel, &cfg) != cudaSuccess) { max_clusters = 0; (void)cudaGetLastError(); }
+            seen[seen_next] = {adaptive, dev, C, smem, max_clusters};
+            seen_next = (seen_next + 1) % 8;
         }
         if (max_clusters > 0) {
             { ProfScope ps("select_cluster", stream);
-              OBC_CUDA_TRY(launch_pdl(select_cluster_kernel, dim3((unsigned)(units * C)), dim3(CL_NT), smem, stream, C, s, scores, idx, seg_cap, keys_in, ad)); }
+              OBC_CUDA_TRY(launch_pdl(kernel, dim3((unsigned)(units * C)), dim3(CL_NT), smem, stream, C, s, scores, idx, seg_cap, keys_in, ad)); }
             return OBC_OK;
         }
         (void)cudaGetLastError();                  // the device cannot host such a cluster: one CTA per head
