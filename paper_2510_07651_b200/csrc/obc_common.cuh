@@ -173,20 +173,38 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(std::forward<Args>(args))...);
 }
 
-// Lets `kernel` use `bytes` of dynamic shared memory on the current device.  The attribute stays with the kernel, so what a
-// host thread has asked for is remembered (per kernel and device) and the call, about a microsecond of host time per
-// launch, is made once.
+// Lets `kernel` use `bytes` of dynamic shared memory on the current device.  The attribute belongs to the kernel and the
+// device, not to the launch or to the host thread, and a smaller value would take from other threads what they count on: so
+// whoever asks sets it to all that the device has left for the kernel (a launch still takes only its own size), and a value
+// that was set is never lowered.  What a host thread has seen set is remembered (per kernel and device), so that the calls,
+// about a microsecond of host time per launch, are made once.  More than the device has is refused, as by the call itself.
 template <typename... KArgs>
 inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
     struct Seen { const void* kernel; int dev; size_t bytes; };
-    thread_local Seen seen[32] = {};
+    constexpr unsigned kSlots = 32;
+    thread_local Seen seen[kSlots] = {};
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    Seen& at = seen[((uintptr_t)kernel >> 4) % 32];
-    if (at.kernel == (const void*)kernel && at.dev == dev && at.bytes >= bytes) return cudaSuccess;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    if (e == cudaSuccess) at = Seen{(const void*)kernel, dev, bytes};
+    const unsigned first = (unsigned)((uintptr_t)kernel >> 4) % kSlots;
+    Seen* at = &seen[first];                               // where the entry goes if there is none and no free slot
+    for (unsigned i = 0; i < kSlots; ++i) {
+        Seen& s = seen[(first + i) % kSlots];
+        if (s.kernel == (const void*)kernel && s.dev == dev) {
+            if (s.bytes >= bytes) return cudaSuccess;
+            at = &s;
+            break;
+        }
+        if (!s.kernel) { at = &s; break; }
+    }
+    int optin = 0;
+    cudaFuncAttributes fa{};
+    if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&fa, kernel)) != cudaSuccess) return e;
+    const size_t all = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
+    if (bytes > all) return cudaErrorInvalidValue;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)all);
+    if (e == cudaSuccess) *at = Seen{(const void*)kernel, dev, all};
     return e;
 }
 
