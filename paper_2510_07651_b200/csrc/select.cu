@@ -812,12 +812,14 @@ gather_kernel(int units, int Hkv, int idx_stride, int vecs, int elem_bytes,
     char* kob = (char*)ko.ptr + ((size_t)b * ko.sb + (size_t)g * ko.sh) * eb;
     char* vob = (char*)vo.ptr + ((size_t)b * vo.sb + (size_t)g * vo.sh) * eb;
     int src[4], j[4], c[4];
+    bool pad[4];                                           // the row exists and its index is negative
     uint4 kv[4], vv[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int e = e0 + u * quarter;
         j[u] = e / vecs; c[u] = e % vecs;
-        src[u] = e < total ? idx[(size_t)unit * idx_stride + j[u]] : -2;         // -2: no row at all
+        src[u] = e < total ? idx[(size_t)unit * idx_stride + j[u]] : -1;
+        pad[u] = e < total && src[u] < 0;
     }
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -831,7 +833,7 @@ gather_kernel(int units, int Hkv, int idx_stride, int vecs, int elem_bytes,
             reinterpret_cast<uint4*>(kob + (size_t)j[u] * ko.st * eb)[c[u]] = kv[u];
             reinterpret_cast<uint4*>(vob + (size_t)j[u] * vo.st * eb)[c[u]] = vv[u];
             if (s_in && c[u] == 0) s_out[(size_t)unit * idx_stride + j[u]] = s_in[(size_t)unit * Nmax + src[u]];
-        } else if (zero_rows && src[u] == -1) {            // padding rows of outputs that nobody has cleared
+        } else if (zero_rows && pad[u]) {            // padding rows of outputs that nobody has cleared
             const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
             if (zero_rows & OBC_ZERO_K) reinterpret_cast<uint4*>(kob + (size_t)j[u] * ko.st * eb)[c[u]] = zero;
             if (zero_rows & OBC_ZERO_V) reinterpret_cast<uint4*>(vob + (size_t)j[u] * vo.st * eb)[c[u]] = zero;

@@ -168,6 +168,24 @@ def test_compact_padding_rows(dtype, kept, stride):
     assert ko2 is mine and torch.equal(ko2[:, :, :kept], ko[:, :, :kept]) and (ko2[:, :, kept:] == 3.0).all() and torch.equal(vo2, vo)
 
 
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_compact_rows_of_any_negative_index_are_zero(dtype):
+    g = torch.Generator(device="cuda").manual_seed(4)
+    k = torch.randn((1, 2, 90, 128), generator=g, device="cuda").to(dtype)
+    s = torch.rand((1, 2, 90), generator=g, device="cuda")
+    idx = torch.tensor([3, -1, 7, -2, -5, 89, -2 ** 31], dtype=torch.int32, device="cuda").repeat(1, 2, 1)
+    filler = [torch.full((1, 2, 7, 128), 7.0, dtype=dtype, device="cuda") for _ in range(3)]        # so that fresh memory is not zero
+    del filler
+    filler = torch.full((1, 2, 7), 7.0, device="cuda")
+    del filler
+    kept = idx[0, 0] >= 0
+    for out, src in zip(api.obc_compact(k, k, idx, scores_in=s), (k, k, s)):
+        assert torch.equal(out[:, :, kept], src[:, :, [3, 7, 89]]) and (out[:, :, ~kept] == 0).all()
+    mine = torch.full((1, 2, 7, 128), 3.0, dtype=dtype, device="cuda")
+    api.obc_compact(k, k, idx, k_out=mine)
+    assert (mine[:, :, ~kept] == 3.0).all()
+
+
 def test_whole_prefill_path_config1():
     # score -> select -> compact end to end; selection compared on the GPU's own fp32 scores
     case, run = synth.config(1)
