@@ -244,6 +244,8 @@ def obc_score_given(q, k, v, o, lse, *, seq_lens=None, scale=0.0, causal=True, v
                     scores=None, workspace=None, mask_lens=None):
     """obc_score from attention outputs the caller already has: o [B,Hq,W,d] (f32 or bf16) and lse
     fp32 [B,Hq,W] (natural log, contiguous) of the window rows; no window attention is recomputed."""
+    if o is None or lse is None:               # (for the native call, o = None would stand for obc_score)
+        raise TypeError("o and lse are required: the window rows' outputs and log-sum-exp")
     return _result(_native().score(q, k, v, o, lse, seq_lens, mask_lens, scale, 1 if causal else 0, variants_mask(variants),
                                    PATHS[path] if isinstance(path, str) else path, scores, workspace), "obc_score_given")
 

@@ -159,3 +159,12 @@ def test_missing_library_fails_loudly(monkeypatch):
     monkeypatch.setattr(api, "LIB_PATH", "/nonexistent/libobcache.so")
     with pytest.raises(OSError):
         api.lib()
+
+
+def test_given_outputs_are_required():
+    # without outputs obc_score_given must not turn into a recompute of the window attention
+    import torch
+    t = torch.zeros((1, 1, 4, 128))
+    for o, lse in ((None, torch.zeros((1, 1, 4))), (t, None), (None, None)):
+        with pytest.raises(TypeError, match="o and lse"):
+            api.obc_score_given(t, t, t, o, lse)
