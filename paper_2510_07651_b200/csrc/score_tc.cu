@@ -50,7 +50,7 @@ constexpr uint32_t OFF_V = OFF_K + NSTAGE * kOperandBytes;        // NSTAGE x 32
 constexpr uint32_t OFF_CONST = OFF_V + NSTAGE * kOperandBytes;    // 16 epilogue warps x 32 float4 (row-pair constants of the warp's half)
 constexpr int NSLOT = 4;                                          // ring depth of the per-tile value norms
 constexpr uint32_t OFF_NV = OFF_CONST + 16 * 32 * 16;             // NSLOT x 128 x (||v||^2, ||v||_1), own-norm kernels only
-constexpr int kNumSums = 6;                                       // running sums a token carries (RowSums)
+constexpr int kNumSums = 7;                                       // running sums a token carries (RowSums)
 constexpr uint32_t OFF_XCH = OFF_NV + NSLOT * TILE * 8;           // [tile parity][2][kNumSums][128] floats: the second half's sums
 constexpr uint32_t OFF_BAR = OFF_XCH + 2 * 2 * kNumSums * TILE * 4;
 constexpr uint32_t kNumBars = 2 * NSTAGE + 2 + 4 + 2 + 2 * NSLOT + 4;
@@ -413,17 +413,23 @@ __device__ __forceinline__ void value_norms(const uint8_t* vt, int tok, float& l
 // instructions per row pair and one exponential per row serve Eq. 4-6 together (the sums over u = a z and
 // b = a (1 + Z) that they replace took ten for Eq. 5 and 6 and thirteen with the rest: 512 rows per head, four sequences of
 // up to 26550 tokens, Eq. 4-6: 265 -> 228 us for pass 2; Eq. 5 and 6 of the 128k layer with 448 rows: 163 -> 157 us).
-// The joint score alone is cheaper in u and b: s1 = sum b^2, s2 = sum u (b t' + u scale |o_r|^2), and the score is
-// |v|^2 s1 + scale s2 with seven instructions per row pair.
-struct RowSums { float2 s1, s2, s3, s4, s5, s6; };
+// The joint score alone is cheaper in u = a z and b = a (1 + Z): s1 = sum b^2, s2 = sum u (b t' + u scale |o_r|^2), and the
+// score is |v|^2 s1 + scale s2 with seven instructions per row pair.
+// S1 + 2 scale S2 + scale^2 S3 stands for a sum of squares and cancels where Z is near -1 in every row that counts, which
+// few rows can bring about (one row: 1e-4 of the token's own score, against 4e-6; no difference from 16 rows on).  Calls with
+// fewer than 64 rows (HILO), whose sums are to be those of 32 bits, therefore keep the squares: S1 = sum a^2, S2 = sum b^2,
+// S3 = sum u^2, S4 = sum u b t', S5 = sum u^2 t', S7 = sum u^2 |o_r|^2, and
+//   Eq. 5   scale^2 (|v|^2 S3 + S5 + S7),   Eq. 6   |v|^2 S2 + scale (S4 + scale S7),
+// with one instruction per row pair more.
+struct RowSums { float2 s1, s2, s3, s4, s5, s6, s7; };
 
-template <unsigned VARS> constexpr bool kWantsA = VARS == OBC_VAR_VK || (VARS & (OBC_VAR_ATTN | OBC_VAR_VATP)) != 0;
+template <unsigned VARS> constexpr bool kSumsA = (VARS & (OBC_VAR_ATTN | OBC_VAR_VATP)) != 0;
 // what the exponent is multiplied with: a^2 alone is wanted, or a
-template <unsigned VARS> constexpr float kExpFactor = kWantsA<VARS> ? 1.f : 2.f;
+template <unsigned VARS, bool HILO = false> constexpr float kExpFactor = HILO || VARS == OBC_VAR_VK || kSumsA<VARS> ? 1.f : 2.f;
 
 // 16 rows of one token: zr = logits, tr = -2 v.o_r, cst = per row pair (-lse2_0, -lse2_1, |o_0|^2, |o_1|^2), the
 // first two times kExpFactor (as sl2); when only the joint score is computed the |o|^2 entries arrive multiplied by scale
-template <unsigned VARS, bool MASKED>
+template <unsigned VARS, bool MASKED, bool HILO>
 __device__ __forceinline__ void score_rows16(const uint32_t (&zr)[16], const uint32_t (&tr)[16], const float4* cst,
                                              float2 sl2, float2 sc, RowSums& S, int ptok, int mask_base, int W, int& wi) {
 #pragma unroll
@@ -444,9 +450,18 @@ __device__ __forceinline__ void score_rows16(const uint32_t (&zr)[16], const uin
             const float2 b = __ffma2_rn(u, sc, a);
             S.s1 = __ffma2_rn(b, b, S.s1);
             S.s2 = __ffma2_rn(u, __ffma2_rn(u, make_float2(cp.z, cp.w), __fmul2_rn(b, t2)), S.s2);
+        } else if (HILO) {
+            const float2 u = __fmul2_rn(a, z), b = __ffma2_rn(u, sc, a), w = __fmul2_rn(u, t2);
+            S.s1 = __ffma2_rn(a, a, S.s1);
+            S.s2 = __ffma2_rn(b, b, S.s2);
+            S.s3 = __ffma2_rn(u, u, S.s3);
+            S.s4 = __ffma2_rn(b, w, S.s4);
+            S.s5 = __ffma2_rn(u, w, S.s5);
+            S.s7 = __ffma2_rn(u, __fmul2_rn(u, make_float2(cp.z, cp.w)), S.s7);
+            if (kSumsA<VARS>) S.s6 = __fadd2_rn(a, S.s6);
         } else {
             float2 c0 = a;                              // a^2 already
-            if (kWantsA<VARS>) { c0 = __fmul2_rn(a, a); S.s6 = __fadd2_rn(a, S.s6); }
+            if (kSumsA<VARS>) { c0 = __fmul2_rn(a, a); S.s6 = __fadd2_rn(a, S.s6); }
             const float2 c1 = __fmul2_rn(c0, z), c2 = __fmul2_rn(c1, z);
             S.s1 = __fadd2_rn(c0, S.s1);
             S.s2 = __fadd2_rn(c1, S.s2);
@@ -458,16 +473,17 @@ __device__ __forceinline__ void score_rows16(const uint32_t (&zr)[16], const uin
 }
 
 // stores the planes of one token from its sums (packed lanes folded)
-template <unsigned VARS>
+template <unsigned VARS, bool HILO = false>
 __device__ __forceinline__ void store_scores(const float (&sum)[kNumSums], float nv, float nv1, float scale, unsigned variants, float* out,
                                              size_t plane, bool live) {
     int pl = 0;
     if (VARS == OBC_VAR_VK) { out[0] = live ? fmaf(nv, sum[0], scale * sum[1]) : 0.f; return; }
     const float s2 = scale * scale;
     if (variants & OBC_VAR_V)    out[(size_t)(pl++) * plane] = live ? nv * sum[0] : 0.f;
-    if (variants & OBC_VAR_K)    out[(size_t)(pl++) * plane] = live ? s2 * fmaf(nv, sum[2], sum[4]) : 0.f;
+    if (variants & OBC_VAR_K)    out[(size_t)(pl++) * plane] = live ? s2 * (fmaf(nv, sum[2], sum[4]) + (HILO ? sum[6] : 0.f)) : 0.f;
     if (variants & OBC_VAR_VK)   out[(size_t)(pl++) * plane] =
-        live ? fmaf(nv, fmaf(s2, sum[2], fmaf(2.f * scale, sum[1], sum[0])), fmaf(scale, sum[3], s2 * sum[4])) : 0.f;
+        !live ? 0.f : HILO ? fmaf(nv, sum[1], scale * fmaf(scale, sum[6], sum[3]))
+                           : fmaf(nv, fmaf(s2, sum[2], fmaf(2.f * scale, sum[1], sum[0])), fmaf(scale, sum[3], s2 * sum[4]));
     if (variants & OBC_VAR_ATTN) out[(size_t)(pl++) * plane] = live ? sum[5] : 0.f;
     if (variants & OBC_VAR_VATP) out[(size_t)(pl++) * plane] = live ? nv1 * sum[5] : 0.f;
 }
@@ -491,7 +507,7 @@ __device__ __forceinline__ void score_chunk(uint32_t zt, uint32_t tt, int chunk_
         }
         tc_ld16(zt + c0, z0);
         tc_wait_ld16x2(z0, t0);
-        score_rows16<VARS, MASKED>(z0, t0, cst + (c0 >> 1), sl2, sc, S, ptok, mask_base, W, wi);
+        score_rows16<VARS, MASKED, HILO>(z0, t0, cst + (c0 >> 1), sl2, sc, S, ptok, mask_base, W, wi);
     }
 }
 
@@ -665,7 +681,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // the chunk's rows in two runs of whole 16-row batches
         const int rows0 = min(p.chunk_rows, (p.chunk_rows / 2 + 15) / 16 * 16);
         const int r_begin = half ? rows0 : 0, r_count = half ? p.chunk_rows - rows0 : rows0;
-        const float ksl = p.scale * kLog2e * kExpFactor<VARS>;
+        const float ksl = p.scale * kLog2e * kExpFactor<VARS, HILO>;
         const float2 sl2 = make_float2(ksl, ksl), sc = make_float2(p.scale, p.scale);
         const size_t plane = (size_t)units * p.Nmax;
         uint32_t item = 0, tile_seq = 0, mine_seq = 0;
@@ -684,7 +700,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             const int Nm = tc_mask_len(p, b);
             const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
             RowSums S;
-            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = make_float2(0.f, 0.f);
+            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
             const uint32_t buf = item & 1;
             float nv = 0.f, nv1 = 0.f;                             // used after the row loop
             if (!OWN_NV && half == 0 && ptok < N) nv = p.nv[(size_t)unit * p.Nmax + ptok];
@@ -694,7 +710,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     const int rp = (r_begin >> 1) + lane;          // row pair of the chunk
                     float4 c4 = lane * 2 < r_count ? p.cpair[(((size_t)unit * p.rows_out) >> 1) + rp] : make_float4(-INFINITY, -INFINITY, 0.f, 0.f);
                     if (VARS == OBC_VAR_VK) { c4.z *= p.scale; c4.w *= p.scale; }
-                    c4.x *= kExpFactor<VARS>; c4.y *= kExpFactor<VARS>;
+                    c4.x *= kExpFactor<VARS, HILO>; c4.y *= kExpFactor<VARS, HILO>;
                     my_const[lane] = c4;
                 }
                 __syncwarp();
@@ -723,7 +739,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (lane == 0) mbar_arrive(bar(BAR_TM_EMPTY + buf));
             ++item;
             // the two row halves of the token meet: the sums of RowSums, packed lanes folded
-            float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y};
+            float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
             // slot xs was last used two of this group's tiles ago; the first half read it before it released the
             // accumulators of the tile after that one, without which the tile at hand could not have been computed
             const uint32_t xs = mine_seq & 1;
@@ -731,7 +747,7 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             if (half == 1) {
 #pragma unroll
                 for (int j = 0; j < kNumSums; ++j) {
-                    const bool used = VARS == OBC_VAR_VK ? j < 2 : j < 5 || kWantsA<VARS>;
+                    const bool used = VARS == OBC_VAR_VK ? j < 2 : j < 5 || (j == 5 ? kSumsA<VARS> : HILO);
                     if (used) xch[j * TILE] = sum[j];
                 }
                 __syncwarp();
@@ -743,10 +759,10 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             ++mine_seq;
 #pragma unroll
             for (int j = 0; j < kNumSums; ++j) {
-                const bool used = VARS == OBC_VAR_VK ? j < 2 : j < 5 || kWantsA<VARS>;
+                const bool used = VARS == OBC_VAR_VK ? j < 2 : j < 5 || (j == 5 ? kSumsA<VARS> : HILO);
                 if (used) sum[j] += xch[j * TILE];
             }
-            if (ptok < p.Nmax) store_scores<VARS>(sum, nv, nv1, p.scale, p.variants, out + ptok, plane, ptok < N);
+            if (ptok < p.Nmax) store_scores<VARS, HILO>(sum, nv, nv1, p.scale, p.variants, out + ptok, plane, ptok < N);
         }
         // padding beyond the last tile of a shorter sequence: zeros
         if (p.seq_lens) {
@@ -986,7 +1002,7 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
             const int ptok = t0 + tok;
             const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
             RowSums S;
-            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = make_float2(0.f, 0.f);
+            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
             for (int v = tw.v0; v < tw.v1; ++v) {
                 const int c = tw.chunk(v);
                 const uint32_t item = 2 * citem + wg, buf = item & 3, cs = citem & 3;
@@ -1020,7 +1036,7 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                 // linear in them), the first into the scores, the others into copies that tc_partial_sum_kernel adds in order
                 if (SPLIT && p.csplit > 1 && threadIdx.x == 128 && tw.ends_pair()) p.copies[(size_t)unit * p.max_pairs + tw.pair] = tw.slot;
                 float* out = (tw.slot > 0 ? p.partial + (size_t)(tw.slot - 1) * __popc(p.variants) * plane : p.scores) + (size_t)unit * p.Nmax;
-                const float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y};
+                const float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
                 store_scores<VARS>(sum, nv, nv1, p.scale, p.variants, out + ptok, plane, ptok < N);
             }
         }

@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 import torch
 
+from oracle import reference as ref
 from paper_2510_07651_b200 import api, synth
 from tests import helpers as H
 
@@ -207,3 +208,28 @@ def test_kernel_spans_are_recorded_and_cleared():
     ws2 = torch.zeros(api.obc_score_workspace(ps), dtype=torch.uint8, device="cuda")
     api.obc_score(q, k, v, variants=["VK"], path="simt", workspace=ws2)
     assert api.obc_score_kernel_spans(ws2) == (0.0, 0.0)
+
+
+@pytest.mark.parametrize("Hq,Hkv,W", [(1, 1, 1), (2, 1, 1), (3, 1, 1)])
+def test_joint_score_near_its_zero(Hq, Hkv, W):
+    """Tokens whose scaled logit is close to -1 for every window row: (1 + Z)^2 is then small against 1 + Z^2, and the joint
+    score keeps its digits only if the square is taken row by row.  The joint score is the same whatever else is asked for,
+    and is off by no more of its own value than a few times what an error of 3e-7 in Z (fp32 logits of magnitude 1, summed
+    over 128 channels) does to it: 2 |1 + Z| |v|^2 3e-7 of a score of at least Z^2 |o|^2."""
+    N, scale = 1500, 128 ** -0.5
+    rng = np.random.default_rng(11)
+    q = np.repeat(rng.standard_normal((1, 1, W, 128)), Hq, 1)
+    k = rng.standard_normal((1, Hkv, N, 128))
+    u = q[0, 0, 0] / np.linalg.norm(q[0, 0, 0])
+    near = -1 + 0.05 * rng.standard_normal(N)
+    k += ((near / (scale * np.linalg.norm(q[0, 0, 0])) - k @ u)[..., None]) * u
+    v = rng.standard_normal((1, Hkv, N, 128))
+    bf = lambda x: synth.bf16_round(x.astype(np.float32))  # noqa: E731
+    (q, qb), (k, kb), (v, vb) = bf(q), bf(k), bf(v)
+    dev = [H.dev_bf16(x) for x in (qb, kb, vb)]
+    want = ref.score(q, k, v, want=("VK",))["VK"][0, 0]
+    got = [api.obc_score(*dev, variants=names)[at, 0, 0].cpu().numpy() for names, at in
+           ((["VK"], 0), (["K", "VK"], 1), (["V", "K", "VK"], 2), (["V", "K", "VK", "ATTN"], 2), (["V", "K", "VK", "ATTN", "VATP"], 2))]
+    assert all(np.array_equal(g, got[0]) or np.abs(g / got[0] - 1).max() < 1e-6 for g in got)
+    own = np.abs(got[0] / want - 1)
+    assert own.max() < 2e-5, own.max()
