@@ -60,6 +60,31 @@ def test_token_sharded_cache_scores_like_the_whole(N, W, Hq, Hkv, dtype, path, c
     assert np.abs(o_all.cpu().numpy() - o_ref).max() <= tol * max(1.0, np.abs(o_ref).max())
 
 
+@pytest.mark.parametrize("Hq,Hkv,W,N,cuts", [
+    (4, 2, 24, 1500, (600, 1490)),        # R = 48; the last shard lies inside the window: its early rows see nothing
+    (2, 2, 7, 900, (450, 896)),           # R = 7
+    (32, 32, 32, 1000, (500, 980)),       # R = 32, many heads
+])
+def test_sharded_cache_with_fewer_than_64_rows_keeps_32_bit_accuracy(Hq, Hkv, W, N, cuts):
+    """bf16 caches, fewer than 64 window rows: a shard's attention is itself a result, in fp32.  Bounds: weights of at most one
+    in fp32, their sum over N tokens and the MMA's or FMA's sums err by a few 2^-24 each, in all below 1e-6 of the norm of O (weights
+    in two bf16 parts, 2^-17 each at most, give 2e-6); the scores hold the tolerance of fp32 caches."""
+    from oracle import reference as ref
+    case = synth.make_prefill("shardfew", B=1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=N + W, hh_frac=0.02)
+    variants = ["V", "K", "VK", "ATTN"]
+    got, o_all, lse_all = _sharded_scores(case, cuts, variants, "auto")
+    want = H.oracle_scores(case, variants)
+    mx = max(np.abs(want[n]).max() for n in ("V", "K", "VK"))
+    for n in variants:
+        H.assert_scores_close(got[n], want[n], "f32", what=f"sharded {n}", mx=None if n == "ATTN" else mx)
+    att = ref.score(case.q, case.k, case.v, want=("ATTN",), return_attention=True)
+    o_ref = att["O"].reshape(1, Hq, W, 128)
+    assert np.linalg.norm(o_all.cpu().numpy() - o_ref) <= 1e-6 * np.linalg.norm(o_ref)
+    q, k, v = H.upload(case)
+    o_one, _ = api.obc_window_attention(q, k, v)
+    assert np.linalg.norm(o_one.cpu().numpy() - o_ref) <= 1e-6 * np.linalg.norm(o_ref)
+
+
 def test_window_attention_with_one_cta_per_row_chunk():
     """2560 window rows per KV head in 20 chunks: pass 1 has one CTA per (unit, chunk), writes the merged results
     itself and no merge kernel runs; in the second shard the early rows see no token at all (their output is 0 and
