@@ -135,7 +135,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
                            SimtPlan* attention_only = nullptr);   // non-null: stop after pass 1 + combine, return the plan
 
 // ---- tensor maps ----------------------------------------------------------------------------------
-// bf16 tensor map of rank 2 or 4 with 128-byte swizzle, innermost dimension = head_dim (128), box
+// bf16 tensor map of rank 2 to 4 with 128-byte swizzle, innermost dimension = head_dim (128), box
 // {64, box_rows, 1, 1}; strides in bytes for dimensions 1..rank-1.  Maps are cached per host thread.
 bool make_map(CUtensorMap* map, const void* base, int rank, const uint64_t* dims, const uint64_t* strides_bytes,
               uint32_t box_rows);

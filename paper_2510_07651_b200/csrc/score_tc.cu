@@ -128,6 +128,20 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
                  ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0, int c1, int c2) {
+    asm volatile("cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
+                 ::"r"(dst), "l"(map), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
+}
+// Pass 2: the window rows from `row` on of a unit (R rows each, one unit after the other).  BY_UNIT, for units whose rows do not
+// fill their last chunk: the map has a dimension for the units, so that the rows that fill it up are zeros and not the next unit's
+// queries, which need not be finite (their weight of 0 would not help).  Elsewhere the map of plain rows, which is
+// the faster one (64 rows x 1024 tokens x 2 heads 13.9 us, 14.0 by unit; 448 rows x 131072 tokens x 4 heads 347.6 and 349.8), and in
+// pass 1, where a row of the MMA's M dimension reaches no other.
+template <bool BY_UNIT>
+__device__ __forceinline__ void load_q(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int row, int unit, int R) {
+    if (BY_UNIT) tma_load_3d(dst, map, bar, x, row, unit);
+    else tma_load_2d(dst, map, bar, x, unit * R + row);
+}
 
 __device__ __forceinline__ void prefetch_tmap(const CUtensorMap* map) {
     asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
@@ -516,7 +530,7 @@ __device__ __forceinline__ void score_chunk(uint32_t zt, uint32_t tt, int chunk_
 // HILO: fewer than 64 window rows.  Such a call is summed in 32 bits throughout: -2 O enters as the sum of two bf16
 // parts, which stand side by side on the MMA's N dimension (at most 2 x 64 rows) and meet in the epilogue.  The
 // kernel stays bound by the K/V tiles it streams, with half of the epilogue's rows idle.
-template <unsigned VARS, bool OWN_NV, bool HILO>
+template <unsigned VARS, bool OWN_NV, bool HILO, bool BY_UNIT>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
                 const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -598,10 +612,9 @@ tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 if (unit != qo_unit) {
                     if (!mbar_wait(bar(BAR_QO_EMPTY), (qo_loads & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
                     mbar_expect_tx(bar(BAR_QO_FULL), qo_bytes);
-                    const int qrow = (b * p.Hkv * p.G + g * p.G) * p.W;
                     const int orow = unit * p.rows_out * (HILO ? 2 : 1);
-                    tma_load_2d(sbase + OFF_Q, &map_q, bar(BAR_QO_FULL), 0, qrow);
-                    tma_load_2d(sbase + OFF_Q + kHalfBytes, &map_q, bar(BAR_QO_FULL), 64, qrow);
+                    load_q<BY_UNIT>(sbase + OFF_Q, &map_q, bar(BAR_QO_FULL), 0, 0, unit, p.R);
+                    load_q<BY_UNIT>(sbase + OFF_Q + kHalfBytes, &map_q, bar(BAR_QO_FULL), 64, 0, unit, p.R);
                     tma_load_2d(sbase + OFF_O, &map_o, bar(BAR_QO_FULL), 0, orow);
                     tma_load_2d(sbase + OFF_O + kHalfBytes, &map_o, bar(BAR_QO_FULL), 64, orow);
                     qo_unit = unit; ++qo_loads;
@@ -810,7 +823,7 @@ constexpr uint32_t kSmemMulti = MC_OFF_TMEM + 16 + 1024;
 
 // SPLIT: the general walk (row chunks of a pair shared by several CTAs, hidden tile pairs skipped); without
 // it every CTA takes whole pairs and every chunk, which is all a short window over a long cache needs.
-template <unsigned VARS, bool SPLIT>
+template <unsigned VARS, bool SPLIT, bool BY_UNIT>
 __global__ void __launch_bounds__(kThreadsMulti, 1)
 tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
                       const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
@@ -881,11 +894,10 @@ tc_pass2_multi_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_co
                     const uint32_t qb = citem & 1;
                     if (!mbar_wait(bar(MC_QO_EMPTY + qb), ((citem >> 1) & 1) ^ 1)) { failed = true; fail_site = __LINE__; break; }
                     mbar_expect_tx(bar(MC_QO_FULL + qb), qo_bytes);
-                    const int qrow = (b * p.Hkv * p.G + g * p.G) * p.W + c * MC_ROWS;
                     const int orow = unit * p.rows_out + c * MC_ROWS;
                     const uint32_t dq = sbase + MC_OFF_QO + qb * kQoBuf, dob = dq + 2 * kHalfB64;
-                    tma_load_2d(dq, &map_q, bar(MC_QO_FULL + qb), 0, qrow);
-                    tma_load_2d(dq + kHalfB64, &map_q, bar(MC_QO_FULL + qb), 64, qrow);
+                    load_q<BY_UNIT>(dq, &map_q, bar(MC_QO_FULL + qb), 0, c * MC_ROWS, unit, p.R);
+                    load_q<BY_UNIT>(dq + kHalfB64, &map_q, bar(MC_QO_FULL + qb), 64, c * MC_ROWS, unit, p.R);
                     tma_load_2d(dob, &map_o, bar(MC_QO_FULL + qb), 0, orow);
                     tma_load_2d(dob + kHalfB64, &map_o, bar(MC_QO_FULL + qb), 64, orow);
                     ++citem;
@@ -1938,13 +1950,19 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     const long long n_tiles = (long long)units * ((s.Nmax + TILE - 1) / TILE);
     const int grid = (int)(n_tiles < sm_count() ? n_tiles : sm_count());
 
+    // the queries of pass 2, by unit where its rows do not fill their last chunk (see load_q)
+    const bool by_unit = s.R % (ch.n_chunks > 1 ? MC_ROWS : ch.chunk_rows) != 0;
+    auto map_queries = [&](CUtensorMap* m, int rows) {
+        const uint64_t rows_of_all[2] = {(uint64_t)kD, (uint64_t)units * s.R}, per_unit[3] = {(uint64_t)kD, (uint64_t)s.R, (uint64_t)units};
+        const uint64_t strides[2] = {(uint64_t)q.st * 2, (uint64_t)s.R * q.st * 2};
+        return make_map(m, q.ptr, by_unit ? 3 : 2, by_unit ? per_unit : rows_of_all, strides, (uint32_t)rows);
+    };
+    auto flag = [](bool f, auto g) { return f ? g(std::true_type{}) : g(std::false_type{}); };
     if (ch.n_chunks > 1) {                               // more than 128 window rows: chunks of 64, K/V tile kept
         CUtensorMap mq64, mo64;
-        const uint64_t qd[2] = {(uint64_t)kD, (uint64_t)s.B * s.Hq * s.W};
-        const uint64_t qs[1] = {(uint64_t)q.st * 2};
         const uint64_t od[2] = {(uint64_t)kD, (uint64_t)units * ch.rows_out};
         const uint64_t os[1] = {(uint64_t)kD * 2};
-        if (!make_map(&mq64, q.ptr, 2, qd, qs, MC_ROWS) || !make_map(&mo64, wsb + plan.off_obf, 2, od, os, MC_ROWS)) {
+        if (!map_queries(&mq64, MC_ROWS) || !make_map(&mo64, wsb + plan.off_obf, 2, od, os, MC_ROWS)) {
             set_last_cuda_error((int)cudaErrorInvalidValue);
             return OBC_ERR_CUDA;
         }
@@ -1966,11 +1984,11 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
             return OBC_OK;
         };
         const bool split = p.csplit > 1 || (s.causal && s.W > MC_ROWS);
-        if (s.variants == OBC_VAR_VK)
-            return split ? launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, true>) : launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, false>);
-        if (!(s.variants & ~kObcVariants))
-            return split ? launch_multi(tc_pass2_multi_kernel<kObcVariants, true>) : launch_multi(tc_pass2_multi_kernel<kObcVariants, false>);
-        return split ? launch_multi(tc_pass2_multi_kernel<kAllVariants, true>) : launch_multi(tc_pass2_multi_kernel<kAllVariants, false>);
+        return flag(split, [&](auto sp) { return flag(by_unit, [&](auto bu) {
+            if (s.variants == OBC_VAR_VK) return launch_multi(tc_pass2_multi_kernel<OBC_VAR_VK, sp.value, bu.value>);
+            if (!(s.variants & ~kObcVariants)) return launch_multi(tc_pass2_multi_kernel<kObcVariants, sp.value, bu.value>);
+            return launch_multi(tc_pass2_multi_kernel<kAllVariants, sp.value, bu.value>);
+        }); });
     }
 
     auto launch = [&](auto kernel) -> obc_status {
@@ -1980,16 +1998,12 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     };
     // pass 1 leaves only ||v||^2; without it, and for the l1 variant, the norms come from the V tiles in pass 2
     const bool own_nv = given || (s.variants & OBC_VAR_VATP);
-    if (s.variants == OBC_VAR_VK) {
-        if (hilo) return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, true>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, true>);
-        return own_nv ? launch(tc_pass2_kernel<OBC_VAR_VK, true, false>) : launch(tc_pass2_kernel<OBC_VAR_VK, false, false>);
-    }
-    if (!(s.variants & ~kObcVariants)) {
-        if (hilo) return own_nv ? launch(tc_pass2_kernel<kObcVariants, true, true>) : launch(tc_pass2_kernel<kObcVariants, false, true>);
-        return own_nv ? launch(tc_pass2_kernel<kObcVariants, true, false>) : launch(tc_pass2_kernel<kObcVariants, false, false>);
-    }
-    if (hilo) return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, true>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, true>);
-    return own_nv ? launch(tc_pass2_kernel<kAllVariants, true, false>) : launch(tc_pass2_kernel<kAllVariants & ~OBC_VAR_VATP, false, false>);
+    if (by_unit && !map_queries(&mq, ch.chunk_rows)) { set_last_cuda_error((int)cudaErrorInvalidValue); return OBC_ERR_CUDA; }
+    return flag(own_nv, [&](auto own) { return flag(hilo, [&](auto hl) { return flag(by_unit, [&](auto bu) {
+        if (s.variants == OBC_VAR_VK) return launch(tc_pass2_kernel<OBC_VAR_VK, own.value, hl.value, bu.value>);
+        if (!(s.variants & ~kObcVariants)) return launch(tc_pass2_kernel<kObcVariants, own.value, hl.value, bu.value>);
+        return launch(tc_pass2_kernel<own.value ? kAllVariants : kAllVariants & ~OBC_VAR_VATP, own.value, hl.value, bu.value>);
+    }); }); });
 }
 
 }  // namespace obc

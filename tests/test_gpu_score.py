@@ -233,3 +233,18 @@ def test_joint_score_near_its_zero(Hq, Hkv, W):
     assert all(np.array_equal(g, got[0]) or np.abs(g / got[0] - 1).max() < 1e-6 for g in got)
     own = np.abs(got[0] / want - 1)
     assert own.max() < 2e-5, own.max()
+
+
+@pytest.mark.parametrize("Hq,Hkv,W,N", [(4, 2, 20, 300), (2, 2, 5, 700), (6, 2, 24, 500), (6, 2, 70, 400)])
+def test_queries_of_a_neighbour_that_are_not_finite(Hq, Hkv, W, N):
+    """Row counts that do not fill the MMA's rows (R = 40, 5, 72 and 210): what fills them up must not be the queries of the
+    next head or sequence, which may be anything (a masked batch item, say)."""
+    case = synth.make_prefill("neighbour", B=2, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=N, hh_frac=0.02)
+    q, k, v = H.upload(case)
+    variants = ["V", "K", "VK", "ATTN"]
+    clean = api.obc_score(q, k, v, variants=variants)
+    for bad in (float("nan"), float("inf")):
+        q2 = q.clone()
+        q2[1] = bad
+        q2[0, Hq // Hkv:] = bad
+        assert torch.equal(api.obc_score(q2, k, v, variants=variants)[:, 0, 0], clean[:, 0, 0])
