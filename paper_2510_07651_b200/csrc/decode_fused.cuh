@@ -115,7 +115,11 @@ decode_fused_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_cons
     }
     copy_failed |= !chunk_wait(&sBar[1], 0);
     if (owns_new && tid >= 16 && tid < 32) sV[staged_piece<N>(next - c0, tid & 15)] = new_row;
-    if (c0 + N > hi)                                       // rows past the live extent may hold anything, and 0 x NaN would spoil the outputs
+    // rows without a live token may hold anything, and 0 x NaN would spoil the outputs: freed slots one by one, those past the
+    // live extent together
+    if (!live && slot < hi)
+        for (int i = 0; i < 16; ++i) sV[staged_piece<N>(tid, i)] = make_uint4(0, 0, 0, 0);
+    if (c0 + N > hi)
         for (int i = tid; i < N * 16; i += N) if (c0 + (i >> 4) >= hi) sV[staged_piece<N>(i >> 4, i & 15)] = make_uint4(0, 0, 0, 0);
     __syncthreads();
 

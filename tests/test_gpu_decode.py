@@ -128,3 +128,33 @@ def test_decode_caches_that_are_views_of_larger_buffers():
     last chunk's rows beyond it must read as zeros although the memory behind them holds NaN."""
     assert _run(B=2, Hq=8, Hkv=2, n0=300, budget=280, cap=333, n_sink=4, n_recent=8, steps=6, strided=True) > 0
 
+
+
+@pytest.mark.parametrize("cap,dead", [
+    (400, (128, 256)),                    # a whole chunk of 128 slots without a live one
+    (3000, (0, 200)), (3000, (512, 768)), # part of a chunk of 256, and a whole one
+    (300, (40, 41)),                      # a single freed slot
+])
+def test_decode_free_slots_may_hold_anything(cap, dead):
+    """Free slots below the highest slot ever used (pos = -1) hold NaN in one cache and zeros in the other: the same step."""
+    g = torch.Generator(device="cuda").manual_seed(cap)
+    k = torch.randn((2, 2, cap, 128), generator=g, device="cuda").bfloat16()
+    v = torch.randn((2, 2, cap, 128), generator=g, device="cuda").bfloat16()
+    q_t = torch.randn((2, 8, 1, 128), generator=g, device="cuda").bfloat16()
+    k_t, v_t = (torch.randn((2, 2, 1, 128), generator=g, device="cuda").bfloat16() for _ in range(2))
+    results = []
+    for fill in (0.0, float("nan")):
+        kc, vc = k.clone(), v.clone()
+        kc[:, :, dead[0]:dead[1]] = fill
+        vc[:, :, dead[0]:dead[1]] = fill
+        pos = torch.arange(cap, dtype=torch.int32, device="cuda").repeat(2, 2, 1)
+        pos[:, :, dead[0]:dead[1]] = -1
+        pos[:, :, cap - 1] = -1
+        live = cap - 1 - (dead[1] - dead[0])
+        state = torch.zeros((2, 2, 4), dtype=torch.int32, device="cuda")
+        state[..., 0] = live; state[..., 1] = cap - 1; state[..., 2] = cap - 1
+        acc = torch.zeros((2, 2, cap), device="cuda")
+        api.obc_decode_step(q_t, k_t, v_t, kc, vc, acc, pos, state, cap + 5, budget=live, n_sink=2, n_recent=16)
+        results.append((acc, pos, state))
+    assert torch.isfinite(results[1][0]).all()
+    assert all(torch.equal(x, y) for x, y in zip(*results))
