@@ -894,13 +894,16 @@ size_t select_workspace_bytes(int B, int Hkv, int Nmax) { return align_up((size_
 // eight, 7.2 with sixteen; of 32768: 8.6 / 8.0).  Above 8192 candidates an SM holds one CTA only: such shares are split
 // further whatever runs side by side (256 heads of 32768: 60 us with two CTAs, 56 with four; 16 heads of 65536: 16.1 with
 // four, 14.9 with eight; of 131072: 36 with eight, 32 with sixteen; 128 heads of 131072: 163 / 172).
-static int select_cluster_size(int units, int Nmax, int* seg_cap) {
+// A pooling kernel so wide that a share and its halo do not fit takes smaller shares.
+static size_t select_cluster_smem(int seg, int pool_kernel) { return sizeof(ClusterShared) + (size_t)seg * 8 + (size_t)pool_kernel * 4 + 32; }
+static int select_cluster_size(int units, int Nmax, int pool_kernel, int* seg_cap) {
+    constexpr size_t kMost = 227 * 1024;                       // dynamic shared memory of a CTA
     auto seg_of = [&](int C) { return ((Nmax + C - 1) / C + 31) / 32 * 32; };
     auto side_by_side = [](int C) { return C == 2 ? 74 : C == 4 ? 33 : C == 8 ? 15 : 7; };     // clusters, one CTA per SM
     int C = 1;
     if (Nmax > 4096)
         while (C < 16 && (units <= side_by_side(2 * C) ? C < 8 || seg_of(C) > 2048 : seg_of(C) > 8192 && (C < 8 || units <= 32))) C *= 2;
-    while (C < 16 && seg_of(C) > CL_MAX_SEG) C *= 2;
+    while (C < 16 && (seg_of(C) > CL_MAX_SEG || select_cluster_smem(seg_of(C), pool_kernel) > kMost)) C *= 2;
     if (seg_of(C) > CL_MAX_SEG) return 0;
     *seg_cap = seg_of(C);
     return C;
@@ -917,9 +920,9 @@ static obc_status launch_select_impl(const SelectShape& s, const float* scores, 
                                      void* ws, cudaStream_t stream) {
     const int units = s.B * s.Hkv;
     int seg_cap = 0;
-    const int C = select_cluster_size(units, s.Nmax, &seg_cap);
+    const int C = select_cluster_size(units, s.Nmax, s.pool_kernel, &seg_cap);
     if (C > 0) {
-        const size_t smem = sizeof(ClusterShared) + (size_t)seg_cap * 8 + (size_t)s.pool_kernel * 4 + 32;
+        const size_t smem = select_cluster_smem(seg_cap, s.pool_kernel);
         const bool adaptive = keys_in != nullptr;
         const auto kernel = adaptive ? select_cluster_kernel<true> : select_cluster_kernel<false>;
         OBC_CUDA_TRY(allow_smem(kernel, smem));

@@ -3,6 +3,7 @@ same fp32 scores."""
 import numpy as np
 import pytest
 import torch
+from scipy.ndimage import maximum_filter1d
 
 from oracle import reference as ref
 from paper_2510_07651_b200 import api, synth
@@ -98,6 +99,17 @@ def test_select_every_pool_width_at_ragged_ends(pool, kern, N):
     scores = rng.random((1, 2, N), dtype=np.float32)
     got, want = _select_both(scores, [N], [N // 3 + 3], 1, 2, pool, kern)
     assert np.array_equal(got.cpu().numpy(), want)
+
+
+def test_select_pool_kernel_that_takes_much_shared_memory():
+    # 33 heads of 131072 would get eight CTAs each, whose shares leave no room for the halo of such a kernel
+    N, kern, budget = 131072, 20001, 300
+    rng = np.random.default_rng(3)
+    scores = rng.random((1, 33, N), dtype=np.float32)
+    pooled = maximum_filter1d(scores, kern, axis=-1, mode="constant", cval=-np.inf)
+    want = ref.select_pipeline(pooled, [N], [budget], 0, 0, "none", 1, budget)
+    idx = api.obc_select(torch.from_numpy(scores).cuda(), budget=budget, pool="max", pool_kernel=kern)
+    assert np.array_equal(idx.cpu().numpy(), want)
 
 
 def test_select_ragged_lengths_and_per_sequence_budgets():
