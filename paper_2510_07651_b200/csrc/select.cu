@@ -598,27 +598,28 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
         }
         __syncthreads();
         cluster.barrier_arrive();                      // this CTA's histograms are clear: others may add to them after their wait
-        // four candidates per thread and step; the top 11 bits of their keys go straight into the first histogram
-        for (int i = tid * 4; i < m; i += CL_NT * 4) {
-            float4 v;
-            if (half <= 3) {
-                v = pool4_staged(stage + i, half, s.pool_mode, s.pool_kernel);
-            } else {
-                float* out = reinterpret_cast<float*>(&v);
-                for (int j = 0; j < 4; ++j) {
-                    const float* at = stage + min(i + j, m - 1);
-                    float val = s.pool_mode == OBC_POOL_MAX ? -INFINITY : 0.f;
-                    if (s.pool_mode == OBC_POOL_MAX) for (int t = 0; t <= 2 * half; ++t) val = fmaxf(val, at[t]);
-                    else for (int t = 0; t <= 2 * half; ++t) val = __fadd_rn(val, at[t]);
-                    out[j] = s.pool_mode == OBC_POOL_MAX ? val : __fdiv_rn(val, (float)s.pool_kernel);
-                }
+        // the top 11 bits of the keys go straight into the first histogram
+        if (half <= 3) {                               // four candidates per thread and step
+            for (int i = tid * 4; i < m; i += CL_NT * 4) {
+                const float4 v = pool4_staged(stage + i, half, s.pool_mode, s.pool_kernel);
+                const uint4 k4 = make_uint4(float_key(v.x), float_key(v.y), float_key(v.z), float_key(v.w));
+                *reinterpret_cast<uint4*>(keys + i) = k4;  // (a share has room for a multiple of 32 keys)
+                atomicAdd(&sh.local[k4.x >> 21], 1u);
+                if (i + 1 < m) atomicAdd(&sh.local[k4.y >> 21], 1u);
+                if (i + 2 < m) atomicAdd(&sh.local[k4.z >> 21], 1u);
+                if (i + 3 < m) atomicAdd(&sh.local[k4.w >> 21], 1u);
             }
-            const uint4 k4 = make_uint4(float_key(v.x), float_key(v.y), float_key(v.z), float_key(v.w));
-            *reinterpret_cast<uint4*>(keys + i) = k4;      // (a share has room for a multiple of 32 keys)
-            atomicAdd(&sh.local[k4.x >> 21], 1u);
-            if (i + 1 < m) atomicAdd(&sh.local[k4.y >> 21], 1u);
-            if (i + 2 < m) atomicAdd(&sh.local[k4.z >> 21], 1u);
-            if (i + 3 < m) atomicAdd(&sh.local[k4.w >> 21], 1u);
+        } else {                                       // one, so that the lanes of a warp read consecutive taps: 64 heads of
+                                                       // 65536, kernels of 9 / 31 / 101 taps: 35 / 47 / 85 us, against 47 / 96 / 250
+                                                       // with four consecutive candidates per thread (four-way bank conflicts)
+            for (int i = tid; i < m; i += CL_NT) {
+                float val = s.pool_mode == OBC_POOL_MAX ? -INFINITY : 0.f;
+                if (s.pool_mode == OBC_POOL_MAX) for (int t = 0; t <= 2 * half; ++t) val = fmaxf(val, stage[i + t]);
+                else for (int t = 0; t <= 2 * half; ++t) val = __fadd_rn(val, stage[i + t]);
+                const uint32_t key = float_key(s.pool_mode == OBC_POOL_MAX ? val : __fdiv_rn(val, (float)s.pool_kernel));
+                keys[i] = key;
+                atomicAdd(&sh.local[key >> 21], 1u);
+            }
         }
     }
     __syncthreads();                               // keys and this CTA's histogram of their top bits are complete
