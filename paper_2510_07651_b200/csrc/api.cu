@@ -12,6 +12,16 @@ namespace obc {
 static thread_local int g_last_cuda_error = 0;
 void set_last_cuda_error(int e) { g_last_cuda_error = e; }
 
+// (a size query may run where there is no device: the plans are then those of a B200)
+int sm_count() {
+    static int n = 0;
+    if (!n) {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 148;
+    }
+    return n;
+}
+
 // ---- optional per-kernel event timing ---------------------------------------------------------
 namespace {
 struct ProfRec { const char* name; cudaEvent_t e0, e1; };

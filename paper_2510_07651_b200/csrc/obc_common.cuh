@@ -28,6 +28,8 @@ struct ProfScope {
     int slot; cudaStream_t stream;
 };
 
+int sm_count();                          // SMs of the device
+
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // ---- internal launch descriptions (plain structs, passed by value to kernels) ---------------

@@ -582,7 +582,7 @@ obc_status launch_pass2_typed(const ScoreShape& s, const SimtPlan& plan, TensorV
 SimtPlan make_simt_plan(const ScoreShape& s, int rows_out, bool want_obf) {
     SimtPlan p{};
     const long long units = (long long)s.B * s.Hkv;
-    const long long slots = 148 * 2;                       // two resident CTAs per SM
+    const long long slots = 2LL * sm_count();              // two resident CTAs per SM
     const bool small = units * ((s.Nmax + 63) / 64) * ((s.R + 31) / 32) < slots;
     const int tn = small ? 32 : 64, rc = small && s.R <= 16 ? 16 : 32;
     const long long chunks = (s.R + rc - 1) / rc;

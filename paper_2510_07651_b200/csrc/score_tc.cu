@@ -1775,15 +1775,6 @@ size_t l2_bytes() {
     return n;
 }
 
-int sm_count() {
-    static int n = 0;
-    if (!n) {
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) n = 148;
-    }
-    return n;
-}
-
 }  // namespace
 
 // Fewer than 64 window rows fill half of the MMA's M dimension at most.  Pass 1 then runs every row twice, the second

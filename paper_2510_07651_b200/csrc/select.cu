@@ -897,13 +897,39 @@ size_t select_workspace_bytes(int B, int Hkv, int Nmax) { return align_up((size_
 // four, 14.9 with eight; of 131072: 36 with eight, 32 with sixteen; 128 heads of 131072: 163 / 172).
 // A pooling kernel so wide that a share and its halo do not fit takes smaller shares.
 static size_t select_cluster_smem(int seg, int pool_kernel) { return sizeof(ClusterShared) + (size_t)seg * 8 + (size_t)pool_kernel * 4 + 32; }
+
+// Clusters of C CTAs, one per SM, that the current device runs at once (74 / 33 / 15 / 7 of 2 / 4 / 8 / 16 on 148 SMs), asked once
+// per host thread and device.
+static int clusters_side_by_side(int C) {
+    thread_local int seen_dev = -1, seen[17];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev != seen_dev) { for (int& x : seen) x = -1; seen_dev = dev; }
+    if (seen[C] < 0) {
+        const auto kernel = select_cluster_kernel<false>;
+        int n = 0, optin = 0;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)C); cfg.blockDim = dim3(CL_NT); cfg.attrs = attr; cfg.numAttrs = 1;
+        if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess) {
+            cfg.dynamicSmemBytes = (size_t)optin;              // all of it (the kernel has no static part): one CTA per SM
+            if (allow_smem(kernel, cfg.dynamicSmemBytes) != cudaSuccess ||
+                cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
+        }
+        seen[C] = n;
+    }
+    return seen[C];
+}
+
 static int select_cluster_size(int units, int Nmax, int pool_kernel, int* seg_cap) {
     constexpr size_t kMost = 227 * 1024;                       // dynamic shared memory of a CTA
     auto seg_of = [&](int C) { return ((Nmax + C - 1) / C + 31) / 32 * 32; };
-    auto side_by_side = [](int C) { return C == 2 ? 74 : C == 4 ? 33 : C == 8 ? 15 : 7; };     // clusters, one CTA per SM
     int C = 1;
     if (Nmax > 4096)
-        while (C < 16 && (units <= side_by_side(2 * C) ? C < 8 || seg_of(C) > 2048 : seg_of(C) > 8192 && (C < 8 || units <= 32))) C *= 2;
+        while (C < 16 && (units <= clusters_side_by_side(2 * C) ? C < 8 || seg_of(C) > 2048 : seg_of(C) > 8192 && (C < 8 || units <= 32))) C *= 2;
     while (C < 16 && (seg_of(C) > CL_MAX_SEG || select_cluster_smem(seg_of(C), pool_kernel) > kMost)) C *= 2;
     if (seg_of(C) > CL_MAX_SEG) return 0;
     *seg_cap = seg_of(C);
@@ -1035,7 +1061,7 @@ obc_status launch_select_adaptive(const SelectShape& s, int n_safe, const float*
     char* w = (char*)ws;
     uint32_t* keys = (uint32_t*)(w + plan.off_keys);
     // about two CTAs per SM: each of them repeats the search through the heads' histograms
-    const long long per = ((long long)units * s.Nmax + 2 * 148 - 1) / (2 * 148);
+    const long long ctas = 2LL * sm_count(), per = ((long long)units * s.Nmax + ctas - 1) / ctas;
     const int chunk = (int)(per < 2048 ? 2048 : (per + AD_NT - 1) / AD_NT * AD_NT);
     const AdaptiveLevels lv{(uint32_t*)(w + plan.off_hist), (uint32_t*)(w + plan.off_above), (uint32_t*)(w + plan.off_digit), counts,
                             (uint32_t)n_safe, chunk, units};
