@@ -59,11 +59,31 @@ def test_ragged_batch_and_odd_tile_counts():
     _check(case, ["V", "K", "VK", "ATTN", "VATP"], tight=2e-2)
 
 
+@pytest.mark.parametrize("path", ["simt", "auto"])
 @pytest.mark.parametrize("causal", [True, False])
-def test_small_shapes_cuda_core_path(causal):
+def test_small_shapes(causal, path):
     case = synth.make_prefill("given-small", B=2, Hq=6, Hkv=2, d=128, W=5, N=[77, 300], dtype="bf16", seed=213,
-                              hh_frac=0.05)                                # R = 15: CUDA-core kernels
-    _check(case, ["V", "K", "VK", "ATTN", "VATP"], causal=causal, tight=2e-2)
+                              hh_frac=0.05)                # R = 15: on CUDA cores, and with -2 O in two bf16 parts on tensor cores
+    _check(case, ["V", "K", "VK", "ATTN", "VATP"], causal=causal, path=path, tight=2e-2)
+
+
+@pytest.mark.parametrize("path", ["simt", "auto"])
+@pytest.mark.parametrize("Hq,Hkv,W,N", [(6, 2, 5, 300), (1, 1, 63, 2000), (32, 32, 32, 900)])
+def test_fewer_than_64_rows_keep_fp32_outputs(Hq, Hkv, W, N, path):
+    """fp32 O beside a bf16 cache: both bf16 parts of -2 O count.  Without the low part the error is 2^-9 of the cross term; with
+    it, and with fp32 sums, the scores hold the tolerance of fp32 caches."""
+    from oracle import reference as ref
+    case = synth.make_prefill("given-f32o", B=1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=217 + N, hh_frac=0.02)
+    out = ref.score(case.q, case.k, case.v, want=("ATTN",), return_attention=True)
+    o = (out["O"].reshape(1, Hq, W, 128) * 3.0).astype(np.float32)            # large enough for the cross term to count
+    lse = (out["m"] + np.log(out["l"])).reshape(1, Hq, W).astype(np.float32)
+    variants = ["V", "K", "VK", "ATTN"]
+    want = ref.score(case.q, case.k, case.v, want=variants, given=(o, lse))
+    q, k, v = H.upload(case)
+    got = api.obc_score_given(q, k, v, torch.from_numpy(o).cuda(), torch.from_numpy(lse).cuda(), variants=variants, path=path).cpu().numpy()
+    mx = max(np.abs(want[n]).max() for n in ("V", "K", "VK"))
+    for n, g in zip(variants, got):
+        H.assert_scores_close(g, want[n], "f32", what=f"{case.name}/{n}/{path}", mx=None if n == "ATTN" else mx)
 
 
 def test_output_dtype_may_differ_from_the_cache():

@@ -120,6 +120,10 @@ def test_one_cta_per_head_and_chunk(N, W, Hq, Hkv):
     # pass 1 writes the merged rows itself, padding rows included: R = 40 (two bf16 parts), 40, 10, 64 and 150 (two chunks)
     case = synth.make_prefill("direct", B=1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=N + W, hh_frac=0.02)
     _check(case, ["K", "VK"], tight=2e-2)
+    if Hq // Hkv * W < 64:                   # both parts of -2 O: the tolerance of 32-bit sums (see test_fewer_than_64_window_rows)
+        want, got = H.oracle_scores(case, ["K", "VK"]), H.gpu_scores(case, ["K", "VK"])
+        for n in ("K", "VK"):
+            H.assert_scores_close(got[n], want[n], "f32", what=f"{case.name}/{n}", mx=np.abs(want["VK"]).max())
 
 
 @pytest.mark.parametrize("N,W,Hq,Hkv,lens", [
@@ -248,3 +252,15 @@ def test_queries_of_a_neighbour_that_are_not_finite(Hq, Hkv, W, N):
         q2[1] = bad
         q2[0, Hq // Hkv:] = bad
         assert torch.equal(api.obc_score(q2, k, v, variants=variants)[:, 0, 0], clean[:, 0, 0])
+
+
+@pytest.mark.parametrize("N,Hq,Hkv", [(1500, 32, 32), (800, 64, 64)])
+def test_fewer_than_64_window_rows_on_many_heads(N, Hq, Hkv):
+    # 1024 and 2048 rows of 32 per head: the merge of the splits takes a warp per row (four splits, two), with both parts of -2 O
+    case = synth.make_prefill("fewmany", B=1, Hq=Hq, Hkv=Hkv, d=128, W=32, N=N, dtype="bf16", seed=N, hh_frac=0.02)
+    case.v, case.v_bits = synth.bf16_round(case.v + 1.0)          # outputs near one in every channel: the cross term weighs more
+    for variants in (["VK"], ["V", "K", "VK", "ATTN", "VATP"]):
+        want, got = H.oracle_scores(case, variants), H.gpu_scores(case, variants)
+        mx = max(np.abs(want[n]).max() for n in variants if n in ("V", "K", "VK"))
+        for n in variants:
+            H.assert_scores_close(got[n], want[n], "f32", what=f"{case.name}/{n}", mx=None if n in ("ATTN", "VATP") else mx)
