@@ -58,7 +58,8 @@ enum { OBC_POOL_NONE = 0, OBC_POOL_AVG = 1, OBC_POOL_MAX = 2 };
 
 /* kernel family used by obc_score */
 enum {
-    OBC_PATH_AUTO = 0,  /* tensor-core kernels when dtype is bf16 (R < 64: with attention weights and outputs in two bf16 parts) */
+    OBC_PATH_AUTO = 0,  /* tensor-core kernels when dtype is bf16 (R < 64: with attention weights and outputs in two bf16 parts,
+                           and obc_window_attention, whose outputs are themselves the result, on CUDA cores) */
     OBC_PATH_SIMT = 1,  /* CUDA-core fp32-FMA kernels (any dtype, any R) */
     OBC_PATH_TC = 2     /* tcgen05 kernels; OBC_ERR_UNSUPPORTED unless the dtype is bf16 and R >= 64 */
 };

@@ -160,8 +160,8 @@ obc_status obc_window_attention(const obc_score_params* p, obc_tensor q, obc_ten
     if (((uintptr_t)workspace & 255) != 0) return OBC_ERR_ALIGN;
     // Fewer than 64 rows on tensor cores carry the attention weights in two bf16 parts.  That is enough for the scores, in which
     // it drowns among the sums' own errors, but here O itself is the fp32 result: 2.0e-6 of its norm off against 2.2e-7 to
-    // 4.6e-7 on CUDA cores, which such calls therefore take (32 heads
-    // of 8191 tokens x 32 rows: 177 us, 39 on tensor cores; 8 heads of 4096 x 32: 29 either way).
+    // 4.6e-7 on CUDA cores, which such calls therefore take (32 heads of 8191 tokens x 32 rows: 177 us, 39 on tensor cores; 8 heads
+    // of 4096 x 32: 29 either way).
     const bool tc = s.R >= 64 && want_tc(p, s, q.dtype, view(q));
     if (p->path == OBC_PATH_TC && !tc) return OBC_ERR_UNSUPPORTED;
     SimtPlan plan;

@@ -529,7 +529,10 @@ __device__ __forceinline__ void score_chunk(uint32_t zt, uint32_t tt, int chunk_
 // caller supplied the attention outputs), so warps 2-3 compute the value norms from the V tiles here.
 // HILO: fewer than 64 window rows.  Such a call is summed in 32 bits throughout: -2 O enters as the sum of two bf16
 // parts, which stand side by side on the MMA's N dimension (at most 2 x 64 rows) and meet in the epilogue.  The
-// kernel stays bound by the K/V tiles it streams, with half of the epilogue's rows idle.
+// kernel stays bound by the K/V tiles it streams, with half of the epilogue's rows idle.  Scores against 64 bits, thirteen
+// shapes of 1 to 63 rows: 0.9e-6 of the norm and 2.6e-6 of the largest, as on CUDA cores.  (The parts leave out 2^-17 of
+// O, which shows where |v - o|^2 is a small difference of large terms: 3 rows x 64 tokens with logits of up to 10, 3.7e-6 of the norm
+// against 1.2e-6.  A third part, 192 columns of T', brought that to 1.9e-6 and cost calls of 63 rows 3 to 6 %.)
 template <unsigned VARS, bool OWN_NV, bool HILO, bool BY_UNIT>
 __global__ void __launch_bounds__(kThreads, 1)
 tc_pass2_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_o,
