@@ -598,28 +598,28 @@ select_cluster_kernel(SelectShape s, const float* __restrict__ scores, int32_t* 
         }
         __syncthreads();
         cluster.barrier_arrive();                      // this CTA's histograms are clear: others may add to them after their wait
-        // the top 11 bits of the keys go straight into the first histogram
-        if (half <= 3) {                               // four candidates per thread and step
-            for (int i = tid * 4; i < m; i += CL_NT * 4) {
-                const float4 v = pool4_staged(stage + i, half, s.pool_mode, s.pool_kernel);
-                const uint4 k4 = make_uint4(float_key(v.x), float_key(v.y), float_key(v.z), float_key(v.w));
-                *reinterpret_cast<uint4*>(keys + i) = k4;  // (a share has room for a multiple of 32 keys)
-                atomicAdd(&sh.local[k4.x >> 21], 1u);
-                if (i + 1 < m) atomicAdd(&sh.local[k4.y >> 21], 1u);
-                if (i + 2 < m) atomicAdd(&sh.local[k4.z >> 21], 1u);
-                if (i + 3 < m) atomicAdd(&sh.local[k4.w >> 21], 1u);
-            }
-        } else {                                       // one, so that the lanes of a warp read consecutive taps: 64 heads of
-                                                       // 65536, kernels of 9 / 31 / 101 taps: 35 / 47 / 85 us, against 47 / 96 / 250
-                                                       // with four consecutive candidates per thread (four-way bank conflicts)
+        // wide kernels beforehand, one candidate per thread and step, so that the lanes of a warp read consecutive taps: 64 heads of
+        // 65536, 9 / 31 / 101 taps: 36 / 47 / 87 us, against 47 / 97 / 250 with four consecutive candidates per thread (four-way bank
+        // conflicts).  (Keys and histogram in the same loop made narrow kernels 0.1 to 0.3 us slower.)
+        if (half > 3) {
+            float* pooled = reinterpret_cast<float*>(keys);
             for (int i = tid; i < m; i += CL_NT) {
-                float val = s.pool_mode == OBC_POOL_MAX ? -INFINITY : 0.f;
+                float val = pad;
                 if (s.pool_mode == OBC_POOL_MAX) for (int t = 0; t <= 2 * half; ++t) val = fmaxf(val, stage[i + t]);
                 else for (int t = 0; t <= 2 * half; ++t) val = __fadd_rn(val, stage[i + t]);
-                const uint32_t key = float_key(s.pool_mode == OBC_POOL_MAX ? val : __fdiv_rn(val, (float)s.pool_kernel));
-                keys[i] = key;
-                atomicAdd(&sh.local[key >> 21], 1u);
+                pooled[i] = s.pool_mode == OBC_POOL_MAX ? val : __fdiv_rn(val, (float)s.pool_kernel);
             }
+            __syncthreads();
+        }
+        // four candidates per thread and step; the top 11 bits of their keys go straight into the first histogram
+        for (int i = tid * 4; i < m; i += CL_NT * 4) {
+            const float4 v = half <= 3 ? pool4_staged(stage + i, half, s.pool_mode, s.pool_kernel) : *reinterpret_cast<const float4*>(keys + i);
+            const uint4 k4 = make_uint4(float_key(v.x), float_key(v.y), float_key(v.z), float_key(v.w));
+            *reinterpret_cast<uint4*>(keys + i) = k4;      // (a share has room for a multiple of 32 keys)
+            atomicAdd(&sh.local[k4.x >> 21], 1u);
+            if (i + 1 < m) atomicAdd(&sh.local[k4.y >> 21], 1u);
+            if (i + 2 < m) atomicAdd(&sh.local[k4.z >> 21], 1u);
+            if (i + 3 < m) atomicAdd(&sh.local[k4.w >> 21], 1u);
         }
     }
     __syncthreads();                               // keys and this CTA's histogram of their top bits are complete
@@ -898,38 +898,41 @@ size_t select_workspace_bytes(int B, int Hkv, int Nmax) { return align_up((size_
 // A pooling kernel so wide that a share and its halo do not fit takes smaller shares.
 static size_t select_cluster_smem(int seg, int pool_kernel) { return sizeof(ClusterShared) + (size_t)seg * 8 + (size_t)pool_kernel * 4 + 32; }
 
-// Clusters of C CTAs, one per SM, that the current device runs at once (74 / 33 / 15 / 7 of 2 / 4 / 8 / 16 on 148 SMs), asked once
-// per host thread and device.
-static int clusters_side_by_side(int C) {
-    thread_local int seen_dev = -1, seen[17];
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (dev != seen_dev) { for (int& x : seen) x = -1; seen_dev = dev; }
-    if (seen[C] < 0) {
-        const auto kernel = select_cluster_kernel<false>;
-        int n = 0, optin = 0;
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.gridDim = dim3((unsigned)C); cfg.blockDim = dim3(CL_NT); cfg.attrs = attr; cfg.numAttrs = 1;
-        if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess) {
-            cfg.dynamicSmemBytes = (size_t)optin;              // all of it (the kernel has no static part): one CTA per SM
-            if (allow_smem(kernel, cfg.dynamicSmemBytes) != cudaSuccess ||
-                cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-                cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
-        }
-        seen[C] = n;
+// How many clusters of 2, 4, 8 and 16 CTAs, one per SM, the current device runs at once (74, 33, 15 and 7 on 148 SMs), asked once per
+// host thread and device.
+struct ClustersAtOnce { int dev, of[4]; };
+static const ClustersAtOnce& clusters_at_once() {
+    thread_local ClustersAtOnce seen{-1, {}};
+    int dev = -1, optin = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess && dev == seen.dev) return seen;
+    const auto kernel = select_cluster_kernel<false>;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.blockDim = dim3(CL_NT); cfg.attrs = attr; cfg.numAttrs = 1;
+    (void)cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cfg.dynamicSmemBytes = (size_t)optin;                      // all of it (the kernel has no static part): one CTA per SM
+    const bool ok = optin > 0 && allow_smem(kernel, cfg.dynamicSmemBytes) == cudaSuccess &&
+                    cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    for (int i = 0; i < 4; ++i) {
+        attr[0].val.clusterDim.x = 2u << i;
+        cfg.gridDim = dim3(2u << i);
+        if (!ok || cudaOccupancyMaxActiveClusters(&seen.of[i], kernel, &cfg) != cudaSuccess) seen.of[i] = 0;
     }
-    return seen[C];
+    (void)cudaGetLastError();
+    seen.dev = dev;
+    return seen;
 }
 
 static int select_cluster_size(int units, int Nmax, int pool_kernel, int* seg_cap) {
     constexpr size_t kMost = 227 * 1024;                       // dynamic shared memory of a CTA
     auto seg_of = [&](int C) { return ((Nmax + C - 1) / C + 31) / 32 * 32; };
     int C = 1;
-    if (Nmax > 4096)
-        while (C < 16 && (units <= clusters_side_by_side(2 * C) ? C < 8 || seg_of(C) > 2048 : seg_of(C) > 8192 && (C < 8 || units <= 32))) C *= 2;
+    if (Nmax > 4096) {
+        const ClustersAtOnce& at_once = clusters_at_once();
+        for (int i = 0; C < 16 && (units <= at_once.of[i] ? C < 8 || seg_of(C) > 2048 : seg_of(C) > 8192 && (C < 8 || units <= 32)); ++i) C *= 2;
+    }
     while (C < 16 && (seg_of(C) > CL_MAX_SEG || select_cluster_smem(seg_of(C), pool_kernel) > kMost)) C *= 2;
     if (seg_of(C) > CL_MAX_SEG) return 0;
     *seg_cap = seg_of(C);
