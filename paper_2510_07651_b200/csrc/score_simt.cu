@@ -1,5 +1,5 @@
-// CUDA-core (fp32 FMA) score kernels: the path for fp32 caches (and for bf16 caches on request, or when the
-// queries' strides rule the tensor-core kernels out).  Two passes over K/V per (batch item, KV head):
+// CUDA-core (fp32 FMA) score kernels: the path for fp32 caches (and for bf16 caches on request, when the queries' strides
+// rule the tensor-core kernels out, and for the window attention of fewer than 64 rows).  Two passes over K/V per (batch item, KV head):
 //
 //   pass 1  split-KV streaming softmax over the window rows: per split, running max / sum of
 //           exp2 and the un-normalised partial output  (Sec. 3: A = softmax(QK^T/sqrt(d)), O = AV)
