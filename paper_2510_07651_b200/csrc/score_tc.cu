@@ -1207,6 +1207,106 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return r;
 }
 
+// zeroes the calling thread's row of a V tile, for the MMAs that follow, if it is row `first` or a later one
+__device__ __forceinline__ void zero_rows_from(uint8_t* tile, int row, int first) {
+    if (row < first) return;
+    uint8_t* at = tile + row * 128;
+#pragma unroll
+    for (int ch = 0; ch < 8; ++ch) {
+        *reinterpret_cast<uint4*>(at + (ch << 4)) = make_uint4(0, 0, 0, 0);
+        *reinterpret_cast<uint4*>(at + kHalfBytes + (ch << 4)) = make_uint4(0, 0, 0, 0);
+    }
+    fence_async_smem();
+}
+
+// The softmax of one 128-token tile, by the thread that owns the row: logits at tS in, P over their first 64 columns out, the running
+// reference m_used and sum l moved on; `has_o`: the warpgroup's accumulator tO holds earlier tiles and follows the reference.
+__device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, int nvis, bool masked, float sl2, bool valid, bool low_part, bool has_o,
+                                             float& m_used, float& l) {
+    // sweep 1: tile maximum of the row (raw logits; the scale is positive)
+    float mt = -INFINITY;
+    {
+        uint32_t sa[32], sb[32];
+        tc_ld32(tS, sa);
+#pragma unroll
+        for (int pc = 0; pc < 4; pc += 2) {
+            tc_wait_ld32(sa);
+            tc_ld32(tS + (pc + 1) * 32, sb);
+            if (masked) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) if (pc * 32 + j >= nvis) sa[j] = 0xff800000u;
+            }
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) mt = fmax3(mt, __uint_as_float(sa[j]), __uint_as_float(sa[j + 1]));
+            tc_wait_ld32(sb);
+            if (pc + 2 < 4) tc_ld32(tS + (pc + 2) * 32, sa);
+            if (masked) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) if ((pc + 1) * 32 + j >= nvis) sb[j] = 0xff800000u;
+            }
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) mt = fmax3(mt, __uint_as_float(sb[j]), __uint_as_float(sb[j + 1]));
+        }
+    }
+    mt *= sl2;
+    const bool need = mt > m_used + kRescaleThreshold;               // also true for the first visible tile
+    const float factor = need ? fast_exp2(m_used - mt) : 1.f;        // m_used = -inf -> 0
+    if (has_o && __any_sync(0xffffffffu, valid && need && m_used != -INFINITY)) {
+        // P.V of this warpgroup's previous tile is complete (the commit that signalled S covers it)
+#pragma unroll 1
+        for (int q4 = 0; q4 < 4; ++q4) {
+            uint32_t ov[32];
+            tc_ld32(tO + q4 * 32, ov);
+            tc_wait_ld32(ov);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * factor);
+            tc_st32(tO + q4 * 32, ov);
+        }
+    }
+    l *= factor;
+    if (need) m_used = mt;
+    const float m_eff = m_used == -INFINITY ? 0.f : m_used;
+    const float2 sl2v = make_float2(sl2, sl2), negm = make_float2(-m_eff, -m_eff);
+
+    // sweep 2: P = exp2(S * scale*log2e - m_used) as bf16 over the first 64 columns of S_w
+    float2 lsum = make_float2(0.f, 0.f);
+    {
+        uint32_t sa[32], sb[32];
+        auto piece = [&](uint32_t* sv, int pc) {
+            uint32_t pk[16];
+#pragma unroll
+            for (int j = 0; j < 32; j += 2) {
+                float2 x = make_float2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1]));
+                x = __ffma2_rn(x, sl2v, negm);
+                if (masked) {
+                    if (pc * 32 + j >= nvis) x.x = -INFINITY;
+                    if (pc * 32 + j + 1 >= nvis) x.y = -INFINITY;
+                }
+                const float2 e = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                lsum = __fadd2_rn(lsum, e);
+                pk[j >> 1] = pack_bf16x2(e.x, e.y);
+                if (low_part) {                                      // P = bf16(P) + bf16(P - bf16(P)): the second term
+                    const float2 h = bf16x2_to_f32x2(pk[j >> 1]);
+                    pk[j >> 1] = pack_bf16x2(e.x - h.x, e.y - h.y);
+                }
+            }
+            tc_st16(tS + pc * 16, pk);
+        };
+        tc_ld32(tS, sa);
+#pragma unroll
+        for (int pc = 0; pc < 4; pc += 2) {
+            tc_wait_ld32(sa);
+            tc_ld32(tS + (pc + 1) * 32, sb);
+            piece(sa, pc);
+            tc_wait_ld32(sb);
+            if (pc + 2 < 4) tc_ld32(tS + (pc + 2) * 32, sa);
+            piece(sb, pc + 1);
+        }
+    }
+    l += lsum.x + lsum.y;
+    tc_wait_st();
+}
+
 // Row chunk of a block (PAIR: pair of consecutive row chunks, in place of a chunk below).  Under a causal window a chunk of rows visits the tiles up to its last row's position, and all
 // of them if it holds the end of a head and the start of the next.  With more CTAs than SMs the chunks that visit most
 // tiles are handed out first: where a head has several chunks, blocks are ordered by the chunk's place counted back from
@@ -1456,97 +1556,8 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             // (a warp whose rows all see the whole tile skips the mask: under a whole-sequence window that is every tile off the diagonal)
             const bool masked = t0 + TILE > first_masked && __any_sync(0xffffffffu, nvis < TILE);
 
-            // sweep 1: tile maximum of the row (raw logits; the scale is positive)
-            float mt = -INFINITY;
-            {
-                uint32_t sa[32], sb[32];
-                tc_ld32(tS, sa);
-#pragma unroll
-                for (int pc = 0; pc < 4; pc += 2) {
-                    tc_wait_ld32(sa);
-                    tc_ld32(tS + (pc + 1) * 32, sb);
-                    if (masked) {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) if (pc * 32 + j >= nvis) sa[j] = 0xff800000u;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 32; j += 2) mt = fmax3(mt, __uint_as_float(sa[j]), __uint_as_float(sa[j + 1]));
-                    tc_wait_ld32(sb);
-                    if (pc + 2 < 4) tc_ld32(tS + (pc + 2) * 32, sa);
-                    if (masked) {
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) if ((pc + 1) * 32 + j >= nvis) sb[j] = 0xff800000u;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 32; j += 2) mt = fmax3(mt, __uint_as_float(sb[j]), __uint_as_float(sb[j + 1]));
-                }
-            }
-            mt *= sl2;
-            const bool need = mt > m_used + kRescaleThreshold;               // also true for the first visible tile
-            const float factor = need ? fast_exp2(m_used - mt) : 1.f;        // m_used = -inf -> 0
-            if (my_tiles > 0 && __any_sync(0xffffffffu, valid && need && m_used != -INFINITY)) {
-                // P.V of this warpgroup's previous tile is complete (the commit that signalled S covers it)
-#pragma unroll 1
-                for (int q4 = 0; q4 < 4; ++q4) {
-                    uint32_t ov[32];
-                    tc_ld32(tO + q4 * 32, ov);
-                    tc_wait_ld32(ov);
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) ov[j] = __float_as_uint(__uint_as_float(ov[j]) * factor);
-                    tc_st32(tO + q4 * 32, ov);
-                }
-            }
-            l *= factor;
-            if (need) m_used = mt;
-            const float m_eff = m_used == -INFINITY ? 0.f : m_used;
-            const float2 sl2v = make_float2(sl2, sl2), negm = make_float2(-m_eff, -m_eff);
-
-            // sweep 2: P = exp2(S * scale*log2e - m_used) as bf16 over the first 64 columns of S_w
-            float2 lsum = make_float2(0.f, 0.f);
-            {
-                uint32_t sa[32], sb[32];
-                auto piece = [&](uint32_t* sv, int pc) {
-                    uint32_t pk[16];
-#pragma unroll
-                    for (int j = 0; j < 32; j += 2) {
-                        float2 x = make_float2(__uint_as_float(sv[j]), __uint_as_float(sv[j + 1]));
-                        x = __ffma2_rn(x, sl2v, negm);
-                        if (masked) {
-                            if (pc * 32 + j >= nvis) x.x = -INFINITY;
-                            if (pc * 32 + j + 1 >= nvis) x.y = -INFINITY;
-                        }
-                        const float2 e = make_float2(fast_exp2(x.x), fast_exp2(x.y));
-                        lsum = __fadd2_rn(lsum, e);
-                        pk[j >> 1] = pack_bf16x2(e.x, e.y);
-                        if (low_part) {                                      // P = bf16(P) + bf16(P - bf16(P)): the second term
-                            const float2 h = bf16x2_to_f32x2(pk[j >> 1]);
-                            pk[j >> 1] = pack_bf16x2(e.x - h.x, e.y - h.y);
-                        }
-                    }
-                    tc_st16(tS + pc * 16, pk);
-                };
-                tc_ld32(tS, sa);
-#pragma unroll
-                for (int pc = 0; pc < 4; pc += 2) {
-                    tc_wait_ld32(sa);
-                    tc_ld32(tS + (pc + 1) * 32, sb);
-                    piece(sa, pc);
-                    tc_wait_ld32(sb);
-                    if (pc + 2 < 4) tc_ld32(tS + (pc + 2) * 32, sa);
-                    piece(sb, pc + 1);
-                }
-            }
-            l += lsum.x + lsum.y;
-            tc_wait_st();
-            if (t0 + TILE > N && t0 + row >= N) {                            // tail: V rows past the sequence must not reach the MMA
-                uint8_t* vrow = smem + OFF_V1 + (i % NST) * kOperandBytes + row * 128;
-#pragma unroll
-                for (int ch = 0; ch < 8; ++ch) {
-                    *reinterpret_cast<uint4*>(vrow + (ch << 4)) = make_uint4(0, 0, 0, 0);
-                    *reinterpret_cast<uint4*>(vrow + kHalfBytes + (ch << 4)) = make_uint4(0, 0, 0, 0);
-                }
-                fence_async_smem();
-            }
+            softmax_tile(tS, tO, nvis, masked, sl2, valid, low_part, my_tiles > 0, m_used, l);
+            if (t0 + TILE > N) zero_rows_from(smem + OFF_V1 + (i % NST) * kOperandBytes, row, N - t0);   // V rows past the sequence must not reach the MMA
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(P1_PFULL + w));
@@ -1755,6 +1766,293 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     }
 }
 
+// =================================================================================================
+// A short cache in one kernel: both passes and the merge between them, for a unit whose tiles have a cluster of CTAs, one
+// tile each.  As three kernels such a call is mostly their beginnings and ends and the second trip of K and V.  A CTA forms the
+// logits, P and its part of O as pass 1 does; row slices of the partial outputs meet in the CTA that owns the slice (over
+// distributed shared memory, added in the order of the tiles), which hands -2 O (HILO: both parts), as the operand image, and the row constants to every
+// CTA of the cluster; the scores of the tile follow from the K, V and Q tiles that are still in shared memory.
+// Bound by that chain (copy, two MMAs around a softmax, two cluster barriers around the merge, MMA, epilogue), not by bytes.  Per call,
+// three kernels / this one: 8 heads on 2 of 1024 tokens x 16 queries 13.9 / 10.6 us, 32 on 8 x 32 queries 16.7 / 14.5, one head of 128 14.7 / 9.1,
+// 7 KV heads of 2048 18.2 / 15.7, 32 of 512 19.3 / 16.1, 74 of 256 19.4 / 12.4.
+//   warps 0-3  softmax; first half of the rows in the score epilogue     warp 8  copies
+//   warps 4-7  value norms; second half of the rows                      warp 9  MMAs
+// TMEM columns: S and P [0, 128)  O [128, 256)  Z^T [256, 384)  T'^T [384, 512)
+// =================================================================================================
+constexpr int kThreadsShort = 320;
+constexpr int SH_MAXC = 16;
+constexpr uint32_t SH_OFF_Q = 0;
+constexpr uint32_t SH_OFF_K = SH_OFF_Q + kOperandBytes;
+constexpr uint32_t SH_OFF_V = SH_OFF_K + kOperandBytes;
+constexpr uint32_t SH_OFF_O = SH_OFF_V + kOperandBytes;            // -2 O of the unit's rows
+constexpr uint32_t SH_OFF_RX = SH_OFF_O + kOperandBytes;           // [source][row of the slice][128] partial outputs, 16-byte pieces XOR-swizzled by the row
+constexpr uint32_t SH_RX_ROWS = 160;                               // sources x slice rows: at most 128 + C - 1, or 2 x (63 + C - 1) with low parts
+constexpr uint32_t SH_OFF_ML = SH_OFF_RX + SH_RX_ROWS * 512;       // [source][row of the slice] (m, l)
+constexpr uint32_t SH_OFF_CONST = SH_OFF_ML + SH_RX_ROWS * 8;      // 64 row pairs of (-lse2_0, -lse2_1, |o_0|^2, |o_1|^2), as the epilogue takes them
+constexpr uint32_t SH_OFF_NV = SH_OFF_CONST + 64 * 16;             // [128] (||v||^2, ||v||_1)
+constexpr uint32_t SH_OFF_XCH = SH_OFF_NV + TILE * 8;              // [kNumSums][128]: the second row half's sums
+constexpr uint32_t SH_OFF_BAR = SH_OFF_XCH + kNumSums * TILE * 4;
+enum { SH_QK = 0, SH_V, SH_S, SH_P, SH_ODONE, SH_T, SH_NBARS };
+constexpr uint32_t SH_OFF_TMEM = SH_OFF_BAR + SH_NBARS * 8;
+constexpr uint32_t kSmemShort = SH_OFF_TMEM + 16 + 1024;
+
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {      // the same place in another CTA of the cluster
+    uint32_t r;
+    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+__device__ __forceinline__ void st_cluster4(uint32_t addr, float4 v) {
+    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
+}
+__device__ __forceinline__ void st_cluster2(uint32_t addr, uint32_t a, uint32_t b) {
+    asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void st_cluster1(uint32_t addr, float a) {
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
+}
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+template <unsigned VARS, bool HILO, bool BY_UNIT>
+__global__ void __launch_bounds__(kThreadsShort, 1)
+tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant__ CUtensorMap map_k,
+                const __grid_constant__ CUtensorMap map_v, const __grid_constant__ TcParams p, int C) {
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    const uint32_t sbase = smem_u32(smem), dbase = sbase & 0x3ffffu;   // (in a cluster the address carries the CTA's rank, which a matrix descriptor has no room for)
+    auto bar = [&](int i) { return sbase + SH_OFF_BAR + 8u * (uint32_t)i; };
+    volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + SH_OFF_TMEM);
+    float* sConst = reinterpret_cast<float*>(smem + SH_OFF_CONST);
+    float2* sNv = reinterpret_cast<float2*>(smem + SH_OFF_NV);
+    float* sXch = reinterpret_cast<float*>(smem + SH_OFF_XCH);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    span_begin(p.span);
+    const int unit = blockIdx.x / C, rank = blockIdx.x % C, b = unit / p.Hkv, g = unit % p.Hkv, t0 = rank * TILE;
+    const int slice = (p.R + C - 1) / C;                               // rows [rank slice, rank slice + slice) are this CTA's to merge
+
+    cluster_arrive();                                                  // (with the wait before the first write to another CTA: that CTA runs)
+    if (threadIdx.x == 0) {
+        prefetch_tmap(&map_k); prefetch_tmap(&map_v); prefetch_tmap(&map_q);
+        for (int i = 0; i < SH_NBARS; ++i) mbar_init(bar(i), i == SH_P ? 4 : 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    if (warp == 8) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + SH_OFF_TMEM), "r"(512u) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    // padding rows: O = 0, weight 0
+    for (int i = threadIdx.x; i < (p.chunk_rows - p.R) * 16 * (HILO ? 2 : 1); i += kThreadsShort) {
+        const int r = p.R + i / 16 % (p.chunk_rows - p.R) + (i / 16 < p.chunk_rows - p.R ? 0 : p.chunk_rows), ch = i & 15;
+        *reinterpret_cast<uint4*>(smem + SH_OFF_O + (ch >> 3) * kHalfBytes + r * 128 + ((ch & 7) << 4)) = make_uint4(0, 0, 0, 0);
+    }
+    for (int r = p.R + (int)threadIdx.x; r < p.chunk_rows; r += kThreadsShort) {
+        sConst[(r >> 1) * 4 + (r & 1)] = -INFINITY; sConst[(r >> 1) * 4 + 2 + (r & 1)] = 0.f;
+    }
+    fence_async_smem();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = *tmem_slot;
+    bool failed = false;
+    int fail_site = 0;                                                 // source line of the wait that gave up (status word)
+    pdl_wait();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *p.status = 0u;           // no wait of this call can have given up yet (each lasts seconds)
+    const int N = tc_seq_len(p, b), Nm = tc_mask_len(p, b);
+    const bool empty = t0 >= N;                                        // a CTA past the end merges its slice and writes zeros
+    const int n_src = min(C, (N + TILE - 1) / TILE);                   // tiles of the unit = partial outputs of a row
+    const uint32_t tS = tmem_base, tO = tmem_base + 128u, tZ = tmem_base + 256u, tT = tmem_base + 384u;
+    auto wait = [&](int i) { if (!failed && !mbar_wait(bar(i), 0)) { failed = true; fail_site = __LINE__; } return !failed; };
+
+    // ---- the tile's partial softmax and output ----------------------------------------------------------------
+    if (!empty) {
+        if (warp == 8) {
+            if (lane == 0) {
+                mbar_expect_tx(bar(SH_QK), kOperandBytes + (uint32_t)p.chunk_rows * (HILO ? 512u : 256u));
+                for (int h = 0; h < 2; ++h) {
+                    load_q<BY_UNIT>(sbase + SH_OFF_Q + h * kHalfBytes, &map_q, bar(SH_QK), h * 64, 0, unit, p.R);
+                    tma_load_4d(sbase + SH_OFF_K + h * kHalfBytes, &map_k, bar(SH_QK), h * 64, t0, g, b);
+                    if (HILO) load_q<BY_UNIT>(sbase + SH_OFF_Q + h * kHalfBytes + kHalfBytes / 2, &map_q, bar(SH_QK), h * 64, 0, unit, p.R);
+                }
+                mbar_expect_tx(bar(SH_V), kOperandBytes);
+                for (int h = 0; h < 2; ++h) tma_load_4d(sbase + SH_OFF_V + h * kHalfBytes, &map_v, bar(SH_V), h * 64, t0, g, b);
+                wait(SH_QK); wait(SH_V);                               // (the copies have landed before the CTA may exit)
+            }
+        } else if (warp == 9) {
+            if (lane == 0) {
+                const uint32_t aq = desc_lo_k(dbase + SH_OFF_Q), ak = desc_lo_k(dbase + SH_OFF_K), av = desc_lo_mn(dbase + SH_OFF_V);
+                if (wait(SH_QK)) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        tc_mma(tS, desc_make(aq + desc_kstep(ks, kHalfBytes)), desc_make(ak + desc_kstep(ks, kHalfBytes)), idesc_bf16(TILE), ks > 0);
+                    tc_commit(bar(SH_S));
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        tc_mma(tZ, desc_make(ak + desc_kstep(ks, kHalfBytes)), desc_make(aq + desc_kstep(ks, kHalfBytes)), idesc_bf16(p.chunk_rows), ks > 0);
+                }
+                if (wait(SH_V) && wait(SH_P)) {
+                    tc_fence_after();
+#pragma unroll
+                    for (int ks = 0; ks < 8; ++ks)
+                        tc_mma_ts(tO, tS + ks * 8, desc_make(av + ks * (2048 >> 4)), idesc_bf16(kD) | (1u << 16), ks > 0);
+                    tc_commit(bar(SH_ODONE));
+                }
+            }
+        } else {
+            const int w = warp >> 2, lane_grp = warp & 3, row = lane_grp * 32 + lane;
+            const uint32_t lane_addr = (uint32_t)(lane_grp * 32) << 16;
+            const bool low_part = HILO && lane_grp >= 2;               // this warp's rows are the second copies of rows 0..63
+            const int r = HILO ? row & 63 : row;
+            const bool valid = r < p.R;
+            const int owner = valid ? r / slice : 0, local = valid ? r % slice : 0;    // of the row's slice
+            const int src = HILO ? 2 * rank + (low_part ? 1 : 0) : rank;
+            const uint32_t rx_row = (uint32_t)(src * slice + local);
+            if (w == 0) {
+                float m = -INFINITY, l = 0.f;
+                if (wait(SH_S)) {
+                    tc_fence_after();
+                    const int last = valid ? (p.causal ? min(Nm - p.W + (r % p.W), N - 1) : N - 1) : -1;   // last visible token
+                    const int nvis = last - t0 + 1;
+                    const bool masked = t0 + TILE > min(p.causal ? Nm - p.W + 1 : N, N) && __any_sync(0xffffffffu, nvis < TILE);
+                    softmax_tile(tS + lane_addr, 0u, nvis, masked, p.scale * kLog2e, valid, low_part, false, m, l);
+                }
+                if (t0 + TILE > N && wait(SH_V)) zero_rows_from(smem + SH_OFF_V, row, N - t0);   // V rows past the sequence must not reach the MMA
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(SH_P));
+                cluster_wait();
+                if (valid) {                                           // (the low part of P adds to O alone)
+                    const uint32_t at = cluster_addr(sbase + SH_OFF_ML + rx_row * 8u, owner);
+                    st_cluster2(at, __float_as_uint(m), low_part ? 0u : __float_as_uint(l));
+                }
+            } else {
+                if (wait(SH_V)) {
+                    float l2, l1;
+                    value_norms<(VARS & OBC_VAR_VATP) != 0>(smem + SH_OFF_V, row, l2, l1);
+                    sNv[row] = make_float2(l2, l1);
+                }
+                cluster_wait();
+            }
+            if (wait(SH_ODONE)) {
+                tc_fence_after();
+                const uint32_t dst = cluster_addr(sbase + SH_OFF_RX + rx_row * 512u, owner);
+#pragma unroll 1
+                for (int q = 0; q < 2; ++q) {                          // warpgroup w: head-dim columns [64 w, 64 w + 64)
+                    uint32_t o[32];
+                    tc_ld32(tO + lane_addr + w * 64u + q * 32u, o);
+                    tc_wait_ld32(o);
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (valid)
+                            st_cluster4(dst + (uint32_t)(((w * 16 + q * 8 + j) ^ (row & 31)) << 4),
+                                        make_float4(__uint_as_float(o[4 * j]), __uint_as_float(o[4 * j + 1]), __uint_as_float(o[4 * j + 2]), __uint_as_float(o[4 * j + 3])));
+                }
+                tc_fence_before();
+            }
+        }
+        if (warp >= 8) { __syncwarp(); cluster_wait(); }
+    } else {
+        cluster_wait();
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();                                                    // the partial outputs of this CTA's slice are here
+    // ---- the slice's rows: merged, and handed to every CTA --------------------------------------------------------
+    if (warp < 8) {
+        const int rows = min(slice, p.R - rank * slice), parts = n_src * (HILO ? 2 : 1);
+        for (int local = warp; local < rows; local += 8) {
+            const int r = rank * slice + local;
+            const float2* ml = reinterpret_cast<const float2*>(smem + SH_OFF_ML) + local;    // part sp: ml[sp * slice]
+            const float2 mine = lane < parts ? ml[lane * slice] : make_float2(-INFINITY, 0.f);
+            const float M = warp_max(mine.x);
+            const float wt = mine.x == -INFINITY ? 0.f : exp2f(mine.x - M);
+            float L = 0.f;
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int sp = 0; sp < parts; ++sp) {
+                const float f = __shfl_sync(0xffffffffu, wt, sp), l = __shfl_sync(0xffffffffu, mine.y, sp);
+                const float4 x = *reinterpret_cast<const float4*>(smem + SH_OFF_RX + (sp * slice + local) * 512 + ((lane ^ (r & 31)) << 4));   // (rows r and r + 64 swizzle alike)
+                L = fmaf(l, f, L);
+                o.x = fmaf(x.x, f, o.x); o.y = fmaf(x.y, f, o.y); o.z = fmaf(x.z, f, o.z); o.w = fmaf(x.w, f, o.w);
+            }
+            if (L > 0.f) { o.x /= L; o.y /= L; o.z /= L; o.w /= L; }
+            const float onorm = warp_sum((o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w));
+            const float lse2 = M + log2f(L);
+            const uint32_t h0 = pack_bf16x2(-2.f * o.x, -2.f * o.y), h1 = pack_bf16x2(-2.f * o.z, -2.f * o.w);
+            const float2 f0 = bf16x2_to_f32x2(h0), f1 = bf16x2_to_f32x2(h1);
+            const uint32_t l0 = pack_bf16x2(fmaf(-2.f, o.x, -f0.x), fmaf(-2.f, o.y, -f0.y)), l1 = pack_bf16x2(fmaf(-2.f, o.z, -f1.x), fmaf(-2.f, o.w, -f1.y));
+            // elements 4 lane .. of row r in the 128-byte swizzle of the operand
+            auto place = [&](int row) { return sbase + SH_OFF_O + (uint32_t)((lane >> 4) * kHalfBytes + row * 128 + ((((lane & 15) >> 1) ^ (row & 7)) << 4) + (lane & 1) * 8); };
+            for (int d = 0; d < C; ++d) {
+                st_cluster2(cluster_addr(place(r), d), h0, h1);
+                if (HILO) st_cluster2(cluster_addr(place(p.chunk_rows + r), d), l0, l1);
+            }
+            if (lane < C) {
+                const uint32_t at = cluster_addr(sbase + SH_OFF_CONST + (uint32_t)((r >> 1) * 16 + (r & 1) * 4), lane);
+                st_cluster1(at, -lse2 * kExpFactor<VARS, HILO>);
+                st_cluster1(at + 8, onorm * (VARS == OBC_VAR_VK ? p.scale : 1.f));
+            }
+        }
+        asm volatile("fence.proxy.async;" ::: "memory");
+    }
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();                                                    // -2 O and the constants are complete; no CTA writes to another from here on
+    // ---- the tile's scores -----------------------------------------------------------------------------------------
+    const size_t plane = (size_t)p.B * p.Hkv * p.Nmax;
+    if (empty) {
+        if (warp < 4 && t0 + (int)threadIdx.x < p.Nmax)
+            for (int pl = 0; pl < __popc(p.variants); ++pl) p.scores[(size_t)pl * plane + (size_t)unit * p.Nmax + t0 + threadIdx.x] = 0.f;
+    } else if (warp == 9) {
+        if (lane == 0 && !failed) {
+            asm volatile("fence.proxy.async;" ::: "memory");
+            tc_fence_after();
+            const uint32_t av = desc_lo_k(dbase + SH_OFF_V), bo = desc_lo_k(dbase + SH_OFF_O);
+#pragma unroll
+            for (int ks = 0; ks < 8; ++ks)
+                tc_mma(tT, desc_make(av + desc_kstep(ks, kHalfBytes)), desc_make(bo + desc_kstep(ks, kHalfBytes)), idesc_bf16(HILO ? 2 * p.chunk_rows : p.chunk_rows), ks > 0);
+            tc_commit(bar(SH_T));
+        }
+    } else if (warp < 8) {
+        const int half = warp >> 2, lane_grp = warp & 3, tok = lane_grp * 32 + lane, ptok = t0 + tok;
+        const int rows0 = min(p.chunk_rows, (p.chunk_rows / 2 + 15) / 16 * 16);        // two runs of whole 16-row batches
+        const int r_begin = half ? rows0 : 0, r_count = half ? p.chunk_rows - rows0 : rows0;
+        const float ksl = p.scale * kLog2e * kExpFactor<VARS, HILO>;
+        const float2 sl2 = make_float2(ksl, ksl), sc = make_float2(p.scale, p.scale);
+        const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
+        RowSums S;
+        S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
+        if (wait(SH_T) && r_count > 0) {
+            tc_fence_after();
+            const float4* cst = reinterpret_cast<const float4*>(sConst) + (r_begin >> 1);
+            const uint32_t zt = tZ + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)r_begin, tt = zt + 128u;
+            if (masked_tile) score_chunk<VARS, true, HILO>(zt, tt, r_count, cst, sl2, sc, S, ptok, Nm - p.W, p.W, r_begin % p.W, p.chunk_rows);
+            else score_chunk<VARS, false, HILO>(zt, tt, r_count, cst, sl2, sc, S, ptok, 0, 0, 0, p.chunk_rows);
+            tc_fence_before();
+        }
+        float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
+        if (half == 1) {
+#pragma unroll
+            for (int j = 0; j < kNumSums; ++j) sXch[j * TILE + tok] = sum[j];
+        }
+        asm volatile("bar.sync 1, 256;" ::: "memory");                 // both warpgroups
+        if (half == 0) {
+#pragma unroll
+            for (int j = 0; j < kNumSums; ++j) sum[j] += sXch[j * TILE + tok];
+            const float2 nv = sNv[tok];
+            if (ptok < p.Nmax)
+                store_scores<VARS, HILO>(sum, nv.x, nv.y, p.scale, p.variants, p.scores + (size_t)unit * p.Nmax + ptok, plane, ptok < N);
+        }
+    }
+    if (failed) atomicCAS(p.status, 0u, (unsigned)(fail_site > 0 ? fail_site : 1));   // the first failure is kept
+    tc_fence_before();
+    __syncthreads();
+    span_end(p.span);
+    if (warp == 8) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    }
+}
+
 // ---- host side ----------------------------------------------------------------------------------
 // Row chunks.  Pass 1 cuts the R window rows into n_chunks pieces of chunk_rows <= 128 (its MMA M
 // dimension).  Pass 2 takes the rows whole when R <= 128 and in pieces of 64 otherwise; rows_out is
@@ -1855,6 +2153,42 @@ static size_t tc_partial_bytes(const ScoreShape& s) {
 
 size_t tc_workspace_bytes(const ScoreShape& s) { return make_tc_plan(s).bytes + tc_partial_bytes(s); }
 
+// How many clusters of 2, 4, 8 and 16 CTAs of tc_short_kernel the current device runs at once, asked once per host thread and device
+static_assert(SH_RX_ROWS >= 128 + SH_MAXC - 1 && SH_RX_ROWS >= 2 * (63 + SH_MAXC - 1), "partial outputs of a slice");
+static int short_clusters(int C) {
+    if (C == 1) return sm_count();
+    thread_local struct { int dev, of[4]; } seen{-1, {}};
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (dev != seen.dev) {
+        const auto kernel = tc_short_kernel<OBC_VAR_VK, false, false>;             // (one CTA per SM, whatever the instantiation)
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.blockDim = dim3(kThreadsShort); cfg.attrs = attr; cfg.numAttrs = 1; cfg.dynamicSmemBytes = kSmemShort;
+        const bool ok = allow_smem(kernel, kSmemShort) == cudaSuccess &&
+                        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+        for (int i = 0; i < 4; ++i) {
+            attr[0].val.clusterDim.x = 2u << i;
+            cfg.gridDim = dim3(2u << i);
+            if (!ok || cudaOccupancyMaxActiveClusters(&seen.of[i], kernel, &cfg) != cudaSuccess) seen.of[i] = 0;
+        }
+        (void)cudaGetLastError();
+        seen.dev = dev;
+    }
+    return seen.of[C == 2 ? 0 : C == 4 ? 1 : C == 8 ? 2 : 3];
+}
+// Cluster size for a call that one kernel serves (tc_short_kernel), or 0: up to 128 window rows, a tile per CTA, all units side by side
+// (a second wave of clusters would take longer than the three kernels' other two: both sides at the kernel).
+static int short_cluster_size(const ScoreShape& s, const TcChunks& ch) {
+    const int tiles = (s.Nmax + TILE - 1) / TILE, units = s.B * s.Hkv;
+    if (ch.n_chunks > 1 || tiles > SH_MAXC) return 0;
+    int C = 1;
+    while (C < tiles) C *= 2;
+    return units <= short_clusters(C) ? C : 0;
+}
+
 obc_status launch_attention_tc(const ScoreShape& s, TensorView q, TensorView k, TensorView v, void* ws, cudaStream_t stream,
                                SimtPlan* plan_out) {
     return launch_score_tc(s, q, k, v, nullptr, ws, stream, nullptr, plan_out);
@@ -1891,7 +2225,10 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     // Smaller caches keep the default policy, so that pass 2 finds in L2 what pass 1 read.
     const bool l2_stream = ch.n_chunks == 1 && !given &&
         (double)units * s.Nmax * kD * 2 * 2 > 0.75 * (double)l2_bytes();
-    if (given) {   // the caller's O and LSE take the place of pass 1 + combine; pass 2 computes the value norms itself
+    const int short_c = given || attention_only ? 0 : short_cluster_size(s, ch);
+    if (short_c) {
+        // everything in one kernel (below)
+    } else if (given) {   // the caller's O and LSE take the place of pass 1 + combine; pass 2 computes the value norms itself
         obc_status st = launch_given_prep(s, plan, *given, ws, stream);
         if (st != OBC_OK) return st;
     } else {       // pass 1 + combine
@@ -1952,6 +2289,22 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         return make_map(m, q.ptr, by_unit ? 3 : 2, by_unit ? per_unit : rows_of_all, strides, (uint32_t)rows);
     };
     auto flag = [](bool f, auto g) { return f ? g(std::true_type{}) : g(std::false_type{}); };
+    if (short_c) {
+        CUtensorMap ms;
+        if (!map_queries(&ms, ch.chunk_rows)) { set_last_cuda_error((int)cudaErrorInvalidValue); return OBC_ERR_CUDA; }
+        auto launch_short = [&](auto kernel) -> obc_status {
+            OBC_CUDA_TRY(allow_smem(kernel, kSmemShort));
+            if (short_c > 8) OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            ProfScope ps("tc_short", stream);
+            OBC_CUDA_TRY(launch_pdl(kernel, dim3(units * short_c), dim3(kThreadsShort), kSmemShort, stream, short_c, ms, mk, mv, p, short_c));
+            return OBC_OK;
+        };
+        return flag(hilo, [&](auto hl) { return flag(by_unit, [&](auto bu) {
+            if (s.variants == OBC_VAR_VK) return launch_short(tc_short_kernel<OBC_VAR_VK, hl.value, bu.value>);
+            if (!(s.variants & ~kObcVariants)) return launch_short(tc_short_kernel<kObcVariants, hl.value, bu.value>);
+            return launch_short(tc_short_kernel<kAllVariants, hl.value, bu.value>);
+        }); });
+    }
     if (ch.n_chunks > 1) {                               // more than 128 window rows: chunks of 64, K/V tile kept
         CUtensorMap mq64, mo64;
         const uint64_t od[2] = {(uint64_t)kD, (uint64_t)units * ch.rows_out};
