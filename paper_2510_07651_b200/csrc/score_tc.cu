@@ -75,8 +75,14 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+template <bool CLUSTER = false>                    // CLUSTER: what other CTAs of the cluster stored before they arrived is visible, too
 __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
     uint32_t ok;
+    if (CLUSTER) {
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+        return ok != 0;
+    }
     asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
                  : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
@@ -97,13 +103,14 @@ __device__ __forceinline__ void span_end(unsigned long long* span) {
     if (threadIdx.x == 96) atomicMax(span + 1, global_ns());
 }
 // bounded wait: false after kWaitNs without completion
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-    if (mbar_try(bar, parity)) return true;
+    if (mbar_try<CLUSTER>(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     for (;;) {
 #pragma unroll 1
         for (int i = 0; i < 64; ++i)
-            if (mbar_try(bar, parity)) return true;
+            if (mbar_try<CLUSTER>(bar, parity)) return true;
         if (global_ns() - t0 > kWaitNs) return false;
     }
 }
@@ -1769,46 +1776,59 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // =================================================================================================
 // A short cache in one kernel: both passes and the merge between them, for a unit whose tiles have a cluster of CTAs, one
 // tile each.  As three kernels such a call is mostly their beginnings and ends and the second trip of K and V.  A CTA forms the
-// logits, P and its part of O as pass 1 does; row slices of the partial outputs meet in the CTA that owns the slice (over
-// distributed shared memory, added in the order of the tiles), which hands -2 O (HILO: both parts), as the operand image, and the row constants to every
-// CTA of the cluster; the scores of the tile follow from the K, V and Q tiles that are still in shared memory.
-// Bound by that chain (copy, two MMAs around a softmax, two cluster barriers around the merge, MMA, epilogue), not by bytes.  Per call,
-// three kernels / this one: 8 heads on 2 of 1024 tokens x 16 queries 13.9 / 10.6 us, 32 on 8 x 32 queries 16.7 / 14.5, one head of 128 14.7 / 9.1,
-// 7 KV heads of 2048 18.2 / 15.7, 32 of 512 19.3 / 16.1, 74 of 256 19.4 / 12.4.
-//   warps 0-3  softmax; first half of the rows in the score epilogue     warp 8  copies
-//   warps 4-7  value norms; second half of the rows                      warp 9  MMAs
+// logits, P and its part of O as pass 1 does; row slices of the partial outputs go to the CTA that owns the slice, which adds them
+// in the order of the tiles and hands -2 O (HILO: both parts), as the operand image, and the row constants to every CTA of the
+// cluster; the scores of the tile follow from the K and V tiles that are still there (Z from before K and Q made room for the staged O).
+// Partial outputs cross the cluster as bulk copies of runs of staged rows, the merged rows as plain stores; both arrive on the
+// receiver's mbarriers, and a CTA that has seen its image complete has neither copies out of its memory nor stores into it under way
+// (its owners have merged what it sent, and all that it receives is counted).
+// The code runs once per launch, from a cold instruction cache: loops are kept short rather than unrolled.
+//   warps 0-7  softmax (64 tokens of the tile per warpgroup), merge, score epilogue (half of the rows per warpgroup)
+//   warp 8  copies     warp 9  MMAs     warps 10-11  value norms
 // TMEM columns: S and P [0, 128)  O [128, 256)  Z^T [256, 384)  T'^T [384, 512)
+// Bound by that chain, not by bytes: at 64 rows x 8 CTAs, cycles of set-up 2.1 k, copies and logits 2.1 k, softmax 2.5 k, P.V 1.3 k, the
+// exchange of partial outputs 2.3 k, merge and hand-out 5.1 k, T' 0.9 k, scores 1.7 k.  Per call, three kernels / this one: 8 heads on 2 of
+// 1024 tokens x 16 queries 13.9 / 10.7 us, 32 on 8 x 32 queries 16.7 / 13.8, one head of 128 tokens 14.8 / 8.8, of 2048 14.5 / 11.8, 7 KV heads of 2048
+// 18.2 / 14.6, 32 of 512 19.3 / 14.9, 74 of 256 19.4 / 12.3.  (Partial outputs and -2 O through the workspace instead, with a device-wide
+// fence before each arrival: 11.7, 14.2, 11.2, 12.5, 14.3, 16.5, 14.8; -2 O alone: 10.9, 14.0, 9.6, 11.9, 14.6, 15.3, 12.6.)
 // =================================================================================================
-constexpr int kThreadsShort = 320;
+constexpr int kThreadsShort = 384;
 constexpr int SH_MAXC = 16;
+constexpr uint32_t SH_PITCH = 528;                                 // a staged row: 128 floats of O, m, l of either half of the tile; no bank conflicts by row or by column
 constexpr uint32_t SH_OFF_Q = 0;
 constexpr uint32_t SH_OFF_K = SH_OFF_Q + kOperandBytes;
-constexpr uint32_t SH_OFF_V = SH_OFF_K + kOperandBytes;
+constexpr uint32_t SH_OFF_STAGE = SH_OFF_Q;                        // [128 accumulator rows], over Q and K once the MMAs have read them
+constexpr uint32_t SH_OFF_XCH = SH_OFF_Q;                          // [kNumSums][128]: the second row half's sums, once the staged rows are with their owners
+constexpr uint32_t SH_OFF_V = SH_OFF_STAGE + 128 * SH_PITCH;
 constexpr uint32_t SH_OFF_O = SH_OFF_V + kOperandBytes;            // -2 O of the unit's rows
-constexpr uint32_t SH_OFF_RX = SH_OFF_O + kOperandBytes;           // [source][row of the slice][128] partial outputs, 16-byte pieces XOR-swizzled by the row
+constexpr uint32_t SH_OFF_RX = SH_OFF_O + kOperandBytes;           // [source][row of the slice]
 constexpr uint32_t SH_RX_ROWS = 160;                               // sources x slice rows: at most 128 + C - 1, or 2 x (63 + C - 1) with low parts
-constexpr uint32_t SH_OFF_ML = SH_OFF_RX + SH_RX_ROWS * 512;       // [source][row of the slice] (m, l)
-constexpr uint32_t SH_OFF_CONST = SH_OFF_ML + SH_RX_ROWS * 8;      // 64 row pairs of (-lse2_0, -lse2_1, |o_0|^2, |o_1|^2), as the epilogue takes them
-constexpr uint32_t SH_OFF_NV = SH_OFF_CONST + 64 * 16;             // [128] (||v||^2, ||v||_1)
-constexpr uint32_t SH_OFF_XCH = SH_OFF_NV + TILE * 8;              // [kNumSums][128]: the second row half's sums
-constexpr uint32_t SH_OFF_BAR = SH_OFF_XCH + kNumSums * TILE * 4;
-enum { SH_QK = 0, SH_V, SH_S, SH_P, SH_ODONE, SH_T, SH_NBARS };
+constexpr uint32_t SH_OFF_ROWS = SH_OFF_RX + SH_RX_ROWS * SH_PITCH; // [128] (-lse2, |o|^2, -, -)
+constexpr uint32_t SH_OFF_CONST = SH_OFF_ROWS + 128 * 16;          // 8 epilogue warps x 32 float4: row-pair constants of the warp's rows
+constexpr uint32_t SH_OFF_MAX = SH_OFF_CONST + 8 * 32 * 16;        // [2][128]: row maxima of the tile's halves
+constexpr uint32_t SH_OFF_NV = SH_OFF_MAX + 2 * 128 * 4;           // [128] (||v||^2, ||v||_1)
+constexpr uint32_t SH_OFF_BAR = SH_OFF_NV + TILE * 8;
+enum { SH_QK = 0, SH_V, SH_S, SH_P, SH_ODONE, SH_STAGED, SH_RX, SH_IMG, SH_NORMS, SH_T, SH_NBARS };
 constexpr uint32_t SH_OFF_TMEM = SH_OFF_BAR + SH_NBARS * 8;
 constexpr uint32_t kSmemShort = SH_OFF_TMEM + 16 + 1024;
+static_assert(SH_OFF_V % 1024 == 0 && kSmemShort <= 227 * 1024, "layout");
+static_assert(SH_RX_ROWS >= 128 + SH_MAXC - 1 && SH_RX_ROWS >= 2 * (63 + SH_MAXC - 1), "partial outputs of a slice");
 
 __device__ __forceinline__ uint32_t cluster_addr(uint32_t addr, int rank) {      // the same place in another CTA of the cluster
     uint32_t r;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-__device__ __forceinline__ void st_cluster4(uint32_t addr, float4 v) {
-    asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
-}
 __device__ __forceinline__ void st_cluster2(uint32_t addr, uint32_t a, uint32_t b) {
     asm volatile("st.shared::cluster.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
-__device__ __forceinline__ void st_cluster1(uint32_t addr, float a) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
+__device__ __forceinline__ void arrive_at_cta(uint32_t remote_bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(remote_bar) : "memory");
+}
+// own shared memory -> another CTA's; the bytes arrive on that CTA's mbarrier
+__device__ __forceinline__ void copy_to_cta(uint32_t dst, uint32_t src, uint32_t bytes, uint32_t dst_bar) {
+    asm volatile("cp.async.bulk.shared::cluster.shared::cta.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                 ::"r"(dst), "r"(src), "r"(bytes), "r"(dst_bar) : "memory");
 }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
@@ -1822,32 +1842,35 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const uint32_t sbase = smem_u32(smem), dbase = sbase & 0x3ffffu;   // (in a cluster the address carries the CTA's rank, which a matrix descriptor has no room for)
     auto bar = [&](int i) { return sbase + SH_OFF_BAR + 8u * (uint32_t)i; };
     volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(smem + SH_OFF_TMEM);
-    float* sConst = reinterpret_cast<float*>(smem + SH_OFF_CONST);
+    float4* sRows = reinterpret_cast<float4*>(smem + SH_OFF_ROWS);
     float2* sNv = reinterpret_cast<float2*>(smem + SH_OFF_NV);
     float* sXch = reinterpret_cast<float*>(smem + SH_OFF_XCH);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     span_begin(p.span);
     const int unit = blockIdx.x / C, rank = blockIdx.x % C, b = unit / p.Hkv, g = unit % p.Hkv, t0 = rank * TILE;
     const int slice = (p.R + C - 1) / C;                               // rows [rank slice, rank slice + slice) are this CTA's to merge
+    const int my_rows = max(min(slice, p.R - rank * slice), 0);
+    const int mergers = p.R / slice * min(slice, 8) + min(p.R % slice, 8);     // warps of the cluster that merge rows: one at least, eight at most per slice
+    constexpr uint32_t kParts = HILO ? 2 : 1;                          // of a partial output, and of -2 O
 
-    cluster_arrive();                                                  // (with the wait before the first write to another CTA: that CTA runs)
     if (threadIdx.x == 0) {
         prefetch_tmap(&map_k); prefetch_tmap(&map_v); prefetch_tmap(&map_q);
-        for (int i = 0; i < SH_NBARS; ++i) mbar_init(bar(i), i == SH_P ? 4 : 1);
+        for (int i = 0; i < SH_NBARS; ++i)
+            mbar_init(bar(i), i == SH_P || i == SH_STAGED ? 8 : i == SH_NORMS ? 2 : i == SH_IMG ? (uint32_t)mergers : 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    cluster_arrive();                                                  // (waited for before the first copy to another CTA: its mbarriers are set up)
     if (warp == 8) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(sbase + SH_OFF_TMEM), "r"(512u) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
     // padding rows: O = 0, weight 0
-    for (int i = threadIdx.x; i < (p.chunk_rows - p.R) * 16 * (HILO ? 2 : 1); i += kThreadsShort) {
-        const int r = p.R + i / 16 % (p.chunk_rows - p.R) + (i / 16 < p.chunk_rows - p.R ? 0 : p.chunk_rows), ch = i & 15;
+    const int pad = p.chunk_rows - p.R;
+    for (int i = threadIdx.x; i < pad * 16 * (int)kParts; i += kThreadsShort) {
+        const int at = i >> 4, r = p.R + at + (at < pad ? 0 : p.chunk_rows - pad), ch = i & 15;
         *reinterpret_cast<uint4*>(smem + SH_OFF_O + (ch >> 3) * kHalfBytes + r * 128 + ((ch & 7) << 4)) = make_uint4(0, 0, 0, 0);
     }
-    for (int r = p.R + (int)threadIdx.x; r < p.chunk_rows; r += kThreadsShort) {
-        sConst[(r >> 1) * 4 + (r & 1)] = -INFINITY; sConst[(r >> 1) * 4 + 2 + (r & 1)] = 0.f;
-    }
+    if ((int)threadIdx.x < pad) sRows[p.R + threadIdx.x] = make_float4(-INFINITY, 0.f, 0.f, 0.f);
     fence_async_smem();
     tc_fence_before();
     __syncthreads();
@@ -1861,186 +1884,252 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const bool empty = t0 >= N;                                        // a CTA past the end merges its slice and writes zeros
     const int n_src = min(C, (N + TILE - 1) / TILE);                   // tiles of the unit = partial outputs of a row
     const uint32_t tS = tmem_base, tO = tmem_base + 128u, tZ = tmem_base + 256u, tT = tmem_base + 384u;
-    auto wait = [&](int i) { if (!failed && !mbar_wait(bar(i), 0)) { failed = true; fail_site = __LINE__; } return !failed; };
+    auto wait = [&](int i, int line) {
+        if (!failed && !(i == SH_IMG ? mbar_wait<true>(bar(i), 0) : mbar_wait(bar(i), 0))) { failed = true; fail_site = line; }
+        return !failed;
+    };
 
-    // ---- the tile's partial softmax and output ----------------------------------------------------------------
-    if (!empty) {
-        if (warp == 8) {
-            if (lane == 0) {
-                mbar_expect_tx(bar(SH_QK), kOperandBytes + (uint32_t)p.chunk_rows * (HILO ? 512u : 256u));
-                for (int h = 0; h < 2; ++h) {
-                    load_q<BY_UNIT>(sbase + SH_OFF_Q + h * kHalfBytes, &map_q, bar(SH_QK), h * 64, 0, unit, p.R);
-                    tma_load_4d(sbase + SH_OFF_K + h * kHalfBytes, &map_k, bar(SH_QK), h * 64, t0, g, b);
-                    if (HILO) load_q<BY_UNIT>(sbase + SH_OFF_Q + h * kHalfBytes + kHalfBytes / 2, &map_q, bar(SH_QK), h * 64, 0, unit, p.R);
-                }
-                mbar_expect_tx(bar(SH_V), kOperandBytes);
-                for (int h = 0; h < 2; ++h) tma_load_4d(sbase + SH_OFF_V + h * kHalfBytes, &map_v, bar(SH_V), h * 64, t0, g, b);
-                wait(SH_QK); wait(SH_V);                               // (the copies have landed before the CTA may exit)
+    if (warp == 8 && lane == 0) {
+        mbar_expect_tx(bar(SH_RX), (uint32_t)(my_rows * (empty ? n_src : n_src - 1)) * kParts * SH_PITCH);   // (its own part stays where it is)
+        if (!empty) {
+            mbar_expect_tx(bar(SH_QK), kOperandBytes + (uint32_t)p.chunk_rows * 256u * kParts);
+            for (int h = 0; h < 2; ++h) {
+                load_q<BY_UNIT>(sbase + SH_OFF_Q + h * kHalfBytes, &map_q, bar(SH_QK), h * 64, 0, unit, p.R);
+                tma_load_4d(sbase + SH_OFF_K + h * kHalfBytes, &map_k, bar(SH_QK), h * 64, t0, g, b);
+                if (HILO) load_q<BY_UNIT>(sbase + SH_OFF_Q + h * kHalfBytes + kHalfBytes / 2, &map_q, bar(SH_QK), h * 64, 0, unit, p.R);
             }
-        } else if (warp == 9) {
-            if (lane == 0) {
-                const uint32_t aq = desc_lo_k(dbase + SH_OFF_Q), ak = desc_lo_k(dbase + SH_OFF_K), av = desc_lo_mn(dbase + SH_OFF_V);
-                if (wait(SH_QK)) {
-                    tc_fence_after();
+            mbar_expect_tx(bar(SH_V), kOperandBytes);
+            for (int h = 0; h < 2; ++h) tma_load_4d(sbase + SH_OFF_V + h * kHalfBytes, &map_v, bar(SH_V), h * 64, t0, g, b);
+        }
+    }
+    __syncwarp();
+    cluster_wait();                                                    // (behind the copies' start)
+
+    if (warp == 8) {
+        // ============================================ copies ================================================
+        // (a wait that gives up anywhere leaves what was not copied as it is: every later wait then gives up as well)
+        if (!empty) {
+            wait(SH_QK, __LINE__); wait(SH_V, __LINE__);
+            const int rows = min(slice, p.R - lane * slice);           // of owner `lane`
+            if (wait(SH_STAGED, __LINE__) && lane < C && lane != rank && rows > 0)
+                for (uint32_t part = 0; part < kParts; ++part)         // (the low part's accumulators are rows 64 ..)
+                    copy_to_cta(cluster_addr(sbase + SH_OFF_RX + (rank * kParts + part) * slice * SH_PITCH, lane),
+                                sbase + SH_OFF_STAGE + (part * 64u + lane * slice) * SH_PITCH, (uint32_t)rows * SH_PITCH, cluster_addr(bar(SH_RX), lane));
+        }
+    } else if (warp == 9) {
+        // ============================================= MMAs =================================================
+        if (lane == 0 && !empty) {
+            const uint32_t aq = desc_lo_k(dbase + SH_OFF_Q), ak = desc_lo_k(dbase + SH_OFF_K);
+            if (wait(SH_QK, __LINE__)) {
+                tc_fence_after();
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        tc_mma(tS, desc_make(aq + desc_kstep(ks, kHalfBytes)), desc_make(ak + desc_kstep(ks, kHalfBytes)), idesc_bf16(TILE), ks > 0);
-                    tc_commit(bar(SH_S));
+                for (int ks = 0; ks < 8; ++ks)
+                    tc_mma(tS, desc_make(aq + desc_kstep(ks, kHalfBytes)), desc_make(ak + desc_kstep(ks, kHalfBytes)), idesc_bf16(TILE), ks > 0);
+                tc_commit(bar(SH_S));
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        tc_mma(tZ, desc_make(ak + desc_kstep(ks, kHalfBytes)), desc_make(aq + desc_kstep(ks, kHalfBytes)), idesc_bf16(p.chunk_rows), ks > 0);
-                }
-                if (wait(SH_V) && wait(SH_P)) {
-                    tc_fence_after();
-#pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)
-                        tc_mma_ts(tO, tS + ks * 8, desc_make(av + ks * (2048 >> 4)), idesc_bf16(kD) | (1u << 16), ks > 0);
-                    tc_commit(bar(SH_ODONE));
-                }
+                for (int ks = 0; ks < 8; ++ks)
+                    tc_mma(tZ, desc_make(ak + desc_kstep(ks, kHalfBytes)), desc_make(aq + desc_kstep(ks, kHalfBytes)), idesc_bf16(p.chunk_rows), ks > 0);
             }
-        } else {
-            const int w = warp >> 2, lane_grp = warp & 3, row = lane_grp * 32 + lane;
-            const uint32_t lane_addr = (uint32_t)(lane_grp * 32) << 16;
+            if (wait(SH_V, __LINE__) && wait(SH_P, __LINE__)) {
+                tc_fence_after();
+                const uint32_t av = desc_lo_mn(dbase + SH_OFF_V);
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks)                         // (P of tokens 64 .. stands over the logits of those)
+                    tc_mma_ts(tO, tS + (ks >> 2) * 64 + (ks & 3) * 8, desc_make(av + ks * (2048 >> 4)), idesc_bf16(kD) | (1u << 16), ks > 0);
+                tc_commit(bar(SH_ODONE));
+            }
+            if (wait(SH_IMG, __LINE__)) {
+                asm volatile("fence.proxy.async;" ::: "memory");       // (the image was written by plain stores)
+                tc_fence_after();
+                const uint32_t av = desc_lo_k(dbase + SH_OFF_V), bo = desc_lo_k(dbase + SH_OFF_O);
+#pragma unroll
+                for (int ks = 0; ks < 8; ++ks)
+                    tc_mma(tT, desc_make(av + desc_kstep(ks, kHalfBytes)), desc_make(bo + desc_kstep(ks, kHalfBytes)), idesc_bf16((int)kParts * p.chunk_rows), ks > 0);
+                tc_commit(bar(SH_T));
+            }
+        }
+    } else if (warp >= 10) {
+        // ========================================== value norms =============================================
+        if (!empty && wait(SH_V, __LINE__)) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+                const int tok = (int)threadIdx.x - 320 + 64 * j;
+                float l2, l1;
+                value_norms<(VARS & OBC_VAR_VATP) != 0>(smem + SH_OFF_V, tok, l2, l1);
+                sNv[tok] = make_float2(l2, l1);
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(bar(SH_NORMS));
+    } else {
+        const int w = warp >> 2, lane_grp = warp & 3, row = lane_grp * 32 + lane;
+        const uint32_t lane_addr = (uint32_t)(lane_grp * 32) << 16;
+        // ================= the tile's softmax and partial output: warpgroup w takes tokens [64 w, 64 w + 64) =================
+        if (!empty) {
             const bool low_part = HILO && lane_grp >= 2;               // this warp's rows are the second copies of rows 0..63
             const int r = HILO ? row & 63 : row;
-            const bool valid = r < p.R;
-            const int owner = valid ? r / slice : 0, local = valid ? r % slice : 0;    // of the row's slice
-            const int src = HILO ? 2 * rank + (low_part ? 1 : 0) : rank;
-            const uint32_t rx_row = (uint32_t)(src * slice + local);
-            if (w == 0) {
-                float m = -INFINITY, l = 0.f;
-                if (wait(SH_S)) {
-                    tc_fence_after();
-                    const int last = valid ? (p.causal ? min(Nm - p.W + (r % p.W), N - 1) : N - 1) : -1;   // last visible token
-                    const int nvis = last - t0 + 1;
-                    const bool masked = t0 + TILE > min(p.causal ? Nm - p.W + 1 : N, N) && __any_sync(0xffffffffu, nvis < TILE);
-                    softmax_tile(tS + lane_addr, 0u, nvis, masked, p.scale * kLog2e, valid, low_part, false, m, l);
+            const float sl2 = p.scale * kLog2e;
+            float* sMax = reinterpret_cast<float*>(smem + SH_OFF_MAX);
+            uint32_t z[32];
+            float mt = -INFINITY, l = 0.f;
+            const int last = r < p.R ? (p.causal ? min(Nm - p.W + (r % p.W), N - 1) : N - 1) : -1;   // last visible token
+            const int nvis = last - t0 - w * 64 + 1;                   // columns j < nvis are visible
+            const bool masked = __any_sync(0xffffffffu, nvis < 64);
+            const uint32_t tSw = tS + lane_addr + w * 64u;
+            auto load_logits = [&](int pc) {
+                tc_ld32(tSw + pc * 32, z);
+                tc_wait_ld32(z);
+                if (masked) {
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) if (pc * 32 + j >= nvis) z[j] = 0xff800000u;
                 }
-                if (t0 + TILE > N && wait(SH_V)) zero_rows_from(smem + SH_OFF_V, row, N - t0);   // V rows past the sequence must not reach the MMA
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(SH_P));
-                cluster_wait();
-                if (valid) {                                           // (the low part of P adds to O alone)
-                    const uint32_t at = cluster_addr(sbase + SH_OFF_ML + rx_row * 8u, owner);
-                    st_cluster2(at, __float_as_uint(m), low_part ? 0u : __float_as_uint(l));
-                }
-            } else {
-                if (wait(SH_V)) {
-                    float l2, l1;
-                    value_norms<(VARS & OBC_VAR_VATP) != 0>(smem + SH_OFF_V, row, l2, l1);
-                    sNv[row] = make_float2(l2, l1);
-                }
-                cluster_wait();
-            }
-            if (wait(SH_ODONE)) {
+            };
+            if (wait(SH_S, __LINE__)) {
                 tc_fence_after();
-                const uint32_t dst = cluster_addr(sbase + SH_OFF_RX + rx_row * 512u, owner);
 #pragma unroll 1
-                for (int q = 0; q < 2; ++q) {                          // warpgroup w: head-dim columns [64 w, 64 w + 64)
-                    uint32_t o[32];
-                    tc_ld32(tO + lane_addr + w * 64u + q * 32u, o);
-                    tc_wait_ld32(o);
+                for (int pc = 0; pc < 2; ++pc) {
+                    load_logits(pc);
+#pragma unroll
+                    for (int j = 0; j < 32; j += 2) mt = fmax3(mt, __uint_as_float(z[j]), __uint_as_float(z[j + 1]));
+                }
+            }
+            sMax[w * 128 + row] = mt;
+            asm volatile("bar.sync 1, 256;" ::: "memory");             // both warpgroups
+            mt = fmaxf(mt, sMax[(w ^ 1) * 128 + row]);
+            const float m = mt == -INFINITY ? mt : mt * sl2;
+            if (!failed) {
+                const float m_eff = m == -INFINITY ? 0.f : m;
+                const float2 sl2v = make_float2(sl2, sl2), negm = make_float2(-m_eff, -m_eff);
+                float2 lsum = make_float2(0.f, 0.f);
+#pragma unroll 1
+                for (int pc = 0; pc < 2; ++pc) {
+                    uint32_t pk[16];
+                    load_logits(pc);
+#pragma unroll
+                    for (int j = 0; j < 32; j += 2) {
+                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(z[j]), __uint_as_float(z[j + 1])), sl2v, negm);
+                        const float2 e = make_float2(fast_exp2(x.x), fast_exp2(x.y));
+                        lsum = __fadd2_rn(lsum, e);
+                        pk[j >> 1] = pack_bf16x2(e.x, e.y);
+                        if (low_part) {                                // P = bf16(P) + bf16(P - bf16(P)): the second term
+                            const float2 h = bf16x2_to_f32x2(pk[j >> 1]);
+                            pk[j >> 1] = pack_bf16x2(e.x - h.x, e.y - h.y);
+                        }
+                    }
+                    tc_st16(tSw + pc * 16, pk);
+                }
+                l = low_part ? 0.f : lsum.x + lsum.y;                  // (the low part of P adds to O alone)
+                tc_wait_st();
+            }
+            if (w == 1 && t0 + TILE > N && wait(SH_V, __LINE__)) zero_rows_from(smem + SH_OFF_V, row, N - t0);   // V rows past the sequence must not reach the MMA
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(SH_P));
+            if (wait(SH_ODONE, __LINE__)) {
+                tc_fence_after();
+                uint8_t* dst = smem + SH_OFF_STAGE + row * SH_PITCH;   // warpgroup w: head-dim columns [64 w, 64 w + 64)
+#pragma unroll 1
+                for (int pc = 0; pc < 2; ++pc) {
+                    tc_ld32(tO + lane_addr + w * 64u + pc * 32u, z);
+                    tc_wait_ld32(z);
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        if (valid)
-                            st_cluster4(dst + (uint32_t)(((w * 16 + q * 8 + j) ^ (row & 31)) << 4),
-                                        make_float4(__uint_as_float(o[4 * j]), __uint_as_float(o[4 * j + 1]), __uint_as_float(o[4 * j + 2]), __uint_as_float(o[4 * j + 3])));
+                        *reinterpret_cast<uint4*>(dst + w * 256 + pc * 128 + j * 16) = make_uint4(z[4 * j], z[4 * j + 1], z[4 * j + 2], z[4 * j + 3]);
                 }
+                float* ml = reinterpret_cast<float*>(dst + 512);       // (m, l of the first half, l of the second, -)
+                if (w == 0) { ml[0] = m; ml[1] = l; } else { ml[2] = l; }
                 tc_fence_before();
             }
+            fence_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(SH_STAGED));
         }
-        if (warp >= 8) { __syncwarp(); cluster_wait(); }
-    } else {
-        cluster_wait();
-    }
-    __syncwarp();
-    cluster_arrive();
-    cluster_wait();                                                    // the partial outputs of this CTA's slice are here
-    // ---- the slice's rows: merged, and handed to every CTA --------------------------------------------------------
-    if (warp < 8) {
-        const int rows = min(slice, p.R - rank * slice), parts = n_src * (HILO ? 2 : 1);
-        for (int local = warp; local < rows; local += 8) {
-            const int r = rank * slice + local;
-            const float2* ml = reinterpret_cast<const float2*>(smem + SH_OFF_ML) + local;    // part sp: ml[sp * slice]
-            const float2 mine = lane < parts ? ml[lane * slice] : make_float2(-INFINITY, 0.f);
-            const float M = warp_max(mine.x);
-            const float wt = mine.x == -INFINITY ? 0.f : exp2f(mine.x - M);
-            float L = 0.f;
-            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (int sp = 0; sp < parts; ++sp) {
-                const float f = __shfl_sync(0xffffffffu, wt, sp), l = __shfl_sync(0xffffffffu, mine.y, sp);
-                const float4 x = *reinterpret_cast<const float4*>(smem + SH_OFF_RX + (sp * slice + local) * 512 + ((lane ^ (r & 31)) << 4));   // (rows r and r + 64 swizzle alike)
-                L = fmaf(l, f, L);
-                o.x = fmaf(x.x, f, o.x); o.y = fmaf(x.y, f, o.y); o.z = fmaf(x.z, f, o.z); o.w = fmaf(x.w, f, o.w);
-            }
-            if (L > 0.f) { o.x /= L; o.y /= L; o.z /= L; o.w /= L; }
-            const float onorm = warp_sum((o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w));
-            const float lse2 = M + log2f(L);
-            const uint32_t h0 = pack_bf16x2(-2.f * o.x, -2.f * o.y), h1 = pack_bf16x2(-2.f * o.z, -2.f * o.w);
-            const float2 f0 = bf16x2_to_f32x2(h0), f1 = bf16x2_to_f32x2(h1);
-            const uint32_t l0 = pack_bf16x2(fmaf(-2.f, o.x, -f0.x), fmaf(-2.f, o.y, -f0.y)), l1 = pack_bf16x2(fmaf(-2.f, o.z, -f1.x), fmaf(-2.f, o.w, -f1.y));
-            // elements 4 lane .. of row r in the 128-byte swizzle of the operand
-            auto place = [&](int row) { return sbase + SH_OFF_O + (uint32_t)((lane >> 4) * kHalfBytes + row * 128 + ((((lane & 15) >> 1) ^ (row & 7)) << 4) + (lane & 1) * 8); };
-            for (int d = 0; d < C; ++d) {
-                st_cluster2(cluster_addr(place(r), d), h0, h1);
-                if (HILO) st_cluster2(cluster_addr(place(p.chunk_rows + r), d), l0, l1);
-            }
-            if (lane < C) {
-                const uint32_t at = cluster_addr(sbase + SH_OFF_CONST + (uint32_t)((r >> 1) * 16 + (r & 1) * 4), lane);
-                st_cluster1(at, -lse2 * kExpFactor<VARS, HILO>);
-                st_cluster1(at + 8, onorm * (VARS == OBC_VAR_VK ? p.scale : 1.f));
+        // ==================== the slice's rows: merged, row by row of a warp, two at a time ====================
+        if ((empty || wait(SH_STAGED, __LINE__)) && wait(SH_RX, __LINE__)) {
+            const int parts = n_src * (int)kParts;
+            auto part_row = [&](int sp, int local) {
+                const int mine = HILO ? sp - 2 * rank : sp - rank;     // 0 (and 1: the low part): this CTA's own
+                return smem + (mine >= 0 && mine < (int)kParts ? SH_OFF_STAGE + (uint32_t)(mine * 64 + rank * slice + local) * SH_PITCH
+                                                               : SH_OFF_RX + (uint32_t)(sp * slice + local) * SH_PITCH);
+            };
+#pragma unroll 1
+            for (int local = warp; local < my_rows; local += 8) {
+                const int r = rank * slice + local;
+                const float4 ml = lane < parts ? *reinterpret_cast<const float4*>(part_row(lane, local) + 512) : make_float4(-INFINITY, 0.f, 0.f, 0.f);
+                const float M = warp_max(ml.x), wt = ml.x == -INFINITY ? 0.f : exp2f(ml.x - M), L = warp_sum((ml.y + ml.z) * wt);
+                float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+                for (int sp = 0; sp < parts; ++sp) {
+                    const float f = __shfl_sync(0xffffffffu, wt, sp);
+                    const float4 x = *reinterpret_cast<const float4*>(part_row(sp, local) + lane * 16);
+                    o.x = fmaf(x.x, f, o.x); o.y = fmaf(x.y, f, o.y); o.z = fmaf(x.z, f, o.z); o.w = fmaf(x.w, f, o.w);
+                }
+                const float inv = L > 0.f ? 1.f / L : 1.f;
+                o.x *= inv; o.y *= inv; o.z *= inv; o.w *= inv;
+                const float onorm = warp_sum((o.x * o.x + o.y * o.y) + (o.z * o.z + o.w * o.w));
+                const uint32_t h0 = pack_bf16x2(-2.f * o.x, -2.f * o.y), h1 = pack_bf16x2(-2.f * o.z, -2.f * o.w);
+                const float2 f0 = bf16x2_to_f32x2(h0), f1 = bf16x2_to_f32x2(h1);   // HILO: and what the high part leaves out
+                const uint32_t e0 = pack_bf16x2(fmaf(-2.f, o.x, -f0.x), fmaf(-2.f, o.y, -f0.y)), e1 = pack_bf16x2(fmaf(-2.f, o.z, -f1.x), fmaf(-2.f, o.w, -f1.y));
+                // elements 4 lane .. of the row in the 128-byte swizzle of the operand
+                auto place = [&](int at) { return sbase + SH_OFF_O + (uint32_t)((lane >> 4) * kHalfBytes + at * 128 + ((((lane & 15) >> 1) ^ (at & 7)) << 4) + (lane & 1) * 8); };
+                const uint32_t hi = place(r), lo = place(p.chunk_rows + r);
+#pragma unroll 2
+                for (int d = 0; d < C; ++d) {
+                    st_cluster2(cluster_addr(hi, d), h0, h1);
+                    if (HILO) st_cluster2(cluster_addr(lo, d), e0, e1);
+                }
+                if (lane < C) st_cluster2(cluster_addr(sbase + SH_OFF_ROWS + (uint32_t)r * 16u, lane), __float_as_uint(-(M + log2f(L))), __float_as_uint(onorm));
             }
         }
-        asm volatile("fence.proxy.async;" ::: "memory");
-    }
-    __syncwarp();
-    cluster_arrive();
-    cluster_wait();                                                    // -2 O and the constants are complete; no CTA writes to another from here on
-    // ---- the tile's scores -----------------------------------------------------------------------------------------
-    const size_t plane = (size_t)p.B * p.Hkv * p.Nmax;
-    if (empty) {
-        if (warp < 4 && t0 + (int)threadIdx.x < p.Nmax)
-            for (int pl = 0; pl < __popc(p.variants); ++pl) p.scores[(size_t)pl * plane + (size_t)unit * p.Nmax + t0 + threadIdx.x] = 0.f;
-    } else if (warp == 9) {
-        if (lane == 0 && !failed) {
+        if (warp < my_rows) {
             asm volatile("fence.proxy.async;" ::: "memory");
-            tc_fence_after();
-            const uint32_t av = desc_lo_k(dbase + SH_OFF_V), bo = desc_lo_k(dbase + SH_OFF_O);
-#pragma unroll
-            for (int ks = 0; ks < 8; ++ks)
-                tc_mma(tT, desc_make(av + desc_kstep(ks, kHalfBytes)), desc_make(bo + desc_kstep(ks, kHalfBytes)), idesc_bf16(HILO ? 2 * p.chunk_rows : p.chunk_rows), ks > 0);
-            tc_commit(bar(SH_T));
+            __syncwarp();
+            if (lane < C) arrive_at_cta(cluster_addr(bar(SH_IMG), lane));
         }
-    } else if (warp < 8) {
-        const int half = warp >> 2, lane_grp = warp & 3, tok = lane_grp * 32 + lane, ptok = t0 + tok;
-        const int rows0 = min(p.chunk_rows, (p.chunk_rows / 2 + 15) / 16 * 16);        // two runs of whole 16-row batches
-        const int r_begin = half ? rows0 : 0, r_count = half ? p.chunk_rows - rows0 : rows0;
-        const float ksl = p.scale * kLog2e * kExpFactor<VARS, HILO>;
-        const float2 sl2 = make_float2(ksl, ksl), sc = make_float2(p.scale, p.scale);
-        const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
-        RowSums S;
-        S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
-        if (wait(SH_T) && r_count > 0) {
-            tc_fence_after();
-            const float4* cst = reinterpret_cast<const float4*>(sConst) + (r_begin >> 1);
-            const uint32_t zt = tZ + ((uint32_t)(lane_grp * 32) << 16) + (uint32_t)r_begin, tt = zt + 128u;
-            if (masked_tile) score_chunk<VARS, true, HILO>(zt, tt, r_count, cst, sl2, sc, S, ptok, Nm - p.W, p.W, r_begin % p.W, p.chunk_rows);
-            else score_chunk<VARS, false, HILO>(zt, tt, r_count, cst, sl2, sc, S, ptok, 0, 0, 0, p.chunk_rows);
-            tc_fence_before();
-        }
-        float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
-        if (half == 1) {
+        // ========================================= the tile's scores =========================================
+        const size_t plane = (size_t)p.B * p.Hkv * p.Nmax;
+        const int tok = row, ptok = t0 + tok;
+        if (empty) {
+            if (w == 0 && ptok < p.Nmax)
+                for (int pl = 0; pl < __popc(p.variants); ++pl) p.scores[(size_t)pl * plane + (size_t)unit * p.Nmax + ptok] = 0.f;
+            wait(SH_IMG, __LINE__);
+        } else {
+            const int rows0 = min(p.chunk_rows, (p.chunk_rows / 2 + 15) / 16 * 16);    // two runs of whole 16-row batches
+            const int r_begin = w ? rows0 : 0, r_count = w ? p.chunk_rows - rows0 : rows0;
+            const float ksl = p.scale * kLog2e * kExpFactor<VARS, HILO>;
+            const float2 sl2 = make_float2(ksl, ksl), sc = make_float2(p.scale, p.scale);
+            const bool masked_tile = p.causal && (t0 + TILE - 1 > Nm - p.W);
+            RowSums S;
+            S.s1 = S.s2 = S.s3 = S.s4 = S.s5 = S.s6 = S.s7 = make_float2(0.f, 0.f);
+            float4* my_const = reinterpret_cast<float4*>(smem + SH_OFF_CONST) + warp * 32;
+            if (wait(SH_IMG, __LINE__) && lane * 2 < r_count) {
+                const float4 c0 = sRows[r_begin + 2 * lane], c1 = sRows[r_begin + 2 * lane + 1];
+                constexpr float kx = kExpFactor<VARS, HILO>;
+                const float ko = VARS == OBC_VAR_VK ? p.scale : 1.f;
+                my_const[lane] = make_float4(c0.x * kx, c1.x * kx, c0.y * ko, c1.y * ko);
+            }
+            __syncwarp();
+            if (wait(SH_T, __LINE__) && r_count > 0) {
+                tc_fence_after();
+                const uint32_t zt = tZ + lane_addr + (uint32_t)r_begin, tt = zt + 128u;
+                if (masked_tile) score_chunk<VARS, true, HILO>(zt, tt, r_count, my_const, sl2, sc, S, ptok, Nm - p.W, p.W, r_begin % p.W, p.chunk_rows);
+                else score_chunk<VARS, false, HILO>(zt, tt, r_count, my_const, sl2, sc, S, ptok, 0, 0, 0, p.chunk_rows);
+                tc_fence_before();
+            }
+            float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
+            if (w == 1) {
 #pragma unroll
-            for (int j = 0; j < kNumSums; ++j) sXch[j * TILE + tok] = sum[j];
-        }
-        asm volatile("bar.sync 1, 256;" ::: "memory");                 // both warpgroups
-        if (half == 0) {
+                for (int j = 0; j < kNumSums; ++j) sXch[j * TILE + tok] = sum[j];
+            }
+            asm volatile("bar.sync 1, 256;" ::: "memory");             // both warpgroups
+            if (w == 0) {
+                wait(SH_NORMS, __LINE__);
+                const float2 nv = sNv[tok];
 #pragma unroll
-            for (int j = 0; j < kNumSums; ++j) sum[j] += sXch[j * TILE + tok];
-            const float2 nv = sNv[tok];
-            if (ptok < p.Nmax)
-                store_scores<VARS, HILO>(sum, nv.x, nv.y, p.scale, p.variants, p.scores + (size_t)unit * p.Nmax + ptok, plane, ptok < N);
+                for (int j = 0; j < kNumSums; ++j) sum[j] += sXch[j * TILE + tok];
+                if (ptok < p.Nmax)
+                    store_scores<VARS, HILO>(sum, nv.x, nv.y, p.scale, p.variants, p.scores + (size_t)unit * p.Nmax + ptok, plane, ptok < N);
+            }
         }
     }
     if (failed) atomicCAS(p.status, 0u, (unsigned)(fail_site > 0 ? fail_site : 1));   // the first failure is kept
@@ -2154,7 +2243,6 @@ static size_t tc_partial_bytes(const ScoreShape& s) {
 size_t tc_workspace_bytes(const ScoreShape& s) { return make_tc_plan(s).bytes + tc_partial_bytes(s); }
 
 // How many clusters of 2, 4, 8 and 16 CTAs of tc_short_kernel the current device runs at once, asked once per host thread and device
-static_assert(SH_RX_ROWS >= 128 + SH_MAXC - 1 && SH_RX_ROWS >= 2 * (63 + SH_MAXC - 1), "partial outputs of a slice");
 static int short_clusters(int C) {
     if (C == 1) return sm_count();
     thread_local struct { int dev, of[4]; } seen{-1, {}};
@@ -2180,7 +2268,8 @@ static int short_clusters(int C) {
     return seen.of[C == 2 ? 0 : C == 4 ? 1 : C == 8 ? 2 : 3];
 }
 // Cluster size for a call that one kernel serves (tc_short_kernel), or 0: up to 128 window rows, a tile per CTA, all units side by side
-// (a second wave of clusters would take longer than the three kernels' other two: both sides at the kernel).
+// (with a second wave of clusters three kernels are the faster ones: 8 heads of 2048 x 32 rows 18.2 / 21.5 us, 4 x 128 rows 20 / 32, 16 of 1024 x 128
+// rows 19.4 / 28.6, 30 of 1000 x 64 rows 20.4 / 24.5, 148 of 256 x 64 rows 22.4 / 25.6; measured with the exchange by plain stores).
 static int short_cluster_size(const ScoreShape& s, const TcChunks& ch) {
     const int tiles = (s.Nmax + TILE - 1) / TILE, units = s.B * s.Hkv;
     if (ch.n_chunks > 1 || tiles > SH_MAXC) return 0;
