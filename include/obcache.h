@@ -174,7 +174,8 @@ obc_status obc_score_status(const void* workspace, void* stream);
  * the window-statistics kernel and of the fused score kernel folds its first and its last reading
  * of the GPU's nanosecond timer into four words of the workspace header; this call synchronises
  * `stream`, returns latest end - earliest start of each kernel in microseconds (host pointers;
- * 0 when nothing was recorded, e.g. on the CUDA-core path) and zeroes the words.  The figures
+ * 0 when nothing was recorded, e.g. on the CUDA-core path; a short cache is scored by one kernel,
+ * whose extent is pass2_us) and zeroes the words.  The figures
  * cover the launches since the words were last zero, so zero the workspace header (or call this
  * once) before the obc_score call to be measured, and measure one call at a time.  Unlike an event
  * pair around the launch, the span leaves out launch latency and keeps the overlap of consecutive
