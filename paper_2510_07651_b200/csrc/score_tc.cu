@@ -1781,7 +1781,9 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 // cluster; the scores of the tile follow from the K and V tiles that are still there (Z from before K and Q made room for the staged O).
 // Partial outputs cross the cluster as bulk copies of runs of staged rows, the merged rows as plain stores; both arrive on the
 // receiver's mbarriers, and a CTA that has seen its image complete has neither copies out of its memory nor stores into it under way
-// (its owners have merged what it sent, and all that it receives is counted).
+// (its owners have merged what it sent, and all that it receives is counted).  A warp whose wait gives up arrives nowhere any more and
+// copies and stores nothing more, so that nobody takes what is missing for complete; its CTA stays until the cluster's other CTAs are
+// done with it (end of the kernel).
 // The code runs once per launch, from a cold instruction cache: loops are kept short rather than unrolled.
 //   warps 0-7  softmax (64 tokens of the tile per warpgroup), merge, score epilogue (half of the rows per warpgroup)
 //   warp 8  copies     warp 9  MMAs     warps 10-11  value norms
@@ -1808,7 +1810,7 @@ constexpr uint32_t SH_OFF_CONST = SH_OFF_ROWS + 128 * 16;          // 8 epilogue
 constexpr uint32_t SH_OFF_MAX = SH_OFF_CONST + 8 * 32 * 16;        // [2][128]: row maxima of the tile's halves
 constexpr uint32_t SH_OFF_NV = SH_OFF_MAX + 2 * 128 * 4;           // [128] (||v||^2, ||v||_1)
 constexpr uint32_t SH_OFF_BAR = SH_OFF_NV + TILE * 8;
-enum { SH_QK = 0, SH_V, SH_S, SH_P, SH_ODONE, SH_STAGED, SH_RX, SH_IMG, SH_NORMS, SH_T, SH_NBARS };
+enum { SH_QK = 0, SH_V, SH_S, SH_P, SH_ODONE, SH_STAGED, SH_RX, SH_IMG, SH_NORMS, SH_T, SH_DRAIN, SH_NBARS };
 constexpr uint32_t SH_OFF_TMEM = SH_OFF_BAR + SH_NBARS * 8;
 constexpr uint32_t kSmemShort = SH_OFF_TMEM + 16 + 1024;
 static_assert(SH_OFF_V % 1024 == 0 && kSmemShort <= 227 * 1024, "layout");
@@ -1884,9 +1886,17 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const bool empty = t0 >= N;                                        // a CTA past the end merges its slice and writes zeros
     const int n_src = min(C, (N + TILE - 1) / TILE);                   // tiles of the unit = partial outputs of a row
     const uint32_t tS = tmem_base, tO = tmem_base + 128u, tZ = tmem_base + 256u, tT = tmem_base + 384u;
-    auto wait = [&](int i, int line) {
+    auto wait_one = [&](int i, int line) {                             // by one thread
         if (!failed && !(i == SH_IMG ? mbar_wait<true>(bar(i), 0) : mbar_wait(bar(i), 0))) { failed = true; fail_site = line; }
         return !failed;
+    };
+    auto wait = [&](int i, int line) {                                 // by a whole warp: its lanes go on together or not at all
+        if (__any_sync(0xffffffffu, !wait_one(i, line)) && !failed) { failed = true; fail_site = line; }
+        return !failed;
+    };
+    auto arrive = [&](int i) {                                         // for a whole warp
+        __syncwarp();
+        if (lane == 0 && !failed) mbar_arrive(bar(i));
     };
 
     if (warp == 8 && lane == 0) {
@@ -1907,7 +1917,6 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
     if (warp == 8) {
         // ============================================ copies ================================================
-        // (a wait that gives up anywhere leaves what was not copied as it is: every later wait then gives up as well)
         if (!empty) {
             wait(SH_QK, __LINE__); wait(SH_V, __LINE__);
             const int rows = min(slice, p.R - lane * slice);           // of owner `lane`
@@ -1920,7 +1929,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // ============================================= MMAs =================================================
         if (lane == 0 && !empty) {
             const uint32_t aq = desc_lo_k(dbase + SH_OFF_Q), ak = desc_lo_k(dbase + SH_OFF_K);
-            if (wait(SH_QK, __LINE__)) {
+            if (wait_one(SH_QK, __LINE__)) {
                 tc_fence_after();
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
@@ -1930,7 +1939,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 for (int ks = 0; ks < 8; ++ks)
                     tc_mma(tZ, desc_make(ak + desc_kstep(ks, kHalfBytes)), desc_make(aq + desc_kstep(ks, kHalfBytes)), idesc_bf16(p.chunk_rows), ks > 0);
             }
-            if (wait(SH_V, __LINE__) && wait(SH_P, __LINE__)) {
+            if (wait_one(SH_V, __LINE__) && wait_one(SH_P, __LINE__)) {
                 tc_fence_after();
                 const uint32_t av = desc_lo_mn(dbase + SH_OFF_V);
 #pragma unroll
@@ -1938,7 +1947,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     tc_mma_ts(tO, tS + (ks >> 2) * 64 + (ks & 3) * 8, desc_make(av + ks * (2048 >> 4)), idesc_bf16(kD) | (1u << 16), ks > 0);
                 tc_commit(bar(SH_ODONE));
             }
-            if (wait(SH_IMG, __LINE__)) {
+            if (wait_one(SH_IMG, __LINE__)) {
                 asm volatile("fence.proxy.async;" ::: "memory");       // (the image was written by plain stores)
                 tc_fence_after();
                 const uint32_t av = desc_lo_k(dbase + SH_OFF_V), bo = desc_lo_k(dbase + SH_OFF_O);
@@ -1959,8 +1968,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 sNv[tok] = make_float2(l2, l1);
             }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar(SH_NORMS));
+        arrive(SH_NORMS);
     } else {
         const int w = warp >> 2, lane_grp = warp & 3, row = lane_grp * 32 + lane;
         const uint32_t lane_addr = (uint32_t)(lane_grp * 32) << 16;
@@ -2023,8 +2031,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
             }
             if (w == 1 && t0 + TILE > N && wait(SH_V, __LINE__)) zero_rows_from(smem + SH_OFF_V, row, N - t0);   // V rows past the sequence must not reach the MMA
             tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(SH_P));
+            arrive(SH_P);
             if (wait(SH_ODONE, __LINE__)) {
                 tc_fence_after();
                 uint8_t* dst = smem + SH_OFF_STAGE + row * SH_PITCH;   // warpgroup w: head-dim columns [64 w, 64 w + 64)
@@ -2041,8 +2048,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 tc_fence_before();
             }
             fence_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(SH_STAGED));
+            arrive(SH_STAGED);
         }
         // ==================== the slice's rows: merged, row by row of a warp, two at a time ====================
         if ((empty || wait(SH_STAGED, __LINE__)) && wait(SH_RX, __LINE__)) {
@@ -2081,7 +2087,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 if (lane < C) st_cluster2(cluster_addr(sbase + SH_OFF_ROWS + (uint32_t)r * 16u, lane), __float_as_uint(-(M + log2f(L))), __float_as_uint(onorm));
             }
         }
-        if (warp < my_rows) {
+        if (warp < my_rows && !failed) {
             asm volatile("fence.proxy.async;" ::: "memory");
             __syncwarp();
             if (lane < C) arrive_at_cta(cluster_addr(bar(SH_IMG), lane));
@@ -2117,13 +2123,12 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 tc_fence_before();
             }
             float sum[kNumSums] = {S.s1.x + S.s1.y, S.s2.x + S.s2.y, S.s3.x + S.s3.y, S.s4.x + S.s4.y, S.s5.x + S.s5.y, S.s6.x + S.s6.y, S.s7.x + S.s7.y};
-            if (w == 1) {
+            if (w == 1 && !failed) {
 #pragma unroll
                 for (int j = 0; j < kNumSums; ++j) sXch[j * TILE + tok] = sum[j];
             }
             asm volatile("bar.sync 1, 256;" ::: "memory");             // both warpgroups
-            if (w == 0) {
-                wait(SH_NORMS, __LINE__);
+            if (w == 0 && wait(SH_NORMS, __LINE__)) {
                 const float2 nv = sNv[tok];
 #pragma unroll
                 for (int j = 0; j < kNumSums; ++j) sum[j] += sXch[j * TILE + tok];
@@ -2134,7 +2139,19 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     }
     if (failed) atomicCAS(p.status, 0u, (unsigned)(fail_site > 0 ? fail_site : 1));   // the first failure is kept
     tc_fence_before();
-    __syncthreads();
+    if (__syncthreads_or(failed)) {
+        // Copies into this CTA or out of it may be under way or still to come from CTAs that are only late.  Those where no wait gave up need
+        // none of this: they saw their image complete, and a thread that has left counts as arrived.  Every wait of the others is bounded.
+        cluster_arrive(); cluster_wait();                              // nobody issues anything more
+        if (threadIdx.x == 0) {                                        // what was issued lands: rows of other CTAs, tiles
+            (void)mbar_wait(bar(SH_RX), 0);
+            if (!empty) { (void)mbar_wait(bar(SH_QK), 0); (void)mbar_wait(bar(SH_V), 0); }
+        } else if (threadIdx.x == 288) {                               // the thread that issued the MMAs
+            tc_commit(bar(SH_DRAIN));
+            (void)mbar_wait(bar(SH_DRAIN), 0);
+        }
+        cluster_arrive(); cluster_wait();                              // ... in every CTA, so that what went out of this one has been read
+    }
     span_end(p.span);
     if (warp == 8) {
         tc_fence_after();
