@@ -1886,18 +1886,12 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
     const bool empty = t0 >= N;                                        // a CTA past the end merges its slice and writes zeros
     const int n_src = min(C, (N + TILE - 1) / TILE);                   // tiles of the unit = partial outputs of a row
     const uint32_t tS = tmem_base, tO = tmem_base + 128u, tZ = tmem_base + 256u, tT = tmem_base + 384u;
-    auto wait_one = [&](int i, int line) {                             // by one thread
+    auto wait = [&](int i, int line) {
         if (!failed && !(i == SH_IMG ? mbar_wait<true>(bar(i), 0) : mbar_wait(bar(i), 0))) { failed = true; fail_site = line; }
         return !failed;
     };
-    auto wait = [&](int i, int line) {                                 // by a whole warp: its lanes go on together or not at all
-        if (__any_sync(0xffffffffu, !wait_one(i, line)) && !failed) { failed = true; fail_site = line; }
-        return !failed;
-    };
-    auto arrive = [&](int i) {                                         // for a whole warp
-        __syncwarp();
-        if (lane == 0 && !failed) mbar_arrive(bar(i));
-    };
+    auto none_failed = [&] { __syncwarp(); return __all_sync(0xffffffffu, !failed) != 0; };   // in the calling warp
+    auto arrive = [&](int i) { if (none_failed() && lane == 0) mbar_arrive(bar(i)); };         // for a whole warp
 
     if (warp == 8 && lane == 0) {
         mbar_expect_tx(bar(SH_RX), (uint32_t)(my_rows * (empty ? n_src : n_src - 1)) * kParts * SH_PITCH);   // (its own part stays where it is)
@@ -1929,7 +1923,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
         // ============================================= MMAs =================================================
         if (lane == 0 && !empty) {
             const uint32_t aq = desc_lo_k(dbase + SH_OFF_Q), ak = desc_lo_k(dbase + SH_OFF_K);
-            if (wait_one(SH_QK, __LINE__)) {
+            if (wait(SH_QK, __LINE__)) {
                 tc_fence_after();
 #pragma unroll
                 for (int ks = 0; ks < 8; ++ks)
@@ -1939,7 +1933,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 for (int ks = 0; ks < 8; ++ks)
                     tc_mma(tZ, desc_make(ak + desc_kstep(ks, kHalfBytes)), desc_make(aq + desc_kstep(ks, kHalfBytes)), idesc_bf16(p.chunk_rows), ks > 0);
             }
-            if (wait_one(SH_V, __LINE__) && wait_one(SH_P, __LINE__)) {
+            if (wait(SH_V, __LINE__) && wait(SH_P, __LINE__)) {
                 tc_fence_after();
                 const uint32_t av = desc_lo_mn(dbase + SH_OFF_V);
 #pragma unroll
@@ -1947,7 +1941,7 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                     tc_mma_ts(tO, tS + (ks >> 2) * 64 + (ks & 3) * 8, desc_make(av + ks * (2048 >> 4)), idesc_bf16(kD) | (1u << 16), ks > 0);
                 tc_commit(bar(SH_ODONE));
             }
-            if (wait_one(SH_IMG, __LINE__)) {
+            if (wait(SH_IMG, __LINE__)) {
                 asm volatile("fence.proxy.async;" ::: "memory");       // (the image was written by plain stores)
                 tc_fence_after();
                 const uint32_t av = desc_lo_k(dbase + SH_OFF_V), bo = desc_lo_k(dbase + SH_OFF_O);
@@ -2087,10 +2081,9 @@ tc_short_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
                 if (lane < C) st_cluster2(cluster_addr(sbase + SH_OFF_ROWS + (uint32_t)r * 16u, lane), __float_as_uint(-(M + log2f(L))), __float_as_uint(onorm));
             }
         }
-        if (warp < my_rows && !failed) {
+        if (warp < my_rows) {
             asm volatile("fence.proxy.async;" ::: "memory");
-            __syncwarp();
-            if (lane < C) arrive_at_cta(cluster_addr(bar(SH_IMG), lane));
+            if (none_failed() && lane < C) arrive_at_cta(cluster_addr(bar(SH_IMG), lane));
         }
         // ========================================= the tile's scores =========================================
         const size_t plane = (size_t)p.B * p.Hkv * p.Nmax;

@@ -15,9 +15,9 @@ def _kernel():
 
 def test_nothing_is_announced_after_a_failed_wait():
     body = _kernel()
-    assert [m for m in re.findall(r"[^\n;]*\bmbar_arrive\(", body) if "!failed" not in m] == []
-    remote = re.findall(r"if \(([^{}]*)\) \{[^{}]*arrive_at_cta\(", body)
-    assert remote and len(remote) == body.count("arrive_at_cta(") and all("!failed" in c for c in remote)
+    arrivals = re.findall(r"[^\n;{}]*\b(?:mbar_arrive|arrive_at_cta)\(", body)
+    assert len(arrivals) == 2 and all("none_failed() &&" in a for a in arrivals)
+    assert re.search(r"none_failed = [^;]*;[^;]*__all_sync\(0xffffffffu, !failed\)", body)
     assert re.search(r"if \(wait\(SH_STAGED, __LINE__\)[^;{}]*\)\s*for \([^;]*;[^;]*;[^)]*\)\s*copy_to_cta\(", body)
     assert re.search(r"wait\(SH_RX, __LINE__\)\) \{(?:(?!\n        \}).)*st_cluster2\(", body, re.S)
 
