@@ -52,6 +52,9 @@ def test_config4_ragged_batch_reduced(path):
     (200, 1, 4, 1, "bf16", True),         # W = 1 (decode-like), R = 4
     (333, 5, 8, 2, "f32", False),         # non-causal
     (1000, 40, 4, 2, "bf16", True),       # R = 80: not a multiple of the row chunk
+    (2333, 5, 8, 2, "bf16", False),       # longer than one kernel takes: pass 1, merge and pass 2, non-causal,
+    (2100, 1, 4, 1, "bf16", True),        # W = 1
+    (2049, 40, 4, 2, "bf16", True),       # and R = 80 with one token in the last tile
 ])
 def test_small_and_degenerate_shapes(N, W, Hq, Hkv, dtype, causal):
     case = synth.make_prefill("edge", B=2, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype=dtype, seed=77 + N,
@@ -88,6 +91,10 @@ def test_tensor_core_row_counts(N, W, Hq, Hkv):
     (3001, 32, 4, 4),        # several tiles per split, no groups
     (1500, 12, 12, 3),       # R = 48: the row halves of pass 2 are 32 and 16
     (700, 63, 1, 1),         # R = 63: the largest row count of this path, one padding row
+    (2177, 1, 7, 1),         # the same row counts beyond 2048 tokens, where pass 1, the merge of its splits and pass 2 are kernels of
+    (2049, 17, 1, 1),        # their own: 9, 15, 0 and 1 padding rows
+    (2500, 12, 12, 3),
+    (2305, 63, 1, 1),
 ])
 def test_fewer_than_64_window_rows(N, W, Hq, Hkv):
     """bf16 caches with fewer than 64 window rows: attention weights and outputs travel as two bf16 parts, so the scores
@@ -115,9 +122,11 @@ def test_full_history_window(N, Hq, Hkv, dtype, path):
     _check(case, ["V", "K", "VK", "ATTN", "VATP"], path=path, tight=2e-2 if dtype == "bf16" else None)
 
 
-@pytest.mark.parametrize("N,W,Hq,Hkv", [(100, 40, 2, 2), (90, 20, 160, 80), (300, 5, 320, 160), (150, 16, 640, 160), (131, 50, 480, 160)])
+@pytest.mark.parametrize("N,W,Hq,Hkv", [(100, 40, 2, 2), (90, 20, 160, 80), (300, 5, 320, 160), (150, 16, 640, 160), (131, 50, 480, 160),
+                                         (100, 40, 170, 170), (90, 20, 340, 170)])
 def test_one_cta_per_head_and_chunk(N, W, Hq, Hkv):
-    # pass 1 writes the merged rows itself, padding rows included: R = 40 (two bf16 parts), 40, 10, 64 and 150 (two chunks)
+    # pass 1 writes the merged rows itself, padding rows included: R = 40 (two bf16 parts), 40, 10, 64, 150 (two chunks), 40 and 40
+    # (the first two have all their heads side by side and are scored by one kernel; the last two are more heads than SMs)
     case = synth.make_prefill("direct", B=1, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=N + W, hh_frac=0.02)
     _check(case, ["K", "VK"], tight=2e-2)
     if Hq // Hkv * W < 64:                   # both parts of -2 O: the tolerance of 32-bit sums (see test_fewer_than_64_window_rows)
@@ -150,19 +159,21 @@ def test_row_chunks_shared_by_several_ctas(N, W, Hq, Hkv, lens):
     _check(case, ["V", "K", "VK", "ATTN"], tight=2e-2)
 
 
-def test_peaky_attention_cancellation_case():
+@pytest.mark.parametrize("N", [2048, 4100])      # one kernel; pass 1, merge and pass 2
+def test_peaky_attention_cancellation_case(N):
     # some attention weights approach 1, so ||v_p - o_i||^2 cancels heavily
-    case = synth.make_prefill("peaky", B=1, Hq=8, Hkv=2, d=128, W=16, N=2048, dtype="bf16", seed=5,
+    case = synth.make_prefill("peaky", B=1, Hq=8, Hkv=2, d=128, W=16, N=N, dtype="bf16", seed=5,
                               hh_frac=0.01, peaky=True)
     _check(case, ["V", "K", "VK"], path="simt")
     _check(case, ["V", "K", "VK"], path="auto")
 
 
-def test_strided_views_and_split_invariance():
+@pytest.mark.parametrize("N", [700, 2600])       # one kernel; pass 1, merge and pass 2
+def test_strided_views_and_split_invariance(N):
     # K/V given as non-contiguous views (token stride 2d) must score like their contiguous copies
-    case = synth.make_prefill("strided", B=1, Hq=4, Hkv=2, d=128, W=8, N=700, dtype="bf16", seed=9)
+    case = synth.make_prefill("strided", B=1, Hq=4, Hkv=2, d=128, W=8, N=N, dtype="bf16", seed=9)
     q, k, v = H.upload(case)
-    wide_k = torch.zeros((1, 2, 700, 256), dtype=torch.bfloat16, device="cuda")
+    wide_k = torch.zeros((1, 2, N, 256), dtype=torch.bfloat16, device="cuda")
     wide_v = torch.zeros_like(wide_k)
     wide_k[..., :128] = k
     wide_v[..., :128] = v
@@ -214,13 +225,14 @@ def test_kernel_spans_are_recorded_and_cleared():
     assert api.obc_score_kernel_spans(ws2) == (0.0, 0.0)
 
 
+@pytest.mark.parametrize("N", [1500, 2600])      # one kernel; pass 1, merge and pass 2
 @pytest.mark.parametrize("Hq,Hkv,W", [(1, 1, 1), (2, 1, 1), (3, 1, 1)])
-def test_joint_score_near_its_zero(Hq, Hkv, W):
+def test_joint_score_near_its_zero(Hq, Hkv, W, N):
     """Tokens whose scaled logit is close to -1 for every window row: (1 + Z)^2 is then small against 1 + Z^2, and the joint
     score keeps its digits only if the square is taken row by row.  The joint score is the same whatever else is asked for,
     and is off by no more of its own value than a few times what an error of 3e-7 in Z (fp32 logits of magnitude 1, summed
     over 128 channels) does to it: 2 |1 + Z| |v|^2 3e-7 of a score of at least Z^2 |o|^2."""
-    N, scale = 1500, 128 ** -0.5
+    scale = 128 ** -0.5
     rng = np.random.default_rng(11)
     q = np.repeat(rng.standard_normal((1, 1, W, 128)), Hq, 1)
     k = rng.standard_normal((1, Hkv, N, 128))
@@ -239,10 +251,12 @@ def test_joint_score_near_its_zero(Hq, Hkv, W):
     assert own.max() < 2e-5, own.max()
 
 
-@pytest.mark.parametrize("Hq,Hkv,W,N", [(4, 2, 20, 300), (2, 2, 5, 700), (6, 2, 24, 500), (6, 2, 70, 400)])
+@pytest.mark.parametrize("Hq,Hkv,W,N", [(4, 2, 20, 300), (2, 2, 5, 700), (6, 2, 24, 500), (6, 2, 70, 400),
+                                         (4, 2, 20, 2300), (2, 2, 5, 2700), (6, 2, 24, 2500)])
 def test_queries_of_a_neighbour_that_are_not_finite(Hq, Hkv, W, N):
-    """Row counts that do not fill the MMA's rows (R = 40, 5, 72 and 210): what fills them up must not be the queries of the
-    next head or sequence, which may be anything (a masked batch item, say)."""
+    """Row counts that do not fill the MMA's rows (R = 40, 5, 72 in one kernel, 210 in the multi-chunk pass 2, and 40, 5, 72 again in
+    pass 1 and the single-chunk pass 2): what fills them up must not be the queries of the next head or sequence, which may be
+    anything (a masked batch item, say)."""
     case = synth.make_prefill("neighbour", B=2, Hq=Hq, Hkv=Hkv, d=128, W=W, N=N, dtype="bf16", seed=N, hh_frac=0.02)
     q, k, v = H.upload(case)
     variants = ["V", "K", "VK", "ATTN"]
@@ -264,3 +278,15 @@ def test_fewer_than_64_window_rows_on_many_heads(N, Hq, Hkv):
         mx = max(np.abs(want[n]).max() for n in variants if n in ("V", "K", "VK"))
         for n in variants:
             H.assert_scores_close(got[n], want[n], "f32", what=f"{case.name}/{n}", mx=None if n in ("ATTN", "VATP") else mx)
+
+
+@pytest.mark.parametrize("W", [8, 20])                           # 32 rows, two bf16 parts; 80, one
+def test_what_stands_past_a_ragged_end_is_not_used(W):
+    lens = [2100, 3000, 130]
+    case = synth.make_prefill("pastend", B=3, Hq=8, Hkv=2, d=128, W=W, N=lens, dtype="bf16", seed=W, hh_frac=0.02)
+    q, k, v = H.upload(case)
+    want = api.obc_score(q, k, v, seq_lens=H.lens_dev(case))
+    for b, n in enumerate(lens):
+        k[b, :, n:] = float("nan")
+        v[b, :, n:] = float("nan")
+    assert torch.equal(api.obc_score(q, k, v, seq_lens=H.lens_dev(case)), want)

@@ -1,5 +1,7 @@
 """Short caches scored by one kernel (a cluster of CTAs per KV head, one 128-token tile each): GPU parity at the edges of
 tiles, clusters and row counts."""
+import ctypes as C
+
 import numpy as np
 import pytest
 import torch
@@ -68,3 +70,62 @@ def test_one_kernel_and_three_agree(B, N):
     want = H.oracle_scores(case, ["VK"])["VK"][0]
     _check(got[0].cpu().numpy(), want, 32, np.abs(want).max())
     assert torch.equal(got, got[:1].expand_as(got))
+
+
+def _kernels(q, k, v):
+    """Scores, and 'one' or 'three': a call by one kernel leaves no extent of a pass 1."""
+    p = api.score_params(q, k)
+    ws = torch.zeros(api.obc_score_workspace(p), dtype=torch.uint8, device="cuda")
+    got = api.obc_score(q, k, v, workspace=ws)
+    api.obc_score_status(ws)
+    first, second = api.obc_score_kernel_spans(ws)
+    assert second > 0
+    return got, "three" if first > 0 else "one"
+
+
+@pytest.mark.parametrize("N,G,W", [(100, 4, 8), (128, 4, 20), (1024, 4, 4), (1100, 7, 16), (2048, 4, 32)])
+def test_which_kernels_run_and_that_they_agree(N, G, W):
+    """One head alone has its cluster on the chip; of more heads than SMs not all have.  The same head is scored by either path, to
+    their common error: 2e-5 where everything is summed in 32 bits, else (P and -2 O rounded to bf16 in either, of other partial sums) 2e-3."""
+    case = synth.make_prefill("paths", B=1, Hq=G, Hkv=1, d=128, W=W, N=N, dtype="bf16", seed=N)
+    q, k, v = H.upload(case)
+    one, path = _kernels(q, k, v)
+    assert path == "one"
+    many = torch.cuda.get_device_properties(0).multi_processor_count + 1
+    three, path = _kernels(*(x.expand(many, -1, -1, -1).contiguous() for x in (q, k, v)))
+    assert path == "three"
+    tight = 2e-5 if G * W < 64 else 2e-3
+    assert ((three - one).abs() <= tight * (one.abs() + 1e-3 * one.abs().max())).all()
+    longer = synth.make_prefill("longer", B=1, Hq=G, Hkv=1, d=128, W=W, N=2049, dtype="bf16", seed=N)
+    assert _kernels(*H.upload(longer))[1] == "three"
+
+
+@pytest.mark.parametrize("N,W,mask", [(300, 16, [310, 1000]), (5, 8, [9, 40]), (700, 30, [700, 729])])
+def test_one_kernel_on_a_shard(N, W, mask):
+    """Tokens that are one shard of a longer sequence: the mask counts from that sequence's end, and the window may be longer than the shard."""
+    case = synth.make_prefill("shard", B=2, Hq=4, Hkv=2, d=128, W=min(W, N), N=N, dtype="bf16", seed=N)
+    _, k, v = H.upload(case)
+    q = torch.randn((2, 4, W, 128), generator=torch.Generator().manual_seed(N)).to(torch.bfloat16).cuda()
+    m = torch.tensor(mask, dtype=torch.int32, device="cuda")
+    out = {}
+    for path in ("auto", "simt"):
+        p = api.score_params(q, k, path=path, mask_lens=m)
+        ws = torch.zeros(api.obc_score_workspace(p), dtype=torch.uint8, device="cuda")
+        out[path] = torch.empty((1, 2, 2, N), device="cuda")
+        torch.cuda.synchronize()
+        assert api.lib().obc_score(C.byref(p), *(api.as_tensor4(x) for x in (q, k, v)), out[path].data_ptr(), ws.data_ptr(), ws.numel(), None) == 0
+        api.obc_score_status(ws)
+        first, second = api.obc_score_kernel_spans(ws)
+        assert first == 0 and (second > 0) == (path == "auto")
+    _check(out["auto"].cpu().numpy(), out["simt"].cpu().numpy(), 2 * W, float(out["simt"].abs().max()))
+
+
+def test_one_kernel_lengths_below_the_window():
+    """A sequence of no tokens scores zero everywhere; one shorter than the window is scored by the rows that see any of it."""
+    case = synth.make_prefill("nothing", B=3, Hq=4, Hkv=2, d=128, W=16, N=400, dtype="bf16", seed=4)
+    q, k, v = H.upload(case)
+    lens = torch.tensor([0, 400, 7], dtype=torch.int32, device="cuda")
+    got = {path: api.obc_score(q, k, v, seq_lens=lens, path=path)[0].cpu().numpy() for path in ("auto", "simt")}
+    assert (got["auto"][0] == 0).all() and (got["auto"][2, :, 7:] == 0).all()
+    for b in (1, 2):
+        _check(got["auto"][b], got["simt"][b], 32, got["simt"][b].max())
