@@ -1775,7 +1775,7 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
 // =================================================================================================
 // A short cache in one kernel: both passes and the merge between them, for a unit whose tiles have a cluster of CTAs, one
-// tile each.  As three kernels such a call is mostly their beginnings and ends and the second trip of K and V.  A CTA forms the
+// tile each (CTAs beyond the tiles, where the cluster has some, take their share of the merge).  As three kernels such a call is mostly their beginnings and ends and the second trip of K and V.  A CTA forms the
 // logits, P and its part of O as pass 1 does; row slices of the partial outputs go to the CTA that owns the slice, which adds them
 // in the order of the tiles and hands -2 O (HILO: both parts), as the operand image, and the row constants to every CTA of the
 // cluster; the scores of the tile follow from the K and V tiles that are still there (Z from before K and Q made room for the staged O).
@@ -2277,15 +2277,23 @@ static int short_clusters(int C) {
     }
     return seen.of[C == 2 ? 0 : C == 4 ? 1 : C == 8 ? 2 : 3];
 }
-// Cluster size for a call that one kernel serves (tc_short_kernel), or 0: up to 128 window rows, a tile per CTA, all units side by side
-// (with a second wave of clusters three kernels are the faster ones: 8 heads of 2048 x 32 rows 18.2 / 21.5 us, 4 x 128 rows 20 / 32, 16 of 1024 x 128
-// rows 19.4 / 28.6, 30 of 1000 x 64 rows 20.4 / 24.5, 148 of 256 x 64 rows 22.4 / 25.6; measured with the exchange by plain stores).
+// Cluster size for a call that one kernel serves (tc_short_kernel), or 0: up to 128 window rows, a tile per CTA, all units side by side.
+// With a second wave of clusters three kernels are the faster ones, us three / one: 8 heads of 2048 x 32 rows 17.2 / 22.9, x 128 rows 19.0 / 27.4, 16 of
+// 1024 x 16 rows 17.1 / 19.1, x 128 rows 18.5 / 26.5, 30 of 1000 x 64 rows 20.0 / 22.3, 34 of 512 x 32 rows 18.4 / 19.3, 148 of 256 x 64 rows 21.9 / 24.5
+// (of single CTAs not always, 149 of 128 x 32 rows 29.3 / 20.4, 160 of 100 x 128 rows 30.6 / 36.8: no line was measured there).
+// Each CTA merges its share of the rows (0.08 us per row), so where the chip has room the cluster has more CTAs than tiles, until a share is
+// 32 rows at most: one head of 128 tokens x 128 rows 14.3 us by three kernels, 17.8 with one CTA, 14.5 with two, 12.9 with four; of 256 tokens 14.7, 15.0
+// with two, 12.9 with four; 74 heads of 128 tokens x 128 rows 17.3, 18.2, 15.3 with two.  Where each unit has one CTA all the same, three kernels
+// are faster for few units and many rows (their time grows by 0.045 us per unit): 90 heads of 128 tokens x 128 rows 17.9 / 18.4 us, 110 19.0 / 18.5; x 112
+// rows 74 17.1 / 17.3, 90 17.7 / 17.4; x 96 rows 90 17.1 / 16.0.
 static int short_cluster_size(const ScoreShape& s, const TcChunks& ch) {
     const int tiles = (s.Nmax + TILE - 1) / TILE, units = s.B * s.Hkv;
     if (ch.n_chunks > 1 || tiles > SH_MAXC) return 0;
     int C = 1;
     while (C < tiles) C *= 2;
-    return units <= short_clusters(C) ? C : 0;
+    if (units > short_clusters(C)) return 0;
+    while (C < SH_MAXC && s.R > 32 * C && units <= short_clusters(2 * C)) C *= 2;
+    return C == 1 && s.R > 32 && s.R > units + 28 ? 0 : C;
 }
 
 obc_status launch_attention_tc(const ScoreShape& s, TensorView q, TensorView k, TensorView v, void* ws, cudaStream_t stream,

@@ -129,3 +129,17 @@ def test_one_kernel_lengths_below_the_window():
     assert (got["auto"][0] == 0).all() and (got["auto"][2, :, 7:] == 0).all()
     for b in (1, 2):
         _check(got["auto"][b], got["simt"][b], 32, got["simt"][b].max())
+
+
+@pytest.mark.parametrize("units,N,R,path", [(1, 128, 128, "one"), (40, 100, 128, "one"), (3, 256, 72, "one"), (90, 128, 128, "three"), (90, 100, 120, "three"),
+                                            (90, 128, 96, "one"), (148, 128, 128, "one"), (20, 30, 36, "one")])
+def test_many_rows_of_few_tokens(units, N, R, path):
+    """A cluster has more CTAs than tiles where there is room for them, up to 32 rows to merge for each; where there is none, few heads of many rows are
+    left to three kernels.  All heads are the same one, so their scores are, too."""
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the routes of a chip with 148 SMs")
+    case = synth.make_prefill("rows", B=1, Hq=4, Hkv=1, d=128, W=R // 4, N=N, dtype="bf16", seed=R, hh_frac=0.02)
+    got, ran = _kernels(*(x.expand(units, -1, -1, -1).contiguous() for x in H.upload(case)))
+    assert ran == path and torch.equal(got, got[:, :1].expand_as(got))
+    want = H.oracle_scores(case, ["VK"])["VK"]
+    _check(got[0, :1].cpu().numpy(), want, R, np.abs(want).max())
