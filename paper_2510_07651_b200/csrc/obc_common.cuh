@@ -180,9 +180,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // whoever asks sets it to all that the device has left for the kernel (a launch still takes only its own size), and a value
 // that was set is never lowered.  What a host thread has seen set is remembered (per kernel and device), so that the calls,
 // about a microsecond of host time per launch, are made once.  More than the device has is refused, as by the call itself.
+// `wide`: clusters of more than 8 CTAs, too.
 template <typename... KArgs>
-inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
-    struct Seen { const void* kernel; int dev; size_t bytes; };
+inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes, bool wide = false) {
+    struct Seen { const void* kernel; int dev; size_t bytes; bool wide; };
     constexpr unsigned kSlots = 32;
     thread_local Seen seen[kSlots] = {};
     int dev = 0;
@@ -193,7 +194,8 @@ inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
     for (unsigned i = 0; i < kSlots; ++i) {
         Seen& s = seen[(first + i) % kSlots];
         if (s.kernel == (const void*)kernel && s.dev == dev) {
-            if (s.bytes >= bytes) return cudaSuccess;
+            if (s.bytes >= bytes && (s.wide || !wide)) return cudaSuccess;
+            wide |= s.wide;
             at = &s;
             break;
         }
@@ -206,7 +208,8 @@ inline cudaError_t allow_smem(void (*kernel)(KArgs...), size_t bytes) {
     const size_t all = (size_t)optin > fa.sharedSizeBytes ? (size_t)optin - fa.sharedSizeBytes : 0;
     if (bytes > all) return cudaErrorInvalidValue;
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)all);
-    if (e == cudaSuccess) *at = Seen{(const void*)kernel, dev, all};
+    if (e == cudaSuccess && wide) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e == cudaSuccess) *at = Seen{(const void*)kernel, dev, all, wide};
     return e;
 }
 

@@ -2252,30 +2252,28 @@ static size_t tc_partial_bytes(const ScoreShape& s) {
 
 size_t tc_workspace_bytes(const ScoreShape& s) { return make_tc_plan(s).bytes + tc_partial_bytes(s); }
 
-// How many clusters of 2, 4, 8 and 16 CTAs of tc_short_kernel the current device runs at once, asked once per host thread and device
+// How many clusters of 2, 4, 8 or 16 CTAs of tc_short_kernel the current device runs at once, asked once per host thread and device (the first
+// kDevices of them); a query that fails is not remembered
 static int short_clusters(int C) {
     if (C == 1) return sm_count();
-    thread_local struct { int dev, of[4]; } seen{-1, {}};
-    int dev = -1;
+    constexpr int kDevices = 16;
+    thread_local struct { bool known; int n; } seen[kDevices][4] = {};
+    int dev = -1, n = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (dev != seen.dev) {
-        const auto kernel = tc_short_kernel<OBC_VAR_VK, false, false>;             // (one CTA per SM, whatever the instantiation)
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.blockDim = dim3(kThreadsShort); cfg.attrs = attr; cfg.numAttrs = 1; cfg.dynamicSmemBytes = kSmemShort;
-        const bool ok = allow_smem(kernel, kSmemShort) == cudaSuccess &&
-                        cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
-        for (int i = 0; i < 4; ++i) {
-            attr[0].val.clusterDim.x = 2u << i;
-            cfg.gridDim = dim3(2u << i);
-            if (!ok || cudaOccupancyMaxActiveClusters(&seen.of[i], kernel, &cfg) != cudaSuccess) seen.of[i] = 0;
-        }
+    const int at = C == 2 ? 0 : C == 4 ? 1 : C == 8 ? 2 : 3;
+    if (dev < kDevices && seen[dev][at].known) return seen[dev][at].n;
+    const auto kernel = tc_short_kernel<OBC_VAR_VK, false, false>;                 // (one CTA per SM, whatever the instantiation)
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.gridDim = dim3((unsigned)C); cfg.blockDim = dim3(kThreadsShort); cfg.attrs = attr; cfg.numAttrs = 1; cfg.dynamicSmemBytes = kSmemShort;
+    if (allow_smem(kernel, kSmemShort, true) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
         (void)cudaGetLastError();
-        seen.dev = dev;
+        return 0;
     }
-    return seen.of[C == 2 ? 0 : C == 4 ? 1 : C == 8 ? 2 : 3];
+    if (dev < kDevices) seen[dev][at] = {true, n};
+    return n;
 }
 // Cluster size for a call that one kernel serves (tc_short_kernel), or 0: up to 128 window rows, a tile per CTA, all units side by side.
 // With a second wave of clusters three kernels are the faster ones, us three / one: 8 heads of 2048 x 32 rows 17.2 / 22.9, x 128 rows 19.0 / 27.4, 16 of
@@ -2309,6 +2307,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     char* wsb = (char*)ws;
     const int units = s.B * s.Hkv;
     const bool hilo = tc_hilo(s);
+    const int short_c = given || attention_only ? 0 : short_cluster_size(s, ch);
     CUtensorMap mq, mo, mk, mv;
     {
         const uint64_t qd[2] = {(uint64_t)kD, (uint64_t)s.B * s.Hq * s.W};
@@ -2320,8 +2319,8 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
                                 (uint64_t)(s.B > 1 ? k.sb : (s.Hkv > 1 ? k.sh * s.Hkv : k.st * s.Nmax)) * 2};
         const uint64_t vs[3] = {(uint64_t)v.st * 2, (uint64_t)(s.Hkv > 1 ? v.sh : v.st * s.Nmax) * 2,
                                 (uint64_t)(s.B > 1 ? v.sb : (s.Hkv > 1 ? v.sh * s.Hkv : v.st * s.Nmax)) * 2};
-        if (!make_map(&mq, q.ptr, 2, qd, qs, (uint32_t)ch.chunk_rows) ||
-            !make_map(&mo, wsb + plan.off_obf, 2, od, os, (uint32_t)(ch.chunk_rows * plan.want_obf)) ||
+        if ((!short_c && (!make_map(&mq, q.ptr, 2, qd, qs, (uint32_t)ch.chunk_rows) ||
+                          !make_map(&mo, wsb + plan.off_obf, 2, od, os, (uint32_t)(ch.chunk_rows * plan.want_obf)))) ||
             !make_map(&mk, k.ptr, 4, kd, ks, TILE) || !make_map(&mv, v.ptr, 4, kd, vs, TILE)) {
             set_last_cuda_error((int)cudaErrorInvalidValue);
             return OBC_ERR_CUDA;
@@ -2332,7 +2331,6 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
     // Smaller caches keep the default policy, so that pass 2 finds in L2 what pass 1 read.
     const bool l2_stream = ch.n_chunks == 1 && !given &&
         (double)units * s.Nmax * kD * 2 * 2 > 0.75 * (double)l2_bytes();
-    const int short_c = given || attention_only ? 0 : short_cluster_size(s, ch);
     if (short_c) {
         // everything in one kernel (below)
     } else if (given) {   // the caller's O and LSE take the place of pass 1 + combine; pass 2 computes the value norms itself
@@ -2400,8 +2398,7 @@ obc_status launch_score_tc(const ScoreShape& s, TensorView q, TensorView k, Tens
         CUtensorMap ms;
         if (!map_queries(&ms, ch.chunk_rows)) { set_last_cuda_error((int)cudaErrorInvalidValue); return OBC_ERR_CUDA; }
         auto launch_short = [&](auto kernel) -> obc_status {
-            OBC_CUDA_TRY(allow_smem(kernel, kSmemShort));
-            if (short_c > 8) OBC_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+            OBC_CUDA_TRY(allow_smem(kernel, kSmemShort, short_c > 8));
             ProfScope ps("tc_short", stream);
             OBC_CUDA_TRY(launch_pdl(kernel, dim3(units * short_c), dim3(kThreadsShort), kSmemShort, stream, short_c, ms, mk, mv, p, short_c));
             return OBC_OK;
