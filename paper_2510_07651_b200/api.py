@@ -257,7 +257,8 @@ def obc_score_status(workspace) -> None:
 
 def obc_score_kernel_spans(workspace) -> tuple[float, float]:
     """Synchronise; return the device-side extents (us) of the window-statistics kernel and of the fused
-    score kernel since the header words were last zero, and zero them.  (0, 0) on the CUDA-core path."""
+    score kernel since the header words were last zero, and zero them.  (0, 0) on the CUDA-core path; a short
+    cache is scored by one kernel, whose extent is the second figure (the first is 0)."""
     p1, p2 = C.c_double(0), C.c_double(0)
     _check(lib().obc_score_kernel_spans(workspace.data_ptr(), _stream(), C.byref(p1), C.byref(p2)),
            "obc_score_kernel_spans")

@@ -1226,7 +1226,8 @@ __device__ __forceinline__ void zero_rows_from(uint8_t* tile, int row, int first
     fence_async_smem();
 }
 
-// The softmax of one 128-token tile, by the thread that owns the row: logits at tS in, P over their first 64 columns out, the running
+// The softmax of one 128-token tile of pass 1, by the thread that owns the row (tc_short_kernel has one of its own: half a tile per warpgroup,
+// and no running reference, since it has a single tile): logits at tS in, P over their first 64 columns out, the running
 // reference m_used and sum l moved on; `has_o`: the warpgroup's accumulator tO holds earlier tiles and follows the reference.
 __device__ __forceinline__ void softmax_tile(uint32_t tS, uint32_t tO, int nvis, bool masked, float sl2, bool valid, bool low_part, bool has_o,
                                              float& m_used, float& l) {
@@ -1775,8 +1776,8 @@ tc_pass1_kernel(const __grid_constant__ CUtensorMap map_q, const __grid_constant
 
 // =================================================================================================
 // A short cache in one kernel: both passes and the merge between them, for a unit whose tiles have a cluster of CTAs, one
-// tile each (CTAs beyond the tiles, where the cluster has some, take their share of the merge).  As three kernels such a call is mostly their beginnings and ends and the second trip of K and V.  A CTA forms the
-// logits, P and its part of O as pass 1 does; row slices of the partial outputs go to the CTA that owns the slice, which adds them
+// tile each (CTAs beyond the tiles, where the cluster has some, take their share of the merge).  As three kernels such a call is mostly
+// their beginnings and ends and the second trip of K and V.  A CTA forms the logits, P and its part of O as pass 1 does; row slices of the partial outputs go to the CTA that owns the slice, which adds them
 // in the order of the tiles and hands -2 O (HILO: both parts), as the operand image, and the row constants to every CTA of the
 // cluster; the scores of the tile follow from the K and V tiles that are still there (Z from before K and Q made room for the staged O).
 // Partial outputs cross the cluster as bulk copies of runs of staged rows, the merged rows as plain stores; both arrive on the
