@@ -2280,6 +2280,8 @@ static int short_clusters(int C) {
 // With a second wave of clusters three kernels are the faster ones, us three / one: 8 heads of 2048 x 32 rows 17.2 / 22.9, x 128 rows 19.0 / 27.4, 16 of
 // 1024 x 16 rows 17.1 / 19.1, x 128 rows 18.5 / 26.5, 30 of 1000 x 64 rows 20.0 / 22.3, 34 of 512 x 32 rows 18.4 / 19.3, 148 of 256 x 64 rows 21.9 / 24.5
 // (of single CTAs not always, 149 of 128 x 32 rows 29.3 / 20.4, 160 of 100 x 128 rows 30.6 / 36.8: no line was measured there).
+// Within one wave the CTAs without a tile that a power of two leaves do not cost what they look like: 1100 tokens (9 tiles of 16 CTAs) x 16 rows, one head 14.7 / 10.8,
+// 7 heads 16.1 / 11.2, x 128 rows 18.1 / 14.0; 600 (5 of 8) x 128 rows, 14 heads 17.7 / 13.9.
 // Each CTA merges its share of the rows (0.08 us per row), so where the chip has room the cluster has more CTAs than tiles, until a share is
 // 32 rows at most: one head of 128 tokens x 128 rows 14.3 us by three kernels, 17.8 with one CTA, 14.5 with two, 12.9 with four; of 256 tokens 14.7, 15.0
 // with two, 12.9 with four; 74 heads of 128 tokens x 128 rows 17.3, 18.2, 15.3 with two.  Where each unit has one CTA all the same, three kernels
